@@ -128,7 +128,11 @@ struct sft_target_s {
   // symmetric Jacobi scaling for the mixed-precision solve (made on first use):
   // sc = diag(M)^-1/2 and the FP32 values of sc_i M_ij sc_j
   double* sc = nullptr;         // [nv]
-  float* val32s = nullptr;      // [nnz]
+  float* val32s = nullptr;      // [nnz] in CSR order (batched solve)
+  int2* jent = nullptr;         // [nnz] off-diagonal entries as jagged diagonals (solve.cu): column, scaled value
+  double* jval = nullptr;       // [nnz] the same entries of M
+  double* mdiag = nullptr;      // [nv] diag(M)
+  uint16_t* rinfo = nullptr;    // [32 ceil(nv / 32)] row and length of each slice lane
   // limit of the solves' device waits (grid barriers), nanoseconds
   uint64_t wait_ns = 2000000000ull;
 };
@@ -189,7 +193,7 @@ sft_status finish_solve(const SolveLate& late, SolveResult* res);
 sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, double tol, int max_iter,
                       cudaStream_t st, int32_t* d_err, SolveResult* res, int cg_mode = SFT_CG_MIXED,
                       SolveLate* late = nullptr, int warm = 0);
-// S = diag(M)^-1/2 and the FP32 values of S M S on the target (made once, cached)
+// S = diag(M)^-1/2 and the FP32 values of S M S in CSR order on the target (made once, kept)
 sft_status scaled_matrix(sft_target_s* t, cudaStream_t st);
 sft_status weighted_sum(const double* w, const double* u, int64_t n, double* out_host, cudaStream_t st);
 constexpr unsigned kWsumBlocks = 304;

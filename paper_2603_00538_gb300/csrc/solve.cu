@@ -4,7 +4,7 @@
 // does not name its solver). Two kernels:
 //   k_pcg       Jacobi-preconditioned CG in FP64 (cg_mode FP64, and the
 //               allocation-free entry point, which takes any SPD CSR matrix);
-//   k_mixed_cg  mixed-precision iterative refinement (default; see below).
+//   k_mixed     mixed-precision iterative refinement (default; see below).
 //
 // One cooperative (co-resident) kernel runs the whole iteration: no host round
 // trip per step. Each k_pcg iteration has two grid barriers:
@@ -230,14 +230,15 @@ __global__ void __launch_bounds__(kSolveThreads) k_pcg(const int32_t* __restrict
 // its attainable accuracy (~ eps32 cond(A)) is far below the per-cycle target.
 // One refinement cycle:
 //   R (FP64)  r = b - M x, t = S r, ||r||_2 (the stopping test) and ||t||_2;
-//   I         c = t / ||t||_2 rounded to FP32 (unit norm), y = 0;
+//   I         c = t / ||t||_2 rounded to FP32 (unit norm), y_0 = 0, y_1 = c / theta;
 //   inner (FP32) on A y = c to ||c - A y||_2 <= eta, eta about the reduction
 //             the stopping test still needs (between 1e-5 and 1/4): the
-//             Chebyshev iteration over the spectrum interval (the step count
-//             the interval fixes for eta; util.cuh), or CG until its
-//             recurrence residual reaches eta when built with
-//             SFT_MIX_CHEBYSHEV=0;
-//   U (FP64)  x += ||t||_2 S y   (so the new residual is ||t|| S^-1 (c - A y)).
+//             Chebyshev iteration over the spectrum interval in its three-term
+//             form  y_{k+1} = y_k + rho' rho (y_k - y_{k-1}) + (2 rho'/delta) (c - A y_k),
+//             K steps (the count the interval fixes for eta; util.cuh) with
+//             K - 1 products by A (y_1 needs none);
+//   U (FP64)  x += ||t||_2 S y   (so the new residual is ||t|| S^-1 (c - A y)),
+//             in the loop of the last step.
 // A warm start takes x as given (||b|| is then reduced separately first) and
 // skips nothing else: the first R phase checks whether x already converged.
 // The FP64 pipe does one SpMV per cycle (2 to 3 cycles) instead of one per
@@ -247,393 +248,607 @@ __global__ void __launch_bounds__(kSolveThreads) k_pcg(const int32_t* __restrict
 // 0.71 / 0.68 ms on the 1.0 M-row 2D / 0.5 M-row 3D systems, 3e-6 and 1e-6
 // 0.74 / 0.71 ms: deeper FP32 solves cost more iterations than the extra
 // refinement cycle they save)
-#ifndef SFT_MIX_ETA_FLOOR
-#define SFT_MIX_ETA_FLOOR 1e-5f
-#endif
-constexpr float kEtaFloor = SFT_MIX_ETA_FLOOR;
-#ifndef SFT_MIX_ROWS_PER_THREAD
-#define SFT_MIX_ROWS_PER_THREAD 3
-#endif
+constexpr float kEtaFloor = 1e-5f;
 
+// Off-diagonal entries of A for the FP32 steps (A's diagonal is 1): rows in
+// slices of 32, each slice's rows sorted by length (longest first) over the
+// lanes of a warp, entry q of the rows that have one stored side by side
+// (jagged diagonals). A warp's load of entry q is one contiguous read with no
+// padding, and the lanes that have it are a prefix, so its place follows from
+// a ballot. Slice s starts at row_ptr[32 s]; rinfo[32 s + lane] = the lane's
+// row in the slice (5 bits) | its off-diagonal count << 5.
+constexpr int kSlice = 32;
+
+// team of blocks that works on one system
+enum : int { kTeamBlock = 0, kTeamCluster = 1, kTeamGrid = 2 };
 
 struct MixCtl {
-  GridBarrier bar;
+  uint32_t arrived;      // grid barrier: arrivals so far (never reset)
   int32_t err;
+  int32_t late[2];       // cluster barriers that overran the wait limit, by parity
   int32_t cycles;
   int32_t iters[kMaxFields];
-  double rel[kMaxFields];
   int32_t conv[kMaxFields];
+  double rel[kMaxFields];
 };
 
+// Barrier over the team with the limit wait_ns on the wait; false when a wait
+// expired (the caller returns). The grid's is one counter that only grows:
+// a release reduction by one thread per block, then acquire polls until
+// phase x blocks have arrived (no reset and no generation word on the way).
+// The cluster's is the hardware barrier, which cannot be left early: an
+// overrun is noted for the next barrier's parity, after which every block
+// sees the same word and leaves.
+template <int TEAM>
+__device__ __forceinline__ bool team_sync(MixCtl* ctl, unsigned nb, unsigned& phase, uint64_t wait_ns) {
+  if constexpr (TEAM == kTeamBlock) {
+    __syncthreads();
+    return true;
+  } else if constexpr (TEAM == kTeamCluster) {
+    __shared__ int ok;
+    ++phase;
+    uint64_t t0 = 0;
+    if (threadIdx.x == 0) t0 = globaltimer_ns();
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (threadIdx.x == 0) {
+      ok = *reinterpret_cast<volatile int32_t*>(&ctl->late[(phase - 1) & 1]) == 0;
+      if (globaltimer_ns() - t0 > wait_ns) {
+        *reinterpret_cast<volatile int32_t*>(&ctl->late[phase & 1]) = 1;
+        set_error(&ctl->err, DEV_BARRIER_TIMEOUT);
+      }
+    }
+    __syncthreads();
+    return ok != 0;
+  } else {
+    __shared__ int ok;
+    ++phase;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      ok = 1;
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->arrived) : "memory");
+      const uint32_t want = phase * nb;
+      const uint64_t t0 = globaltimer_ns();
+      for (;;) {
+        const int32_t e = *reinterpret_cast<volatile int32_t*>(&ctl->err);
+        uint32_t got;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&ctl->arrived) : "memory");
+        if ((int32_t)(got - want) >= 0) break;
+        if (e != 0) { ok = 0; break; }
+        if (globaltimer_ns() - t0 > wait_ns) {
+          set_error(&ctl->err, DEV_BARRIER_TIMEOUT);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    __syncthreads();
+    return ok != 0;
+  }
+}
+
+// a row's NR interleaved FP32 values
 template <int NR>
-__device__ __forceinline__ void block_partials_d(const double (&v)[NR][2], int nrhs, double* part) {
-  __shared__ double sh[kSolveThreads / 32][NR][2];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void ld_row(const float* p, float (&v)[NR]) {
+  if constexpr (NR == 1) {
+    v[0] = *p;
+  } else if constexpr (NR == 2) {
+    const float2 a = *reinterpret_cast<const float2*>(p);
+    v[0] = a.x; v[1] = a.y;
+  } else {
 #pragma unroll
-  for (int f = 0; f < NR; ++f) {
-    if (f >= nrhs) break;
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const double w = warp_sum<double>(v[f][c]);
-      if (lane == 0) sh[warp][f][c] = w;
+    for (int q = 0; q < NR; q += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(p + q);
+      v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
     }
   }
-  __syncthreads();
-  if (threadIdx.x < nrhs * 2) {
-    const int f = threadIdx.x >> 1, c = threadIdx.x & 1;
-    double s = 0.0;
-    for (int w = 0; w < kSolveThreads / 32; ++w) s += sh[w][f][c];
-    part[((int64_t)blockIdx.x * nrhs + f) * 2 + c] = s;
+}
+template <int NR>
+__device__ __forceinline__ void st_row(float* p, const float (&v)[NR]) {
+  if constexpr (NR == 1) {
+    *p = v[0];
+  } else if constexpr (NR == 2) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < NR; q += 4) *reinterpret_cast<float4*>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
   }
-  __syncthreads();
 }
 
-template <int NR>
-__device__ __forceinline__ void block_partials_f(const float (&v)[NR], int nrhs, float* part) {
-  __shared__ float sh[kSolveThreads / 32][NR];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Where a block keeps the Chebyshev iterates y. kTeamBlock: all in its shared
+// memory. kTeamCluster: each block's rows in its shared memory, read by the
+// others through the cluster's distributed shared memory (an L2 round trip
+// costs about three times as much: 4.0 k cycles per step through L2 against
+// 1.3 k). kTeamGrid with OWN: the block's rows in its shared memory and a
+// copy in global memory for the other blocks; without OWN (more rows than
+// fit): global memory only.
+template <int TEAM, bool OWN>
+struct YRef {
+  float* sm;           // [2][rows][NR] own rows (shared)
+  const float* glob;   // the current y in global memory (grid)
+  int64_t r0;
+  int rows;            // rows of a block
+  int NRv;
+
+  // column -> reference kept in an entry
+  __device__ __forceinline__ int translate(int col) const {
+    if constexpr (TEAM == kTeamBlock) {
+      return col;
+    } else if constexpr (TEAM == kTeamCluster) {
+      const uint32_t rank = (uint32_t)col / (uint32_t)rows, loc = (uint32_t)col - rank * (uint32_t)rows;
+      uint32_t addr = (uint32_t)__cvta_generic_to_shared(sm) + loc * (uint32_t)NRv * 4u;
+      asm("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(addr) : "r"(rank));
+      return (int)addr;
+    } else if constexpr (OWN) {
+      const int64_t l = col - r0;
+      return l >= 0 && l < rows ? (int)l : ~col;
+    } else {
+      return col;
+    }
+  }
+};
+
+// a row's NR interleaved values of the current y by its reference; `cur` is
+// the current half of the own rows (shared memory), `half` its byte offset
+template <int NR, int TEAM, bool OWN>
+__device__ __forceinline__ void ld_y(const float* cur, uint32_t half, const float* glob, int ref, float (&v)[NR]) {
+  if constexpr (TEAM == kTeamBlock) {
+    ld_row<NR>(cur + ref * NR, v);
+  } else if constexpr (TEAM == kTeamCluster) {
+    const uint32_t ad = (uint32_t)ref + half;
+    if constexpr (NR == 1) {
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v[0]) : "r"(ad));
+    } else if constexpr (NR == 2) {
+      asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(ad));
+    } else {
 #pragma unroll
-  for (int f = 0; f < NR; ++f) {
-    if (f >= nrhs) break;
-    const float w = warp_sum<float>(v[f]);
-    if (lane == 0) sh[warp][f] = w;
+      for (int q = 0; q < NR; q += 4)
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v[q]), "=f"(v[q + 1]), "=f"(v[q + 2]), "=f"(v[q + 3])
+                     : "r"(ad + 4u * q));
+    }
+  } else if constexpr (OWN) {
+    if (ref >= 0) ld_row<NR>(cur + ref * NR, v);
+    else ld_row<NR>(glob + (int64_t)(~ref) * NR, v);
+  } else {
+    // written by other blocks before the last barrier: plain loads (cached in
+    // L1, where neighbouring rows share the lines)
+    ld_row<NR>(glob + (int64_t)ref * NR, v);
   }
-  __syncthreads();
-  if (threadIdx.x < nrhs) {
-    float s = 0.f;
-    for (int w = 0; w < kSolveThreads / 32; ++w) s += sh[w][threadIdx.x];
-    part[(int64_t)blockIdx.x * nrhs + threadIdx.x] = s;
-  }
-  __syncthreads();
 }
 
-// sum the FP32 partials [nblocks][nrhs] in a fixed order (identical in all blocks)
-template <int NR>
-__device__ __forceinline__ void reduce_partials_f(const float* part, int nblocks, int nrhs, float* sh_tot) {
-  __shared__ float shw[kSolveThreads / 32][NR];
-  float acc[NR];
+// w += (A - I) y for the lane's row of a slice: `len` entries, the slice's
+// longest row has `maxlen`. U entries at a time, so U gathers are in flight.
+template <int NR, int TEAM, bool OWN, bool HELD>
+__device__ __forceinline__ void slice_product(const int2* ent, const YRef<TEAM, OWN>& Y, const float* cur, uint32_t half,
+                                              int len, int maxlen, int lane, float (&w)[NR]) {
+  constexpr int U = NR <= 2 ? 8 : 4;
+  const int2* e0 = ent + lane;
+  for (int q = 0; q < maxlen; q += U) {
+    int2 e[U];
+    float g[U][NR];
 #pragma unroll
-  for (int f = 0; f < NR; ++f) acc[f] = 0.f;
-  for (int bidx = threadIdx.x; bidx < nblocks; bidx += blockDim.x) {
-    const float* pb = part + (int64_t)bidx * nrhs;
+    for (int u = 0; u < U; ++u) {
+      const bool has = len > q + u;
+      e[u] = make_int2(0, 0);
+      if (has) e[u] = *e0;
+      e0 += __popc(__ballot_sync(0xffffffffu, has));
+    }
 #pragma unroll
-    for (int f = 0; f < NR; ++f)
-      if (f < nrhs) acc[f] += __ldcg(pb + f);
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int u = 0; u < U; ++u) {
 #pragma unroll
-  for (int f = 0; f < NR; ++f) {
-    if (f >= nrhs) break;
-    const float w = warp_sum<float>(acc[f]);
-    if (lane == 0) shw[warp][f] = w;
+      for (int f = 0; f < NR; ++f) g[u][f] = 0.f;
+      if (len > q + u) ld_y<NR, TEAM, OWN>(cur, half, Y.glob, HELD ? e[u].x : Y.translate(e[u].x), g[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int f = 0; f < NR; ++f) w[f] = __fmaf_rn(__int_as_float(e[u].y), g[u][f], w[f]);
   }
-  __syncthreads();
-  if (threadIdx.x < nrhs) {
-    float t = 0.f;
-    for (int w = 0; w < kSolveThreads / 32; ++w) t += shw[w][threadIdx.x];
-    sh_tot[threadIdx.x] = t;
-  }
-  __syncthreads();
 }
 
-// NR: compile-time bound on the number of right-hand sides (nrhs <= NR).
-// Four resident blocks per SM (64 registers a thread): 0.69 ms on the 1.0 M-row
-// 2D system against 0.78 ms with the compiler's own register choice (48 and
-// spills). Interleaving 2, 4 or 8 of a thread's rows (overlapping their load
-// chains) measured no better (0.69 / 0.71 / 0.91 ms).
+// Sum of V values (a power of two up to 32) over the lanes of a warp: at each
+// of the first log2 V steps a lane hands over half of its values and keeps
+// the other half, so the V sums take V - 1 + 5 - log2 V additions instead of
+// 5 V (an FP64 warp instruction occupies this GPU's FP64 pipe for 16 cycles).
+// Lane l returns the sum of value l / (32 / V).
+template <int V>
+__device__ __forceinline__ double warp_sums(double (&v)[V], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int h = V / 2; h >= 1; h >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double give = up ? v[k] : v[k + h];
+      const double keep = up ? v[k + h] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+    o >>= 1;
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
+struct MixArgs {
+  const int32_t* rp;      // row starts of M
+  const int2* jent;       // off-diagonal entries as jagged diagonals: {column, FP32 value bits of A},
+  const double* jval;     //   the same entries of M,
+  const double* mdiag;    //   its diagonal,
+  const uint16_t* rinfo;  //   rows and lengths of the slices' lanes
+  const double* sc;       // diag(M)^-1/2
+  int64_t n;
+  int nrhs;
+  const double* b;        // [nrhs][n]
+  double* x;
+  double* t;              // [nrhs][n]
+  float* ya;              // [n][NR] (grid)
+  float* yb;
+  float* c;               // [n][NR], when it is not held in shared memory
+  double* partd;          // [2][2 nrhs][blocks]: the warm start's, the cycles'
+  MixCtl* ctl;
+  double tol;
+  int max_iter;
+  int warm;
+  uint64_t wait_ns;
+  float lmax;
+  int spb;                // slices per block
+  int cap;                // entries held in shared memory
+  int c_smem;             // c held in shared memory
+  int r_smem;             // rinfo held in shared memory
+};
+
+// blocks hold as much of their part of A as fits in shared memory for the
+// whole solve: bytes of it
+constexpr uint32_t kMixSmemMax = 212u * 1024u;
+constexpr int kMaxStaged = 1024;   // slices a block may hold
 template <int NR>
-__global__ void __launch_bounds__(kSolveThreads, 4) k_mixed_cg(
-    const int32_t* __restrict__ rp, const int32_t* __restrict__ col, const double* __restrict__ val,
-    const float* __restrict__ aval, const double* __restrict__ sc, int64_t n, int nrhs,
-    const double* __restrict__ b, double* x, double* t, float* r, float* p, float* q, float* y, double* partd,
-    float* partf, MixCtl* ctl, double tol, int max_iter, int warm, uint64_t wait_ns, float lmax) {
-  __shared__ double totd[kMaxFields * 2];
-  __shared__ float totf[NR];
-  __shared__ double bnorm[NR], prev[NR], sig[NR], isig[NR];
-  __shared__ float eta2[NR], rr[NR], alpha[NR], beta[NR];
-  __shared__ int live[NR], act[NR], conv[NR], ksteps[NR], stop;
-  const ChebCoef ch = cheb_coef(lmax);
+constexpr int kMixThreads = NR <= 2 ? 1024 : 512;
+
+// One block per SM. Each block owns spb consecutive slices of rows for the
+// whole solve and keeps what it can of them in shared memory: its part of A,
+// its rows of y, c and rinfo. So a step reads from L2 only the neighbours'
+// rows of y and the part of A that does not fit (none up to about 0.6 M rows
+// in 2D, 0.25 M in 3D).
+// What bounds it: small systems the chain of barrier, gather and row update
+// (a step takes 1.8 k cycles on a block, 3.1 k on a cluster, 5 k on the
+// grid), large ones the shared-memory loads and issue of the steps (12 us a
+// step at 1.0 M rows) and the FP64 pipe of the residual (38 us a cycle there
+// against 25 of pure FP64 work). Kernel time, before (grid of 4 blocks per SM
+// over CSR rows, all vectors in L2) and now: 1.0 M rows 2D 648 -> 431 us,
+// 0.51 M 3D 574 -> 429, 0.37 M 2D 350 -> 177, 10 k 2D 179 -> 62, 784 2D
+// 140 -> 46, 227 k 3D with 8 fields 1,739 -> 618.
+template <int NR, int TEAM, bool OWN>
+__global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
+  constexpr int T = kMixThreads<NR>, W = T / 32, V = 2 * NR;
+  constexpr bool YSM = TEAM != kTeamGrid || OWN;   // own rows of y in shared memory
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ int32_t s_off[kMaxStaged + 1];     // start of each held slice in ent
+  __shared__ double shw[W][V];
+  __shared__ double shtot[V];
+  __shared__ double bn2[NR], prev2[NR], sig[NR], isig[NR];
+  __shared__ int live[NR], act[NR], conv[NR], ks[NR], itf[NR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned nb = gridDim.x;
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int f = 0; f < NR; ++f) {
-      live[f] = f < nrhs;
-      act[f] = 0;
-      conv[f] = 0;
+  const int64_t n = a.n;
+  const int nrhs = NR == 1 ? 1 : a.nrhs;
+  const int64_t s0 = (int64_t)blockIdx.x * a.spb;
+  const int64_t nslices = (n + kSlice - 1) / kSlice;
+  const int nsl = (int)(s0 >= nslices ? 0 : (nslices - s0 < a.spb ? nslices - s0 : a.spb));
+  const int64_t r0 = s0 * kSlice;
+  const int64_t r1 = r0 + (int64_t)nsl * kSlice < n ? r0 + (int64_t)nsl * kSlice : n;
+  const int rows = a.spb * kSlice;
+  float* const ysm = reinterpret_cast<float*>(dsm);   // [2][rows][NR]
+  int2* const ent = reinterpret_cast<int2*>(ysm + (YSM ? (int64_t)2 * rows * NR : 0));
+  float* const csm = reinterpret_cast<float*>(ent + a.cap);
+  uint16_t* const rsm = reinterpret_cast<uint16_t*>(csm + (a.c_smem ? (int64_t)rows * NR : 0));
+  float* const cg = a.c + r0 * NR;
+  MixCtl* ctl = a.ctl;
+  unsigned phase = 0;
+  const ChebCoef ch = cheb_coef(a.lmax);
+  const float inv_acosh = 1.f / acoshf(ch.s1);
+  YRef<TEAM, OWN> Y;
+  Y.sm = ysm;
+  Y.glob = a.ya;
+  Y.r0 = r0;
+  Y.rows = rows;
+  Y.NRv = NR;
+
+  // hold rinfo and the leading slices of A
+  if (a.r_smem)
+    for (int i = tid; i < nsl * kSlice; i += T) rsm[i] = a.rinfo[r0 + i];
+  const int ncand = nsl < kMaxStaged ? nsl : kMaxStaged;
+  for (int sl = warp; sl < ncand; sl += W) {
+    const int cnt = __reduce_add_sync(0xffffffffu, a.rinfo[r0 + sl * kSlice + lane] >> 5);
+    if (lane == 0) s_off[sl + 1] = cnt;
+  }
+  if (tid == 0) s_off[0] = 0;
+  if (tid < NR) {
+    live[tid] = tid < nrhs;
+    act[tid] = 0;
+    conv[tid] = 0;
+    itf[tid] = 0;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int base = 0;
+    for (int q = 0; q < ncand; q += 32) {
+      const int k = q + lane;
+      const int v = k < ncand ? s_off[k + 1] : 0;
+      const int inc = warp_inclusive_scan<int>(v, lane) + base;
+      if (k < ncand) s_off[k + 1] = inc;
+      base = __shfl_sync(0xffffffffu, inc, 31);
     }
   }
   __syncthreads();
-  int it = 0, cyc = 0;
-  if (warm) {
+  int nheld = 0;
+  for (int k = 0; k < ncand; k += 32) {  // slices whose entries all fit (a prefix)
+    const bool fits = k + lane < ncand && s_off[k + lane + 1] <= a.cap;
+    nheld += __popc(__ballot_sync(0xffffffffu, fits));
+  }
+  for (int sl = warp; sl < nheld; sl += W) {
+    const int o = s_off[sl], cnt = s_off[sl + 1] - o;
+    const int2* src = a.jent + __ldg(a.rp + r0 + sl * kSlice);
+#pragma unroll 4
+    for (int k = lane; k < cnt; k += 32) {
+      int2 e = __ldg(src + k);
+      e.x = Y.translate(e.x);
+      ent[o + k] = e;
+    }
+  }
+  __syncthreads();
+
+  // per-block partial sums -> global; after the barrier every block adds all
+  // of them in the same order (totals in shtot)
+  auto put_partials = [&](double (&v)[V], double* part) {
+    const double ws = warp_sums<V>(v, lane);
+    if (lane % (32 / V) == 0) shw[warp][lane / (32 / V)] = ws;
+    __syncthreads();
+    if (warp < 2 * nrhs) {
+      const double s = warp_sum<double>(lane < W ? shw[lane][warp] : 0.0);
+      if (lane == 0) part[(int64_t)warp * nb + blockIdx.x] = s;
+    }
+  };
+  auto get_totals = [&](const double* part) {
+    if (warp < 2 * nrhs) {
+      double s = 0.0;
+      for (int k = lane; k < (int)nb; k += 32) s += __ldcg(part + (int64_t)warp * nb + k);
+      s = warp_sum<double>(s);
+      if (lane == 0) shtot[warp] = s;
+    }
+    __syncthreads();
+  };
+
+  if (a.warm) {
     // warm start from the x given: ||b|| for the stopping test first
-    double v[NR][2];
+    double v[V];
 #pragma unroll
-    for (int f = 0; f < NR; ++f) v[f][0] = v[f][1] = 0.0;
-    for (int64_t i = tid; i < n; i += nthreads) {
+    for (int f = 0; f < V; ++f) v[f] = 0.0;
+    for (int64_t i = r0 + tid; i < r1; i += T)
 #pragma unroll
       for (int f = 0; f < NR; ++f) {
         if (f >= nrhs) break;
-        const double bi = b[(int64_t)f * n + i];
-        v[f][0] += bi * bi;
+        const double bi = a.b[(int64_t)f * n + i];
+        v[2 * f] += bi * bi;
       }
-    }
-    block_partials_d<NR>(v, nrhs, partd);
-    if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
-    reduce_partials(partd, nb, nrhs, totd);
-    if (threadIdx.x == 0)
-      for (int f = 0; f < nrhs; ++f) bnorm[f] = sqrt(totd[2 * f]);
+    put_partials(v, a.partd);
+    if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
+    get_totals(a.partd);
+    if (tid < nrhs) bn2[tid] = shtot[2 * tid];
     __syncthreads();
   }
+
+  double* const part = a.partd + (int64_t)nb * 2 * nrhs;
+  int it = 0, cyc = 0;
   for (;; ++cyc) {
     // R: true residual in FP64 (x = 0 in the first cycle unless warm)
-    double v[NR][2];
+    double v[V];
 #pragma unroll
-    for (int f = 0; f < NR; ++f) v[f][0] = v[f][1] = 0.0;
-    for (int64_t i = tid; i < n; i += nthreads) {
-      const double si = sc[i];
-      int32_t k0 = 0, k1 = 0;
-      if (cyc > 0 || warm) {
-        k0 = __ldg(rp + i);
-        k1 = __ldg(rp + i + 1);
-      }
+    for (int f = 0; f < V; ++f) v[f] = 0.0;
+    auto residual = [&](int64_t i, const double (&s)[NR], bool zero_x) {
+      const double si = a.sc[i];
 #pragma unroll
       for (int f = 0; f < NR; ++f) {
         if (f >= nrhs) break;
         if (!live[f]) continue;
-        const int64_t o = (int64_t)f * n;
-        double s = 0.0;
-        // x was written by other blocks before the grid barrier (plain loads)
-        for (int32_t k = k0; k < k1; ++k) s += __ldg(val + k) * x[o + __ldg(col + k)];
-        if (cyc == 0 && !warm) x[o + i] = 0.0;
-        const double ri = b[o + i] - s;
+        const int64_t o = (int64_t)f * n + i;
+        if (zero_x) a.x[o] = 0.0;
+        const double ri = a.b[o] - s[f];
         const double ti = si * ri;
-        t[o + i] = ti;
-        v[f][0] += ri * ri;
-        v[f][1] += ti * ti;
+        a.t[o] = ti;
+        v[2 * f] += ri * ri;
+        v[2 * f + 1] += ti * ti;
       }
-    }
-    block_partials_d<NR>(v, nrhs, partd);
-    if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
-    reduce_partials(partd, nb, nrhs, totd);
-    if (threadIdx.x == 0) {
-      bool any = false;
-      for (int f = 0; f < nrhs; ++f) {
-        act[f] = 0;
-        if (!live[f]) continue;
-        const double rn = sqrt(totd[2 * f]), tn = sqrt(totd[2 * f + 1]);
-        if (cyc == 0 && !warm) bnorm[f] = rn;
-        if (blockIdx.x == 0) {
-          ctl->rel[f] = bnorm[f] > 0.0 ? rn / bnorm[f] : 0.0;
-          ctl->iters[f] = it;
-        }
-        if (rn <= tol * bnorm[f]) {
-          live[f] = 0;
-          conv[f] = 1;
-          continue;
-        }
-        // a cycle that did not halve the residual (FP64 rounding floor) or a
-        // residual on rows without diagonal ends the field unconverged
-        if ((cyc > 0 && rn > 0.5 * prev[f]) || !(tn > 0.0)) {
-          live[f] = 0;
-          continue;
-        }
-        prev[f] = rn;
-        sig[f] = tn;
-        isig[f] = 1.0 / tn;
-        const double e = fmin(0.25, fmax((double)kEtaFloor, 0.1 * tol * bnorm[f] / rn));
-        eta2[f] = (float)(e * e);
-        ksteps[f] = cheb_steps(e, ch.s1);
-        act[f] = 1;
-        any = true;
-      }
-      stop = !any || it >= max_iter;
-    }
-    __syncthreads();
-    if (stop) break;
-
-    if constexpr (kMixCheb) {
-      // I: c = t / ||t|| in FP32, r = c, y = 0, d = c / theta (in p)
-      const float ith = 1.f / ch.theta;
-      for (int64_t i = tid; i < n; i += nthreads) {
+    };
+    if (cyc > 0 || a.warm) {
+      for (int sl = warp; sl < nsl; sl += W) {
+        const int64_t rb = r0 + (int64_t)sl * kSlice;
+        const int ri = a.r_smem ? rsm[sl * kSlice + lane] : a.rinfo[rb + lane];
+        const int64_t i = rb + (ri & 31);
+        const int len = ri >> 5;
+        const int maxlen = __shfl_sync(0xffffffffu, len, 0);
+        double s[NR];
 #pragma unroll
-        for (int f = 0; f < NR; ++f) {
-          if (f >= nrhs) break;
-          if (!act[f]) continue;
-          const int64_t k = (int64_t)f * n + i;
-          const float ci = (float)(t[k] * isig[f]);
-          r[k] = ci;
-          y[k] = 0.f;
-          p[k] = ci * ith;
+        for (int f = 0; f < NR; ++f) s[f] = 0.0;
+        // x was written by other blocks before the barrier (plain loads)
+        if (i < n) {
+          const double d = a.mdiag[i];
+#pragma unroll
+          for (int f = 0; f < NR; ++f)
+            if (f < nrhs) s[f] = d * a.x[(int64_t)f * n + i];
         }
-      }
-      if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
-      // Chebyshev steps; d alternates between p and q (the SpMV of a step
-      // reads the d every block wrote in the step before)
-      float rho = 1.f / ch.s1;
-      const float idl = 2.f / ch.delta;
-      auto steps_left = [&](int s) {  // fields that take step s
-        unsigned mm = 0u;
+        const int32_t base = __ldg(a.rp + rb);
+        const int2* e0 = a.jent + base + lane;
+        const double* m0 = a.jval + base + lane;
+        constexpr int U = NR <= 2 ? 4 : 2;
+        for (int q = 0; q < maxlen; q += U) {
+          int col[U];
+          double m[U];
 #pragma unroll
-        for (int f = 0; f < NR; ++f)
-          if (f < nrhs && act[f] && s < ksteps[f]) mm |= 1u << f;
-        return it < max_iter ? mm : 0u;
-      };
-      for (int s = 0;; ++s) {
-        const unsigned m = steps_left(s);
-        if (!m) break;
-        const float rn1 = 1.f / (2.f * ch.s1 - rho);
-        const float c1 = rn1 * rho, c2 = rn1 * idl;
-        const float* dc = (s & 1) ? q : p;
-        float* dn = (s & 1) ? p : q;
-        for (int64_t i = tid; i < n; i += nthreads) {
-          const int32_t k0 = __ldg(rp + i), k1 = __ldg(rp + i + 1);
-#pragma unroll
-          for (int f = 0; f < NR; ++f) {
-            if (f >= nrhs) break;
-            if (!((m >> f) & 1u)) continue;
-            const int64_t o = (int64_t)f * n;
-            const float* df = dc + o;
-            float w = 0.f;
-            // d was written by other blocks before the grid barrier (plain loads)
-            for (int32_t k = k0; k < k1; ++k) w += __ldg(aval + k) * df[__ldg(col + k)];
-            const float di = df[i];
-            y[o + i] += di;
-            const float ri = r[o + i] - w;
-            r[o + i] = ri;
-            dn[o + i] = c1 * di + c2 * ri;
+          for (int u = 0; u < U; ++u) {
+            const bool has = len > q + u;
+            col[u] = 0;
+            m[u] = 0.0;
+            if (has) {
+              col[u] = __ldg(&e0->x);
+              m[u] = __ldg(m0);
+            }
+            const int step = __popc(__ballot_sync(0xffffffffu, has));
+            e0 += step;
+            m0 += step;
           }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (len > q + u) {
+#pragma unroll
+              for (int f = 0; f < NR; ++f)
+                if (f < nrhs) s[f] += m[u] * a.x[(int64_t)f * n + col[u]];
+            }
         }
-        rho = rn1;
-        ++it;
-        // the next step's SpMV reads the d of other blocks; after the last
-        // step U touches only the thread's own rows, so no barrier
-        if (!steps_left(s + 1)) break;
-        if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
+        if (i < n) residual(i, s, false);
       }
     } else {
-      // I: unit-norm FP32 right-hand side, zero iterate and directions
-      float vf[NR];
+      double s[NR];
 #pragma unroll
-      for (int f = 0; f < NR; ++f) vf[f] = 0.f;
-      for (int64_t i = tid; i < n; i += nthreads) {
-#pragma unroll
-        for (int f = 0; f < NR; ++f) {
-          if (f >= nrhs) break;
-          if (!act[f]) continue;
-          const int64_t k = (int64_t)f * n + i;
-          const float ci = (float)(t[k] * isig[f]);
-          r[k] = ci;
-          y[k] = 0.f;
-          p[k] = 0.f;
-          q[k] = 0.f;
-          vf[f] += ci * ci;
+      for (int f = 0; f < NR; ++f) s[f] = 0.0;
+      for (int64_t i = r0 + tid; i < r1; i += T) residual(i, s, true);
+    }
+    put_partials(v, part);
+    if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
+    get_totals(part);
+    if (tid < nrhs) {
+      const int f = tid;
+      act[f] = 0;
+      ks[f] = 0;
+      if (live[f]) {
+        // tests on the squared norms (no square root or quotient on the way)
+        const double rn2 = shtot[2 * f], tn2 = shtot[2 * f + 1];
+        if (cyc == 0 && !a.warm) bn2[f] = rn2;
+        const double b2 = bn2[f], last2 = prev2[f];
+        prev2[f] = rn2;
+        itf[f] = it;
+        if (rn2 <= a.tol * a.tol * b2) {
+          live[f] = 0;
+          conv[f] = 1;
+        } else if ((cyc > 0 && rn2 > 0.25 * last2) || !(tn2 > 0.0)) {
+          // a cycle that did not halve the residual (FP64 rounding floor) or a
+          // residual on rows without diagonal ends the field unconverged
+          live[f] = 0;
+        } else {
+          const double is = rsqrt(tn2);
+          isig[f] = is;
+          sig[f] = tn2 * is;
+          const float e = fminf(0.25f, fmaxf(kEtaFloor, (float)(0.1 * a.tol) * sqrtf((float)(b2 / rn2))));
+          ks[f] = max(1, (int)ceilf(acoshf(1.f / e) * inv_acosh));
+          act[f] = 1;
         }
-      }
-      block_partials_f<NR>(vf, nrhs, partf);
-      if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
-      reduce_partials_f<NR>(partf, nb, nrhs, totf);
-      if (threadIdx.x == 0)
-        for (int f = 0; f < nrhs; ++f) {
-          rr[f] = totf[f];
-          beta[f] = 0.f;
-        }
-      __syncthreads();
-
-      // CG in FP32 on A y = c
-      for (;;) {
-        bool any = false;
-#pragma unroll
-        for (int f = 0; f < NR; ++f)
-          if (f < nrhs) any = any || act[f];
-        if (!any || it >= max_iter) break;
-        // phase A: w = A r, p = r + beta p, q = w + beta q (= A p), partial (p, q)
-#pragma unroll
-        for (int f = 0; f < NR; ++f) vf[f] = 0.f;
-        for (int64_t i = tid; i < n; i += nthreads) {
-          const int32_t k0 = __ldg(rp + i), k1 = __ldg(rp + i + 1);
-#pragma unroll
-          for (int f = 0; f < NR; ++f) {
-            if (f >= nrhs) break;
-            if (!act[f]) continue;
-            const int64_t o = (int64_t)f * n;
-            const float* rf = r + o;
-            float s = 0.f;
-            // r was written by other blocks before the grid barrier (plain loads)
-            for (int32_t k = k0; k < k1; ++k) s += __ldg(aval + k) * rf[__ldg(col + k)];
-            const float bt = beta[f];
-            const int64_t k = o + i;
-            const float pn = rf[i] + bt * p[k];
-            const float qn = s + bt * q[k];
-            p[k] = pn;
-            q[k] = qn;
-            vf[f] += pn * qn;
-          }
-        }
-        block_partials_f<NR>(vf, nrhs, partf);
-        if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
-        reduce_partials_f<NR>(partf, nb, nrhs, totf);
-        if (threadIdx.x == 0)
-          for (int f = 0; f < nrhs; ++f) alpha[f] = act[f] ? rr[f] / totf[f] : 0.f;
-        __syncthreads();
-        // phase B: y += alpha p, r -= alpha q, partial (r, r)
-#pragma unroll
-        for (int f = 0; f < NR; ++f) vf[f] = 0.f;
-        for (int64_t i = tid; i < n; i += nthreads) {
-#pragma unroll
-          for (int f = 0; f < NR; ++f) {
-            if (f >= nrhs) break;
-            if (!act[f]) continue;
-            const int64_t k = (int64_t)f * n + i;
-            const float a = alpha[f];
-            y[k] += a * p[k];
-            const float ri = r[k] - a * q[k];
-            r[k] = ri;
-            vf[f] += ri * ri;
-          }
-        }
-        block_partials_f<NR>(vf, nrhs, partf);
-        if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
-        reduce_partials_f<NR>(partf, nb, nrhs, totf);
-        ++it;
-        if (threadIdx.x == 0)
-          for (int f = 0; f < nrhs; ++f) {
-            if (!act[f]) continue;
-            const float rn = totf[f];
-            beta[f] = rn / rr[f];
-            rr[f] = rn;
-            if (rn <= eta2[f]) act[f] = 0;
-          }
-        __syncthreads();
       }
     }
+    __syncthreads();
+    // every active field takes the largest step count (more steps only
+    // reduce its residual further)
+    int K = 0;
+#pragma unroll
+    for (int f = 0; f < NR; ++f)
+      if (f < nrhs && act[f] && ks[f] > K) K = ks[f];
+    if (K == 0 || it >= a.max_iter) break;
+    if (K > a.max_iter - it) K = a.max_iter - it;
 
-    // U: x += ||t|| S y for every field that ran this cycle
-    for (int64_t i = tid; i < n; i += nthreads) {
-      const double si = sc[i];
+    // U for one row: x += ||t|| S y
+    auto update_x = [&](int64_t i, const float (&y)[NR]) {
+      const double si = a.sc[i];
 #pragma unroll
       for (int f = 0; f < NR; ++f) {
         if (f >= nrhs) break;
-        if (!live[f]) continue;
-        const int64_t k = (int64_t)f * n + i;
-        x[k] += (sig[f] * si) * (double)y[k];
+        if (act[f]) a.x[(int64_t)f * n + i] += (sig[f] * si) * f2d(y[f]);
+      }
+    };
+    // I: c = t / ||t|| in FP32, y_1 = c / theta
+    const float ith = 1.f / ch.theta;
+    for (int64_t i = r0 + tid; i < r1; i += T) {
+      float c[NR], y[NR];
+#pragma unroll
+      for (int f = 0; f < NR; ++f) {
+        c[f] = 0.f;
+        if (f < nrhs && act[f]) c[f] = (float)(a.t[(int64_t)f * n + i] * isig[f]);
+        y[f] = c[f] * ith;
+      }
+      if (K == 1) {
+        update_x(i, y);
+      } else {
+        st_row<NR>((a.c_smem ? csm : cg) + (i - r0) * NR, c);
+        if constexpr (YSM) st_row<NR>(ysm + (i - r0) * NR, y);
+        if constexpr (TEAM == kTeamGrid) st_row<NR>(a.ya + i * NR, y);
       }
     }
-    if (!grid_sync(&ctl->bar, nb, &ctl->err, wait_ns)) return;
+    if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
+    float rho = 1.f / ch.s1;
+    const float idl = 2.f / ch.delta;
+    for (int k = 1; k < K; ++k) {   // y_{k+1} from y_k and y_{k-1} (whose place it takes)
+      const float rn1 = 1.f / (2.f * ch.s1 - rho);
+      const float c1 = rn1 * rho, c2 = rn1 * idl;
+      const int h = (k & 1) ^ 1;    // half of the buffers that holds y_k
+      const float* cur = ysm + (h ? (int64_t)rows * NR : 0);
+      float* nxt = ysm + (h ? 0 : (int64_t)rows * NR);
+      const uint32_t half = h ? (uint32_t)rows * NR * 4u : 0u;
+      Y.glob = h ? a.yb : a.ya;
+      float* gn = h ? a.ya : a.yb;
+      const bool last = k + 1 == K;
+      for (int sl = warp; sl < nsl; sl += W) {
+        const int64_t rb = r0 + (int64_t)sl * kSlice;
+        const int ri = a.r_smem ? rsm[sl * kSlice + lane] : a.rinfo[rb + lane];
+        const int64_t i = rb + (ri & 31);
+        const int loc = sl * kSlice + (ri & 31);
+        const int len = ri >> 5;
+        const int maxlen = __shfl_sync(0xffffffffu, len, 0);
+        const bool valid = i < n;
+        float c[NR], y0[NR], y1[NR], w[NR];
+#pragma unroll
+        for (int f = 0; f < NR; ++f) c[f] = y0[f] = y1[f] = w[f] = 0.f;
+        if (valid) {
+          if constexpr (YSM) {
+            ld_row<NR>(cur + loc * NR, y1);
+            if (k > 1) ld_row<NR>(nxt + loc * NR, y0);
+          } else {
+            ld_row<NR>(Y.glob + i * NR, y1);
+            if (k > 1) ld_row<NR>(gn + i * NR, y0);
+          }
+          ld_row<NR>((a.c_smem ? csm : cg) + (int64_t)loc * NR, c);
+        }
+        if (sl < nheld) slice_product<NR, TEAM, OWN, true>(ent + s_off[sl], Y, cur, half, len, maxlen, lane, w);
+        else slice_product<NR, TEAM, OWN, false>(a.jent + __ldg(a.rp + rb), Y, cur, half, len, maxlen, lane, w);
+#pragma unroll
+        for (int f = 0; f < NR; ++f) y0[f] = y1[f] + (c1 * (y1[f] - y0[f]) + c2 * (c[f] - (y1[f] + w[f])));
+        if (valid) {
+          if (last) {
+            update_x(i, y0);
+          } else {
+            if constexpr (YSM) st_row<NR>(nxt + loc * NR, y0);
+            if constexpr (TEAM == kTeamGrid) st_row<NR>(gn + i * NR, y0);
+          }
+        }
+      }
+      rho = rn1;
+      if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
+    }
+    it += K;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    ctl->cycles = cyc;
-    for (int f = 0; f < nrhs; ++f) ctl->conv[f] = conv[f];
+  if (blockIdx.x == 0 && tid < nrhs) {
+    if (tid == 0) ctl->cycles = cyc;
+    ctl->iters[tid] = itf[tid];
+    ctl->rel[tid] = bn2[tid] > 0.0 ? sqrt(prev2[tid] / bn2[tid]) : 0.0;
+    ctl->conv[tid] = conv[tid];
   }
 }
 
-// S = diag(M)^-1/2 (0 on a row without diagonal) and the FP32 scaled values
+// S = diag(M)^-1/2 (0 on a row without diagonal)
 __global__ void k_jacobi_sqrt(const double* __restrict__ dinv, int64_t n, double* __restrict__ sc) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     sc[i] = sqrt(dinv[i]);
 }
 
+// FP32 values of S M S in CSR order (the batched solve)
 __global__ void k_scaled_values(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                                 const double* __restrict__ val, const double* __restrict__ sc, int64_t n,
                                 float* __restrict__ out) {
@@ -643,15 +858,98 @@ __global__ void k_scaled_values(const int32_t* __restrict__ rp, const int32_t* _
   }
 }
 
-sft_status scaled_matrix(sft_target_s* t, cudaStream_t st) {
-  if (t->val32s) return SFT_OK;
+// the off-diagonal entries of S M S as jagged diagonals: one warp per slice
+__global__ void k_scaled_slices(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                const double* __restrict__ val, const double* __restrict__ sc, int64_t n,
+                                int64_t nslices, int2* __restrict__ jent, double* __restrict__ jval,
+                                double* __restrict__ mdiag, uint16_t* __restrict__ rinfo) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
+    const int64_t i = s * kSlice + lane;
+    int32_t k0 = 0, k1 = 0;
+    if (i < n) {
+      k0 = __ldg(rp + i);
+      k1 = __ldg(rp + i + 1);
+    }
+    const int mylen = k1 > k0 ? k1 - k0 - 1 : 0;   // a non-empty row has its diagonal
+    // rank of the row by length (longest first, ties by row)
+    int rank = 0;
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+      const int o = __shfl_sync(0xffffffffu, mylen, l);
+      rank += o > mylen || (o == mylen && l < lane);
+    }
+    // the row that lane takes: the inverse of the ranks
+    int row = 0;
+#pragma unroll
+    for (int l = 0; l < 32; ++l)
+      if (__shfl_sync(0xffffffffu, rank, l) == lane) row = l;
+    const int len = __shfl_sync(0xffffffffu, mylen, row);
+    const int32_t q0 = __shfl_sync(0xffffffffu, k0, row), q1 = __shfl_sync(0xffffffffu, k1, row);
+    const int32_t base = __shfl_sync(0xffffffffu, k0, 0);
+    const int maxlen = __shfl_sync(0xffffffffu, len, 0);
+    const int32_t me = (int32_t)(s * kSlice) + row;
+    const double si = len > 0 ? __ldg(sc + me) : 0.0;
+    rinfo[s * kSlice + lane] = (uint16_t)(row | (len << 5));
+    int32_t k = q0;
+    int32_t out = base + lane;
+    double diag = 0.0;
+    for (int q = 0; q < maxlen; ++q) {
+      const bool has = len > q;
+      if (has) {
+        int32_t c = __ldg(col + k);
+        if (c == me) {   // the diagonal is kept apart
+          diag = __ldg(val + k);
+          c = __ldg(col + ++k);
+        }
+        const double m = __ldg(val + k);
+        jent[out] = make_int2(c, __float_as_int((float)(m * si * __ldg(sc + c))));
+        jval[out] = m;
+        ++k;
+      }
+      out += __popc(__ballot_sync(0xffffffffu, has));
+    }
+    if (me < n) {
+      // a diagonal after the row's last off-diagonal entry was not passed
+      if (diag == 0.0 && k < q1) diag = __ldg(val + k);
+      mdiag[me] = diag;
+    }
+  }
+}
+
+static sft_status jacobi_scale(sft_target_s* t, cudaStream_t st) {
+  if (t->sc) return SFT_OK;
   const int64_t n = t->nv;
   SFT_CUDA(dalloc(&t->sc, (size_t)n, st));
-  SFT_CUDA(dalloc(&t->val32s, (size_t)std::max<int64_t>(t->nnz, 1), st));
   const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
   ::sft::note_launch(), k_jacobi_sqrt<<<nb, 256, 0, st>>>(t->dinv, n, t->sc);
   SFT_CUDA(cudaGetLastError());
+  return SFT_OK;
+}
+
+sft_status scaled_matrix(sft_target_s* t, cudaStream_t st) {
+  if (t->val32s) return SFT_OK;
+  const int64_t n = t->nv;
+  if (sft_status r = jacobi_scale(t, st)) return r;
+  SFT_CUDA(dalloc(&t->val32s, (size_t)std::max<int64_t>(t->nnz, 1), st));
+  const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
   ::sft::note_launch(), k_scaled_values<<<nb, 256, 0, st>>>(t->row_ptr, t->col, t->val, t->sc, n, t->val32s);
+  SFT_CUDA(cudaGetLastError());
+  return SFT_OK;
+}
+
+static sft_status scaled_slices(sft_target_s* t, cudaStream_t st) {
+  if (t->jent) return SFT_OK;
+  const int64_t n = t->nv, ns = (n + kSlice - 1) / kSlice;
+  if (sft_status r = jacobi_scale(t, st)) return r;
+  SFT_CUDA(dalloc(&t->rinfo, (size_t)(ns * kSlice), st));
+  SFT_CUDA(dalloc(&t->jval, (size_t)std::max<int64_t>(t->nnz, 1), st));
+  SFT_CUDA(dalloc(&t->mdiag, (size_t)n, st));
+  SFT_CUDA(dalloc(&t->jent, (size_t)std::max<int64_t>(t->nnz, 1), st));
+  const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ns + 7) / 8, 152 * 16));
+  ::sft::note_launch(), k_scaled_slices<<<nb, 256, 0, st>>>(t->row_ptr, t->col, t->val, t->sc, n, ns, t->jent,
+                                                           t->jval, t->mdiag, t->rinfo);
   SFT_CUDA(cudaGetLastError());
   return SFT_OK;
 }
@@ -670,66 +968,146 @@ sft_status finish_solve(const SolveLate& late, SolveResult* res) {
   if (!late.pending) return SFT_OK;
   MixCtl h;
   std::memcpy(&h, late.host, sizeof(MixCtl));
-  if (h.err != 0) return fail(SFT_ERR_DEVICE_STATUS, "CG kernel: grid barrier wait expired");
+  if (h.err != 0) return fail(SFT_ERR_DEVICE_STATUS, "solve kernel: a barrier wait expired");
   mix_result(h, late.nrhs, res);
+  return SFT_OK;
+}
+
+// Work (nonzeros x fields) up to which one block, or one cluster of
+// kClusterBlocks, takes the system. A step on one block needs no barrier
+// beyond its own, one on a cluster the hardware's (0.3 us) and distributed
+// shared memory, one on the grid a counter in L2 (1.2 us); against that stand
+// the FP64 phases (two lanes a clock on an SM) and the shared-memory loads of
+// few SMs. Measured, kernel time on a block / a cluster / the grid: 784 rows
+// 2D 46 / 50 / 76 us, 729 rows 3D 60 / 63 / 101; 2,025 rows 2D 87 / 51 / 77;
+// 10,201 rows 2D - / 62 / 81, 22,801 - / 95 / 83; 4,913 rows 3D - / 84 / 106,
+// 15,625 - / 135 / 108; 8 fields of 1,681 rows 2D - / 86 / 114, of 6,561
+// - / 128 / 118.
+constexpr int64_t kBlockWork = 10000;
+constexpr int64_t kClusterWork = 110000;
+constexpr int kClusterBlocks = 16;
+
+// Attributes of the solve kernels on the current device, set once per device;
+// false when a cluster of kClusterBlocks cannot be resident there.
+template <int NR>
+static sft_status mixed_attributes(int dev, bool* cluster_ok) {
+  static std::mutex mu;
+  static int state[64] = {0};  // 0 unset, 1 no cluster, 2 cluster
+  std::lock_guard<std::mutex> lk(mu);
+  int local = 0;
+  int& s = dev >= 0 && dev < 64 ? state[dev] : local;
+  if (s == 0) {
+    const void* k[4] = {(const void*)k_mixed<NR, kTeamBlock, true>, (const void*)k_mixed<NR, kTeamCluster, true>,
+                        (const void*)k_mixed<NR, kTeamGrid, true>, (const void*)k_mixed<NR, kTeamGrid, false>};
+    for (const void* f : k)
+      SFT_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmemMax));
+    SFT_CUDA(cudaFuncSetAttribute(k[1], cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterBlocks);
+    cfg.blockDim = dim3(kMixThreads<NR>);
+    cfg.dynamicSmemBytes = kMixSmemMax;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kClusterBlocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, k[1], &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    s = e == cudaSuccess && fit > 0 ? 2 : 1;
+  }
+  *cluster_ok = s == 2;
   return SFT_OK;
 }
 
 template <int NR>
 static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, double* x, double tol, int max_iter,
                                cudaStream_t st, SolveResult* res, SolveLate* late, int warm) {
-  const int64_t n = t->nv;
-  // largest eigenvalue bound of S M S: 2 for triangles, 5/2 for tetrahedra
-  float lmax = t->dim == 2 ? 2.f : 2.5f;
+  const int64_t n = t->nv, ns = (n + kSlice - 1) / kSlice;
   int dev = 0, sms = 0;
   SFT_CUDA(cudaGetDevice(&dev));
   SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int per_sm = 0;
-  SFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mixed_cg<NR>, kSolveThreads, 0));
-  if (per_sm < 1) return fail(SFT_ERR_CUDA, "solver kernel cannot be resident");
-  per_sm = std::min(per_sm, 4);
-  // as many resident blocks as ~3 rows per thread allows: measured 0.78 /
-  // 0.71 ms (1.0 M-row 2D / 0.5 M-row 3D systems) at 3 rows, 0.78 / 0.76 at
-  // 6, 1.04 / 1.06 at 12 (the FP32 phases are latency-bound, not FP64-bound)
-  constexpr int64_t kRows = SFT_MIX_ROWS_PER_THREAD;
-  const int64_t want = (n + kSolveThreads * kRows - 1) / (kSolveThreads * kRows);
-  const unsigned nblocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * sms, want));
+  bool cluster = false;
+  if (sft_status r = mixed_attributes<NR>(dev, &cluster)) return r;
+  const int64_t work = std::max<int64_t>(t->nnz, n) * NR;
+  const int team = work <= kBlockWork ? kTeamBlock : (cluster && work <= kClusterWork ? kTeamCluster : kTeamGrid);
+  const int64_t most = team == kTeamBlock ? 1 : (team == kTeamCluster ? kClusterBlocks : sms);
+  MixArgs a;
+  a.spb = (int)((ns + most - 1) / most);
+  // the cluster keeps its size; a grid leaves out blocks that would own no slice
+  const unsigned nblocks = (unsigned)(team == kTeamGrid ? (ns + a.spb - 1) / a.spb : most);
+  const int64_t rows = (int64_t)a.spb * kSlice;
+  // own rows of y in shared memory, and c and rinfo beside them, where they
+  // leave room for A
+  const bool own = rows * NR * 8 <= 128 * 1024;
+  a.c_smem = own && rows * NR * 12 <= 128 * 1024;
+  a.r_smem = rows * 2 <= 32 * 1024;
+  const int64_t fixed = (own ? rows * NR * 8 : 0) + (a.c_smem ? rows * NR * 4 : 0) + (a.r_smem ? rows * 2 : 0);
+  // shared memory for the block's share of A (with room for uneven shares)
+  const int64_t want = t->nnz * a.spb / std::max<int64_t>(ns, 1) * 5 / 4 + 1024;
+  a.cap = (int)(std::min<int64_t>(want, ((int64_t)kMixSmemMax - fixed) / 8) & ~(int64_t)1);  // 16-byte multiple
+  const size_t smem = (size_t)a.cap * 8 + (size_t)fixed;
+  const void* kern = team == kTeamBlock     ? (const void*)k_mixed<NR, kTeamBlock, true>
+                     : team == kTeamCluster ? (const void*)k_mixed<NR, kTeamCluster, true>
+                     : own                  ? (const void*)k_mixed<NR, kTeamGrid, true>
+                                            : (const void*)k_mixed<NR, kTeamGrid, false>;
   const size_t vec = (size_t)n * nrhs;
   DevBuf<double> tb(st), partd(st);
-  DevBuf<float> rb(st), pb(st), qb(st), yb(st), partf(st);
+  DevBuf<float> ya(st), yb(st), cb(st);
   DevBuf<MixCtl> ctl(st);
   SFT_CUDA(tb.alloc(vec));
-  SFT_CUDA(rb.alloc(vec));
-  SFT_CUDA(pb.alloc(vec));
-  SFT_CUDA(qb.alloc(vec));
-  SFT_CUDA(yb.alloc(vec));
-  SFT_CUDA(partd.alloc((size_t)nblocks * nrhs * 2));
-  SFT_CUDA(partf.alloc((size_t)nblocks * nrhs));
-  MixCtl* c = nullptr;
+  SFT_CUDA(ya.alloc(team == kTeamGrid ? (size_t)n * NR : 1));
+  SFT_CUDA(yb.alloc(team == kTeamGrid ? (size_t)n * NR : 1));
+  SFT_CUDA(cb.alloc(a.c_smem ? 1 : (size_t)n * NR));
+  SFT_CUDA(partd.alloc((size_t)nblocks * nrhs * 4));
   if (late) {
     SFT_CUDA(late->buf.alloc(sizeof(MixCtl)));
-    c = reinterpret_cast<MixCtl*>(late->buf.p);
+    a.ctl = reinterpret_cast<MixCtl*>(late->buf.p);
   } else {
     SFT_CUDA(ctl.alloc(1));
-    c = ctl.p;
+    a.ctl = ctl.p;
   }
-  SFT_CUDA(cudaMemsetAsync(c, 0, sizeof(MixCtl), st));
-  const int32_t* rp = t->row_ptr;
-  const int32_t* col = t->col;
-  const double* val = t->val;
-  const float* aval = t->val32s;
-  const double* sc = t->sc;
-  double* tp = tb.p;
-  float *r = rb.p, *p = pb.p, *q = qb.p, *y = yb.p;
-  double* pd = partd.p;
-  float* pf = partf.p;
-  void* args[] = {(void*)&rp, (void*)&col, (void*)&val, (void*)&aval, (void*)&sc, (void*)&n, (void*)&nrhs,
-                  (void*)&b, (void*)&x, (void*)&tp, (void*)&r, (void*)&p, (void*)&q, (void*)&y,
-                  (void*)&pd, (void*)&pf, (void*)&c, (void*)&tol, (void*)&max_iter, (void*)&warm,
-                  (void*)&t->wait_ns, (void*)&lmax};
-  const cudaError_t le = (::sft::note_launch(), cudaLaunchCooperativeKernel((const void*)k_mixed_cg<NR>, nblocks,
-                                                                           kSolveThreads, args, 0, st));
-  if (le != cudaSuccess) return cuda_fail(le, "cudaLaunchCooperativeKernel(k_mixed_cg)");
+  SFT_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(MixCtl), st));
+  a.rp = t->row_ptr;
+  a.jent = t->jent;
+  a.jval = t->jval;
+  a.mdiag = t->mdiag;
+  a.rinfo = t->rinfo;
+  a.sc = t->sc;
+  a.n = n;
+  a.nrhs = nrhs;
+  a.b = b;
+  a.x = x;
+  a.t = tb.p;
+  a.ya = ya.p;
+  a.yb = yb.p;
+  a.c = cb.p;
+  a.partd = partd.p;
+  a.tol = tol;
+  a.max_iter = max_iter;
+  a.warm = warm;
+  a.wait_ns = t->wait_ns;
+  a.lmax = t->dim == 2 ? 2.f : 2.5f;  // largest eigenvalue bound of S M S
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nblocks);
+  cfg.blockDim = dim3(kMixThreads<NR>);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  if (team == kTeamCluster) {
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kClusterBlocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  } else {
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = team == kTeamGrid;
+  }
+  cfg.attrs = &attr;
+  cfg.numAttrs = team == kTeamBlock ? 0 : 1;
+  void* args[] = {(void*)&a};
+  const cudaError_t le = (::sft::note_launch(), cudaLaunchKernelExC(&cfg, kern, args));
+  if (le != cudaSuccess) return cuda_fail(le, "launch of the mixed-precision solve");
   if (late) {
     late->bytes = sizeof(MixCtl);
     late->nrhs = nrhs;
@@ -739,7 +1117,7 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
   MixCtl h;
   SFT_CUDA(cudaMemcpyAsync(&h, ctl.p, sizeof(MixCtl), cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaStreamSynchronize(st));
-  if (h.err != 0) return fail(SFT_ERR_DEVICE_STATUS, "CG kernel: grid barrier wait expired");
+  if (h.err != 0) return fail(SFT_ERR_DEVICE_STATUS, "solve kernel: a barrier wait expired");
   mix_result(h, nrhs, res);
   return SFT_OK;
 }
@@ -760,7 +1138,7 @@ sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, dou
   }
   if (warm && cg_mode != SFT_CG_MIXED) return fail(SFT_ERR_UNSUPPORTED, "a warm start needs cg_mode MIXED");
   if (cg_mode == SFT_CG_MIXED) {
-    if (sft_status r = scaled_matrix(t, st)) return r;
+    if (sft_status r = scaled_slices(t, st)) return r;
     if (nrhs == 1) return launch_mixed<1>(t, nrhs, b, x, tol, max_iter, st, res, late, warm);
     if (nrhs == 2) return launch_mixed<2>(t, nrhs, b, x, tol, max_iter, st, res, late, warm);
     if (nrhs <= 4) return launch_mixed<4>(t, nrhs, b, x, tol, max_iter, st, res, late, warm);
