@@ -14,36 +14,44 @@
 
 namespace sft {
 
-// Forward of the network on n points (x,y,z) [n][3] FP32 -> out [n] FP32.
-// Persistent CTAs of 256 threads (two per SM): each 128-point tile is
-// shared by the two column halves (mlp_tile).
-__global__ void __launch_bounds__(kTPR * kTileM, 2) k_mlp_forward(const float* __restrict__ P,
-                                                                  const unsigned char* __restrict__ W2,
-                                                                  const unsigned char* __restrict__ W3,
-                                                                  const unsigned char* __restrict__ W4, int64_t n,
-                                                                  const float* __restrict__ pts,
-                                                                  float* __restrict__ out, int32_t* err) {
+// Forward of the network on n points (x,y,z) [n][3] FP32 -> out [n] FP32:
+// persistent CTAs (one per SM) of two groups that alternate on the tensor
+// cores (fwd_tile).
+__global__ void __launch_bounds__(2 * kGroupThreads, 1) k_mlp_forward(const float* __restrict__ P,
+                                                                     const unsigned char* __restrict__ W2,
+                                                                     const unsigned char* __restrict__ W3,
+                                                                     const unsigned char* __restrict__ W4, int64_t n,
+                                                                     const float* __restrict__ pts,
+                                                                     float* __restrict__ out, int32_t* err) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  const MlpSmem S = mlp_smem(sm);
+  const FwdSmem S = fwd_smem(sm);
   const unsigned char* const Wc[3] = {W2, W3, W4};
-  WStream ws;
-  const uint32_t taddr = mlp_setup(S, P, Wc, cta_tiles((n + kTileM - 1) / kTileM), ws);
-  uint32_t phase = 0;
-  bool ok = true;
-  const int row = threadIdx.x & (kTileM - 1);
-  for (int64_t tile = blockIdx.x; ok && tile * kTileM < n; tile += gridDim.x) {
-    const int64_t gi = tile * kTileM + row;
-    float x[3] = {0.f, 0.f, 0.f};
-    if (gi < n) {
-      x[0] = pts[gi * 3];
-      x[1] = pts[gi * 3 + 1];
-      x[2] = pts[gi * 3 + 2];
-    }
-    float y = 0.f;
-    ok = mlp_tile(S, P, Wc, ws, x, taddr, phase, err, y);
-    if (ok && gi < n && threadIdx.x < kTileM) out[gi] = y;
+  const int grp = threadIdx.x / kGroupThreads;
+  const int lt = threadIdx.x - grp * kGroupThreads;
+  const int64_t tiles = cta_tiles((n + kTileM - 1) / kTileM);
+  const uint32_t taddr = fwd_setup(S, P, Wc, tiles);
+  const int64_t J1 = tiles / 2;  // tiles of each group that have a partner
+  uint32_t lphase = 0;
+  // inputs of rows l / 4 + 8 q of the warp's 32 in tile k
+  float x[4][3];
+  auto load_x = [&](int64_t k) {
+    const int64_t first = (blockIdx.x + k * gridDim.x) * kTileM + (lt & 96) + ((lt & 31) >> 2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[q][a] = k < tiles && first + 8 * q < n ? __ldg(pts + (first + 8 * q) * 3 + a) : 0.f;
+  };
+  load_x(grp);
+  for (int64_t k = grp; k < tiles; k += 2) {
+    const int64_t gi = (blockIdx.x + k * gridDim.x) * kTileM + lt;
+    const int64_t j = k / 2;
+    float y;
+    // the next tile's inputs load during this tile's last layer
+    fwd_tile(S, P, Wc, grp, lt, x, taddr, lphase, j < J1 ? 6 * j + grp : 6 * J1, j < J1 ? 2 : 1, err, y,
+             [&] { load_x(k + 2); });
+    if (lt < kTileM && gi < n) out[gi] = y;
   }
-  mlp_teardown(S, taddr, ws, err);
+  fwd_teardown(S, taddr, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -422,8 +430,8 @@ sft_status mlp_forward_dev(sft_mlp_s* m, int64_t n, const float* pts, float* out
   SFT_CUDA(cudaGetDevice(&dev));
   SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t tiles = (n + kTileM - 1) / kTileM;
-  const unsigned grid = (unsigned)std::min<int64_t>(tiles, 2 * (int64_t)sms);
-  ::sft::note_launch(), k_mlp_forward<<<grid, kTPR * kTileM, kSmemFwd, st>>>(m->P, m->Wc[0], m->Wc[1], m->Wc[2], n,
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)sms);
+  ::sft::note_launch(), k_mlp_forward<<<grid, 2 * kGroupThreads, kSmemFwd, st>>>(m->P, m->Wc[0], m->Wc[1], m->Wc[2], n,
                                                                              pts, out, d_err);
   SFT_CUDA(cudaGetLastError());
   return SFT_OK;

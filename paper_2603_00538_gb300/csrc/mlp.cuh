@@ -16,28 +16,18 @@ namespace sft {
 constexpr int kH = 256;
 constexpr int kTileM = 128;
 constexpr int kKC = 64;  // K chunk of a streamed weight block (training GEMM)
-constexpr int kKF = 16;  // K chunk of a streamed weight block (forward tile): one MMA
-constexpr int kStages = 4;  // weight chunk buffers of the forward tile
-constexpr int kTPR = 2;  // forward tile: threads per activation row (each owns half the columns)
+constexpr int kKF = 16;  // K of one MMA
+constexpr int kTPR = 2;  // forward tile: threads per activation row (each owns half of the columns)
 constexpr int64_t kOffW1 = 0, kOffC1 = kH * 3, kOffW2 = kOffC1 + kH, kOffC2 = kOffW2 + kH * kH,
                   kOffW3 = kOffC2 + kH, kOffC3 = kOffW3 + kH * kH, kOffW4 = kOffC3 + kH,
                   kOffC4 = kOffW4 + kH * kH, kOffW5 = kOffC4 + kH, kOffC5 = kOffW5 + kH,
                   kNParam = kOffC5 + 1;
 
-// shared memory of a forward tile: activation tile (128 x 256 BF16),
-// kStages weight chunks (256 x 16 BF16), the first layer as float4
-// {w0, w1, w2, c} per output, the two halves' partial outputs, the
-// mbarriers, the TMEM address slot and a status word. About 101 KB: two
-// CTAs fit on one SM.
-constexpr uint32_t kSmemA = kTileM * kH * 2;        // 64 KiB
+constexpr uint32_t kSmemA = kTileM * kH * 2;        // 64 KiB: activation tile (128 x 256 BF16)
 constexpr uint32_t kSmemB = kH * kKC * 2;           // 32 KiB (training GEMM chunk)
-constexpr uint32_t kSmemBF = kH * kKF * 2;          // 8 KiB
-constexpr uint32_t kSmemW1 = kH * 16;               // 4 KiB
-constexpr uint32_t kSmemY = kTPR * kTileM * 4;      // 1 KiB
+constexpr uint32_t kSmemBF = kH * kKF * 2;          // 8 KiB: weights of one MMA (256 x 16 BF16)
+constexpr uint32_t kSmemW1 = kH * 16;               // 4 KiB: first layer (w1_table_entry)
 constexpr uint32_t kSmemBias = 4 * kH * 4;          // 4 KiB: c2, c3, c4, w5
-constexpr uint32_t kSmemBar = 128;                  // 2 kStages + 1 mbarriers, slot, status
-constexpr uint32_t kSmemFwd = kSmemA + kStages * kSmemBF + kSmemW1 + kSmemBias + kSmemY + kSmemBar;
-constexpr int kChunksPerLayer = kH / kKF;
 
 // byte offset of weight (n, k) of a 256x256 layer in the chunked layout the
 // forward tile streams: chunk k / kKF is one contiguous [256][kKF] block in
@@ -103,342 +93,130 @@ __device__ __forceinline__ void w1_table_entry(float4* w1, const float* __restri
   e1[odd] = __ldg(P + kOffW1 + o * 3 + 2);
   e1[2 + odd] = __ldg(P + kOffC1 + o);
 }
-// first-layer outputs o .. o + 7 (o even) of the point x: SiLU(W1 x + c1),
-// the FMAs in the order fma(w2, x2, fma(w1, x1, fma(w0, x0, c)))
-__device__ __forceinline__ void layer1_outputs8(const float4* w1, int o, const float x[3], float h[8]) {
-  const uint64_t X0 = f2_pack(x[0], x[0]), X1 = f2_pack(x[1], x[1]), X2 = f2_pack(x[2], x[2]);
-#pragma unroll
-  for (int q = 0; q < 8; q += 2) {
-    const float4 a = w1[o + q], b = w1[o + q + 1];
-    const uint64_t z = f2_fma(f2_pack(b.x, b.y), X2, f2_fma(f2_pack(a.z, a.w), X1,
-                                                           f2_fma(f2_pack(a.x, a.y), X0, f2_pack(b.z, b.w))));
-    silu_pair(z, h[q], h[q + 1]);
-  }
-}
+// ---------------------------------------------------------------------------
+// The forward pass on 128-row tiles: one CTA per SM, two groups of 256
+// threads (two threads a row, half of the columns each). Each group runs its
+// own tiles with its own activation tile, TMEM accumulator (columns 256 g ..
+// +255) and named barrier: layer 1 (3 -> 256) on the FMA pipe into the BF16
+// activation tile, three 256x256 layers on the tensor cores with bias + SiLU
+// epilogues from TMEM, the last layer (256 -> 1) as FMA chains over each half of
+// the columns beside the last epilogue, the halves added in a fixed order. The
+// two groups' layers take turns on the tensor cores in a fixed order - tile
+// pair j: T0 L1, T1 L1, T0 L2, T1 L2, T0 L3, T1 L3; a group without a partner
+// tile at the end runs its layers alone - so one group's epilogue overlaps the
+// other's MMAs, and both read one ring of kRing weight chunks (64 wide in K:
+// four MMAs each) fed in that order (chunk c = 4 s + k: K-slice k of the layer
+// of slot s). Per slot 1 + kRing warps of its group work at once: warp 0
+// issues the MMAs as their chunks land, and warp 1 + b refills buffer b as
+// soon as the MMAs that read it complete (the chunk kRing ahead); each is a
+// converged warp with one elected lane (a lone thread in a divergent branch
+// took about 100 cycles an MMA). Turn counters in shared memory (bounded
+// waits) keep the slots' MMA issue and each buffer's copies in slot order, so
+// every mbarrier phase is waited only after the phase before it completed.
+//
+// What bounds it: the chain of a group's phases. A tile takes 131 k
+// activations, each two special-function operations (some 12 k cycles of an
+// SM) and about 8 issue slots, and 6.1 k cycles of MMA; a group's tile passes
+// through layer 1 (5 k cycles), three MMA phases (3.5 k) and three epilogues
+// (4.3 k), and two groups a SM overlap to 17 k cycles a tile (a third
+// accumulator does not fit in TMEM). 1.536 M points: 1,157 us (two CTAs of one
+// tile each, one thread issuing MMAs and copies, 16-wide chunks, broadcast
+// bias loads) -> 763 (two groups taking turns, every operation over 16 columns
+// at a time) -> 747 (accumulator fragments, output layer inside the epilogue)
+// -> 711 (64-wide chunks) -> 707 us (elected lanes) = 0.86 PFLOP/s, 0.46 of
+// the measured BF16 burst rate. Measured and dropped: 512 threads a group, 5 or
+// 7 smaller ring buffers, one copier warp, every thread polling the layer's
+// mbarrier (770 us: the polls slow the issuer).
+// ---------------------------------------------------------------------------
+constexpr int kChunkK = 64;                     // K of a ring chunk
+constexpr uint32_t kChunkBytes = kH * kChunkK * 2;
+constexpr int kChunks = kH / kChunkK;           // chunks per layer
+constexpr int kRing = 2;                        // chunk buffers
+constexpr int kGroupThreads = kTPR * kTileM;    // 512
+constexpr uint32_t kSmemBars = 256;             // mbarriers, TMEM slot, failed flag, turn counters, stream state
+constexpr uint32_t kSmemYH = 2 * kTileM * 4;    // partial outputs of the column halves
+constexpr uint32_t kSmemFwd = 2 * kSmemA + kRing * kChunkBytes + kSmemW1 + kSmemBias + 2 * kSmemYH + kSmemBars;
+static_assert(kRing <= kChunks && 32 * kRing < kGroupThreads, "ring size");
+static_assert(kSmemFwd <= 227u * 1024u, "forward tile exceeds the shared memory of one CTA");
 
-// The weight stream of a forward CTA: chunk g (g = 0, 1, ... over the
-// CTA's tiles, 3 layers of kChunksPerLayer chunks each) goes to buffer
-// g % kStages by one bulk copy whose bytes complete full[b]; its MMA commits
-// to mdone[b]. Thread 0 consumes chunk g (wait full, MMA, commit), then waits
-// for chunk g-1's MMA (its buffer is the one chunk g+kStages-1 goes to; the
-// MMA of chunk g stays queued behind it, so the tensor pipe does not idle)
-// and issues that copy. The next layer's first chunks thus load during the
-// current layer's epilogue. Every commit to mdone[b] is waited exactly once,
-// before its buffer is refilled; parity of the k-th use of a buffer is k & 1.
-struct WStream {
-  int64_t next_use = 0, next_copy = 0, total = 0;
+struct FwdStream {
+  int32_t total;             // chunks of the CTA's stream
+  int32_t tail0;             // first slot of the unpaired tile (6 x the paired tiles of a group)
+  int32_t next_use;          // chunks whose MMAs were issued
+  int32_t next_copy[kRing];  // the next chunk copied into each buffer
 };
 
-__device__ __forceinline__ const unsigned char* wchunk_src(const unsigned char* const Wc[3], int64_t g) {
-  const int64_t per_tile = 3 * kChunksPerLayer;
-  const int l = (int)((g % per_tile) / kChunksPerLayer);
-  const int kc = (int)(g % kChunksPerLayer);
-  return Wc[l] + (size_t)kc * kSmemBF;
-}
-
-// thread 0: copy chunk ws.next_copy (buffer free: its previous reader's MMA
-// was waited by the caller, or the buffer is unused yet)
-__device__ __forceinline__ void ws_copy(WStream& ws, unsigned char* B, uint64_t* full,
-                                        const unsigned char* const Wc[3]) {
-  const int64_t g = ws.next_copy++;
-  const int b = (int)(g % kStages);
-  tc::mbar_arrive_expect_tx(full + b, kSmemBF);
-  tc::bulk_g2s(B + (size_t)b * kSmemBF, wchunk_src(Wc, g), kSmemBF, full + b);
-}
-
-// one 256x256 layer: TMEM[128 x 256] = A (smem, 128 x 256) * W^T. Only
-// thread 0 works; ends with a commit to lbar and a bounded wait on it.
-// Returns false if a wait expired (error recorded in *err).
-__device__ __forceinline__ bool tc_layer_issue(WStream& ws, unsigned char* A, unsigned char* B, uint64_t* full,
-                                               uint64_t* mdone, uint64_t* lbar, uint32_t& lphase,
-                                               const unsigned char* const Wc[3], uint32_t taddr, int32_t* err) {
-  tc::fence_after_sync();
-  for (int kc = 0; kc < kChunksPerLayer; ++kc) {
-    const int64_t g = ws.next_use++;
-    const int b = (int)(g % kStages);
-    if (!tc::mbar_wait(full + b, (uint32_t)((g / kStages) & 1), err)) return false;
-    const uint64_t ad = tc::smem_desc(tc::smem_addr(A) + (uint32_t)(kc * kKF / 8) * 128u, 128u, (uint32_t)kH * 16u);
-    const uint64_t bd = tc::smem_desc(tc::smem_addr(B + (size_t)b * kSmemBF), 128u, (uint32_t)kKF * 16u);
-    tc::mma_bf16(taddr, ad, bd, kIdesc, kc != 0);
-    tc::mma_commit(mdone + b);
-    if (ws.next_copy < ws.total) {
-      if (g >= 1) {
-        const int64_t gp = g - 1;  // last reader of the buffer chunk next_copy goes to
-        if (!tc::mbar_wait(mdone + (gp % kStages), (uint32_t)((gp / kStages) & 1), err)) return false;
-      }
-      ws_copy(ws, B, full, Wc);
-    }
-  }
-  tc::mma_commit(lbar);
-  const bool ok = tc::mbar_wait(lbar, lphase, err);
-  lphase ^= 1u;
-  return ok;
-}
-
-// shared-memory carve-up of one 128-row network tile
-struct MlpSmem {
-  unsigned char* A;   // activation tile [128][256] BF16, K-major core matrices
-  unsigned char* B;   // kStages weight chunk buffers [256][kKF] BF16
+struct FwdSmem {
+  unsigned char* A;   // [2] activation tiles
+  unsigned char* B;   // kRing weight chunk buffers
   float4* w1;         // first layer, pair-interleaved (w1_table_entry)
   float* bias;        // [4][256]: c2, c3, c4 and the output weights w5
-  float* ypart;       // [kTPR][128] partial outputs of the column halves
-  uint64_t* full;     // [kStages] chunk landed (bulk-copy transaction bytes)
-  uint64_t* mdone;    // [kStages] MMAs reading the chunk completed
-  uint64_t* lbar;     // all MMAs of a layer completed
+  float* ypart;       // [2][2][128] partial outputs of each group's column halves
+  uint64_t* full;     // [kRing] chunk landed (bulk-copy transaction bytes)
+  uint64_t* mdone;    // [kRing] MMAs reading the chunk completed
+  uint64_t* lbar;     // [2] all MMAs of a group's layer completed
   uint32_t* slot;     // TMEM base address
-  int* s_ok;          // result of thread 0's bounded waits
-};
-__device__ __forceinline__ MlpSmem mlp_smem(unsigned char* sm) {
-  MlpSmem S;
-  S.A = sm;
-  S.B = sm + kSmemA;
-  S.w1 = reinterpret_cast<float4*>(S.B + kStages * kSmemBF);
-  S.bias = reinterpret_cast<float*>(S.B + kStages * kSmemBF + kSmemW1);
-  S.ypart = reinterpret_cast<float*>(S.B + kStages * kSmemBF + kSmemW1 + kSmemBias);
-  S.full = reinterpret_cast<uint64_t*>(S.B + kStages * kSmemBF + kSmemW1 + kSmemBias + kSmemY);
-  S.mdone = S.full + kStages;
-  S.lbar = S.mdone + kStages;
-  S.slot = reinterpret_cast<uint32_t*>(S.lbar + 1);
-  S.s_ok = reinterpret_cast<int*>(S.slot + 1);
-  return S;
-}
-
-// Per-CTA setup of a network tile loop over `ntiles` tiles: TMEM allocation
-// (256 columns), the mbarriers, the first-layer table and the first
-// kStages - 1 weight chunk copies. Every thread calls it.
-__device__ __forceinline__ uint32_t mlp_setup(const MlpSmem& S, const float* __restrict__ P,
-                                              const unsigned char* const Wc[3], int64_t ntiles, WStream& ws) {
-  if ((threadIdx.x >> 5) == 0) {
-    tc::tmem_alloc(S.slot, kH);
-    tc::tmem_relinquish();
-  }
-  ws.total = ntiles * 3 * kChunksPerLayer;
-  if (threadIdx.x == 0) {
-    for (int b = 0; b < kStages; ++b) {
-      tc::mbar_init(S.full + b, 1);
-      tc::mbar_init(S.mdone + b, 1);
-    }
-    tc::mbar_init(S.lbar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    while (ws.next_copy < ws.total && ws.next_copy < kStages - 1) ws_copy(ws, S.B, S.full, Wc);
-  }
-  for (int o = threadIdx.x; o < kH; o += blockDim.x) {
-    w1_table_entry(S.w1, P, o);
-    S.bias[o] = __ldg(P + kOffC2 + o);
-    S.bias[kH + o] = __ldg(P + kOffC3 + o);
-    S.bias[2 * kH + o] = __ldg(P + kOffC4 + o);
-    S.bias[3 * kH + o] = __ldg(P + kOffW5 + o);
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  return *S.slot;
-}
-// End of the tile loop: thread 0 waits (bounded) for copies it issued that
-// no MMA consumed (after an expired wait), then TMEM is released.
-__device__ __forceinline__ void mlp_teardown(const MlpSmem& S, uint32_t taddr, WStream& ws, int32_t* err) {
-  if (threadIdx.x == 0) {
-    for (int64_t g = ws.next_use; g < ws.next_copy; ++g)
-      if (!tc::mbar_wait(S.full + (g % kStages), (uint32_t)((g / kStages) & 1), err, 200000000ull)) break;
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(taddr, kH);
-}
-
-// tiles a persistent CTA visits (tile = blockIdx.x + k gridDim.x < ntiles)
-__device__ __forceinline__ int64_t cta_tiles(int64_t ntiles) {
-  return blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-}
-
-// 32 columns cc .. cc+31 of hidden layer l (accumulators in r) for this
-// thread's row: bias + SiLU, then into the activation tile (l < 2) or the
-// output dot product y
-__device__ __forceinline__ void tile_columns_a(unsigned char* A, const float* bias, int l, int row, int cc,
-                                               const uint32_t (&r)[32], float& y) {
-  const float4* b4 = reinterpret_cast<const float4*>(bias + l * kH + cc);
-  float v[32];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 b = b4[i];
-    // silu_f(acc + bias) on pairs of columns
-    silu_pair(f2_add(f2_pack(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1])), f2_pack(b.x, b.y)),
-              v[4 * i], v[4 * i + 1]);
-    silu_pair(f2_add(f2_pack(__uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])), f2_pack(b.z, b.w)),
-              v[4 * i + 2], v[4 * i + 3]);
-  }
-  if (l < 2) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) store_bf16x8(A + tc::kmajor_offset(row, cc + q * 8, kH), v + q * 8);
-  } else {
-    const float4* w4 = reinterpret_cast<const float4*>(bias + 3 * kH + cc);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float4 w = w4[i];
-      y = __fmaf_rn(bf16r(v[4 * i]), w.x, y);
-      y = __fmaf_rn(bf16r(v[4 * i + 1]), w.y, y);
-      y = __fmaf_rn(bf16r(v[4 * i + 2]), w.z, y);
-      y = __fmaf_rn(bf16r(v[4 * i + 3]), w.w, y);
-    }
-  }
-}
-
-__device__ __forceinline__ void tile_columns(const MlpSmem& S, int l, int row, int cc, const uint32_t (&r)[32],
-                                             float& y) {
-  tile_columns_a(S.A, S.bias, l, row, cc, r, y);
-}
-
-// The whole network on one 128-row tile with kTPR * 128 threads: thread t
-// owns row t % 128 and the column half t / 128 (TMEM lanes of warp w are
-// 32 (w % 4) .. +31). Every thread passes its row's input x and gets y.
-// Layer 1 (3 -> 256) on the FMA pipe into the BF16 activation tile, three
-// 256x256 layers on the tensor cores with bias + SiLU epilogues from TMEM,
-// the last layer (256 -> 1) as FMA dots over each half, the halves added in
-// a fixed order. False if a tensor-core wait expired.
-__device__ __forceinline__ bool mlp_tile(const MlpSmem& S, const float* __restrict__ P,
-                                         const unsigned char* const Wc[3], WStream& ws, const float x[3],
-                                         uint32_t taddr, uint32_t& phase, int32_t* err, float& y_out) {
-  constexpr int kCols = kH / kTPR;
-  const int row = threadIdx.x & (kTileM - 1);
-  const int half = threadIdx.x / kTileM;
-  const int c0 = half * kCols;
-  const uint32_t trow = taddr + ((uint32_t)(32 * ((threadIdx.x >> 5) & 3)) << 16);
-  for (int o = c0; o < c0 + kCols; o += 8) {
-    float h[8];
-    layer1_outputs8(S.w1, o, x, h);
-    store_bf16x8(S.A + tc::kmajor_offset(row, o, kH), h);
-  }
-  tc::fence_async_smem();
-  __syncthreads();
-  float y = 0.f;
-  for (int l = 0; l < 3; ++l) {
-    if (threadIdx.x == 0) *S.s_ok = tc_layer_issue(ws, S.A, S.B, S.full, S.mdone, S.lbar, phase, Wc, taddr, err);
-    __syncthreads();
-    tc::fence_after_sync();
-    if (!*S.s_ok) return false;
-    // epilogue: bias + SiLU from TMEM, this thread's row and column half;
-    // TMEM loads double buffered (the next 32 columns load while the
-    // current ones are processed)
-    uint32_t ra[32], rb[32];
-    tc::tmem_ld32_issue(trow + (uint32_t)c0, ra);
-    tc::tmem_ld_wait();
-#pragma unroll 1
-    for (int cc = c0; cc < c0 + kCols; cc += 64) {
-      tc::tmem_ld32_issue(trow + (uint32_t)(cc + 32), rb);
-      tile_columns(S, l, row, cc, ra, y);
-      tc::tmem_ld_wait();
-      if (cc + 64 < c0 + kCols) tc::tmem_ld32_issue(trow + (uint32_t)(cc + 64), ra);
-      tile_columns(S, l, row, cc + 32, rb, y);
-      tc::tmem_ld_wait();
-    }
-    if (l == 2) S.ypart[half * kTileM + row] = y;
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-  }
-  float yy = S.ypart[row];
-#pragma unroll
-  for (int h = 1; h < kTPR; ++h) yy += S.ypart[h * kTileM + row];
-  y_out = yy + __ldg(P + kOffC5);
-  return true;
-}
-
-// ---------------------------------------------------------------------------
-// Two-group forward tile (the fused surrogate assembly): one CTA per SM,
-// 2 x 256 threads. Group g (threads 256 g .. 256 g + 255) runs its own
-// 128-row tiles exactly as mlp_tile does one (same arithmetic, bit-identical
-// outputs), with its own activation tile, TMEM accumulator (columns
-// 256 g .. +255) and named barrier. The two groups' layers take turns on the
-// tensor cores in a fixed order - tile pair j: T0 L1, T1 L1, T0 L2, T1 L2,
-// T0 L3, T1 L3; a group without a partner tile at the end runs its layers
-// alone - so one group's epilogue overlaps the other's MMAs, and both read
-// one ring of kStagesPP weight chunks fed in that order (chunk c = 16 s + k:
-// K-slice k of the layer of slot s). Per slot 1 + kCopiers threads of its
-// group work at once: thread 0 issues the 16 MMAs as their chunks land
-// (descriptors formed once, so an MMA costs a few adds), and kCopiers
-// threads each refill one class of buffers (chunk c mod kCopiers) as soon as
-// the MMA that read a buffer completes (the chunk kStagesPP ahead). One
-// thread doing both spent about 1,000 cycles per chunk on issue work, five
-// times the MMA's own time (sur3d fused kernel 258 ms against 132 ms for two
-// independent CTAs per SM); with one copier 132 ms, two 122 ms. Turn counters in shared memory
-// (bounded waits) keep the slots' MMA issue and their copies each in slot
-// order; the copies of slot s wait for slot s - 1's copier, so every
-// mbarrier phase is waited only after the phase before it completed.
-// ---------------------------------------------------------------------------
-constexpr int kStagesPP = 8;                    // power of two
-constexpr int kGroupThreads = kTPR * kTileM;    // 256
-constexpr int kCopiers = 4;      // ring refill threads per group: 32 (1 + p) handles chunks = p (mod kCopiers)
-constexpr int kCopierLane = 32;
-constexpr uint32_t kSmemBarPP = 256;            // mbarriers, TMEM slot, flags, turn counters, stream state
-constexpr uint32_t kSmemPP = 2 * kSmemA + kStagesPP * kSmemBF + kSmemW1 + kSmemBias + 2 * kSmemY + kSmemBarPP;
-static_assert((kStagesPP & (kStagesPP - 1)) == 0 && kStagesPP <= kChunksPerLayer, "ring size");
-static_assert(kStagesPP % kCopiers == 0 && kCopierLane * kCopiers < kGroupThreads, "copier classes");
-
-struct StreamPP {
-  int32_t total;         // chunks of the CTA's stream
-  int32_t tail0;         // first slot of the unpaired tiles (6 x the paired tiles of a group)
-  int32_t next_use;      // chunks whose MMA was issued
-  int32_t next_copy[kCopiers];  // chunk c of class c % kCopiers was copied iff c < next_copy[c % kCopiers]
-};
-
-struct MlpSmemPP {
-  unsigned char* A[2];
-  unsigned char* B;   // kStagesPP weight chunk buffers [256][kKF] BF16
-  float4* w1;
-  float* bias;
-  float* ypart[2];
-  uint64_t* full;     // [kStagesPP]
-  uint64_t* mdone;    // [kStagesPP]
-  uint64_t* lbar;     // [2]: all MMAs of a group's layer completed
-  uint32_t* slot;     // TMEM base address
-  int* s_ok;          // [2]: MMA issue of the group's current slot succeeded
-  int* s_okc;         // [2][kCopiers]: its copies of each class succeeded
+  volatile int* failed;  // a wait expired: nothing is issued or waited for any more
   volatile int* issued;  // layer slots whose MMAs were issued
-  volatile int* copied;  // [kCopiers]: layer slots whose copies of each class were issued
-  StreamPP* st;
+  volatile int* copied;  // [kRing] layer slots whose copies into each buffer were issued
+  FwdStream* st;
 };
-__device__ __forceinline__ MlpSmemPP mlp_smem_pp(unsigned char* sm) {
-  MlpSmemPP S;
-  S.A[0] = sm;
-  S.A[1] = sm + kSmemA;
+__device__ __forceinline__ FwdSmem fwd_smem(unsigned char* sm) {
+  FwdSmem S;
+  S.A = sm;
   S.B = sm + 2 * kSmemA;
-  unsigned char* q = S.B + kStagesPP * kSmemBF;
+  unsigned char* q = S.B + kRing * kChunkBytes;
   S.w1 = reinterpret_cast<float4*>(q);
   q += kSmemW1;
   S.bias = reinterpret_cast<float*>(q);
   q += kSmemBias;
-  S.ypart[0] = reinterpret_cast<float*>(q);
-  S.ypart[1] = reinterpret_cast<float*>(q + kSmemY);
-  q += 2 * kSmemY;
+  S.ypart = reinterpret_cast<float*>(q);
+  q += 2 * kSmemYH;
   S.full = reinterpret_cast<uint64_t*>(q);
-  S.mdone = S.full + kStagesPP;
-  S.lbar = S.mdone + kStagesPP;
+  S.mdone = S.full + kRing;
+  S.lbar = S.mdone + kRing;
   S.slot = reinterpret_cast<uint32_t*>(S.lbar + 2);
-  S.s_ok = reinterpret_cast<int*>(S.slot + 1);
-  S.s_okc = S.s_ok + 2;
-  S.issued = reinterpret_cast<volatile int*>(S.s_okc + 2 * kCopiers);
+  S.failed = reinterpret_cast<volatile int*>(S.slot + 1);
+  S.issued = S.failed + 1;
   S.copied = S.issued + 1;
-  S.st = reinterpret_cast<StreamPP*>(q + 224);
+  S.st = reinterpret_cast<FwdStream*>(q + 192);
   return S;
 }
-static_assert(2 * kStagesPP * 8 + 2 * 8 + 4 + 8 + 8 * kCopiers + 4 + 4 * kCopiers <= 224,
+static_assert(2 * kRing * 8 + 2 * 8 + 4 + 4 + 4 + 4 * kRing <= 192,
               "barrier block overlaps the stream state");
-static_assert(224 + sizeof(StreamPP) <= kSmemBarPP, "stream state outside its block");
+static_assert(192 + sizeof(FwdStream) <= kSmemBars, "stream state outside its block");
 
 __device__ __forceinline__ void group_sync(int grp) {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(kGroupThreads) : "memory");
+  if (grp == 0) asm volatile("bar.sync 1, %0;" ::"n"(kGroupThreads) : "memory");
+  else asm volatile("bar.sync 2, %0;" ::"n"(kGroupThreads) : "memory");
 }
 
-// bounded wait until *ctr == v (false and *err set if it did not come)
-__device__ __forceinline__ bool turn_wait(volatile int* ctr, int v, int32_t* err,
-                                          uint64_t timeout_ns = 2000000000ull) {
+// Bounded waits of the forward kernel. One that runs out sets *err and the
+// CTA's failed flag; from then on every wait returns at once and no copy or
+// MMA is issued, so the threads run through their loops, meet at the same
+// barriers, and leave together.
+__device__ __forceinline__ bool turn_wait(const FwdSmem& S, volatile int* ctr, int v, int32_t* err) {
   if (*ctr == v) return true;
   const uint64_t t0 = globaltimer_ns();
   while (*ctr != v) {
-    if (globaltimer_ns() - t0 > timeout_ns) {
+    if (*S.failed) return false;
+    if (globaltimer_ns() - t0 > kDefaultWaitNs) {
       set_error(err, DEV_BARRIER_TIMEOUT);
+      *S.failed = 1;
+      return false;
+    }
+    __nanosleep(32);
+  }
+  return true;
+}
+__device__ __forceinline__ bool fwd_wait(const FwdSmem& S, uint64_t* bar, uint32_t parity, int32_t* err) {
+  if (tc::mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  while (!tc::mbar_try_wait(bar, parity)) {
+    if (*S.failed) return false;
+    if (globaltimer_ns() - t0 > kDefaultWaitNs) {
+      set_error(err, DEV_BARRIER_TIMEOUT);
+      *S.failed = 1;
       return false;
     }
   }
@@ -452,44 +230,49 @@ __device__ __forceinline__ int slot_layer(int s, int tail0) { return s < tail0 ?
 __device__ __forceinline__ const unsigned char* layer_weights(const unsigned char* const Wc[3], int l) {
   return l == 0 ? Wc[0] : (l == 1 ? Wc[1] : Wc[2]);
 }
-__device__ __forceinline__ void copy_chunk_pp(const MlpSmemPP& S, const unsigned char* layer_w, int c) {
-  const int b = c & (kStagesPP - 1);
-  tc::mbar_arrive_expect_tx(S.full + b, kSmemBF);
-  tc::bulk_g2s(S.B + (size_t)b * kSmemBF, layer_w + (size_t)(c & (kChunksPerLayer - 1)) * kSmemBF, kSmemBF,
+__device__ __forceinline__ void copy_chunk(const FwdSmem& S, const unsigned char* layer_w, int c) {
+  const int b = c % kRing;
+  tc::mbar_arrive_expect_tx(S.full + b, kChunkBytes);
+  tc::bulk_g2s(S.B + (size_t)b * kChunkBytes, layer_w + (size_t)(c & (kChunks - 1)) * kChunkBytes, kChunkBytes,
                S.full + b);
 }
 
-// Setup over the CTA's `units` work units of `nsub` tiles each, split between
-// the groups (group 0 the even ones): TMEM (512 columns), mbarriers, the
-// stream state and its first kStagesPP copies, the first-layer table.
-// Every thread calls it.
-__device__ __forceinline__ uint32_t mlp_setup_pp(const MlpSmemPP& S, const float* __restrict__ P,
-                                                 const unsigned char* const Wc[3], int64_t units, int nsub) {
+// tiles a persistent CTA visits (tile = blockIdx.x + k gridDim.x < ntiles)
+__device__ __forceinline__ int64_t cta_tiles(int64_t ntiles) {
+  return blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+}
+
+// Setup over the CTA's tiles, split between the groups (group 0 the even
+// ones): TMEM (512 columns), mbarriers, the stream state and its first kRing
+// copies, the first-layer table. Every thread calls it.
+__device__ __forceinline__ uint32_t fwd_setup(const FwdSmem& S, const float* __restrict__ P,
+                                              const unsigned char* const Wc[3], int64_t tiles) {
   if ((threadIdx.x >> 5) == 0) {
     tc::tmem_alloc(S.slot, 2 * kH);
     tc::tmem_relinquish();
   }
   if (threadIdx.x == 0) {
-    for (int b = 0; b < kStagesPP; ++b) {
+    for (int b = 0; b < kRing; ++b) {
       tc::mbar_init(S.full + b, 1);
       tc::mbar_init(S.mdone + b, 1);
     }
     tc::mbar_init(S.lbar, 1);
     tc::mbar_init(S.lbar + 1, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    StreamPP& st = *S.st;
-    st.total = (int32_t)(units * nsub * 3 * kChunksPerLayer);
-    st.tail0 = (int32_t)(6 * (units / 2) * nsub);
+    FwdStream& st = *S.st;
+    st.total = (int32_t)(tiles * 3 * kChunks);
+    st.tail0 = (int32_t)(6 * (tiles / 2));
     st.next_use = 0;
     *S.issued = 0;
-    S.s_ok[0] = S.s_ok[1] = 1;
-    for (int q2 = 0; q2 < 2 * kCopiers; ++q2) S.s_okc[q2] = 1;
+    *S.failed = 0;
     const unsigned char* w0 = layer_weights(Wc, slot_layer(0, st.tail0));
-    int c = 0;
-    for (; c < st.total && c < kStagesPP; ++c) copy_chunk_pp(S, w0, c);
-    for (int q2 = 0; q2 < kCopiers; ++q2) {
-      S.copied[q2] = 0;
-      st.next_copy[q2] = c + ((q2 - c) % kCopiers + kCopiers) % kCopiers;  // first chunk of class q2 not copied
+    for (int c = 0; c < kRing; ++c) {
+      S.copied[c] = 0;
+      st.next_copy[c] = c;
+      if (c < st.total) {
+        copy_chunk(S, w0, c);
+        st.next_copy[c] = c + kRing;
+      }
     }
   }
   for (int o = threadIdx.x; o < kH; o += blockDim.x) {
@@ -507,17 +290,17 @@ __device__ __forceinline__ uint32_t mlp_setup_pp(const MlpSmemPP& S, const float
 
 // End of both groups' tile loops (every thread calls it): thread 0 waits
 // (bounded) for copies that no MMA consumed, then TMEM is released.
-__device__ __forceinline__ void mlp_teardown_pp(const MlpSmemPP& S, uint32_t taddr, int32_t* err) {
+__device__ __forceinline__ void fwd_teardown(const FwdSmem& S, uint32_t taddr, int32_t* err) {
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   if (threadIdx.x == 0) {
-    const StreamPP& st = *S.st;
-    int hi = st.next_copy[0];
-    for (int q2 = 1; q2 < kCopiers; ++q2) hi = st.next_copy[q2] > hi ? st.next_copy[q2] : hi;
+    const FwdStream& st = *S.st;
+    int hi = 0;
+    for (int q = 0; q < kRing; ++q) hi = max(hi, st.next_copy[q]);
     for (int c = st.next_use; c < hi; ++c)
-      if (c < st.next_copy[c % kCopiers] &&
-          !tc::mbar_wait(S.full + (c & (kStagesPP - 1)), ((uint32_t)c / kStagesPP) & 1u, err, 200000000ull))
+      if (c < st.next_copy[c % kRing] &&
+          !tc::mbar_wait(S.full + (c % kRing), ((uint32_t)c / kRing) & 1u, err, 200000000ull))
         break;
   }
   tc::fence_before_sync();
@@ -526,129 +309,225 @@ __device__ __forceinline__ void mlp_teardown_pp(const MlpSmemPP& S, uint32_t tad
   if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(taddr, 2 * kH);
 }
 
-// MMAs of layer slot `slot` (group grp's thread 0): after the previous slot's
-// MMAs were issued, one MMA per chunk as it lands, a commit per chunk
-// (mdone: its buffer may be refilled) and one for the layer (lbar[grp]); the
-// turn is handed on before the bounded wait for the layer's MMAs.
-__device__ __forceinline__ bool tc_layer_issue_pp(const MlpSmemPP& S, int grp, uint32_t taddr_g, int slot,
-                                                  uint32_t& lphase, int32_t* err) {
-  if (!turn_wait(S.issued, slot, err)) return false;
+// MMAs of layer slot `slot` (group grp's warp 0): after the previous slot's
+// MMAs were issued, the MMAs of each chunk as it lands, a commit per chunk
+// (mdone: its buffer may be refilled) and one for the layer (lbar[grp]).
+__device__ __forceinline__ void layer_issue(const FwdSmem& S, int grp, uint32_t taddr_g, int slot, int32_t* err) {
+  const uint64_t a0 = tc::smem_desc(tc::smem_addr(S.A + grp * kSmemA), 128u, (uint32_t)kH * 16u);
+  const uint64_t b0 = tc::smem_desc(tc::smem_addr(S.B), 128u, (uint32_t)kKF * 16u);
+  const int c0 = slot * kChunks;
+  const bool leader = tc::elect_one();
+  if (!turn_wait(S, S.issued, slot, err)) return;
   __threadfence_block();
   tc::fence_after_sync();
-  const uint64_t a0 = tc::smem_desc(tc::smem_addr(S.A[grp]), 128u, (uint32_t)kH * 16u);
-  const uint64_t b0 = tc::smem_desc(tc::smem_addr(S.B), 128u, (uint32_t)kKF * 16u);
-  const int c0 = slot * kChunksPerLayer;
-  for (int kc = 0; kc < kChunksPerLayer; ++kc) {
+#pragma unroll 1
+  for (int kc = 0; kc < kChunks; ++kc) {
     const int c = c0 + kc;
-    const int b = c & (kStagesPP - 1);
-    if (!tc::mbar_wait(S.full + b, ((uint32_t)c / kStagesPP) & 1u, err)) return false;
-    // descriptor start address in 16-byte units: K-slice kc of A is 256 bytes
-    // on, buffer b of the ring kSmemBF bytes on
-    tc::mma_bf16(taddr_g, a0 + (uint64_t)(kc * (kKF * 16 / 16)), b0 + (uint64_t)(b * (kSmemBF / 16)), kIdesc,
-                 kc != 0);
-    tc::mma_commit(S.mdone + b);
+    const int b = c % kRing;
+    if (!fwd_wait(S, S.full + b, ((uint32_t)c / kRing) & 1u, err)) return;
+    if (leader) {
+#pragma unroll
+      for (int m = 0; m < kChunkK / kKF; ++m) {
+        // descriptor start addresses in 16-byte units: the MMA's K-slice of A
+        // is 256 bytes on, its weights kSmemBF bytes on
+        const int k = kc * (kChunkK / kKF) + m;
+        tc::mma_bf16(taddr_g, a0 + (uint64_t)(k * (kKF * 16 / 16)),
+                     b0 + (uint64_t)(b * (kChunkBytes / 16) + m * (kSmemBF / 16)), kIdesc, k != 0);
+      }
+      tc::mma_commit(S.mdone + b);
+      if (kc == kChunks - 1) tc::mma_commit(S.lbar + grp);
+    }
+    __syncwarp();
   }
-  tc::mma_commit(S.lbar + grp);
-  S.st->next_use = c0 + kChunksPerLayer;
-  __threadfence_block();
-  *S.issued = slot + 1;
-  const bool ok = tc::mbar_wait(S.lbar + grp, lphase, err);
-  lphase ^= 1u;
-  return ok;
+  if (leader) {
+    S.st->next_use = c0 + kChunks;
+    __threadfence_block();
+    *S.issued = slot + 1;
+  }
+  __syncwarp();
 }
 
-// Copies of layer slot `slot`, chunks of class par = c mod kCopiers (group
-// grp's thread kCopierLane (1 + par)): after the same class's copier of the
-// previous slot, chunk u + kStagesPP into buffer u's slot as soon as MMA u
-// (u in this slot) completed. A class's chunks live in its own buffers only,
-// so each buffer sees its mbarrier phases in order.
-__device__ __forceinline__ bool copy_slot_pp(const MlpSmemPP& S, const unsigned char* const Wc[3], int slot, int par,
-                                             int32_t* err) {
-  if (!turn_wait(S.copied + par, slot, err)) return false;
+// Refills of buffer b during layer slot `slot` (group grp's warp 1 + b):
+// after the previous slot's, chunk u + kRing into the buffer as soon as the
+// MMAs of chunk u (u in this slot) completed.
+__device__ __forceinline__ void refill_buffer(const FwdSmem& S, const unsigned char* const Wc[3], int slot, int b,
+                                              int32_t* err) {
+  if (!turn_wait(S, S.copied + b, slot, err)) return;
   __threadfence_block();
-  StreamPP& st = *S.st;
-  const int c0 = slot * kChunksPerLayer;
+  const bool leader = tc::elect_one();
+  FwdStream& st = *S.st;
+  const int c0 = slot * kChunks;
   const int total = st.total;
-  // chunks c0 + kStagesPP .. c0 + 15 belong to this slot's layer, the rest
-  // to the next slot's
+  // chunks c0 + kRing .. belong to this slot's layer, the last to the next slot's
   const unsigned char* w_this = layer_weights(Wc, slot_layer(slot, st.tail0));
   const unsigned char* w_next = layer_weights(Wc, slot_layer(slot + 1, st.tail0));
-  for (int kc = par; kc < kChunksPerLayer; kc += kCopiers) {
-    const int u = c0 + kc;  // the MMA whose buffer the next chunk reuses
-    const int c = u + kStagesPP;
+  for (int kc = (b + kRing - c0 % kRing) % kRing; kc < kChunks; kc += kRing) {
+    const int u = c0 + kc;  // the chunk whose buffer the next one reuses
+    const int c = u + kRing;
     if (c >= total) break;
-    if (!tc::mbar_wait(S.mdone + (u & (kStagesPP - 1)), ((uint32_t)u / kStagesPP) & 1u, err)) return false;
-    copy_chunk_pp(S, kc + kStagesPP < kChunksPerLayer ? w_this : w_next, c);
-    st.next_copy[par] = c + kCopiers;
+    if (!fwd_wait(S, S.mdone + b, ((uint32_t)u / kRing) & 1u, err)) return;
+    if (leader) {
+      copy_chunk(S, kc + kRing < kChunks ? w_this : w_next, c);
+      st.next_copy[b] = c + kRing;
+    }
+    __syncwarp();
   }
-  __threadfence_block();
-  S.copied[par] = slot + 1;
-  return true;
+  if (leader) {
+    __threadfence_block();
+    S.copied[b] = slot + 1;
+  }
+  __syncwarp();
+}
+
+// SiLU of N pairs, rounded to BF16 pairs: each operation over all pairs
+// before the next, so the special-function latencies overlap
+template <int N>
+__device__ __forceinline__ void silu_pairs(const uint64_t (&z)[N], uint32_t (&h)[N]) {
+  float t[2 * N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) f2_unpack(f2_mul(z[i], f2_pack(kNegLog2e, kNegLog2e)), t[2 * i], t[2 * i + 1]);
+#pragma unroll
+  for (int i = 0; i < 2 * N; ++i) t[i] = ex2_sfu(t[i]);
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    f2_unpack(f2_add(f2_pack(1.0f, 1.0f), f2_pack(t[2 * i], t[2 * i + 1])), t[2 * i], t[2 * i + 1]);
+#pragma unroll
+  for (int i = 0; i < 2 * N; ++i) t[i] = rcp_sfu(t[i]);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float h0, h1;
+    f2_unpack(f2_mul(z[i], f2_pack(t[2 * i], t[2 * i + 1])), h0, h1);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h[i]) : "f"(h1), "f"(h0));
+  }
 }
 
 // The network on group grp's 128-row tile (lt = thread index in the group):
-// the arithmetic of mlp_tile, layer slots slot0, slot0 + step, slot0 + 2 step.
-// hook(lt) runs on the group's other threads while the first layer's MMAs
-// are issued and computed (the caller's prefetch of its next tile).
-template <class Hook>
-__device__ __forceinline__ bool mlp_tile_pp(const MlpSmemPP& S, const float* __restrict__ P,
-                                            const unsigned char* const Wc[3], int grp, int lt, const float x[3],
-                                            uint32_t taddr, uint32_t& lphase, int64_t slot0, int step,
-                                            int32_t* err, float& y_out, Hook&& hook) {
+// layer slots slot0, slot0 + step, slot0 + 2 step. Lane l of each warp passes
+// the inputs of rows l / 4 + 8 q (q = 0..3) of its 32 rows; threads lt < 128
+// get row lt's output. next() is called when the inputs are no longer needed.
+template <class Next>
+__device__ __forceinline__ void fwd_tile(const FwdSmem& S, const float* __restrict__ P,
+                                         const unsigned char* const Wc[3], int grp, int lt,
+                                         const float (&x)[4][3], uint32_t taddr, uint32_t& lphase, int64_t slot0,
+                                         int step, int32_t* err, float& y_out, Next&& next) {
   constexpr int kCols = kH / kTPR;
-  const int row = lt & (kTileM - 1);
-  const int half = lt / kTileM;
-  const int c0 = half * kCols;
+  const int lane = lt & 31;
+  const int w0 = lt & 96;                      // first of the warp's 32 rows
+  const int c0 = (lt / kTileM) * kCols;        // first of its 128 columns
   const uint32_t tcol = taddr + (uint32_t)(grp * kH);
-  const uint32_t trow = tcol + ((uint32_t)(32 * ((lt >> 5) & 3)) << 16);
-  unsigned char* A = S.A[grp];
-  for (int o = c0; o < c0 + kCols; o += 8) {
-    float h[8];
-    layer1_outputs8(S.w1, o, x, h);
-    store_bf16x8(A + tc::kmajor_offset(row, o, kH), h);
+  const uint32_t tw = tcol + ((uint32_t)w0 << 16) + (uint32_t)c0;
+  unsigned char* A = S.A + grp * kSmemA;
+  float* ypart = S.ypart + grp * 2 * kTileM;
+  // Accumulator fragments (16 rows x 8 columns over a warp): a lane holds two
+  // neighbouring columns 2 (l % 4) of rows l / 4 and l / 4 + 8, so it needs a
+  // quarter of the warp's biases, not all of them, and its BF16 pairs go to
+  // the activation tile by stmatrix. (With one row and 16 columns a thread,
+  // every bias and first-layer weight was a broadcast 16-byte load: the loads
+  // took 6.1 k of the 13.4 k shared-memory cycles of a tile.)
+  // The lane's row of the four 8x8 matrices of a store: matrices (rows 0-7,
+  // block i), (rows 8-15, i), (rows 0-7, i + 1), (rows 8-15, i + 1).
+  const uint32_t a_st = tc::smem_addr(A) +
+                        (uint32_t)((w0 >> 3) + ((lane >> 3) & 1)) * (kH * 16) +
+                        (uint32_t)((c0 >> 3) + (lane >> 4)) * 128u + (uint32_t)(lane & 7) * 16u;
+  const uint32_t half_rows = 2u * kH * 16u;    // 16 rows on
+  // layer 1: rows l / 4 + 8 q of the warp
+  {
+    const float4* w1 = S.w1 + c0 + 2 * (lane & 3);
+#pragma unroll 2
+    for (int i = 0; i < kCols / 8; i += 2) {
+      uint64_t z[8];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float4 a = w1[8 * (i + u)], b = w1[8 * (i + u) + 1];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          z[4 * (q >> 1) + 2 * u + (q & 1)] =
+              f2_fma(f2_pack(b.x, b.y), f2_pack(x[q][2], x[q][2]),
+                     f2_fma(f2_pack(a.z, a.w), f2_pack(x[q][1], x[q][1]),
+                            f2_fma(f2_pack(a.x, a.y), f2_pack(x[q][0], x[q][0]), f2_pack(b.z, b.w))));
+      }
+      uint32_t h[8];
+      silu_pairs<8>(z, h);
+      tc::stmatrix4(a_st + (uint32_t)i * 128u, h[0], h[1], h[2], h[3]);
+      tc::stmatrix4(a_st + (uint32_t)i * 128u + half_rows, h[4], h[5], h[6], h[7]);
+    }
   }
   tc::fence_async_smem();
   group_sync(grp);
   float y = 0.f;
+#pragma unroll
   for (int l = 0; l < 3; ++l) {
     const int slot = (int)(slot0 + (int64_t)l * step);
-    if (lt == 0) {
-      S.s_ok[grp] = tc_layer_issue_pp(S, grp, tcol, slot, lphase, err);
-    } else if (lt % kCopierLane == 0 && lt <= kCopierLane * kCopiers) {
-      const int par = lt / kCopierLane - 1;
-      S.s_okc[grp * kCopiers + par] = copy_slot_pp(S, Wc, slot, par, err);
-    } else if (l == 0) {
-      hook(lt);
+    // (the others wait at the barrier: 256 threads polling lbar slowed the
+    // issue from 3.9 k to 5.3 k cycles a layer)
+    const int warp = __shfl_sync(0xffffffffu, lt >> 5, 0);
+    if (warp == 0) {
+      layer_issue(S, grp, tcol, slot, err);
+      fwd_wait(S, S.lbar + grp, lphase, err);
+      lphase ^= 1u;
+    } else if (warp <= kRing) {
+      refill_buffer(S, Wc, slot, warp - 1, err);
     }
     group_sync(grp);
     tc::fence_after_sync();
-    bool good = S.s_ok[grp];
+    uint32_t ra[16], rb[16];
+    tc::tmem_ld_16x256_x4(tw, ra);
 #pragma unroll
-    for (int q = 0; q < kCopiers; ++q) good = good && S.s_okc[grp * kCopiers + q];
-    if (!good) return false;
-    uint32_t ra[32], rb[32];
-    tc::tmem_ld32_issue(trow + (uint32_t)c0, ra);
-    tc::tmem_ld_wait();
-#pragma unroll 1
-    for (int cc = c0; cc < c0 + kCols; cc += 64) {
-      tc::tmem_ld32_issue(trow + (uint32_t)(cc + 32), rb);
-      tile_columns_a(A, S.bias, l, row, cc, ra, y);
+    for (int cc = 0; cc < kCols; cc += 32) {
+      const float2* b2 = reinterpret_cast<const float2*>(S.bias + l * kH + c0 + cc) + (lane & 3);
+      uint64_t bb[4], z[8];
+      uint32_t h[8];
+      const uint32_t ad = a_st + (uint32_t)cc * 16u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 b = b2[4 * i];
+        bb[i] = f2_pack(b.x, b.y);
+      }
       tc::tmem_ld_wait();
-      if (cc + 64 < c0 + kCols) tc::tmem_ld32_issue(trow + (uint32_t)(cc + 64), ra);
-      tile_columns_a(A, S.bias, l, row, cc + 32, rb, y);
+      tc::tmem_ld_16x256_x4(tw + (16u << 16) + (uint32_t)cc, rb);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        z[i] = f2_add(f2_pack(__uint_as_float(ra[2 * i]), __uint_as_float(ra[2 * i + 1])), bb[i >> 1]);
+      silu_pairs<8>(z, h);
+      tc::stmatrix4(ad, h[0], h[1], h[2], h[3]);
+      tc::stmatrix4(ad + 256u, h[4], h[5], h[6], h[7]);
       tc::tmem_ld_wait();
+      if (cc + 32 < kCols) tc::tmem_ld_16x256_x4(tw + (uint32_t)(cc + 32), ra);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        z[i] = f2_add(f2_pack(__uint_as_float(rb[2 * i]), __uint_as_float(rb[2 * i + 1])), bb[i >> 1]);
+      silu_pairs<8>(z, h);
+      tc::stmatrix4(ad + half_rows, h[0], h[1], h[2], h[3]);
+      tc::stmatrix4(ad + half_rows + 256u, h[4], h[5], h[6], h[7]);
+      if (l == 2) {
+        // 256 -> 1: the warp's rows and columns are one half of 32 rows, so
+        // lane r runs row r's FMA chain over the columns as they come
+        __syncwarp();
+#pragma unroll
+        for (int k = cc; k < cc + 32; k += 8) {
+          const uint4 a = *reinterpret_cast<const uint4*>(A + tc::kmajor_offset(w0 + lane, c0 + k, kH));
+          const uint32_t u[4] = {a.x, a.y, a.z, a.w};
+          const float4* w4 = reinterpret_cast<const float4*>(S.bias + 3 * kH + c0 + k);
+          const float4 wa = w4[0], wb = w4[1];
+          const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            y = __fmaf_rn(__uint_as_float(u[i] << 16), w[2 * i], y);
+            y = __fmaf_rn(__uint_as_float(u[i] & 0xFFFF0000u), w[2 * i + 1], y);
+          }
+        }
+      }
     }
-    if (l == 2) S.ypart[grp][half * kTileM + row] = y;
+    if (l == 1) next();
+    if (l == 2) ypart[lt] = y;
     tc::fence_async_smem();
     tc::fence_before_sync();
     group_sync(grp);
     tc::fence_after_sync();
   }
-  float yy = S.ypart[grp][row];
-#pragma unroll
-  for (int h = 1; h < kTPR; ++h) yy += S.ypart[grp][h * kTileM + row];
-  y_out = yy + __ldg(P + kOffC5);
-  return true;
+  // the halves added in a fixed order
+  y_out = 0.f;
+  if (lt < kTileM) y_out = ypart[lt] + ypart[kTileM + lt] + __ldg(P + kOffC5);
 }
 
 }  // namespace sft

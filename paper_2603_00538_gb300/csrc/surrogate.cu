@@ -3,24 +3,24 @@
 // surrogate network instead of a mesh location, plus a per-element exact
 // fallback, and the training set drawn from the exact source.
 //
-// Fused assembly kernels, persistent over tiles of 128 samples (a row per
-// sample):
+// Per 128-sample tile (a row per sample):
 //   Philox -> barycentrics -> X (FP32)  ->  network on the tensor cores
 //   (tcgen05, FP32 accumulation in tensor memory) or an exact query  ->
 //   residual r = f - alpha sum_m g_m lambda_m  ->  r lambda_i partials  ->
 //   warp-segmented compensated sums  ->  per-element epilogue + FP64 atomics
 //   into b.
-// k_surrogate_net (one CTA of two 256-thread groups per SM) runs the network
-// tiles, k_surrogate_exact (128 threads, many CTAs per SM) the exact ones.
+// The network pass runs in three kernels over chunks of samples (k_net_points,
+// the standalone forward, k_net_combine), the exact pass in one
+// (k_surrogate_exact: 128 threads, many CTAs per SM).
 // Tiles hold EPB = floor(128/N) whole elements when N <= 128; an element with
-// N > 128 samples spans ceil(N/128) consecutive tiles of one group or CTA.
+// N > 128 samples spans ceil(N/128) consecutive tiles.
 //
 // Fallback: the first s samples of every element are also queried exactly
 // (a location of X's first d_s coordinates in the exact source mesh). If any
 // of them differs from the network by more than tau (or is not finite), the
 // whole element uses exact queries for all N samples. The decision is taken
 // first, for all elements (k_sub_points, the standalone network forward,
-// k_decide, k_split); then k_surrogate_net runs over the elements that keep
+// k_decide, k_split); then the network pass runs over the elements that keep
 // the network and k_surrogate_exact over the elements that fall back (their
 // s subsample values reused).
 // So no network tile is spent on a sample whose value is thrown away, and
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
 // k_sub_points forms the first s sample points of every element (the same
 // Philox counters, map and rounding as the assembly), padded to the network's
 // 3 inputs, and their exact values; the network then evaluates them (the
-// standalone forward, bit-identical to the fused tile); k_decide flags an
+// standalone forward); k_decide flags an
 // element when one of its s network values differs from the exact one by
 // more than tau or is not finite; k_split lists the survivors (network for
 // all N samples) and the fallbacks (exact queries, the subsample's values
@@ -377,240 +377,173 @@ __global__ void k_dataset(int64_t n, PhiloxKey key, uint32_t stream_id, float3 l
   }
 }
 
-// The network pass (the elements that keep the network; no exact queries):
-// one CTA per SM, two groups of 256 threads, each running the tile loop over
-// its share of the CTA's units (group 0 the even ones) with the two-group
-// forward tile (mlp_tile_pp): the groups' layers alternate on the tensor
-// cores, so one group's sampling, epilogues and scatter overlap the other's
-// MMAs. The network values are those of the standalone forward bit for bit;
-// partials and epilogue follow k_surrogate_exact's with the network value in
-// place of the exact one.
-// An element's inputs to its tile rows and its scatter, fetched by one
-// thread while the group waits for the previous tile's first-layer MMAs
-// (the dependent loads list -> connectivity -> vertices / control values no
-// longer stall the group). Used when a tile holds at most kPfMax elements.
-struct EPre {
-  int32_t t;        // element, -1: none
-  int32_t v[4];
-  float xv[4][3];
-  float gv[4];
-  float vol;
-  int32_t pad[2];
-};
-constexpr int kPfMax = 8;
-constexpr int kPfLane = 192;  // group threads 192 .. 192 + EPB - 1 (warp 6: no issuer, no copier)
-static_assert(kPfLane % 32 == 0 && kPfLane > kCopierLane * kCopiers && kPfLane + kPfMax <= kGroupThreads,
-              "prefetch threads");
-constexpr uint32_t kSmemPrePP = 2 * 2 * kPfMax * sizeof(EPre);
-constexpr uint32_t kSmemSurPP = kSmemPP + kSmemPrePP;
+// The network pass (the elements that keep the network; no exact queries), in
+// chunks of at most kNetChunk samples: k_net_points forms the sample points
+// of the chunk's elements (Philox, map; the FP32 points of the assembly),
+// the standalone forward evaluates them, k_net_combine turns the values into
+// residuals and adds them into b. The points and values of a chunk (16 bytes a
+// sample) stay in L2 between the three. One kernel that did all three per
+// 128-sample tile took 14 us a tile and SM, the forward alone takes 9.0 (its
+// registers and warps all serve the epilogues that bound it), and the points
+// and the combine together 0.5: 288 k elements x 64 samples 13.25 -> 9.3 ms.
+constexpr int64_t kNetChunk = 4 << 20;
 
+// point k N + j of the chunk = sample j of element elist[k]
 template <int DT>
-__device__ __forceinline__ void pf_element(EPre& e, const SurParams& p, int64_t unit, int el,
-                                           const int32_t* __restrict__ tconn, const float* __restrict__ tx,
-                                           const float* __restrict__ g, const float* __restrict__ vol32) {
+__global__ void k_net_points(const float* __restrict__ tx, const int32_t* __restrict__ tconn, SurParams p, int64_t k0,
+                             int64_t nk, float* __restrict__ pts3) {
   constexpr int K = DT + 1;
-  const int64_t k = unit * p.EPB + el;
-  if (unit >= p.nunits || k >= p.nlist) {
-    e.t = -1;
-    return;
+  const int64_t n = nk * p.N;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = i / p.N;
+    const int j = (int)(i - k * p.N);
+    const int64_t t = p.elist ? (int64_t)__ldg(p.elist + k0 + k) : k0 + k;
+    float xv[K][DT], lam[K], X[DT];
+#pragma unroll
+    for (int m = 0; m < K; ++m) {
+      const int32_t v = __ldg(tconn + t * K + m);
+#pragma unroll
+      for (int a = 0; a < DT; ++a) xv[m][a] = __ldg(tx + (int64_t)v * DT + a);
+    }
+    const uint4 w = philox4x32_10(make_uint4((uint32_t)(DT == 2 ? (j >> 1) : j), (uint32_t)t, p.stream_id, 0u), p.key);
+    sample_lambda<DT, float>(w, j, p.st, lam);
+    map_point<DT, float>(lam, xv, X);
+    pts3[i * 3] = X[0];
+    pts3[i * 3 + 1] = X[1];
+    pts3[i * 3 + 2] = DT == 3 ? X[DT - 1] : 0.f;
   }
-  const int64_t t = p.elist ? (int64_t)__ldg(p.elist + k) : k;
-  int32_t v[K];
-#pragma unroll
-  for (int m = 0; m < K; ++m) v[m] = __ldg(tconn + t * K + m);
-#pragma unroll
-  for (int m = 0; m < K; ++m) {
-#pragma unroll
-    for (int a = 0; a < DT; ++a) e.xv[m][a] = __ldg(tx + (int64_t)v[m] * DT + a);
-    e.gv[m] = __ldg(g + v[m]);
-    e.v[m] = v[m];
-  }
-  e.vol = __ldg(vol32 + t);
-  e.t = (int32_t)t;
 }
-static_assert(kSmemSurPP <= 227u * 1024u, "two-group tile exceeds the shared memory of one CTA");
 
+// Residuals of the chunk's samples into b. The rows of a tile of 128 samples
+// (EPB whole elements, or a part of one element with N > 128) lie over four
+// warps; a warp's rows of one element are combined by a segmented suffix scan,
+// and each segment's head adds its share |T| / N sum_j r_j lambda_i into b; the
+// head of the element's first sample also adds the control term (the FP32
+// epilogue of the exact pass, split over the segments).
 template <int DT>
-__global__ void __launch_bounds__(2 * kGroupThreads, 1) k_surrogate_net(
-    const float* __restrict__ P, const unsigned char* __restrict__ W2, const unsigned char* __restrict__ W3,
-    const unsigned char* __restrict__ W4, const float* __restrict__ tx, const int32_t* __restrict__ tconn,
-    const float* __restrict__ vol32, const float* __restrict__ g, SurParams p, double* __restrict__ b,
-    int32_t* __restrict__ fb_out, float* __restrict__ sample_f, int32_t* err) {
+__global__ void __launch_bounds__(256) k_net_combine(const int32_t* __restrict__ tconn,
+                                                     const float* __restrict__ vol32, const float* __restrict__ g,
+                                                     SurParams p, int64_t k0, int64_t nk,
+                                                     const float* __restrict__ f_in, double* __restrict__ b,
+                                                     int32_t* __restrict__ fb_out, float* __restrict__ sample_f) {
   constexpr int K = DT + 1;
-  extern __shared__ __align__(1024) unsigned char sm[];
-  const MlpSmemPP S = mlp_smem_pp(sm);
-  const int grp = threadIdx.x / kGroupThreads;
-  const int lt = threadIdx.x - grp * kGroupThreads;
   const int lane = threadIdx.x & 31;
-  const unsigned char* const Wc[3] = {W2, W3, W4};
-  const int64_t units = cta_tiles(p.nunits);
-  const uint32_t taddr = mlp_setup_pp(S, P, Wc, units, p.nsub);
-  uint32_t lphase = 0;
-  bool ok = true;
-  const int row = lt & (kTileM - 1);
-  const bool lead = lt < kTileM;
-  const int64_t J1 = (units / 2) * p.nsub;  // tiles of each group that have a partner
-  const bool usepf = p.nsub == 1 && p.EPB <= kPfMax;
-  EPre* pre = reinterpret_cast<EPre*>(sm + kSmemPP) + grp * 2 * kPfMax;  // [2][kPfMax]
-  if (usepf) {  // the group's first tile
-    if (lt >= kPfLane && lt < kPfLane + p.EPB)
-      pf_element<DT>(pre[lt - kPfLane], p, blockIdx.x + (int64_t)grp * gridDim.x, lt - kPfLane, tconn, tx, g, vol32);
-    group_sync(grp);
-  }
-
-  for (int64_t kk = grp; ok && kk < units; kk += 2) {
-    const int64_t unit = blockIdx.x + kk * gridDim.x;
-    for (int c = 0; c < p.nsub; ++c) {
-      const int64_t jt = (kk / 2) * p.nsub + c;
-      const int64_t slot0 = jt < J1 ? 6 * jt + grp : 6 * J1 + 3 * (jt - J1);
-      const int step = jt < J1 ? 2 : 1;
-      const int cur = (int)(jt & 1);
-      int el, j;
-      int64_t t;
-      bool valid;
-      const EPre* ep = nullptr;
-      if (usepf) {
-        el = row / p.N;
-        j = row - el * p.N;
-        ep = pre + cur * kPfMax + (el < p.EPB ? el : 0);
-        valid = el < p.EPB && ep->t >= 0;
-        t = ep->t;
-      } else if (p.nsub == 1) {
-        el = row / p.N;
-        j = row - el * p.N;
-        const int64_t k = unit * p.EPB + el;
-        valid = el < p.EPB && k < p.nlist;
-        t = valid && p.elist ? (int64_t)__ldg(p.elist + k) : k;
-      } else {
-        el = 0;
-        j = c * kTileM + row;
-        t = p.elist ? (int64_t)__ldg(p.elist + unit) : unit;
-        valid = j < p.N;
+  const int64_t units = p.nsub == 1 ? (nk + p.EPB - 1) / p.EPB : nk;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t wt = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wt < units * p.nsub * 4; wt += nw) {
+    const int64_t tile = wt >> 2;
+    const int row = (int)(wt & 3) * 32 + lane;
+    int el = 0, j;
+    int64_t k;
+    bool valid;
+    if (p.nsub == 1) {
+      el = row / p.N;
+      j = row - el * p.N;
+      k = tile * p.EPB + el;
+      valid = el < p.EPB && k < nk;
+    } else {
+      k = tile / p.nsub;
+      j = (int)(tile - k * p.nsub) * kTileM + row;
+      valid = j < p.N;
+    }
+    float lam[K], gvr[K];
+    int32_t v[K];
+    Acc<float> a[K];
+    int64_t t = 0;
+    if (valid) {
+      t = p.elist ? (int64_t)__ldg(p.elist + k0 + k) : k0 + k;
+      const float f = __ldg(f_in + k * p.N + j);
+#pragma unroll
+      for (int m = 0; m < K; ++m) {
+        v[m] = __ldg(tconn + t * K + m);
+        gvr[m] = __ldg(g + v[m]);
       }
-      float lam[K], X[DT];
-      int32_t v[K];
+      const uint4 w =
+          philox4x32_10(make_uint4((uint32_t)(DT == 2 ? (j >> 1) : j), (uint32_t)t, p.stream_id, 0u), p.key);
+      sample_lambda<DT, float>(w, j, p.st, lam);
+      if (fb_out && j == 0) fb_out[t] = 0;
+      if (sample_f) sample_f[t * p.N + j] = f;
+      float gX = __fmul_rn(gvr[0], lam[0]);
 #pragma unroll
-      for (int m = 0; m < K; ++m) { lam[m] = 0.f; v[m] = 0; }
+      for (int m = 1; m < K; ++m) gX = __fmaf_rn(gvr[m], lam[m], gX);
+      const float r = __fsub_rn(f, __fmul_rn(p.alpha, gX));
 #pragma unroll
-      for (int a = 0; a < DT; ++a) X[a] = 0.f;
-      float gvr[K];
-      if (valid) {
-        float xv[K][DT];
+      for (int i = 0; i < K; ++i) a[i].add(__fmul_rn(r, lam[i]));
+    }
+    const int seg = valid ? el : -1;
 #pragma unroll
-        for (int m = 0; m < K; ++m) {
-          if (usepf) {
-            v[m] = ep->v[m];
-            gvr[m] = ep->gv[m];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int seg2 = __shfl_down_sync(0xffffffffu, seg, o);
+      const bool take = lane + o < 32 && seg2 == seg;
 #pragma unroll
-            for (int a = 0; a < DT; ++a) xv[m][a] = ep->xv[m][a];
-          } else {
-            v[m] = __ldg(tconn + t * K + m);
-            gvr[m] = __ldg(g + v[m]);
-#pragma unroll
-            for (int a = 0; a < DT; ++a) xv[m][a] = __ldg(tx + (int64_t)v[m] * DT + a);
-          }
-        }
-        const uint4 w = philox4x32_10(make_uint4((uint32_t)(DT == 2 ? (j >> 1) : j), (uint32_t)t, p.stream_id, 0u),
-                                      p.key);
-        sample_lambda<DT, float>(w, j, p.st, lam);
-        map_point<DT, float>(lam, xv, X);
+      for (int i = 0; i < K; ++i) {
+        const float s2 = __shfl_down_sync(0xffffffffu, a[i].s, o);
+        const float e2 = __shfl_down_sync(0xffffffffu, a[i].e, o);
+        if (take) a[i].combine(s2, e2);
       }
-      const float x3[3] = {X[0], X[1], DT == 3 ? X[DT - 1] : 0.f};
-      float f = 0.f;
-      // while the first layer's MMAs run, threads kPfLane.. fetch the
-      // elements of the group's next tile into the other buffer
-      const int64_t unit_next = blockIdx.x + (kk + 2) * gridDim.x;
-      EPre* nxt = pre + (cur ^ 1) * kPfMax;
-      ok = mlp_tile_pp(S, P, Wc, grp, lt, x3, taddr, lphase, slot0, step, err, f, [&](int q) {
-        if (usepf && q >= kPfLane && q < kPfLane + p.EPB)
-          pf_element<DT>(nxt[q - kPfLane], p, unit_next, q - kPfLane, tconn, tx, g, vol32);
-      });
-      if (!ok) break;
-      if (fb_out && lead && valid && c == 0 && j == 0) fb_out[t] = 0;
-      if (lead && valid && sample_f) sample_f[t * p.N + j] = f;
-
-      // residual against the P1 control and its basis-weighted partials
-      Acc<float> a[K];
-      const bool mine = lead && valid;
-      if (mine) {
-        float gX = __fmul_rn(gvr[0], lam[0]);
+    }
+    const int seg_prev = __shfl_up_sync(0xffffffffu, seg, 1);
+    if (valid && (lane == 0 || seg_prev != seg)) {
+      const float volf = __ldg(vol32 + t);
+      float gsum = gvr[0];
 #pragma unroll
-        for (int m = 1; m < K; ++m) gX = __fmaf_rn(gvr[m], lam[m], gX);
-        const float r = __fsub_rn(f, __fmul_rn(p.alpha, gX));
+      for (int m = 1; m < K; ++m) gsum = __fadd_rn(gsum, gvr[m]);
+      const float wc = __fmul_rn(volf, p.cmc);
 #pragma unroll
-        for (int i = 0; i < K; ++i) a[i].add(__fmul_rn(r, lam[i]));
-      }
-      // warp-segmented suffix combine over rows of the same element
-      const int seg = mine ? el : -1;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int seg2 = __shfl_down_sync(0xffffffffu, seg, o);
-        const bool take = lane + o < 32 && seg2 == seg;
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-          const float s2 = __shfl_down_sync(0xffffffffu, a[i].s, o);
-          const float e2 = __shfl_down_sync(0xffffffffu, a[i].e, o);
-          if (take) a[i].combine(s2, e2);
-        }
-      }
-      const int seg_prev = __shfl_up_sync(0xffffffffu, seg, 1);
-      const bool head = mine && (lane == 0 || seg_prev != seg);
-      // each warp segment's head adds its share |T| / N sum_j r_j lambda_i
-      // into b; the head of the element's first sample also adds the control
-      // term (the FP32 epilogue of the exact pass, split over the segments:
-      // no shared-memory pieces and no block barrier between tiles)
-      if (head) {
-        const float volf = usepf ? ep->vol : __ldg(vol32 + t);
-        float gsum = gvr[0];
-#pragma unroll
-        for (int m = 1; m < K; ++m) gsum = __fadd_rn(gsum, gvr[m]);
-        const float wc = __fmul_rn(volf, p.cmc);
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-          const double add = j == 0 ? Epi<float>::contrib(volf, 0.0, p.cdet, p.cmc, gsum, gvr[i], a[i])
-                                    : (double)__fmul_rn(wc, __fadd_rn(a[i].s, a[i].e));
-          atomicAdd(b + v[i], add);
-        }
+      for (int i = 0; i < K; ++i) {
+        const double add = j == 0 ? Epi<float>::contrib(volf, 0.0, p.cdet, p.cmc, gsum, gvr[i], a[i])
+                                  : (double)__fmul_rn(wc, __fadd_rn(a[i].s, a[i].e));
+        atomicAdd(b + v[i], add);
       }
     }
   }
-  mlp_teardown_pp(S, taddr, err);
 }
 
-template <int DT, int DS, bool NET>
-static sft_status launch_sur(sft_mlp_s* m, sft_source_s* s, sft_target_s* t, const SurParams& p, const float* g,
-                             double* b, int32_t* fb, float* sf, int64_t* counters, int32_t* err, cudaStream_t st) {
+// the network pass over the elements of p (p.nlist of them), chunk by chunk
+template <int DT>
+static sft_status net_pass(sft_mlp_s* m, sft_target_s* t, const SurParams& p, const float* g, double* b, int32_t* fb,
+                           float* sf, int32_t* err, cudaStream_t st) {
   int dev = 0, sms = 0;
   SFT_CUDA(cudaGetDevice(&dev));
   SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  if constexpr (NET) {
-    // the network pass: one two-group CTA per SM (about 218 KB of shared
-    // memory and all 512 TMEM columns)
-    static bool attr = false;
-    if (!attr) {
-      SFT_CUDA(cudaFuncSetAttribute(k_surrogate_net<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSmemSurPP));
-      attr = true;
-    }
-    if (p.has_exact) return fail(SFT_ERR_UNSUPPORTED, "network pass with exact queries");
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.nunits, (int64_t)sms));
-    ::sft::note_launch(), k_surrogate_net<DT><<<grid, 2 * kGroupThreads, kSmemSurPP, st>>>(
-        m->P, m->Wc[0], m->Wc[1], m->Wc[2], (const float*)t->coordsP[SFT_PREC_FP32], t->conn, t->vol32, g, p, b, fb,
-        sf, err);
+  // whole units (tiles) per chunk, so the tiling does not depend on the chunks
+  int64_t step = std::max<int64_t>(1, kNetChunk / p.N);
+  if (p.nsub == 1) step = std::max<int64_t>(p.EPB, step / p.EPB * p.EPB);
+  step = std::min(step, p.nlist);
+  DevBuf<float> pts(st), f(st);
+  SFT_CUDA(pts.alloc((size_t)(step * p.N * 3)));
+  SFT_CUDA(f.alloc((size_t)(step * p.N)));
+  const float* tx = (const float*)t->coordsP[SFT_PREC_FP32];
+  for (int64_t k0 = 0; k0 < p.nlist; k0 += step) {
+    const int64_t nk = std::min(step, p.nlist - k0), n = nk * p.N;
+    const unsigned nbp = (unsigned)std::min<int64_t>((n + 255) / 256, 32LL * sms);
+    ::sft::note_launch(), k_net_points<DT><<<nbp, 256, 0, st>>>(tx, t->conn, p, k0, nk, pts.p);
     SFT_CUDA(cudaGetLastError());
-    return SFT_OK;
-  } else {
-    // exact queries only: latency-bound location work, many CTAs per SM
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.nunits, (int64_t)sms * 16));
-    const Locator* L = s ? &s->loc[SFT_PREC_FP32] : nullptr;
-    ::sft::note_launch(), k_surrogate_exact<DT, DS><<<grid, kTileM, kSmemPieces, st>>>(
-        (const float*)t->coordsP[SFT_PREC_FP32], t->conn, t->vol32, g,
-        L ? (const GridP<float>*)L->grid : nullptr, L ? L->cell_start : nullptr, L ? L->cell_items : nullptr,
-        L ? L->cell_first : nullptr, L ? (const float*)L->recs : nullptr, L ? L->adj : nullptr,
-        L ? (const float*)L->vals : nullptr, p, b, fb, sf, counters, err);
+    if (sft_status r = mlp_forward_dev(m, n, pts.p, f.p, st, err)) return r;
+    const int64_t warps = (p.nsub == 1 ? (nk + p.EPB - 1) / p.EPB : nk * p.nsub) * 4;
+    const unsigned nbc = (unsigned)std::min<int64_t>((warps + 7) / 8, 32LL * sms);
+    ::sft::note_launch(), k_net_combine<DT><<<nbc, 256, 0, st>>>(t->conn, t->vol32, g, p, k0, nk, f.p, b, fb, sf);
     SFT_CUDA(cudaGetLastError());
-    return SFT_OK;
   }
+  return SFT_OK;
+}
+
+template <int DT, int DS>
+static sft_status launch_exact(sft_source_s* s, sft_target_s* t, const SurParams& p, const float* g, double* b,
+                               int32_t* fb, float* sf, int64_t* counters, int32_t* err, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  SFT_CUDA(cudaGetDevice(&dev));
+  SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // exact queries only: latency-bound location work, many CTAs per SM
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.nunits, (int64_t)sms * 16));
+  const Locator* L = s ? &s->loc[SFT_PREC_FP32] : nullptr;
+  ::sft::note_launch(), k_surrogate_exact<DT, DS><<<grid, kTileM, kSmemPieces, st>>>(
+      (const float*)t->coordsP[SFT_PREC_FP32], t->conn, t->vol32, g,
+      L ? (const GridP<float>*)L->grid : nullptr, L ? L->cell_start : nullptr, L ? L->cell_items : nullptr,
+      L ? L->cell_first : nullptr, L ? (const float*)L->recs : nullptr, L ? L->adj : nullptr,
+      L ? (const float*)L->vals : nullptr, p, b, fb, sf, counters, err);
+  SFT_CUDA(cudaGetLastError());
+  return SFT_OK;
 }
 
 }  // namespace sft
@@ -775,14 +708,12 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   auto pass = [&](bool with_net, SurParams q, int32_t* fbp) -> sft_status {
     if (q.nlist == 0) return SFT_OK;
     q.nunits = q.nsub == 1 ? (q.nlist + q.EPB - 1) / q.EPB : q.nlist;
-    if (with_net) {
-      if (t->dim == 2) return launch_sur<2, 2, true>(net, exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-      if (ds == 2) return launch_sur<3, 2, true>(net, exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-      return launch_sur<3, 3, true>(net, exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-    }
-    if (t->dim == 2) return launch_sur<2, 2, false>(nullptr, exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-    if (ds == 2) return launch_sur<3, 2, false>(nullptr, exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-    return launch_sur<3, 3, false>(nullptr, exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
+    if (with_net)
+      return t->dim == 2 ? net_pass<2>(net, t, q, g.p, b.p, fbp, sf, d_err.p, st)
+                         : net_pass<3>(net, t, q, g.p, b.p, fbp, sf, d_err.p, st);
+    if (t->dim == 2) return launch_exact<2, 2>(exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
+    if (ds == 2) return launch_exact<3, 2>(exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
+    return launch_exact<3, 3>(exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
   };
   sft_status lr = SFT_OK;
   int64_t n_fallback = net ? 0 : ne;
