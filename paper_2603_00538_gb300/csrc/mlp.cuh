@@ -15,7 +15,6 @@ namespace sft {
 
 constexpr int kH = 256;
 constexpr int kTileM = 128;
-constexpr int kKC = 64;  // K chunk of a streamed weight block (training GEMM)
 constexpr int kKF = 16;  // K of one MMA
 constexpr int kTPR = 2;  // forward tile: threads per activation row (each owns half of the columns)
 constexpr int64_t kOffW1 = 0, kOffC1 = kH * 3, kOffW2 = kOffC1 + kH, kOffC2 = kOffW2 + kH * kH,
@@ -24,7 +23,6 @@ constexpr int64_t kOffW1 = 0, kOffC1 = kH * 3, kOffW2 = kOffC1 + kH, kOffC2 = kO
                   kNParam = kOffC5 + 1;
 
 constexpr uint32_t kSmemA = kTileM * kH * 2;        // 64 KiB: activation tile (128 x 256 BF16)
-constexpr uint32_t kSmemB = kH * kKC * 2;           // 32 KiB (training GEMM chunk)
 constexpr uint32_t kSmemBF = kH * kKF * 2;          // 8 KiB: weights of one MMA (256 x 16 BF16)
 constexpr uint32_t kSmemW1 = kH * 16;               // 4 KiB: first layer (w1_table_entry)
 constexpr uint32_t kSmemBias = 4 * kH * 4;          // 4 KiB: c2, c3, c4, w5
@@ -73,13 +71,6 @@ __device__ __forceinline__ float silu_grad(float z) {
   return sg * __fmaf_rn(z, 1.0f - sg, 1.0f);
 }
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
-__device__ __forceinline__ void store_bf16x8(unsigned char* dst, const float* v) {
-  __align__(16) __nv_bfloat16 h[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) h[i] = __float2bfloat16_rn(v[i]);
-  *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h);
-}
 
 // The first layer in shared memory, pair-interleaved for the packed FMAs:
 // outputs 2m and 2m + 1 take entries 2m = {W1[2m][0], W1[2m+1][0], W1[2m][1],
@@ -141,7 +132,7 @@ static_assert(kSmemFwd <= 227u * 1024u, "forward tile exceeds the shared memory 
 
 struct FwdStream {
   int32_t total;             // chunks of the CTA's stream
-  int32_t tail0;             // first slot of the unpaired tile (6 x the paired tiles of a group)
+  int32_t tail0;             // first slot of the unpaired tile (2 x layers x the paired tiles of a group)
   int32_t next_use;          // chunks whose MMAs were issued
   int32_t next_copy[kRing];  // the next chunk copied into each buffer
 };
@@ -223,13 +214,22 @@ __device__ __forceinline__ bool fwd_wait(const FwdSmem& S, uint64_t* bar, uint32
   return true;
 }
 
-// layer of slot s in the two-group order
-__device__ __forceinline__ int slot_layer(int s, int tail0) { return s < tail0 ? (s % 6) >> 1 : (s - tail0) % 3; }
-
-// the weights of layer l (a select, not an indexed local array)
-__device__ __forceinline__ const unsigned char* layer_weights(const unsigned char* const Wc[3], int l) {
-  return l == 0 ? Wc[0] : (l == 1 ? Wc[1] : Wc[2]);
-}
+// the chunked weights of the NL tensor-core layers of a tile, in their order
+template <int NL>
+struct LayerWeights {
+  const unsigned char* w[NL];
+  // layer l (selects, not an indexed local array)
+  __device__ __forceinline__ const unsigned char* of(int l) const {
+    const unsigned char* r = w[0];
+#pragma unroll
+    for (int q = 1; q < NL; ++q) r = l == q ? w[q] : r;
+    return r;
+  }
+  // layer of slot s in the two-group order
+  __device__ __forceinline__ const unsigned char* of_slot(int s, int tail0) const {
+    return of(s < tail0 ? (s % (2 * NL)) >> 1 : (s - tail0) % NL);
+  }
+};
 __device__ __forceinline__ void copy_chunk(const FwdSmem& S, const unsigned char* layer_w, int c) {
   const int b = c % kRing;
   tc::mbar_arrive_expect_tx(S.full + b, kChunkBytes);
@@ -245,8 +245,9 @@ __device__ __forceinline__ int64_t cta_tiles(int64_t ntiles) {
 // Setup over the CTA's tiles, split between the groups (group 0 the even
 // ones): TMEM (512 columns), mbarriers, the stream state and its first kRing
 // copies, the first-layer table. Every thread calls it.
-__device__ __forceinline__ uint32_t fwd_setup(const FwdSmem& S, const float* __restrict__ P,
-                                              const unsigned char* const Wc[3], int64_t tiles) {
+template <int NL>
+__device__ __forceinline__ uint32_t fwd_setup(const FwdSmem& S, const float* __restrict__ P, const LayerWeights<NL>& Wc,
+                                              int64_t tiles) {
   if ((threadIdx.x >> 5) == 0) {
     tc::tmem_alloc(S.slot, 2 * kH);
     tc::tmem_relinquish();
@@ -260,12 +261,12 @@ __device__ __forceinline__ uint32_t fwd_setup(const FwdSmem& S, const float* __r
     tc::mbar_init(S.lbar + 1, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     FwdStream& st = *S.st;
-    st.total = (int32_t)(tiles * 3 * kChunks);
-    st.tail0 = (int32_t)(6 * (tiles / 2));
+    st.total = (int32_t)(tiles * NL * kChunks);
+    st.tail0 = (int32_t)(2 * NL * (tiles / 2));
     st.next_use = 0;
     *S.issued = 0;
     *S.failed = 0;
-    const unsigned char* w0 = layer_weights(Wc, slot_layer(0, st.tail0));
+    const unsigned char* w0 = Wc.of_slot(0, st.tail0);
     for (int c = 0; c < kRing; ++c) {
       S.copied[c] = 0;
       st.next_copy[c] = c;
@@ -350,7 +351,8 @@ __device__ __forceinline__ void layer_issue(const FwdSmem& S, int grp, uint32_t 
 // Refills of buffer b during layer slot `slot` (group grp's warp 1 + b):
 // after the previous slot's, chunk u + kRing into the buffer as soon as the
 // MMAs of chunk u (u in this slot) completed.
-__device__ __forceinline__ void refill_buffer(const FwdSmem& S, const unsigned char* const Wc[3], int slot, int b,
+template <int NL>
+__device__ __forceinline__ void refill_buffer(const FwdSmem& S, const LayerWeights<NL>& Wc, int slot, int b,
                                               int32_t* err) {
   if (!turn_wait(S, S.copied + b, slot, err)) return;
   __threadfence_block();
@@ -359,8 +361,8 @@ __device__ __forceinline__ void refill_buffer(const FwdSmem& S, const unsigned c
   const int c0 = slot * kChunks;
   const int total = st.total;
   // chunks c0 + kRing .. belong to this slot's layer, the last to the next slot's
-  const unsigned char* w_this = layer_weights(Wc, slot_layer(slot, st.tail0));
-  const unsigned char* w_next = layer_weights(Wc, slot_layer(slot + 1, st.tail0));
+  const unsigned char* w_this = Wc.of_slot(slot, st.tail0);
+  const unsigned char* w_next = Wc.of_slot(slot + 1, st.tail0);
   for (int kc = (b + kRing - c0 % kRing) % kRing; kc < kChunks; kc += kRing) {
     const int u = c0 + kc;  // the chunk whose buffer the next one reuses
     const int c = u + kRing;
@@ -401,113 +403,177 @@ __device__ __forceinline__ void silu_pairs(const uint64_t (&z)[N], uint32_t (&h)
   }
 }
 
-// The network on group grp's 128-row tile (lt = thread index in the group):
-// layer slots slot0, slot0 + step, slot0 + 2 step. Lane l of each warp passes
-// the inputs of rows l / 4 + 8 q (q = 0..3) of its 32 rows; threads lt < 128
-// get row lt's output. next() is called when the inputs are no longer needed.
-template <class Next>
-__device__ __forceinline__ void fwd_tile(const FwdSmem& S, const float* __restrict__ P,
-                                         const unsigned char* const Wc[3], int grp, int lt,
-                                         const float (&x)[4][3], uint32_t taddr, uint32_t& lphase, int64_t slot0,
-                                         int step, int32_t* err, float& y_out, Next&& next) {
-  constexpr int kCols = kH / kTPR;
-  const int lane = lt & 31;
-  const int w0 = lt & 96;                      // first of the warp's 32 rows
-  const int c0 = (lt / kTileM) * kCols;        // first of its 128 columns
-  const uint32_t tcol = taddr + (uint32_t)(grp * kH);
-  const uint32_t tw = tcol + ((uint32_t)w0 << 16) + (uint32_t)c0;
-  unsigned char* A = S.A + grp * kSmemA;
-  float* ypart = S.ypart + grp * 2 * kTileM;
-  // Accumulator fragments (16 rows x 8 columns over a warp): a lane holds two
-  // neighbouring columns 2 (l % 4) of rows l / 4 and l / 4 + 8, so it needs a
-  // quarter of the warp's biases, not all of them, and its BF16 pairs go to
-  // the activation tile by stmatrix. (With one row and 16 columns a thread,
-  // every bias and first-layer weight was a broadcast 16-byte load: the loads
-  // took 6.1 k of the 13.4 k shared-memory cycles of a tile.)
-  // The lane's row of the four 8x8 matrices of a store: matrices (rows 0-7,
-  // block i), (rows 8-15, i), (rows 0-7, i + 1), (rows 8-15, i + 1).
-  const uint32_t a_st = tc::smem_addr(A) +
-                        (uint32_t)((w0 >> 3) + ((lane >> 3) & 1)) * (kH * 16) +
-                        (uint32_t)((c0 >> 3) + (lane >> 4)) * 128u + (uint32_t)(lane & 7) * 16u;
-  const uint32_t half_rows = 2u * kH * 16u;    // 16 rows on
-  // layer 1: rows l / 4 + 8 q of the warp
-  {
-    const float4* w1 = S.w1 + c0 + 2 * (lane & 3);
+// A thread's place in its group's tile. Accumulator fragments (16 rows x 8
+// columns over a warp): a lane holds two neighbouring columns 2 (l % 4) of
+// rows l / 4 and l / 4 + 8, so it needs a quarter of the warp's biases, not
+// all of them, and its BF16 pairs go to the activation tile by stmatrix. (With
+// one row and 16 columns a thread, every bias and first-layer weight was a
+// broadcast 16-byte load: the loads took 6.1 k of the 13.4 k shared-memory
+// cycles of a tile.)
+struct TileLane {
+  static constexpr int kCols = kH / kTPR;
+  int grp, lt, lane, warp;
+  int w0;              // first of the warp's 32 rows
+  int c0;              // first of its 128 columns
+  uint32_t tcol, tw;   // TMEM: the group's accumulator, the warp's part of it
+  unsigned char* A;    // the group's activation tile
+  // the lane's row of the four 8x8 matrices of a store or load: matrices (rows
+  // 0-7, block i), (rows 8-15, i), (rows 0-7, i + 1), (rows 8-15, i + 1)
+  uint32_t a_st;
+  static constexpr uint32_t kHalfRows = 2u * kH * 16u;  // 16 rows on
+};
+__device__ __forceinline__ TileLane tile_lane(const FwdSmem& S, uint32_t taddr) {
+  TileLane t;
+  t.grp = threadIdx.x / kGroupThreads;
+  t.lt = threadIdx.x - t.grp * kGroupThreads;
+  t.lane = t.lt & 31;
+  t.warp = __shfl_sync(0xffffffffu, t.lt >> 5, 0);
+  t.w0 = t.lt & 96;
+  t.c0 = (t.lt / kTileM) * TileLane::kCols;
+  t.tcol = taddr + (uint32_t)(t.grp * kH);
+  t.tw = t.tcol + ((uint32_t)t.w0 << 16) + (uint32_t)t.c0;
+  t.A = S.A + t.grp * kSmemA;
+  t.a_st = tc::smem_addr(t.A) + (uint32_t)((t.w0 >> 3) + ((t.lane >> 3) & 1)) * (kH * 16) +
+           (uint32_t)((t.c0 >> 3) + (t.lane >> 4)) * 128u + (uint32_t)(t.lane & 7) * 16u;
+  return t;
+}
+
+// layer 1 of rows l / 4 + 8 q of the warp (inputs x[q]) into the activation tile
+__device__ __forceinline__ void tile_layer1(const FwdSmem& S, const TileLane& t, const float (&x)[4][3]) {
+  const float4* w1 = S.w1 + t.c0 + 2 * (t.lane & 3);
 #pragma unroll 2
-    for (int i = 0; i < kCols / 8; i += 2) {
-      uint64_t z[8];
+  for (int i = 0; i < TileLane::kCols / 8; i += 2) {
+    uint64_t z[8];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const float4 a = w1[8 * (i + u)], b = w1[8 * (i + u) + 1];
+    for (int u = 0; u < 2; ++u) {
+      const float4 a = w1[8 * (i + u)], b = w1[8 * (i + u) + 1];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          z[4 * (q >> 1) + 2 * u + (q & 1)] =
-              f2_fma(f2_pack(b.x, b.y), f2_pack(x[q][2], x[q][2]),
-                     f2_fma(f2_pack(a.z, a.w), f2_pack(x[q][1], x[q][1]),
-                            f2_fma(f2_pack(a.x, a.y), f2_pack(x[q][0], x[q][0]), f2_pack(b.z, b.w))));
-      }
-      uint32_t h[8];
-      silu_pairs<8>(z, h);
-      tc::stmatrix4(a_st + (uint32_t)i * 128u, h[0], h[1], h[2], h[3]);
-      tc::stmatrix4(a_st + (uint32_t)i * 128u + half_rows, h[4], h[5], h[6], h[7]);
+      for (int q = 0; q < 4; ++q)
+        z[4 * (q >> 1) + 2 * u + (q & 1)] =
+            f2_fma(f2_pack(b.x, b.y), f2_pack(x[q][2], x[q][2]),
+                   f2_fma(f2_pack(a.z, a.w), f2_pack(x[q][1], x[q][1]),
+                          f2_fma(f2_pack(a.x, a.y), f2_pack(x[q][0], x[q][0]), f2_pack(b.z, b.w))));
     }
+    uint32_t h[8];
+    silu_pairs<8>(z, h);
+    tc::stmatrix4(t.a_st + (uint32_t)i * 128u, h[0], h[1], h[2], h[3]);
+    tc::stmatrix4(t.a_st + (uint32_t)i * 128u + TileLane::kHalfRows, h[4], h[5], h[6], h[7]);
   }
+}
+
+// the activation tile is written: make it visible to the tensor cores
+__device__ __forceinline__ void tile_written(const TileLane& t) {
   tc::fence_async_smem();
-  group_sync(grp);
+  tc::fence_before_sync();
+  group_sync(t.grp);
+  tc::fence_after_sync();
+}
+
+// One tensor-core layer of the group's tile: warp 0 issues, warps 1 .. kRing
+// refill the ring, other(t) runs on the last warp; all meet when the layer's
+// MMAs are complete. (The others wait at the barrier: 256 threads polling lbar
+// slowed the issue from 3.9 k to 5.3 k cycles a layer.)
+template <int NL, class Other>
+__device__ __forceinline__ void tile_mma(const FwdSmem& S, const TileLane& t, const LayerWeights<NL>& Wc, int slot,
+                                         uint32_t& lphase, int32_t* err, Other&& other) {
+  static_assert(kRing < kGroupThreads / 32 - 1, "a warp per role");
+  if (t.warp == 0) {
+    layer_issue(S, t.grp, t.tcol, slot, err);
+    fwd_wait(S, S.lbar + t.grp, lphase, err);
+    lphase ^= 1u;
+  } else if (t.warp <= kRing) {
+    refill_buffer<NL>(S, Wc, slot, t.warp - 1, err);
+  } else if (t.warp == kGroupThreads / 32 - 1) {
+    other();
+  }
+  group_sync(t.grp);
+  tc::fence_after_sync();
+}
+
+// f(cc, hh, r): accumulator fragments of columns cc .. cc + 31 of the warp's,
+// rows 16 hh .. 16 hh + 15 (r as tc::tmem_ld_16x256_x4), the next loads in
+// flight meanwhile; pre(cc) before the wait for the first of them (bias loads)
+template <class Pre, class F>
+__device__ __forceinline__ void tile_fragments(const TileLane& t, Pre&& pre, F&& f) {
+  uint32_t ra[16], rb[16];
+  tc::tmem_ld_16x256_x4(t.tw, ra);
+#pragma unroll
+  for (int cc = 0; cc < TileLane::kCols; cc += 32) {
+    pre(cc);
+    tc::tmem_ld_wait();
+    tc::tmem_ld_16x256_x4(t.tw + (16u << 16) + (uint32_t)cc, rb);
+    f(cc, 0, ra);
+    tc::tmem_ld_wait();
+    if (cc + 32 < TileLane::kCols) tc::tmem_ld_16x256_x4(t.tw + (uint32_t)(cc + 32), ra);
+    f(cc, 1, rb);
+  }
+}
+
+// the lane's biases of 32 columns (bias: the layer's, at the first of them)
+__device__ __forceinline__ void load_bias(const TileLane& t, const float* bias, uint64_t (&bb)[4]) {
+  const float2* b2 = reinterpret_cast<const float2*>(bias) + (t.lane & 3);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 b = b2[4 * i];
+    bb[i] = f2_pack(b.x, b.y);
+  }
+}
+// acc + bias of eight column pairs
+__device__ __forceinline__ void add_bias(const uint64_t (&bb)[4], const uint32_t (&r)[16], uint64_t (&z)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    z[i] = f2_add(f2_pack(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), bb[i >> 1]);
+}
+
+// store of one fragment set to the activation tile
+__device__ __forceinline__ void put_fragments(const TileLane& t, int cc, int hh, const uint32_t (&h)[8]) {
+  const uint32_t ad = t.a_st + (uint32_t)cc * 16u + (hh ? TileLane::kHalfRows : 0u);
+  tc::stmatrix4(ad, h[0], h[1], h[2], h[3]);
+  tc::stmatrix4(ad + 256u, h[4], h[5], h[6], h[7]);
+}
+
+// inputs of rows l / 4 + 8 q of the warp's 32 in the tile that starts at point `first`
+__device__ __forceinline__ void tile_inputs(const TileLane& t, const float* __restrict__ pts, int64_t first, int64_t n,
+                                            float (&x)[4][3]) {
+  const int64_t i0 = first + t.w0 + (t.lane >> 2);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) x[q][a] = i0 + 8 * q < n ? __ldg(pts + (i0 + 8 * q) * 3 + a) : 0.f;
+}
+
+// The network on the group's 128-row tile: layer slots slot0, slot0 + step,
+// slot0 + 2 step. Lane l of each warp passes the inputs of rows l / 4 + 8 q
+// (q = 0..3) of its 32 rows; threads lt < 128 get row lt's output. next() is
+// called when the inputs are no longer needed.
+template <class Next>
+__device__ __forceinline__ void fwd_tile(const FwdSmem& S, const TileLane& t, const float* __restrict__ P,
+                                         const LayerWeights<3>& Wc, const float (&x)[4][3], uint32_t& lphase,
+                                         int64_t slot0, int step, int32_t* err, float& y_out, Next&& next) {
+  float* ypart = S.ypart + t.grp * 2 * kTileM;
+  tile_layer1(S, t, x);
+  tile_written(t);
   float y = 0.f;
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    const int slot = (int)(slot0 + (int64_t)l * step);
-    // (the others wait at the barrier: 256 threads polling lbar slowed the
-    // issue from 3.9 k to 5.3 k cycles a layer)
-    const int warp = __shfl_sync(0xffffffffu, lt >> 5, 0);
-    if (warp == 0) {
-      layer_issue(S, grp, tcol, slot, err);
-      fwd_wait(S, S.lbar + grp, lphase, err);
-      lphase ^= 1u;
-    } else if (warp <= kRing) {
-      refill_buffer(S, Wc, slot, warp - 1, err);
-    }
-    group_sync(grp);
-    tc::fence_after_sync();
-    uint32_t ra[16], rb[16];
-    tc::tmem_ld_16x256_x4(tw, ra);
-#pragma unroll
-    for (int cc = 0; cc < kCols; cc += 32) {
-      const float2* b2 = reinterpret_cast<const float2*>(S.bias + l * kH + c0 + cc) + (lane & 3);
-      uint64_t bb[4], z[8];
+    tile_mma<3>(S, t, Wc, (int)(slot0 + (int64_t)l * step), lphase, err, [] {});
+    uint64_t bb[4];
+    tile_fragments(t, [&](int cc) { load_bias(t, S.bias + l * kH + t.c0 + cc, bb); },
+                   [&](int cc, int hh, const uint32_t (&r)[16]) {
+      uint64_t z[8];
       uint32_t h[8];
-      const uint32_t ad = a_st + (uint32_t)cc * 16u;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 b = b2[4 * i];
-        bb[i] = f2_pack(b.x, b.y);
-      }
-      tc::tmem_ld_wait();
-      tc::tmem_ld_16x256_x4(tw + (16u << 16) + (uint32_t)cc, rb);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        z[i] = f2_add(f2_pack(__uint_as_float(ra[2 * i]), __uint_as_float(ra[2 * i + 1])), bb[i >> 1]);
+      add_bias(bb, r, z);
       silu_pairs<8>(z, h);
-      tc::stmatrix4(ad, h[0], h[1], h[2], h[3]);
-      tc::stmatrix4(ad + 256u, h[4], h[5], h[6], h[7]);
-      tc::tmem_ld_wait();
-      if (cc + 32 < kCols) tc::tmem_ld_16x256_x4(tw + (uint32_t)(cc + 32), ra);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        z[i] = f2_add(f2_pack(__uint_as_float(rb[2 * i]), __uint_as_float(rb[2 * i + 1])), bb[i >> 1]);
-      silu_pairs<8>(z, h);
-      tc::stmatrix4(ad + half_rows, h[0], h[1], h[2], h[3]);
-      tc::stmatrix4(ad + half_rows + 256u, h[4], h[5], h[6], h[7]);
-      if (l == 2) {
+      put_fragments(t, cc, hh, h);
+      if (l == 2 && hh == 1) {
         // 256 -> 1: the warp's rows and columns are one half of 32 rows, so
         // lane r runs row r's FMA chain over the columns as they come
         __syncwarp();
 #pragma unroll
         for (int k = cc; k < cc + 32; k += 8) {
-          const uint4 a = *reinterpret_cast<const uint4*>(A + tc::kmajor_offset(w0 + lane, c0 + k, kH));
+          const uint4 a = *reinterpret_cast<const uint4*>(t.A + tc::kmajor_offset(t.w0 + t.lane, t.c0 + k, kH));
           const uint32_t u[4] = {a.x, a.y, a.z, a.w};
-          const float4* w4 = reinterpret_cast<const float4*>(S.bias + 3 * kH + c0 + k);
+          const float4* w4 = reinterpret_cast<const float4*>(S.bias + 3 * kH + t.c0 + k);
           const float4 wa = w4[0], wb = w4[1];
           const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
@@ -517,26 +583,22 @@ __device__ __forceinline__ void fwd_tile(const FwdSmem& S, const float* __restri
           }
         }
       }
-    }
+    });
     if (l == 1) next();
-    if (l == 2) ypart[lt] = y;
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    group_sync(grp);
-    tc::fence_after_sync();
+    if (l == 2) ypart[t.lt] = y;
+    tile_written(t);
   }
   // the halves added in a fixed order
   y_out = 0.f;
-  if (lt < kTileM) y_out = ypart[lt] + ypart[kTileM + lt] + __ldg(P + kOffC5);
+  if (t.lt < kTileM) y_out = ypart[t.lt] + ypart[kTileM + t.lt] + __ldg(P + kOffC5);
 }
 
 }  // namespace sft
 
 struct sft_mlp_s {
   float* P = nullptr;                                  // FP32 parameters (master)
-  __nv_bfloat16* W[3] = {nullptr, nullptr, nullptr};   // BF16 copies of W2, W3, W4 ([out][in])
-  __nv_bfloat16* WT[3] = {nullptr, nullptr, nullptr};  // BF16 transposes ([in][out]) for the backward pass
-  unsigned char* Wc[3] = {nullptr, nullptr, nullptr};  // BF16 in the forward tile's chunked layout
+  unsigned char* Wc[3] = {nullptr, nullptr, nullptr};   // BF16 W2, W3, W4 in the tile's chunked layout
+  unsigned char* WTc[3] = {nullptr, nullptr, nullptr};  // BF16 transposes in the same layout (the backward pass)
   float* grad = nullptr;                               // FP32 gradient of the mean loss
   float* m1 = nullptr;                                 // Adam moments
   float* m2 = nullptr;

@@ -88,13 +88,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
-// ---- cp.async (16-byte global -> shared) ----
-__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src_gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // ---- descriptors ----
 // Shared-memory matrix descriptor, no swizzle, K-major canonical layout made
 // of 8-row x 16-byte core matrices: lbo = byte step between core matrices
@@ -108,11 +101,16 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   // base offset 0, leading-byte-offset mode 0, layout type 0 (no swizzle)
   return d;
 }
-// Instruction descriptor of kind::f16: D FP32, A and B BF16, both K-major.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
+// The same tile read with its other index as K (MN-major canonical layout: a
+// core matrix is 8 K rows of 8 contiguous M or N values): sbo = byte step
+// between core matrices along M (or N), lbo = along K.
+// Instruction descriptor of kind::f16: D FP32, A and B BF16, both K-major, or
+// both MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool mn_major = false) {
   return (1u << 4)                       // D format: F32
          | (1u << 7)                     // A format: BF16
          | (1u << 10)                    // B format: BF16
+         | (mn_major ? (3u << 15) : 0u)  // A and B MN-major
          | ((uint32_t)(N >> 3) << 17)    // N / 8
          | ((uint32_t)(M >> 4) << 24);   // M / 16
 }
@@ -133,43 +131,12 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-// ---- TMEM -> registers: 32 lanes x 32 consecutive 32-bit columns per warp ----
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Split form for software pipelining: tmem_ld32_issue starts the load; the
-// registers are valid only after tmem_ld_wait (which waits for all of this
-// thread's outstanding TMEM loads). Callers read them only after the wait.
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
+// ---- TMEM -> registers ----
 // 16 lanes x 32 consecutive columns, as four 16x8 accumulator fragments: of
 // fragment i a lane gets columns 8 i + 2 (l % 4) + {0, 1} of lanes l / 4
-// (r[4 i], r[4 i + 1]) and l / 4 + 8 (r[4 i + 2], r[4 i + 3]); issued only, as
-// tmem_ld32_issue
+// (r[4 i], r[4 i + 1]) and l / 4 + 8 (r[4 i + 2], r[4 i + 3]). It starts the load:
+// the registers are valid only after tmem_ld_wait (which waits for all of the
+// thread's outstanding TMEM loads)
 __device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
@@ -186,6 +153,24 @@ __device__ __forceinline__ void stmatrix4(uint32_t saddr, uint32_t a, uint32_t b
                "r"(d)
                : "memory");
 }
+// the fragments back (the addresses as stmatrix4)
+__device__ __forceinline__ void ldmatrix4(uint32_t saddr, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a), "=r"(b), "=r"(c), "=r"(d)
+               : "r"(saddr)
+               : "memory");
+}
+// shared -> global bulk copy of the issuing thread (16-byte aligned, a multiple
+// of 16 bytes) and the wait until its source may be overwritten / it is done
+__device__ __forceinline__ void bulk_s2g(void* dst_gmem, uint32_t src_saddr, uint32_t bytes) {
+  asm volatile(
+      "cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\t"
+      "cp.async.bulk.commit_group;" ::"l"(dst_gmem), "r"(src_saddr), "r"(bytes)
+      : "memory");
+}
+__device__ __forceinline__ void bulk_s2g_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_s2g_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // byte offset of element (row, k) in a no-swizzle K-major tile with K columns
