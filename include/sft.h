@@ -479,7 +479,9 @@ sft_status sft_target_mass(sft_target tgt, int64_t* nnz_out, int64_t* row_ptr_ou
  * *_destroy and by finished calls for later calls instead of returning them
  * to the driver at each synchronisation (creating and destroying meshes in a
  * loop then maps no new memory). This returns the pools' unused blocks to
- * the driver; memory in use is untouched. The paper has no counterpart. */
+ * the driver, and the page-locked status buffers and timing events kept idle
+ * between calls (at most 16 sets); memory in use is untouched. The paper has
+ * no counterpart. */
 sft_status sft_trim_memory(void);
 
 const char* sft_status_str(sft_status s);

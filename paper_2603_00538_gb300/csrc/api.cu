@@ -250,40 +250,36 @@ sft_status sft_transfer(sft_source s, sft_target t, const sft_options* o, double
   const int64_t nv = t->nv, ne = t->ne;
   const size_t psz = prec == SFT_PREC_FP32 ? 4 : 8;
   Events ev;
-  if (ev.ok) cudaEventRecord(ev.e[0], st);
-  DevBuf<int32_t> d_err(st);
-  SFT_CUDA(d_err.alloc(1));
-  SFT_CUDA(cudaMemsetAsync(d_err.p, 0, sizeof(int32_t), st));
-  if (sft_status r = build_locator(s, prec, st, d_err.p)) return r;
+  ev.record(0, st);
+  // one allocation: the status words and b (zeroed together), g and the
+  // outputs staged for the host
+  Carve lay;
+  const size_t vec = (size_t)nv * nf;
+  lay.add(sizeof(CallStatus));
+  const size_t o_b = lay.add(sizeof(double) * vec), zeroed = lay.total;
+  const size_t o_g = lay.add(psz * vec);
+  const size_t o_u = lay.add(o->out_device ? 0 : sizeof(double) * vec);
+  const size_t o_g64 = lay.add(g_out && prec == SFT_PREC_FP32 ? sizeof(double) * vec : 0);
+  const size_t o_se = lay.add(o->sample_elem_out && !o->out_device ? sizeof(int32_t) * (size_t)(ne * nmax) : 0);
+  DevBuf<char> ws(st);
+  SFT_CUDA(ws.alloc(lay.total));
+  CallStatus* status = (CallStatus*)ws.p;
+  double* b = (double*)(ws.p + o_b);
+  char* g = ws.p + o_g;
+  SFT_CUDA(cudaMemsetAsync(ws.p, 0, zeroed, st));
+  if (sft_status r = build_locator(s, prec, st, &status->err)) return r;
   if (sft_status r = target_coordsP(t, prec, st)) return r;
-  if (ev.ok) cudaEventRecord(ev.e[1], st);
-
-  DevBuf<char> g(st);
-  DevBuf<double> b(st), u_tmp(st);
-  DevBuf<int64_t> counters(st);
-  DevBuf<int32_t> se_tmp(st);
-  SFT_CUDA(g.alloc(psz * nv * nf));
-  SFT_CUDA(b.alloc((size_t)nv * nf));
-  SFT_CUDA(counters.alloc(3));
-  SFT_CUDA(cudaMemsetAsync(b.p, 0, sizeof(double) * nv * nf, st));
-  SFT_CUDA(cudaMemsetAsync(counters.p, 0, sizeof(int64_t) * 3, st));
+  ev.record(1, st);
 
   // step 1: control values g = f^s at the target nodes
-  if (sft_status r = locate_points(s, prec, nv, t->coordsP[prec], prec == SFT_PREC_FP64, nullptr, g.p,
-                                   prec == SFT_PREC_FP64, nv, counters.p, st, nf))
+  if (sft_status r = locate_points(s, prec, nv, t->coordsP[prec], prec == SFT_PREC_FP64, nullptr, g,
+                                   prec == SFT_PREC_FP64, nv, status->counters, st, nf))
     return r;
-  if (ev.ok) cudaEventRecord(ev.e[2], st);
+  ev.record(2, st);
 
   // steps 2-6: fused sampling / query / control / scatter
   int32_t* se = nullptr;
-  if (o->sample_elem_out) {
-    if (o->out_device) {
-      se = o->sample_elem_out;
-    } else {
-      SFT_CUDA(se_tmp.alloc((size_t)(ne * nmax)));
-      se = se_tmp.p;
-    }
-  }
+  if (o->sample_elem_out) se = o->out_device ? o->sample_elem_out : (int32_t*)(ws.p + o_se);
   AssembleArgs a;
   a.prec = prec;
   a.nf = nf;
@@ -291,54 +287,48 @@ sft_status sft_transfer(sft_source s, sft_target t, const sft_options* o, double
   a.seed = o->seed;
   a.stream_id = o->stream_id;
   a.alpha = o->alpha;
-  a.g = g.p;
-  a.b = b.p;
+  a.g = g;
+  a.b = b;
   a.sample_elem = se;
-  a.counters = counters.p;
+  a.counters = status->counters;
   a.sampling = o->sampling;
   a.adapt_ref = o->adapt_ref_measure;
   if (sft_status r = launch_assembly(s, t, a, st)) return r;
-  if (ev.ok) cudaEventRecord(ev.e[3], st);
+  ev.record(3, st);
 
   // step 7: M u = b
   double* u_dev = u_out;
   if (!o->out_device) {
-    SFT_CUDA(u_tmp.alloc((size_t)nv * nf));
-    u_dev = u_tmp.p;
+    u_dev = (double*)(ws.p + o_u);
     if (o->cg_warm_start)
-      SFT_CUDA(cudaMemcpyAsync(u_dev, u_out, sizeof(double) * nv * nf, cudaMemcpyHostToDevice, st));
+      SFT_CUDA(cudaMemcpyAsync(u_dev, u_out, sizeof(double) * vec, cudaMemcpyHostToDevice, st));
   }
   SolveResult sr;
-  SolveLate late(st);  // the solve's status is read with the final readback below
-  if (sft_status r = mass_solve(t, nf, b.p, u_dev, o->cg_tol, o->cg_max_iter, st, d_err.p, &sr, o->cg_mode, &late,
+  SolveLate late(status->solve);  // the solve's status is read with the final readback below
+  if (sft_status r = mass_solve(t, nf, b, u_dev, o->cg_tol, o->cg_max_iter, st, &status->err, &sr, o->cg_mode, &late,
                                 o->cg_warm_start))
     return r;
-  if (ev.ok) cudaEventRecord(ev.e[4], st);
+  ev.record(4, st);
 
   const cudaMemcpyKind d2o = o->out_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  if (!o->out_device) SFT_CUDA(cudaMemcpyAsync(u_out, u_dev, sizeof(double) * nv * nf, d2o, st));
-  if (b_out) SFT_CUDA(cudaMemcpyAsync(b_out, b.p, sizeof(double) * nv * nf, d2o, st));
+  if (!o->out_device) SFT_CUDA(cudaMemcpyAsync(u_out, u_dev, sizeof(double) * vec, d2o, st));
+  if (b_out) SFT_CUDA(cudaMemcpyAsync(b_out, b, sizeof(double) * vec, d2o, st));
   if (g_out) {
     if (prec == SFT_PREC_FP64) {
-      SFT_CUDA(cudaMemcpyAsync(g_out, g.p, sizeof(double) * nv * nf, d2o, st));
+      SFT_CUDA(cudaMemcpyAsync(g_out, g, sizeof(double) * vec, d2o, st));
     } else {
-      DevBuf<double> g64(st);
-      SFT_CUDA(g64.alloc((size_t)nv * nf));
-      if (sft_status r = convert_coords(g.p, SFT_F32, g64.p, SFT_PREC_FP64, nv * nf, st)) return r;
-      SFT_CUDA(cudaMemcpyAsync(g_out, g64.p, sizeof(double) * nv * nf, d2o, st));
-      SFT_CUDA(cudaStreamSynchronize(st));
+      if (sft_status r = convert_coords(g, SFT_F32, ws.p + o_g64, SFT_PREC_FP64, (int64_t)vec, st)) return r;
+      SFT_CUDA(cudaMemcpyAsync(g_out, ws.p + o_g64, sizeof(double) * vec, d2o, st));
     }
   }
   if (se && !o->out_device)
     SFT_CUDA(cudaMemcpyAsync(o->sample_elem_out, se, sizeof(int32_t) * ne * nmax, d2o, st));
-  int64_t hc[3] = {0, 0, 0};
-  int32_t herr = 0;
-  SFT_CUDA(cudaMemcpyAsync(hc, counters.p, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  SFT_CUDA(cudaMemcpyAsync(&herr, d_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  if (late.pending) SFT_CUDA(cudaMemcpyAsync(late.host, late.buf.p, late.bytes, cudaMemcpyDeviceToHost, st));
-  if (ev.ok) cudaEventRecord(ev.e[5], st);
+  SFT_CUDA(cudaMemcpyAsync(&ev.host(), status, sizeof(CallStatus), cudaMemcpyDeviceToHost, st));
+  ev.record(5, st);
   SFT_CUDA(cudaStreamSynchronize(st));
-  if (sft_status r = finish_solve(late, &sr)) return r;
+  const int64_t* hc = ev.host().counters;
+  const int32_t herr = ev.host().err;
+  if (sft_status r = finish_solve(late, ev.host(), &sr)) return r;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
     stats->cg_iters = sr.iters;
@@ -374,15 +364,22 @@ sft_status sft_conservation_error(sft_source s, sft_target t, const double* u, i
   // both reductions read back together (one wait on the stream)
   const size_t ni = s->integral_valid ? 0 : (size_t)kIntegralBlocks * kMaxFields;
   DevBuf<double> part(st);
-  SFT_CUDA(part.alloc(ni + kWsumBlocks));
+  SFT_CUDA(part.alloc(ni + kWsumBlocks + kMaxFields + 1));
+  double* const sums = part.p + ni + kWsumBlocks;
   if (ni)
     if (sft_status r = source_integrals_launch(s, part.p, st)) return r;
   if (sft_status r = weighted_sum_launch(t->lumped, ud, t->nv, part.p + ni, st)) return r;
-  std::vector<double> h(ni + kWsumBlocks);
-  SFT_CUDA(cudaMemcpyAsync(h.data(), part.p, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
+  if (sft_status r = final_sums_launch(part.p, ni ? s->nf : 0, part.p + ni, (int)kWsumBlocks, sums, st)) return r;
+  Events kit;
+  double* const h = reinterpret_cast<double*>(kit.host().solve);
+  static_assert(sizeof(double) * (kMaxFields + 1) <= sizeof(CallStatus::solve), "sums");
+  SFT_CUDA(cudaMemcpyAsync(h, sums, sizeof(double) * (kMaxFields + 1), cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaStreamSynchronize(st));
-  if (ni) source_integrals_finish(s, h.data());
-  const double it = weighted_sum_finish(h.data() + ni);
+  if (ni) {
+    for (int f = 0; f < s->nf; ++f) s->integral[f] = h[f];
+    s->integral_valid = true;
+  }
+  const double it = h[kMaxFields];
   const double is = s->integral[field];
   out3[0] = std::fabs(is - it) / std::fabs(is);
   out3[1] = is;

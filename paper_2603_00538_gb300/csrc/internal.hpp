@@ -53,20 +53,54 @@ struct DevBuf {
   ~DevBuf() { dfree(p, s); }
 };
 
-struct Events {
-  cudaEvent_t e[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  bool ok = false;
-  Events() {
-    ok = true;
-    for (auto& x : e) ok = ok && cudaEventCreate(&x) == cudaSuccess;
+// Byte offsets of several arrays in one allocation (each 256-byte aligned)
+struct Carve {
+  size_t total = 0;
+  size_t add(size_t bytes) {
+    const size_t o = total;
+    total += (bytes + 255) & ~(size_t)255;
+    return o;
   }
-  ~Events() {
-    for (auto& x : e)
-      if (x) cudaEventDestroy(x);
+};
+
+// Status words of one call: on the device beside the call's work arrays
+// (zeroed with them), read back in one copy.
+struct CallStatus {
+  int32_t err;
+  int32_t pad;
+  int64_t counters[3];
+  alignas(16) unsigned char solve[256];  // the solve's control block (solve.cu)
+};
+
+// Host resources of one call: timing events and a page-locked copy of the
+// status words (a copy to pageable memory costs the call some 10 us more).
+// Kits are lent out for the length of a call, one caller at a time, and at
+// most kMaxKits idle ones per process are kept (util.cu); sft_trim_memory
+// frees those.
+struct CallKit {
+  int dev = 0;
+  cudaEvent_t e[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  CallStatus* host = nullptr;  // page-locked, or &own
+  CallStatus own;
+  bool timing = false;
+};
+CallKit* kit_acquire();
+void kit_release(CallKit* k);
+
+struct Events {
+  CallKit* kit;
+  bool ok;
+  Events() : kit(kit_acquire()), ok(kit->timing) {}
+  ~Events() { kit_release(kit); }
+  Events(const Events&) = delete;
+  Events& operator=(const Events&) = delete;
+  CallStatus& host() { return *kit->host; }
+  void record(int i, cudaStream_t st) {
+    if (ok) cudaEventRecord(kit->e[i], st);
   }
   float ms(int a, int b) const {
     float t = 0.f;
-    if (ok && cudaEventElapsedTime(&t, e[a], e[b]) != cudaSuccess) {
+    if (ok && cudaEventElapsedTime(&t, kit->e[a], kit->e[b]) != cudaSuccess) {
       t = -1.f;
       cudaGetLastError();  // timing unavailable: do not leave a sticky error behind
     }
@@ -143,12 +177,12 @@ sft_status build_locator(sft_source_s* s, int prec, cudaStream_t st, int32_t* d_
 sft_status locate_points(sft_source_s* s, int prec, int64_t n, const void* pts, int pts_are_double,
                          int32_t* elem_out, void* val_out, int val_is_double, int64_t val_stride,
                          int64_t* d_counters, cudaStream_t st, int nf_out = -1, void* mu_out = nullptr);
-sft_status source_integrals(sft_source_s* s, cudaStream_t st);
-// the same split in launch (partials [kIntegralBlocks][kMaxFields] on the
-// device) and the host's fixed-order sum of the copied partials
+// integrals of every source field and a weighted sum: per-block partials
+// ([kIntegralBlocks][kMaxFields], [kWsumBlocks]) and their final sums in a
+// fixed order (out[0 .. kMaxFields - 1] the fields, out[kMaxFields] the sum)
 constexpr unsigned kIntegralBlocks = 152 * 8;
 sft_status source_integrals_launch(sft_source_s* s, double* part, cudaStream_t st);
-void source_integrals_finish(sft_source_s* s, const double* hpart);
+sft_status final_sums_launch(const double* part, int nf, const double* wpart, int n_w, double* out, cudaStream_t st);
 sft_status refresh_value_copies(sft_source_s* s, cudaStream_t st);
 // target.cu
 sft_status build_target(sft_target_s* t, cudaStream_t st, int32_t* d_err);
@@ -178,27 +212,24 @@ sft_status launch_assembly(sft_source_s* s, sft_target_s* t, const AssembleArgs&
 // solve.cu
 struct SolveResult { int iters; double rel_resid; int converged; };
 // Deferred solve status: with a SolveLate, mass_solve returns without waiting
-// for the kernel (mixed mode); the caller copies `bytes` from buf to host in
-// its own final readback and then calls finish_solve.
+// for the kernel (mixed mode); its control block is the zeroed `dev` of the
+// caller's CallStatus, and the caller calls finish_solve with the copy it read
+// back.
 struct SolveLate {
-  explicit SolveLate(cudaStream_t st) : buf(st) {}
-  DevBuf<unsigned char> buf;
-  alignas(16) unsigned char host[256];
-  size_t bytes = 0;
+  explicit SolveLate(unsigned char* d) : dev(d) {}
+  unsigned char* dev;
   int nrhs = 0;
   bool pending = false;
 };
-sft_status finish_solve(const SolveLate& late, SolveResult* res);
+sft_status finish_solve(const SolveLate& late, const CallStatus& host, SolveResult* res);
 // cg_mode: SFT_CG_MIXED (FP64 refinement around FP32 CG) or SFT_CG_FP64
 sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, double tol, int max_iter,
                       cudaStream_t st, int32_t* d_err, SolveResult* res, int cg_mode = SFT_CG_MIXED,
                       SolveLate* late = nullptr, int warm = 0);
 // S = diag(M)^-1/2 and the FP32 values of S M S in CSR order on the target (made once, kept)
 sft_status scaled_matrix(sft_target_s* t, cudaStream_t st);
-sft_status weighted_sum(const double* w, const double* u, int64_t n, double* out_host, cudaStream_t st);
 constexpr unsigned kWsumBlocks = 304;
 sft_status weighted_sum_launch(const double* w, const double* u, int64_t n, double* part, cudaStream_t st);
-double weighted_sum_finish(const double* hpart);
 // conversions
 sft_status convert_coords(const void* in, int in_dtype, void* out, int out_prec, int64_t n, cudaStream_t st);
 }  // namespace sft

@@ -567,11 +567,12 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
                                                                                cell_count.p, nullptr, nullptr, mask.p);
   SFT_CUDA(cudaGetLastError());
   SFT_CUDA(exclusive_scan_i32_to_i64(cell_count.p, start64.p, L.ncells, st));
-  int32_t herr = 0;
-  int64_t total = 0;
-  SFT_CUDA(cudaMemcpyAsync(&herr, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  SFT_CUDA(cudaMemcpyAsync(&total, start64.p + L.ncells, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+  Events kit;
+  SFT_CUDA(cudaMemcpyAsync(&kit.host().err, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  SFT_CUDA(cudaMemcpyAsync(&kit.host().counters[0], start64.p + L.ncells, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaStreamSynchronize(st));
+  const int32_t herr = kit.host().err;
+  const int64_t total = kit.host().counters[0];
   if (herr != 0)
     return fail(SFT_ERR_MESH, herr == DEV_NONFINITE  ? "non-finite source coordinate"
                               : herr == DEV_BAD_INDEX ? "source connectivity index out of range"
@@ -785,23 +786,24 @@ sft_status source_integrals_launch(sft_source_s* s, double* part, cudaStream_t s
   return SFT_OK;
 }
 
-void source_integrals_finish(sft_source_s* s, const double* hpart) {
-  for (int f = 0; f < s->nf; ++f) {
-    double t = 0.0;
-    for (unsigned b = 0; b < kIntegralBlocks; ++b) t += hpart[(size_t)b * kMaxFields + f];
-    s->integral[f] = t;
-  }
-  s->integral_valid = true;
+// Final sums in a fixed order: warp f < nf adds field f's partials, warp
+// kMaxFields the n_w partials of a weighted sum, into out[0 .. kMaxFields]
+__global__ void __launch_bounds__(32 * (kMaxFields + 1)) k_final_sums(const double* __restrict__ part, int nf,
+                                                                     const double* __restrict__ wpart, int n_w,
+                                                                     double* __restrict__ out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+  if (warp < nf)
+    for (unsigned k = lane; k < kIntegralBlocks; k += 32) s += part[(int64_t)k * kMaxFields + warp];
+  if (warp == kMaxFields)
+    for (int k = lane; k < n_w; k += 32) s += wpart[k];
+  s = warp_sum<double>(s);
+  if (lane == 0) out[warp] = s;
 }
 
-sft_status source_integrals(sft_source_s* s, cudaStream_t st) {
-  DevBuf<double> part(st);
-  SFT_CUDA(part.alloc((size_t)kIntegralBlocks * kMaxFields));
-  if (sft_status r = source_integrals_launch(s, part.p, st)) return r;
-  std::vector<double> h((size_t)kIntegralBlocks * kMaxFields);
-  SFT_CUDA(cudaMemcpyAsync(h.data(), part.p, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
-  SFT_CUDA(cudaStreamSynchronize(st));
-  source_integrals_finish(s, h.data());
+sft_status final_sums_launch(const double* part, int nf, const double* wpart, int n_w, double* out, cudaStream_t st) {
+  ::sft::note_launch(), k_final_sums<<<1, 32 * (kMaxFields + 1), 0, st>>>(part, nf, wpart, n_w, out);
+  SFT_CUDA(cudaGetLastError());
   return SFT_OK;
 }
 

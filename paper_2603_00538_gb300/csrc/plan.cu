@@ -163,35 +163,42 @@ sft_status sft_plan_transfer(sft_plan pl, double* u_out, double* b_out, double* 
   const size_t psz = prec == SFT_PREC_FP32 ? 4 : 8;
   const Locator& L = s->loc[prec];
   Events ev;
-  if (ev.ok) cudaEventRecord(ev.e[0], st);
-  DevBuf<int32_t> d_err(st);
-  DevBuf<char> g(st);
-  DevBuf<double> b(st), u_tmp(st);
-  SFT_CUDA(d_err.alloc(1));
-  SFT_CUDA(g.alloc(psz * nv * nf));
-  SFT_CUDA(b.alloc((size_t)nv * nf));
-  SFT_CUDA(cudaMemsetAsync(d_err.p, 0, sizeof(int32_t), st));
-  SFT_CUDA(cudaMemsetAsync(b.p, 0, sizeof(double) * nv * nf, st));
-  if (ev.ok) cudaEventRecord(ev.e[1], st);
+  ev.record(0, st);
+  // one allocation: the status words and b (zeroed together), g and the
+  // outputs staged for the host
+  Carve lay;
+  const size_t vec = (size_t)nv * nf;
+  lay.add(sizeof(CallStatus));
+  const size_t o_b = lay.add(sizeof(double) * vec), zeroed = lay.total;
+  const size_t o_g = lay.add(psz * vec);
+  const size_t o_u = lay.add(o.out_device ? 0 : sizeof(double) * vec);
+  const size_t o_g64 = lay.add(g_out && prec == SFT_PREC_FP32 ? sizeof(double) * vec : 0);
+  DevBuf<char> ws(st);
+  SFT_CUDA(ws.alloc(lay.total));
+  CallStatus* status = (CallStatus*)ws.p;
+  double* b = (double*)(ws.p + o_b);
+  char* g = ws.p + o_g;
+  SFT_CUDA(cudaMemsetAsync(ws.p, 0, zeroed, st));
+  ev.record(1, st);
   // step 1 online: control values from the recorded node locations
   const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nv + 255) / 256, 152 * 16));
   if (t->dim == 2) {
     if (prec == SFT_PREC_FP32)
       ::sft::note_launch(), k_plan_control<2, float><<<nb, 256, 0, st>>>(pl->node_elem, (const float*)pl->node_mu, nv,
-                                                                        (const float*)L.vals, s->nf, nf, (float*)g.p);
+                                                                        (const float*)L.vals, s->nf, nf, (float*)g);
     else
       ::sft::note_launch(), k_plan_control<2, double><<<nb, 256, 0, st>>>(pl->node_elem, (const double*)pl->node_mu, nv,
-                                                                         (const double*)L.vals, s->nf, nf, (double*)g.p);
+                                                                         (const double*)L.vals, s->nf, nf, (double*)g);
   } else {
     if (prec == SFT_PREC_FP32)
       ::sft::note_launch(), k_plan_control<3, float><<<nb, 256, 0, st>>>(pl->node_elem, (const float*)pl->node_mu, nv,
-                                                                        (const float*)L.vals, s->nf, nf, (float*)g.p);
+                                                                        (const float*)L.vals, s->nf, nf, (float*)g);
     else
       ::sft::note_launch(), k_plan_control<3, double><<<nb, 256, 0, st>>>(pl->node_elem, (const double*)pl->node_mu, nv,
-                                                                         (const double*)L.vals, s->nf, nf, (double*)g.p);
+                                                                         (const double*)L.vals, s->nf, nf, (double*)g);
   }
   SFT_CUDA(cudaGetLastError());
-  if (ev.ok) cudaEventRecord(ev.e[2], st);
+  ev.record(2, st);
   // steps 2-6 online
   AssembleArgs a;
   a.prec = prec;
@@ -200,48 +207,44 @@ sft_status sft_plan_transfer(sft_plan pl, double* u_out, double* b_out, double* 
   a.seed = o.seed;
   a.stream_id = o.stream_id;
   a.alpha = o.alpha;
-  a.g = g.p;
-  a.b = b.p;
+  a.g = g;
+  a.b = b;
   a.sample_elem = pl->samp_elem;
   a.counters = nullptr;
   a.mode = kAsmCached;
   a.pmu = pl->samp_mu;
   a.sampling = o.sampling;
   if (sft_status r = launch_assembly(s, t, a, st)) return r;
-  if (ev.ok) cudaEventRecord(ev.e[3], st);
+  ev.record(3, st);
   // step 7
   double* u_dev = u_out;
   if (!o.out_device) {
-    SFT_CUDA(u_tmp.alloc((size_t)nv * nf));
-    u_dev = u_tmp.p;
+    u_dev = (double*)(ws.p + o_u);
     if (o.cg_warm_start)
       SFT_CUDA(cudaMemcpyAsync(u_dev, u_out, sizeof(double) * nv * nf, cudaMemcpyHostToDevice, st));
   }
   SolveResult sr;
-  SolveLate late(st);  // the solve's status is read with the final readback
-  if (sft_status r = mass_solve(t, nf, b.p, u_dev, o.cg_tol, o.cg_max_iter, st, d_err.p, &sr, o.cg_mode, &late,
+  SolveLate late(status->solve);  // the solve's status is read with the final readback
+  if (sft_status r = mass_solve(t, nf, b, u_dev, o.cg_tol, o.cg_max_iter, st, &status->err, &sr, o.cg_mode, &late,
                                 o.cg_warm_start))
     return r;
-  if (ev.ok) cudaEventRecord(ev.e[4], st);
+  ev.record(4, st);
   const cudaMemcpyKind d2o = o.out_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   if (!o.out_device) SFT_CUDA(cudaMemcpyAsync(u_out, u_dev, sizeof(double) * nv * nf, d2o, st));
-  if (b_out) SFT_CUDA(cudaMemcpyAsync(b_out, b.p, sizeof(double) * nv * nf, d2o, st));
-  DevBuf<double> g64(st);
+  if (b_out) SFT_CUDA(cudaMemcpyAsync(b_out, b, sizeof(double) * nv * nf, d2o, st));
   if (g_out) {
     if (prec == SFT_PREC_FP64) {
-      SFT_CUDA(cudaMemcpyAsync(g_out, g.p, sizeof(double) * nv * nf, d2o, st));
+      SFT_CUDA(cudaMemcpyAsync(g_out, g, sizeof(double) * nv * nf, d2o, st));
     } else {
-      SFT_CUDA(g64.alloc((size_t)nv * nf));
-      if (sft_status r = convert_coords(g.p, SFT_F32, g64.p, SFT_PREC_FP64, nv * nf, st)) return r;
-      SFT_CUDA(cudaMemcpyAsync(g_out, g64.p, sizeof(double) * nv * nf, d2o, st));
+      if (sft_status r = convert_coords(g, SFT_F32, ws.p + o_g64, SFT_PREC_FP64, (int64_t)vec, st)) return r;
+      SFT_CUDA(cudaMemcpyAsync(g_out, ws.p + o_g64, sizeof(double) * nv * nf, d2o, st));
     }
   }
-  int32_t herr = 0;
-  SFT_CUDA(cudaMemcpyAsync(&herr, d_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  if (late.pending) SFT_CUDA(cudaMemcpyAsync(late.host, late.buf.p, late.bytes, cudaMemcpyDeviceToHost, st));
-  if (ev.ok) cudaEventRecord(ev.e[5], st);
+  SFT_CUDA(cudaMemcpyAsync(&ev.host(), status, sizeof(CallStatus), cudaMemcpyDeviceToHost, st));
+  ev.record(5, st);
   SFT_CUDA(cudaStreamSynchronize(st));
-  if (sft_status r = finish_solve(late, &sr)) return r;
+  const int32_t herr = ev.host().err;
+  if (sft_status r = finish_solve(late, ev.host(), &sr)) return r;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
     stats->cg_iters = sr.iters;

@@ -954,7 +954,7 @@ static sft_status scaled_slices(sft_target_s* t, cudaStream_t st) {
   return SFT_OK;
 }
 
-static_assert(sizeof(MixCtl) <= sizeof(SolveLate::host), "status block larger than its host copy");
+static_assert(sizeof(MixCtl) <= sizeof(CallStatus::solve), "control block larger than its place in the call's status");
 
 static void mix_result(const MixCtl& h, int nrhs, SolveResult* res) {
   for (int f = 0; f < nrhs; ++f) {
@@ -964,10 +964,10 @@ static void mix_result(const MixCtl& h, int nrhs, SolveResult* res) {
   }
 }
 
-sft_status finish_solve(const SolveLate& late, SolveResult* res) {
+sft_status finish_solve(const SolveLate& late, const CallStatus& host, SolveResult* res) {
   if (!late.pending) return SFT_OK;
   MixCtl h;
-  std::memcpy(&h, late.host, sizeof(MixCtl));
+  std::memcpy(&h, host.solve, sizeof(MixCtl));
   if (h.err != 0) return fail(SFT_ERR_DEVICE_STATUS, "solve kernel: a barrier wait expired");
   mix_result(h, late.nrhs, res);
   return SFT_OK;
@@ -1052,23 +1052,21 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
                      : team == kTeamCluster ? (const void*)k_mixed<NR, kTeamCluster, true>
                      : own                  ? (const void*)k_mixed<NR, kTeamGrid, true>
                                             : (const void*)k_mixed<NR, kTeamGrid, false>;
-  const size_t vec = (size_t)n * nrhs;
-  DevBuf<double> tb(st), partd(st);
-  DevBuf<float> ya(st), yb(st), cb(st);
-  DevBuf<MixCtl> ctl(st);
-  SFT_CUDA(tb.alloc(vec));
-  SFT_CUDA(ya.alloc(team == kTeamGrid ? (size_t)n * NR : 1));
-  SFT_CUDA(yb.alloc(team == kTeamGrid ? (size_t)n * NR : 1));
-  SFT_CUDA(cb.alloc(a.c_smem ? 1 : (size_t)n * NR));
-  SFT_CUDA(partd.alloc((size_t)nblocks * nrhs * 4));
+  Carve lay;  // one allocation for the work vectors
+  const size_t o_ctl = lay.add(late ? 0 : sizeof(MixCtl));
+  const size_t o_t = lay.add(sizeof(double) * (size_t)n * nrhs);
+  const size_t o_part = lay.add(sizeof(double) * (size_t)nblocks * nrhs * 4);
+  const size_t o_ya = lay.add(team == kTeamGrid ? sizeof(float) * (size_t)n * NR : 0);
+  const size_t o_yb = lay.add(team == kTeamGrid ? sizeof(float) * (size_t)n * NR : 0);
+  const size_t o_c = lay.add(a.c_smem ? 0 : sizeof(float) * (size_t)n * NR);
+  DevBuf<char> ws(st);
+  SFT_CUDA(ws.alloc(lay.total));
   if (late) {
-    SFT_CUDA(late->buf.alloc(sizeof(MixCtl)));
-    a.ctl = reinterpret_cast<MixCtl*>(late->buf.p);
+    a.ctl = reinterpret_cast<MixCtl*>(late->dev);  // zeroed by the caller
   } else {
-    SFT_CUDA(ctl.alloc(1));
-    a.ctl = ctl.p;
+    a.ctl = reinterpret_cast<MixCtl*>(ws.p + o_ctl);
+    SFT_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(MixCtl), st));
   }
-  SFT_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(MixCtl), st));
   a.rp = t->row_ptr;
   a.jent = t->jent;
   a.jval = t->jval;
@@ -1079,11 +1077,11 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
   a.nrhs = nrhs;
   a.b = b;
   a.x = x;
-  a.t = tb.p;
-  a.ya = ya.p;
-  a.yb = yb.p;
-  a.c = cb.p;
-  a.partd = partd.p;
+  a.t = reinterpret_cast<double*>(ws.p + o_t);
+  a.ya = reinterpret_cast<float*>(ws.p + o_ya);
+  a.yb = reinterpret_cast<float*>(ws.p + o_yb);
+  a.c = reinterpret_cast<float*>(ws.p + o_c);
+  a.partd = reinterpret_cast<double*>(ws.p + o_part);
   a.tol = tol;
   a.max_iter = max_iter;
   a.warm = warm;
@@ -1109,13 +1107,13 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
   const cudaError_t le = (::sft::note_launch(), cudaLaunchKernelExC(&cfg, kern, args));
   if (le != cudaSuccess) return cuda_fail(le, "launch of the mixed-precision solve");
   if (late) {
-    late->bytes = sizeof(MixCtl);
     late->nrhs = nrhs;
     late->pending = true;
     return SFT_OK;  // the work buffers are freed in stream order
   }
-  MixCtl h;
-  SFT_CUDA(cudaMemcpyAsync(&h, ctl.p, sizeof(MixCtl), cudaMemcpyDeviceToHost, st));
+  Events kit;
+  MixCtl& h = *reinterpret_cast<MixCtl*>(kit.host().solve);
+  SFT_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(MixCtl), cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaStreamSynchronize(st));
   if (h.err != 0) return fail(SFT_ERR_DEVICE_STATUS, "solve kernel: a barrier wait expired");
   mix_result(h, nrhs, res);
@@ -1216,23 +1214,6 @@ __global__ void k_wsum_partial(const double* __restrict__ w, const double* __res
 sft_status weighted_sum_launch(const double* w, const double* u, int64_t n, double* part, cudaStream_t st) {
   ::sft::note_launch(), k_wsum_partial<<<kWsumBlocks, 256, 0, st>>>(w, u, n, part);
   SFT_CUDA(cudaGetLastError());
-  return SFT_OK;
-}
-
-double weighted_sum_finish(const double* hpart) {
-  double t = 0.0;
-  for (unsigned k = 0; k < kWsumBlocks; ++k) t += hpart[k];
-  return t;
-}
-
-sft_status weighted_sum(const double* w, const double* u, int64_t n, double* out_host, cudaStream_t st) {
-  DevBuf<double> part(st);
-  SFT_CUDA(part.alloc(kWsumBlocks));
-  if (sft_status r = weighted_sum_launch(w, u, n, part.p, st)) return r;
-  std::vector<double> h(kWsumBlocks);
-  SFT_CUDA(cudaMemcpyAsync(h.data(), part.p, sizeof(double) * kWsumBlocks, cudaMemcpyDeviceToHost, st));
-  SFT_CUDA(cudaStreamSynchronize(st));
-  *out_host = weighted_sum_finish(h.data());
   return SFT_OK;
 }
 

@@ -629,24 +629,24 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   const int64_t nv = t->nv, ne = t->ne;
   const int N = o->samples_per_elem;
   Events ev;
-  if (ev.ok) cudaEventRecord(ev.e[0], st);
-  DevBuf<int32_t> d_err(st), fb_tmp(st);
+  ev.record(0, st);
+  DevBuf<int32_t> fb_tmp(st);
   DevBuf<float> g(st), pts3(st), sf_tmp(st);
   DevBuf<double> b(st), u_tmp(st);
-  DevBuf<int64_t> counters(st);
-  SFT_CUDA(d_err.alloc(1));
-  SFT_CUDA(cudaMemsetAsync(d_err.p, 0, sizeof(int32_t), st));
+  DevBuf<CallStatus> status(st);
+  SFT_CUDA(status.alloc(1));
+  SFT_CUDA(cudaMemsetAsync(status.p, 0, sizeof(CallStatus), st));
+  int32_t* const d_err = &status.p->err;
+  int64_t* const counters = status.p->counters;
   if (exact) {
-    if (sft_status r = build_locator(exact, SFT_PREC_FP32, st, d_err.p)) return r;
+    if (sft_status r = build_locator(exact, SFT_PREC_FP32, st, d_err)) return r;
   }
   if (sft_status r = target_coordsP(t, SFT_PREC_FP32, st)) return r;
   SFT_CUDA(g.alloc((size_t)nv));
   SFT_CUDA(b.alloc((size_t)nv));
-  SFT_CUDA(counters.alloc(3));
   SFT_CUDA(cudaMemsetAsync(b.p, 0, sizeof(double) * nv, st));
-  SFT_CUDA(cudaMemsetAsync(counters.p, 0, sizeof(int64_t) * 3, st));
   const float* tx = (const float*)t->coordsP[SFT_PREC_FP32];
-  if (ev.ok) cudaEventRecord(ev.e[1], st);
+  ev.record(1, st);
 
   // step 1: control values at the target nodes (network, or exact without one)
   const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nv + 255) / 256, 152 * 16));
@@ -654,7 +654,7 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
     SFT_CUDA(pts3.alloc((size_t)nv * 3));
     ::sft::note_launch(), k_pad3<<<nb, 256, 0, st>>>(tx, nv, t->dim, pts3.p);
     SFT_CUDA(cudaGetLastError());
-    if (sft_status r = mlp_forward_dev(net, nv, pts3.p, g.p, st, d_err.p)) return r;
+    if (sft_status r = mlp_forward_dev(net, nv, pts3.p, g.p, st, d_err)) return r;
   } else {
     const Locator& L = exact->loc[SFT_PREC_FP32];
 #define SFT_EN(DSV)                                                                                             \
@@ -663,12 +663,12 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
                                                               (const float*)L.recs,                             \
                                                               L.adj, (const float*)L.vals, exact->nf,           \
                                                               so->exact_field, so->exact_cost,                  \
-                                                              g.p, counters.p)
+                                                              g.p, counters)
     if (exact->dim == 2) SFT_EN(2); else SFT_EN(3);
 #undef SFT_EN
     SFT_CUDA(cudaGetLastError());
   }
-  if (ev.ok) cudaEventRecord(ev.e[2], st);
+  ev.record(2, st);
 
   // steps 2-6: fused sample / network / fallback / scatter
   SurParams p{};
@@ -709,11 +709,11 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
     if (q.nlist == 0) return SFT_OK;
     q.nunits = q.nsub == 1 ? (q.nlist + q.EPB - 1) / q.EPB : q.nlist;
     if (with_net)
-      return t->dim == 2 ? net_pass<2>(net, t, q, g.p, b.p, fbp, sf, d_err.p, st)
-                         : net_pass<3>(net, t, q, g.p, b.p, fbp, sf, d_err.p, st);
-    if (t->dim == 2) return launch_exact<2, 2>(exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-    if (ds == 2) return launch_exact<3, 2>(exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
-    return launch_exact<3, 3>(exact, t, q, g.p, b.p, fbp, sf, counters.p, d_err.p, st);
+      return t->dim == 2 ? net_pass<2>(net, t, q, g.p, b.p, fbp, sf, d_err, st)
+                         : net_pass<3>(net, t, q, g.p, b.p, fbp, sf, d_err, st);
+    if (t->dim == 2) return launch_exact<2, 2>(exact, t, q, g.p, b.p, fbp, sf, counters, d_err, st);
+    if (ds == 2) return launch_exact<3, 2>(exact, t, q, g.p, b.p, fbp, sf, counters, d_err, st);
+    return launch_exact<3, 3>(exact, t, q, g.p, b.p, fbp, sf, counters, d_err, st);
   };
   sft_status lr = SFT_OK;
   int64_t n_fallback = net ? 0 : ne;
@@ -736,13 +736,13 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   ::sft::note_launch(), k_sub_points<DTV, DSV><<<nbs, 128, 0, st>>>(                                                  \
       tx, t->conn, ne, sub, p.key, p.stream_id, p.st, (const GridP<float>*)L.grid, L.cell_start, L.cell_items,     \
       L.cell_first, (const float*)L.recs, L.adj, (const float*)L.vals, exact->nf, so->exact_field, so->exact_cost, s_pts.p,      \
-      s_fe.p, counters.p)
+      s_fe.p, counters)
     if (t->dim == 2) SFT_SP(2, 2);
     else if (ds == 2) SFT_SP(3, 2);
     else SFT_SP(3, 3);
 #undef SFT_SP
     SFT_CUDA(cudaGetLastError());
-    if (sft_status r = mlp_forward_dev(net, nsp, s_pts.p, s_y.p, st, d_err.p)) return r;
+    if (sft_status r = mlp_forward_dev(net, nsp, s_pts.p, s_y.p, st, d_err)) return r;
     const unsigned nbe = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ne + 255) / 256, 152 * 16));
     ::sft::note_launch(), k_decide<<<nbe, 256, 0, st>>>(s_y.p, s_fe.p, ne, sub, so->tau, s_flag.p, fb);
     SFT_CUDA(cudaGetLastError());
@@ -775,7 +775,7 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
     lr = pass(net != nullptr, q, fb);
   }
   if (lr) return lr;
-  if (ev.ok) cudaEventRecord(ev.e[3], st);
+  ev.record(3, st);
 
   // step 7: M u = b
   double* u_dev = u_out;
@@ -785,11 +785,11 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
     if (o->cg_warm_start) SFT_CUDA(cudaMemcpyAsync(u_dev, u_out, sizeof(double) * nv, cudaMemcpyHostToDevice, st));
   }
   SolveResult sr;
-  SolveLate late(st);  // the solve's status is read with the final readback
-  if (sft_status r = mass_solve(t, 1, b.p, u_dev, o->cg_tol, o->cg_max_iter, st, d_err.p, &sr, o->cg_mode, &late,
+  SolveLate late(status.p->solve);  // the solve's status is read with the final readback
+  if (sft_status r = mass_solve(t, 1, b.p, u_dev, o->cg_tol, o->cg_max_iter, st, d_err, &sr, o->cg_mode, &late,
                                 o->cg_warm_start))
     return r;
-  if (ev.ok) cudaEventRecord(ev.e[4], st);
+  ev.record(4, st);
 
   const cudaMemcpyKind d2o = o->out_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   if (!o->out_device) SFT_CUDA(cudaMemcpyAsync(u_out, u_dev, sizeof(double) * nv, d2o, st));
@@ -802,14 +802,12 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   }
   if (fb && !o->out_device) SFT_CUDA(cudaMemcpyAsync(so->fallback_out, fb, sizeof(int32_t) * ne, d2o, st));
   if (sf && !o->out_device) SFT_CUDA(cudaMemcpyAsync(so->sample_f_out, sf, sizeof(float) * ne * N, d2o, st));
-  int64_t hc[3] = {0, 0, 0};
-  int32_t herr = 0;
-  SFT_CUDA(cudaMemcpyAsync(hc, counters.p, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  SFT_CUDA(cudaMemcpyAsync(&herr, d_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  if (late.pending) SFT_CUDA(cudaMemcpyAsync(late.host, late.buf.p, late.bytes, cudaMemcpyDeviceToHost, st));
-  if (ev.ok) cudaEventRecord(ev.e[5], st);
+  SFT_CUDA(cudaMemcpyAsync(&ev.host(), status.p, sizeof(CallStatus), cudaMemcpyDeviceToHost, st));
+  ev.record(5, st);
   SFT_CUDA(cudaStreamSynchronize(st));
-  if (sft_status r = finish_solve(late, &sr)) return r;
+  const int64_t* hc = ev.host().counters;
+  const int32_t herr = ev.host().err;
+  if (sft_status r = finish_solve(late, ev.host(), &sr)) return r;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
     stats->cg_iters = sr.iters;

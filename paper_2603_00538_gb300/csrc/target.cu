@@ -238,7 +238,6 @@ static sft_status build_target_t(sft_target_s* t, cudaStream_t st, int32_t* d_er
   else
     ::sft::note_launch(), k_volumes<D, float><<<blocks_for(t->ne), 256, 0, st>>>((const float*)t->coords, t->conn, t->nv, t->ne, t->vol, t->vol32, wfac, inc_count, d_err);
   SFT_CUDA(cudaGetLastError());
-  int32_t herr = 0;
   // no host check here: every later kernel only follows connectivity of
   // elements whose indices are all in range, and the error flag is read with
   // the row count below
@@ -288,10 +287,12 @@ static sft_status build_target_t(sft_target_s* t, cudaStream_t st, int32_t* d_er
                                                            tmp_val, tmp_lump);
   SFT_CUDA(cudaGetLastError());
   SFT_CUDA(exclusive_scan_i32_to_i64(row_len, off64, t->nv, st));
-  int64_t nnz = 0;
-  SFT_CUDA(cudaMemcpyAsync(&nnz, off64 + t->nv, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  SFT_CUDA(cudaMemcpyAsync(&herr, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  Events kit;
+  SFT_CUDA(cudaMemcpyAsync(&kit.host().counters[0], off64 + t->nv, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+  SFT_CUDA(cudaMemcpyAsync(&kit.host().err, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaStreamSynchronize(st));
+  const int64_t nnz = kit.host().counters[0];
+  const int32_t herr = kit.host().err;
   if (herr || nnz >= (int64_t)INT32_MAX) {
     dfree(off64, st);
     dfree(inc_start, st);

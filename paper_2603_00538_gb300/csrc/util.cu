@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <mutex>
+#include <vector>
 #include "internal.hpp"
 
 namespace sft {
@@ -43,7 +44,58 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
+// idle call kits
+constexpr size_t kMaxKits = 16;
+static std::mutex g_kit_mu;
+static std::vector<CallKit*> g_kits;
+
+static void kit_free(CallKit* k) {
+  for (auto& x : k->e)
+    if (x) cudaEventDestroy(x);
+  if (k->host != &k->own) cudaFreeHost(k->host);
+  delete k;
+}
+
+CallKit* kit_acquire() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  {
+    std::lock_guard<std::mutex> lk(g_kit_mu);
+    for (size_t i = 0; i < g_kits.size(); ++i)
+      if (g_kits[i]->dev == dev) {
+        CallKit* k = g_kits[i];
+        g_kits.erase(g_kits.begin() + (long)i);
+        return k;
+      }
+  }
+  auto* k = new CallKit();
+  k->dev = dev;
+  k->timing = true;
+  for (auto& x : k->e) k->timing = k->timing && cudaEventCreate(&x) == cudaSuccess;
+  void* p = nullptr;
+  k->host = cudaMallocHost(&p, sizeof(CallStatus)) == cudaSuccess ? (CallStatus*)p : &k->own;
+  cudaGetLastError();
+  return k;
+}
+
+void kit_release(CallKit* k) {
+  {
+    std::lock_guard<std::mutex> lk(g_kit_mu);
+    if (g_kits.size() < kMaxKits) {
+      g_kits.push_back(k);
+      return;
+    }
+  }
+  kit_free(k);
+}
+
 void trim_pools() {
+  std::vector<CallKit*> idle;
+  {
+    std::lock_guard<std::mutex> lk(g_kit_mu);
+    idle.swap(g_kits);
+  }
+  for (CallKit* k : idle) kit_free(k);
   std::lock_guard<std::mutex> lk(g_pool_mu);
   for (auto& pool : g_pool)
     if (pool) cudaMemPoolTrimTo(pool, 0);
