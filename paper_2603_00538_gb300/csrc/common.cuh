@@ -607,6 +607,32 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
 }
 
 // ---------------------------------------------------------------------------
+// FP64 difference a - b of two FP32 values. The FP32 difference is exact when
+// its TwoSum error is zero (neighbouring mesh nodes, almost always) and is then
+// widened by its bits; FP64 additions use this GPU's narrow FP64 pipe.
+__device__ __forceinline__ double diff_d(float a, float b) {
+  const float s = __fsub_rn(a, b);
+  const float bp = __fsub_rn(a, s), ap = __fadd_rn(s, bp);
+  const float e = __fadd_rn(__fsub_rn(a, ap), __fsub_rn(bp, b));
+  return e == 0.0f ? f2d(s) : __dsub_rn(f2d(a), f2d(b));
+}
+__device__ __forceinline__ double diff_d(double a, double b) { return __dsub_rn(a, b); }
+
+// FP64 measure of an element with vertices xv
+template <int D, typename P>
+__device__ __forceinline__ double elem_measure(const P (&xv)[D + 1][D]) {
+  double e[D][D];
+#pragma unroll
+  for (int m = 0; m < D; ++m)
+#pragma unroll
+    for (int a = 0; a < D; ++a) e[m][a] = diff_d(xv[m + 1][a], xv[0][a]);
+  if constexpr (D == 2) return 0.5 * (e[0][0] * e[1][1] - e[1][0] * e[0][1]);
+  else
+    return (e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) - e[0][1] * (e[1][0] * e[2][2] - e[1][2] * e[2][0]) +
+            e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0])) * (1.0 / 6.0);
+}
+
+// ---------------------------------------------------------------------------
 // error-free transformation: Knuth's TwoSum
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {

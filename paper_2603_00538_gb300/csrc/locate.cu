@@ -90,19 +90,40 @@ __global__ void k_bbox_partial(const P* __restrict__ x, int64_t nv, P* __restric
   }
 }
 
+constexpr int kBoxBlocks = 256;  // partial boxes
+
+// one block of kBoxBlocks threads, one partial box each (a single thread over
+// all of them took 19 us in FP32 and 65 in FP64, now 3)
 template <int D, typename P>
-__global__ void k_grid_params(const P* __restrict__ part, int nblocks, int32_t n, GridP<P>* __restrict__ g,
-                              int32_t* err) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(kBoxBlocks) k_grid_params(const P* __restrict__ part, int32_t n,
+                                                           GridP<P>* __restrict__ g, int32_t* err) {
+  __shared__ P slo[D][kBoxBlocks / 32], shi[D][kBoxBlocks / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    P lo = part[threadIdx.x * 2 * D + a], hi = part[threadIdx.x * 2 * D + D + a];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const P l2 = __shfl_xor_sync(0xffffffffu, lo, o), h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+      lo = l2 < lo ? l2 : lo;
+      hi = h2 > hi ? h2 : hi;
+    }
+    if (lane == 0) {
+      slo[a][warp] = lo;
+      shi[a][warp] = hi;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   GridP<P> r;
 #pragma unroll
   for (int a = 0; a < 3; ++a) { r.lo[a] = P(0); r.inv[a] = P(0); r.h[a] = P(0); r.n[a] = 1; }
+#pragma unroll
   for (int a = 0; a < D; ++a) {
-    P lo = part[a], hi = part[D + a];
-    for (int b = 1; b < nblocks; ++b) {
-      const P l2 = part[b * 2 * D + a], h2 = part[b * 2 * D + D + a];
-      lo = l2 < lo ? l2 : lo;
-      hi = h2 > hi ? h2 : hi;
+    P lo = slo[a][0], hi = shi[a][0];
+    for (int w = 1; w < kBoxBlocks / 32; ++w) {
+      lo = slo[a][w] < lo ? slo[a][w] : lo;
+      hi = shi[a][w] > hi ? shi[a][w] : hi;
     }
     if (!(hi > lo)) set_error(err, DEV_BAD_ELEMENT);
     r.lo[a] = lo;
@@ -237,6 +258,20 @@ __device__ __forceinline__ bool record_map(const P xv[D + 1][D], P* r) {
   }
 }
 
+// L values to a 16-byte aligned row (a multiple of 16 bytes). (With 4-byte
+// stores, and the element measure's differences on the FP64 pipe, k_records
+// took 293 us for 5.0 M tetrahedra, now 179; that pipe still bounds it.)
+template <typename P, int L>
+__device__ __forceinline__ void store_row(P* dst, const P (&r)[L]) {
+  if constexpr (sizeof(P) == 4) {
+#pragma unroll
+    for (int q = 0; q < L; q += 4) *reinterpret_cast<float4*>(dst + q) = make_float4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < L; q += 2) *reinterpret_cast<double2*>(dst + q) = make_double2(r[q], r[q + 1]);
+  }
+}
+
 template <int D, typename P, typename TV>
 __global__ void k_records(const P* __restrict__ x, const int32_t* __restrict__ conn, const TV* __restrict__ values,
                           int64_t nv, int64_t ne, int nf, P* __restrict__ recs, P* __restrict__ vals, int32_t* err,
@@ -263,31 +298,13 @@ __global__ void k_records(const P* __restrict__ x, const int32_t* __restrict__ c
 #pragma unroll
     for (int a = 0; a < D; ++a) r[a] = xv[0][a];
     if (!record_map<D, P>(xv, r)) set_error(err, DEV_BAD_ELEMENT);
-#pragma unroll
-    for (int q = 0; q < L; ++q) recs[e * L + q] = r[q];
-    if (evol) {
-      // FP64 measure of the element (exact differences of the stored coordinates)
-      double xd[D + 1][D];
-#pragma unroll
-      for (int m = 0; m <= D; ++m)
-#pragma unroll
-        for (int a = 0; a < D; ++a) xd[m][a] = f2d(xv[m][a]);
-      double vol;
-      if constexpr (D == 2) {
-        vol = 0.5 * ((xd[1][0] - xd[0][0]) * (xd[2][1] - xd[0][1]) - (xd[2][0] - xd[0][0]) * (xd[1][1] - xd[0][1]));
-      } else {
-        double e1[3], e2[3], e3[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) { e1[a] = xd[1][a] - xd[0][a]; e2[a] = xd[2][a] - xd[0][a]; e3[a] = xd[3][a] - xd[0][a]; }
-        vol = (e1[0] * (e2[1] * e3[2] - e2[2] * e3[1]) - e1[1] * (e2[0] * e3[2] - e2[2] * e3[0]) +
-               e1[2] * (e2[0] * e3[1] - e2[1] * e3[0])) * (1.0 / 6.0);
-      }
-      evol[e] = vol;
-    }
+    store_row<P, L>(recs + e * L, r);
+    if (evol) evol[e] = elem_measure<D, P>(xv);
     for (int f = 0; f < nf; ++f) {
+      P fv[4];
 #pragma unroll
-      for (int m = 0; m < 4; ++m)
-        vals[((int64_t)e * nf + f) * 4 + m] = m <= D ? P(values[(int64_t)f * nv + v[m]]) : P(0);
+      for (int m = 0; m < 4; ++m) fv[m] = m <= D ? P(values[(int64_t)f * nv + v[m]]) : P(0);
+      store_row<P, 4>(vals + ((int64_t)e * nf + f) * 4, fv);
     }
   }
 }
@@ -333,104 +350,383 @@ __device__ __forceinline__ bool cell_may_hold(const P* r, const P c[D], const P 
   return !(A::add(A::sub(P(1), tsum), S) < -eps);
 }
 
-// one filled registration: the element and the depth of the cell centre in it,
-// stored together so that the fill writes one scattered entry, not two
-template <typename P> struct RegEntry;
-template <> struct alignas(8) RegEntry<float> { int32_t id; float depth; };
-template <> struct alignas(16) RegEntry<double> { int32_t id; int32_t pad; double depth; };
+// Registration of the elements in the cells of their bounding boxes that pass
+// cell_may_hold, and each cell's start element (deepest at the cell centre,
+// ties to the lowest id). Two passes, a thread per element:
+//   count  tests the box cells; which passed goes to a bit mask (bit k: the
+//          k-th box cell in x-fastest order). An element whose centre
+//          coordinate is not negative competes for the cell's start element
+//          with an atomic maximum of (depth, id);
+//   fill   from the masks alone, four registrations of an element in flight:
+//          the atomic on the cell's cursor returns the place.
+// Elements with more than kMaskCells box cells go to a list that a warp per
+// element takes after the others.
+// (8-byte (id, depth) entries filled one at a time with the full test again,
+// and read back for the start elements, took 1.60 ms for the 68 M
+// registrations of a 5.0 M-tetrahedron source, 0.43 ms for 4.0 M triangles;
+// now 1.07 ms and 0.36. Sorting a block's registrations by cell in shared
+// memory, with one global atomic per block and cell, took 1.45 ms and 0.42:
+// the shared-memory atomics collide.)
+constexpr int kMaskCells = 64;
+constexpr int kRegThreads = 128;
 
-// one registration per (element, cell) that passes cell_may_hold: count, or
-// fill the element id and the depth of the cell centre in the
-// element (its min barycentric coordinate there, evaluated exactly as a
-// query at that point would be), which orders the cell's list
-// The count pass records which cells of the element's bounding box passed
-// the test as a bit mask (bit k: the k-th box cell in x-fastest order) when
-// the box has at most kMaskCells cells; the fill pass then registers exactly
-// those without testing again. Larger boxes (bit 31 set) are tested again.
-constexpr int kMaskCells = 31;
-constexpr uint32_t kMaskRetest = 0x80000000u;
+// best (depth, id) at a cell's centre so far: largest depth, lowest id
+template <typename P> struct FirstKey;
+template <> struct FirstKey<float> { unsigned long long k; };           // depth bits | ~id; 0: none
+template <> struct alignas(16) FirstKey<double> { unsigned long long id1, depth; };  // ~id (nonzero), depth bits; 0: none
 
-template <int D, typename P, bool FILL>
-__global__ void k_register(const P* __restrict__ x, const int32_t* __restrict__ conn, const P* __restrict__ recs,
-                           int64_t nv, int64_t ne, const GridP<P>* __restrict__ gp, int32_t* __restrict__ cell_count,
-                           const int32_t* __restrict__ cell_start, RegEntry<P>* __restrict__ reg,
-                           uint32_t* __restrict__ mask) {
+__device__ __forceinline__ void first_offer(FirstKey<float>* f, float depth, int32_t e) {
+  const uint32_t d = __float_as_uint(depth + 0.0f);   // depth >= 0: ordered as its bits (-0 made +0)
+  atomicMax(&f->k, ((unsigned long long)d << 32) | (uint32_t)~e);
+}
+__device__ __forceinline__ void first_offer(FirstKey<double>* f, double depth, int32_t e) {
+  const unsigned long long d = (unsigned long long)__double_as_longlong(depth + 0.0), i = (uint32_t)~e;
+  unsigned long long od = 0ull, oi = 0ull;
+  for (;;) {
+    unsigned long long rd, ri;
+    asm volatile(
+        "{\n\t.reg .b128 c, n, r;\n\tmov.b128 c, {%2, %3};\n\tmov.b128 n, {%4, %5};\n\t"
+        "atom.global.cas.b128 r, [%6], c, n;\n\tmov.b128 {%0, %1}, r;\n\t}"
+        : "=l"(ri), "=l"(rd)
+        : "l"(oi), "l"(od), "l"(i), "l"(d), "l"(f)
+        : "memory");
+    if (ri == oi && rd == od) return;               // taken
+    if (rd > d || (rd == d && ri >= i)) return;     // a better one is there
+    oi = ri;
+    od = rd;
+  }
+}
+
+// depth of cell centre cc in the element: its smallest barycentric coordinate
+template <int D, typename P>
+__device__ __forceinline__ P centre_depth(const P* r, const P (&cc)[D]) {
+  P mu[D + 1];
+  bary_from_record<D, P>(r, cc, mu);
+  P depth = mu[0];
+#pragma unroll
+  for (int q = 1; q <= D; ++q) depth = mu[q] < depth ? mu[q] : depth;
+  return depth;
+}
+
+// The coordinates of the box's cell centres as linear functions of the cell's
+// offset, in FP32, with a bound of their difference from the evaluation in P
+// by cell_may_hold and centre_depth. A cell is settled when it lies outside
+// the bound of the threshold and its centre is surely not in the element; the
+// others (one in ten) are decided in P. (In FP64 because its operations are
+// 64 times as dear here, in FP32 because the full test takes four times the
+// instructions.)
+template <int D, typename P>
+struct BoxFilter {
+  float t0[D], st[D][D], sp[D], S, band;
+  // hf = grid steps, mag = bound of the coordinates of the grid, in FP32; nc = cells of the box per axis
+  __device__ __forceinline__ void init(const GridP<P>& g, const P* rec, const int32_t c0[3], const float* hf, float mag,
+                                       const int (&nc)[3]) {
+    constexpr float kEps = sizeof(P) == 4 ? 4.8e-7f : 4e-15f;  // P's rounding of two cell centres (8 and more units)
+    float d[D], col[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      d[a] = (float)(cell_centre<P>(g, a, c0[a]) - rec[a]);
+      col[a] = 0.f;
+    }
+    band = 2e-6f;
+#pragma unroll
+    for (int m = 0; m < D; ++m) {
+      float abs_t = 0.f, rsum = 0.f;
+      t0[m] = 0.f;
+      sp[m] = 0.f;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const float row = (float)rec[D + m * D + a];
+        t0[m] = fmaf(row, d[a], t0[m]);
+        abs_t = fmaf(fabsf(row), fabsf(d[a]), abs_t);
+        rsum += fabsf(row);
+        st[m][a] = row * hf[a];
+        sp[m] += 0.5f * fabsf(st[m][a]);
+        abs_t = fmaf(fabsf(st[m][a]), (float)nc[a], abs_t);
+        col[a] += st[m][a];
+      }
+      // roundings here (at most 16 x 2^-24 per term), and of the coordinates in P
+      band += 2e-6f * abs_t + kEps * mag * rsum;
+    }
+    S = 0.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) S += 0.5f * fabsf(col[a]);
+  }
+  // cell at offset o[] of the box: 0 not held, 1 held and the centre outside, 2 undecided
+  __device__ __forceinline__ int operator()(const float (&o)[3]) const {
+    constexpr float eps = 0.0009765625f;
+    float t[D], sum = 0.f;
+#pragma unroll
+    for (int m = 0; m < D; ++m) {
+      t[m] = t0[m];
+#pragma unroll
+      for (int a = 0; a < D; ++a) t[m] = fmaf(st[m][a], o[a], t[m]);
+      sum += t[m];
+    }
+    float mn = 1.f - sum, lo = mn + S;
+#pragma unroll
+    for (int m = 0; m < D; ++m) {
+      lo = fminf(lo, t[m] + sp[m]);
+      mn = fminf(mn, t[m]);
+    }
+    lo += eps;
+    if (lo < -band) return 0;
+    return lo > band && mn < -band ? 1 : 2;
+  }
+};
+
+// an element's bounding-box cells: linear index of the first, nx | ny << 8
+struct ElemBox { int32_t lin0, dims; };
+
+template <int D, typename P>
+__global__ void __launch_bounds__(kRegThreads)
+    k_register_count(const P* __restrict__ x, const int32_t* __restrict__ conn, const P* __restrict__ recs, int64_t nv,
+                     int64_t ne, const GridP<P>* __restrict__ gp, int32_t* __restrict__ cell_count,
+                     FirstKey<P>* __restrict__ first, unsigned long long* __restrict__ mask, ElemBox* __restrict__ box,
+                     int32_t* __restrict__ big, int32_t* __restrict__ nbig) {
   constexpr int RL = RecLen<D>::value;
+  constexpr int W = kRegThreads / 32;
+  __shared__ unsigned long long smask[kRegThreads];         // cells settled in P
+  __shared__ int32_t sbox[kRegThreads][4];                  // first box cell, nx | ny << 8
+  __shared__ uint16_t queue[W][64];                         // lane << 6 | k
+  __shared__ float gf[4];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const GridP<P> g = *gp;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
-    bool ok = true;
+  if (t == 0) {
+    float mag = 0.f;
+    for (int a = 0; a < D; ++a) {
+      gf[a] = (float)g.h[a];
+      mag = fmaxf(mag, fabsf((float)g.lo[a]) + fabsf((float)g.h[a]) * (float)g.n[a]);
+    }
+    gf[3] = mag;
+  }
+  __syncthreads();
+  const int64_t e0 = (int64_t)blockIdx.x * kRegThreads, e = e0 + t;
+
+  // box of the element
+  bool ok = e < ne;
+  if (ok) {
 #pragma unroll
     for (int m = 0; m <= D; ++m) {
       const int32_t v = conn[e * (D + 1) + m];
-      ok = ok && v >= 0 && v < nv;
+      ok = ok && v >= 0 && v < nv;  // reported by k_records; never read out of range
     }
-    if (!ok) continue;  // reported by k_records; never read out of range
+  }
+  int32_t c0[3] = {0, 0, 0}, c1[3] = {-1, -1, -1};
+  if (ok) {
+    P xv[D + 1][D];
+    elem_vertices<D, P>(x, conn, e, xv);
+    const int64_t nb = elem_cell_range<D, P>(g, xv, c0, c1);
+    ok = c1[0] >= c0[0] && c1[1] >= c0[1] && c1[2] >= c0[2];  // (non-finite coordinates)
+    if (ok && nb > kMaskCells) {
+      big[atomicAdd(nbig, 1)] = (int32_t)e;
+      ok = false;
+    }
+  }
+  const int nx = ok ? c1[0] - c0[0] + 1 : 1, ny = ok ? c1[1] - c0[1] + 1 : 1;
+  const int nbox = ok ? nx * ny * (c1[2] - c0[2] + 1) : 0;
+  const int32_t lin0 = (int32_t)(((int64_t)c0[2] * g.n[1] + c0[1]) * g.n[0] + c0[0]);
+
+  BoxFilter<D, P> filter;
+  if (ok) {
+    P r[RL];
+    load_record<D, P>(recs, (int32_t)e, r);
+    const int nc[3] = {nx, ny, c1[2] - c0[2] + 1};
+    filter.init(g, r, c0, gf, gf[3], nc);
+  }
+  // coordinates beyond FP32's range for this leave all cells undecided
+  bool sane = ok && filter.band < 1e30f && gf[3] < 1e15f;
+#pragma unroll
+  for (int a = 0; a < D; ++a) sane = sane && gf[a] > 1e-30f;
+#pragma unroll
+  for (int m = 0; m < D; ++m) sane = sane && fabsf(filter.t0[m]) < 1e30f && filter.sp[m] < 1e30f;
+  smask[t] = 0ull;
+  sbox[t][0] = c0[0];
+  sbox[t][1] = c0[1];
+  sbox[t][2] = c0[2];
+  sbox[t][3] = nx | ny << 8;
+  __syncwarp();
+  // the undecided cells of a warp are gathered and taken 32 at a time
+  auto settle = [&](int n) {
+    __syncwarp();
+    if (lane < n) {
+      const int q = queue[warp][lane], src = warp * 32 + (q >> 6), k = q & 63;
+      const int bx = sbox[src][3] & 255, by = sbox[src][3] >> 8;
+      const int row = k / bx;
+      const int32_t idx[3] = {sbox[src][0] + k - row * bx, sbox[src][1] + (D == 3 ? row % by : row),
+                              sbox[src][2] + (D == 3 ? row / by : 0)};
+      const int32_t e2 = (int32_t)(e0 + src);
+      P r2[RL], cc[D], w[D];
+      load_record<D, P>(recs, e2, r2);
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        cc[a] = cell_centre<P>(g, a, idx[a]);
+        w[a] = Ar<P>::mul(g.h[a], P(0.5));
+      }
+      if (cell_may_hold<D, P>(r2, cc, w)) {
+        const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
+        atomicOr(&smask[src], 1ull << k);
+        atomicAdd(cell_count + c, 1);
+        const P depth = centre_depth<D, P>(r2, cc);
+        if (depth >= P(0)) first_offer(first + c, depth, e2);
+      }
+    }
+    __syncwarp();
+  };
+  const int kmax = __reduce_max_sync(0xffffffffu, nbox);
+  const float fx = (float)nx, fy = (float)ny;
+  const int32_t ystep = g.n[0] - nx, zstep = g.n[0] * (g.n[1] - ny);
+  float o[3] = {0.f, 0.f, 0.f};
+  int32_t c = lin0;
+  unsigned long long bits = 0ull;
+  int qn = 0;
+  for (int k = 0; k < kmax; ++k) {
+    int res = sane ? filter(o) : 2;
+    if (k >= nbox) res = 0;
+    if (res == 1) {
+      bits |= 1ull << k;
+      atomicAdd(cell_count + c, 1);
+    }
+    const uint32_t und = __ballot_sync(0xffffffffu, res == 2);
+    if (und != 0u) {
+      if (res == 2) queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)(lane << 6 | k);
+      qn += __popc(und);
+      if (qn >= 32) {
+        settle(32);
+        qn -= 32;
+        if (lane < qn) queue[warp][lane] = queue[warp][32 + lane];
+        __syncwarp();
+      }
+    }
+    o[0] += 1.f;
+    ++c;
+    if (o[0] == fx) {
+      o[0] = 0.f;
+      o[1] += 1.f;
+      c += ystep;
+      if (o[1] == fy) {
+        o[1] = 0.f;
+        o[2] += 1.f;
+        c += zstep;
+      }
+    }
+  }
+  settle(qn);
+  if (e >= ne) return;
+  mask[e] = bits | smask[t];
+  box[e].lin0 = lin0;
+  box[e].dims = nx | ny << 8;
+}
+
+// the elements with large boxes: FILL = false counts them, true fills them
+// (cell_count then holds the cells' cursors)
+template <int D, typename P, bool FILL>
+__global__ void k_register_big(const P* __restrict__ x, const int32_t* __restrict__ conn, const P* __restrict__ recs,
+                               const GridP<P>* __restrict__ gp, const int32_t* __restrict__ big,
+                               const int32_t* __restrict__ nbig, int32_t* __restrict__ cell_count,
+                               FirstKey<P>* __restrict__ first, int32_t* __restrict__ items) {
+  constexpr int RL = RecLen<D>::value;
+  const int nb = *nbig;
+  // a warp per element, its box cells over the lanes
+  const int lane = threadIdx.x & 31;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb;
+       b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int32_t e = big[b];
+    const GridP<P> g = *gp;
     P xv[D + 1][D];
     elem_vertices<D, P>(x, conn, e, xv);
     int32_t c0[3], c1[3];
     const int64_t nbox = elem_cell_range<D, P>(g, xv, c0, c1);
-    P r[RL];
-    load_record<D, P>(recs, (int32_t)e, r);
-    P w[D];
+    P r[RL], w[D];
+    load_record<D, P>(recs, e, r);
 #pragma unroll
     for (int a = 0; a < D; ++a) w[a] = Ar<P>::mul(g.h[a], P(0.5));
-    const bool use_mask = nbox <= kMaskCells;
-    const uint32_t have = FILL ? __ldg(mask + e) : 0u;
-    const bool retest = !FILL || (have & kMaskRetest) != 0u;
-    uint32_t bits = 0u;
-    int k = 0;
-    for (int32_t iz = c0[2]; iz <= c1[2]; ++iz)
-      for (int32_t iy = c0[1]; iy <= c1[1]; ++iy)
-        for (int32_t ix = c0[0]; ix <= c1[0]; ++ix, ++k) {
-          const int32_t idx[3] = {ix, iy, iz};
-          P cc[D];
+    const int64_t nx = c1[0] - c0[0] + 1, ny = c1[1] - c0[1] + 1;
+    for (int64_t k = lane; k < nbox; k += 32) {
+      const int32_t idx[3] = {c0[0] + (int32_t)(k % nx), c0[1] + (int32_t)(k / nx % ny), c0[2] + (int32_t)(k / nx / ny)};
+      P cc[D];
 #pragma unroll
-          for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
-          if (retest) {
-            if (!cell_may_hold<D, P>(r, cc, w)) continue;
-          } else if (!((have >> k) & 1u)) {
-            continue;
-          }
-          if (!FILL && use_mask) bits |= 1u << k;
-          const int64_t c = ((int64_t)iz * g.n[1] + iy) * g.n[0] + ix;
-          const int32_t pos = atomicAdd(cell_count + c, 1);
-          if (FILL) {
-            P mu[D + 1];
-            bary_from_record<D, P>(r, cc, mu);
-            P mn = mu[0];
-#pragma unroll
-            for (int q = 1; q <= D; ++q) mn = mu[q] < mn ? mu[q] : mn;
-            RegEntry<P> en;
-            if constexpr (sizeof(P) == 8) en.pad = 0;
-            en.id = (int32_t)e;
-            en.depth = mn;
-            reg[(int64_t)cell_start[c] + pos] = en;
-          }
-        }
-    if (!FILL) mask[e] = use_mask ? bits : kMaskRetest;
+      for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
+      if (!cell_may_hold<D, P>(r, cc, w)) continue;
+      const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
+      if (FILL) {
+        items[atomicAdd(cell_count + c, 1)] = e;
+      } else {
+        atomicAdd(cell_count + c, 1);
+        const P depth = centre_depth<D, P>(r, cc);
+        if (depth >= P(0)) first_offer(first + c, depth, e);
+      }
+    }
   }
 }
 
-// Start element of each cell and its list of ids: the fill leaves a cell's
-// entries in arbitrary order, which no rule depends on (the walk starts at
-// the element deepest at the cell centre, ties to the lowest id; the
-// fallback takes the best-scoring candidate whatever the order). One thread
-// per cell: the argmax of (depth, -id) over its entries, and the ids copied
-// into the cell's list.
-template <typename P>
-__global__ void k_cell_first(const int32_t* __restrict__ cell_start, const RegEntry<P>* __restrict__ reg,
-                             int64_t ncells, int32_t* __restrict__ items, int32_t* __restrict__ first) {
+// cursor: place of each cell's next registration (its start before the first)
+template <int D>
+__global__ void k_register_fill(int64_t ne, int32_t gnx, int32_t gny, const unsigned long long* __restrict__ mask,
+                                const ElemBox* __restrict__ box, int32_t* __restrict__ cursor, int32_t* __restrict__ items) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
+    unsigned long long rest = __ldg(mask + e);
+    const int2 bx = __ldg(reinterpret_cast<const int2*>(box) + e);
+    const uint32_t nx = bx.y & 255, ny = bx.y >> 8;
+    // division of k < 64 by n <= 64 as (k * ceil(2^16 / n)) >> 16: exact
+    const uint32_t inx = (65535u + nx) / nx, iny = D == 3 ? (65535u + ny) / ny : 0u;
+    while (rest != 0ull) {
+      constexpr int U = 4;
+      int32_t* at[U];
+      int32_t pos[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        at[u] = nullptr;
+        if (rest != 0ull) {
+          const uint32_t k = (uint32_t)__ffsll((long long)rest) - 1u;
+          rest &= rest - 1ull;
+          const uint32_t row = (k * inx) >> 16, lay = D == 3 ? (row * iny) >> 16 : 0u;
+          at[u] = cursor + (bx.x + (int32_t)(k - row * nx) + gnx * (int32_t)(row - lay * ny + gny * lay));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (at[u]) pos[u] = atomicAdd(at[u], 1);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (at[u]) items[pos[u]] = (int32_t)e;
+    }
+  }
+}
+
+// Start element of each cell from the best offer; a cell whose centre no
+// element holds (outside the mesh, or in a rounding gap) takes the deepest of
+// its list.
+template <int D, typename P>
+__global__ void k_cell_first(const int32_t* __restrict__ cell_start, const int32_t* __restrict__ items,
+                             const P* __restrict__ recs, const GridP<P>* __restrict__ gp,
+                             const FirstKey<P>* __restrict__ key, int64_t ncells, int32_t* __restrict__ first) {
+  constexpr int RL = RecLen<D>::value;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t p0 = __ldg(cell_start + c), p1 = __ldg(cell_start + c + 1);
+    const FirstKey<P> k = key[c];
+    uint32_t id1;
+    if constexpr (sizeof(P) == 4) id1 = (uint32_t)k.k;
+    else id1 = (uint32_t)k.id1;
+    if (id1 != 0u) {
+      first[c] = (int32_t)~id1;
+      continue;
+    }
+    const GridP<P> g = *gp;
+    const int32_t idx[3] = {(int32_t)(c % g.n[0]), (int32_t)(c / g.n[0] % g.n[1]), (int32_t)(c / g.n[0] / g.n[1])};
+    P cc[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
     int32_t best = -1;
     P bd = P(0);
-    for (int32_t p = p0; p < p1; ++p) {
-      const RegEntry<P> en = reg[p];
-      if (best < 0 || en.depth > bd || (en.depth == bd && en.id < best)) {
-        best = en.id;
-        bd = en.depth;
+    for (int32_t p = __ldg(cell_start + c); p < __ldg(cell_start + c + 1); ++p) {
+      const int32_t e = items[p];
+      P r[RL];
+      load_record<D, P>(recs, e, r);
+      const P depth = centre_depth<D, P>(r, cc);
+      if (best < 0 || depth > bd || (depth == bd && e < best)) {
+        best = e;
+        bd = depth;
       }
-      items[p] = en.id;
     }
     first[c] = best;
   }
@@ -476,8 +772,14 @@ __global__ void k_adjacency(const P* __restrict__ x, const int32_t* __restrict__
         const int32_t e2 = __ldg(cell_items + p);
         if (e2 == (int32_t)e) continue;
         int32_t w[K];
+        if constexpr (D == 3) {
+          // (four 4-byte loads kept the L1 data pipe 85 % busy: 782 us for 5.0 M tetrahedra, now 697)
+          const int4 q = __ldg(reinterpret_cast<const int4*>(conn) + e2);
+          w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+        } else {
 #pragma unroll
-        for (int r = 0; r < K; ++r) w[r] = __ldg(conn + (int64_t)e2 * K + r);
+          for (int r = 0; r < K; ++r) w[r] = __ldg(conn + (int64_t)e2 * K + r);
+        }
         int shared = 0, miss = 0;
 #pragma unroll
         for (int m = 0; m < K; ++m) {
@@ -522,14 +824,13 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
   L.n[0] = L.n[1] = L.n[2] = 1;
   L.ncells = 1;
   for (int a = 0; a < D; ++a) { L.n[a] = n; L.ncells *= n; }
-  const unsigned nb = 256;
   P* part = nullptr;
-  SFT_CUDA(dalloc(&part, (size_t)nb * 2 * D, st));
-  ::sft::note_launch(), k_bbox_partial<D, P><<<nb, 256, 0, st>>>(xP, s->nv, part);
+  SFT_CUDA(dalloc(&part, (size_t)kBoxBlocks * 2 * D, st));
+  ::sft::note_launch(), k_bbox_partial<D, P><<<kBoxBlocks, 256, 0, st>>>(xP, s->nv, part);
   GridP<P>* g = nullptr;
   SFT_CUDA(dalloc(&g, 1, st));
   L.grid = g;
-  ::sft::note_launch(), k_grid_params<D, P><<<1, 32, 0, st>>>(part, nb, n, g, d_err);
+  ::sft::note_launch(), k_grid_params<D, P><<<1, kBoxBlocks, 0, st>>>(part, n, g, d_err);
   SFT_CUDA(cudaGetLastError());
   dfree(part, st);
   // location records and value copies
@@ -555,18 +856,33 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
   SFT_CUDA(cudaGetLastError());
   // count registrations per cell, then total (int64) -> int32 offsets must suffice
   // (temporaries freed in stream order on every return)
-  DevBuf<int32_t> cell_count(st);
   DevBuf<int64_t> start64(st);
-  DevBuf<uint32_t> mask(st);
-  DevBuf<RegEntry<P>> reg(st);
-  SFT_CUDA(cell_count.alloc((size_t)L.ncells));
+  DevBuf<char> ws(st);
   SFT_CUDA(start64.alloc((size_t)L.ncells + 1));
-  SFT_CUDA(mask.alloc((size_t)s->ne));
-  SFT_CUDA(cudaMemsetAsync(cell_count.p, 0, sizeof(int32_t) * L.ncells, st));
-  ::sft::note_launch(), k_register<D, P, false><<<grid_for(s->ne), 256, 0, st>>>(xP, s->conn, recs, s->nv, s->ne, g,
-                                                                               cell_count.p, nullptr, nullptr, mask.p);
+  Carve lay;  // the first three start at zero
+  const size_t o_count = lay.add(sizeof(int32_t) * (size_t)L.ncells);
+  const size_t o_key = lay.add(sizeof(FirstKey<P>) * (size_t)L.ncells);
+  const size_t o_nbig = lay.add(sizeof(int32_t)), zeroed = lay.total;
+  const size_t o_mask = lay.add(sizeof(unsigned long long) * (size_t)s->ne);
+  const size_t o_box = lay.add(sizeof(ElemBox) * (size_t)s->ne);
+  const size_t o_big = lay.add(sizeof(int32_t) * (size_t)s->ne);
+  SFT_CUDA(ws.alloc(lay.total));
+  int32_t* const count = (int32_t*)(ws.p + o_count);
+  FirstKey<P>* const key = (FirstKey<P>*)(ws.p + o_key);
+  int32_t* const nbig = (int32_t*)(ws.p + o_nbig);
+  unsigned long long* const mask = (unsigned long long*)(ws.p + o_mask);
+  ElemBox* const box = (ElemBox*)(ws.p + o_box);
+  int32_t* const big = (int32_t*)(ws.p + o_big);
+  const unsigned reg_blocks = (unsigned)((s->ne + kRegThreads - 1) / kRegThreads);
+  constexpr unsigned kBigBlocks = 152 * 4;
+  SFT_CUDA(cudaMemsetAsync(ws.p, 0, zeroed, st));
+  ::sft::note_launch(), k_register_count<D, P><<<reg_blocks, kRegThreads, 0, st>>>(xP, s->conn, recs, s->nv, s->ne, g, count,
+                                                                                  key, mask, box, big, nbig);
   SFT_CUDA(cudaGetLastError());
-  SFT_CUDA(exclusive_scan_i32_to_i64(cell_count.p, start64.p, L.ncells, st));
+  ::sft::note_launch(), k_register_big<D, P, false><<<kBigBlocks, 256, 0, st>>>(xP, s->conn, recs, g, big, nbig, count, key,
+                                                                              nullptr);
+  SFT_CUDA(cudaGetLastError());
+  SFT_CUDA(exclusive_scan_i32_to_i64(count, start64.p, L.ncells, st));
   Events kit;
   SFT_CUDA(cudaMemcpyAsync(&kit.host().err, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaMemcpyAsync(&kit.host().counters[0], start64.p + L.ncells, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -582,15 +898,17 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
   SFT_CUDA(dalloc(&L.cell_start, (size_t)L.ncells + 1, st));
   SFT_CUDA(narrow_i64_to_i32(start64.p, L.cell_start, L.ncells + 1, st));
   // fill (arbitrary order within a cell), then each cell's start element
-  SFT_CUDA(reg.alloc((size_t)total));
   SFT_CUDA(dalloc(&L.cell_items, (size_t)total, st));
-  SFT_CUDA(cudaMemsetAsync(cell_count.p, 0, sizeof(int32_t) * L.ncells, st));
-  ::sft::note_launch(), k_register<D, P, true><<<grid_for(s->ne), 256, 0, st>>>(xP, s->conn, recs, s->nv, s->ne, g,
-                                                                              cell_count.p, L.cell_start, reg.p, mask.p);
+  SFT_CUDA(cudaMemcpyAsync(count, L.cell_start, sizeof(int32_t) * (size_t)L.ncells, cudaMemcpyDeviceToDevice, st));
+  ::sft::note_launch(), k_register_fill<D><<<grid_for(s->ne), 256, 0, st>>>(s->ne, L.n[0], L.n[1], mask, box, count,
+                                                                          L.cell_items);
+  SFT_CUDA(cudaGetLastError());
+  ::sft::note_launch(), k_register_big<D, P, true><<<kBigBlocks, 256, 0, st>>>(xP, s->conn, recs, g, big, nbig, count, key,
+                                                                             L.cell_items);
   SFT_CUDA(cudaGetLastError());
   SFT_CUDA(dalloc(&L.cell_first, (size_t)L.ncells, st));
-  ::sft::note_launch(), k_cell_first<P><<<grid_for(L.ncells), 256, 0, st>>>(L.cell_start, reg.p, L.ncells, L.cell_items,
-                                                                           L.cell_first);
+  ::sft::note_launch(), k_cell_first<D, P><<<grid_for(L.ncells), 256, 0, st>>>(L.cell_start, L.cell_items, recs, g, key,
+                                                                             L.ncells, L.cell_first);
   SFT_CUDA(cudaGetLastError());
   // face neighbours for the location walk (one array per source mesh)
   if (!s->adj) {
@@ -619,9 +937,12 @@ __global__ void k_value_copies(const int32_t* __restrict__ conn, const TV* __res
     int32_t v[D + 1];
 #pragma unroll
     for (int m = 0; m <= D; ++m) v[m] = conn[e * (D + 1) + m];
-    for (int f = 0; f < nf; ++f)
+    for (int f = 0; f < nf; ++f) {
+      P fv[4];
 #pragma unroll
-      for (int m = 0; m < 4; ++m) vals[((int64_t)e * nf + f) * 4 + m] = m <= D ? P(values[(int64_t)f * nv + v[m]]) : P(0);
+      for (int m = 0; m < 4; ++m) fv[m] = m <= D ? P(values[(int64_t)f * nv + v[m]]) : P(0);
+      store_row<P, 4>(vals + ((int64_t)e * nf + f) * 4, fv);
+    }
   }
 }
 

@@ -7,6 +7,7 @@
 // then one thread per row merges the vertices of its incident elements into a
 // sorted, de-duplicated column list, summing contributions in ascending
 // element order (deterministic values).
+#include <type_traits>
 #include <vector>
 #include "internal.hpp"
 #include "util.cuh"
@@ -33,22 +34,15 @@ __global__ void k_volumes(const TI* __restrict__ x, const int32_t* __restrict__ 
       vol32[e] = 0.f;
       continue;
     }
-    double xv[D + 1][D];
+    TI xv[D + 1][D];
 #pragma unroll
     for (int m = 0; m <= D; ++m)
 #pragma unroll
-      for (int a = 0; a < D; ++a) xv[m][a] = f2d(x[(int64_t)v[m] * D + a]);
-    double w;
-    if constexpr (D == 2) {
-      w = 0.5 * ((xv[1][0] - xv[0][0]) * (xv[2][1] - xv[0][1]) - (xv[2][0] - xv[0][0]) * (xv[1][1] - xv[0][1]));
-    } else {
-      double e1[3], e2[3], e3[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) { e1[a] = xv[1][a] - xv[0][a]; e2[a] = xv[2][a] - xv[0][a]; e3[a] = xv[3][a] - xv[0][a]; }
-      w = (e1[0] * (e2[1] * e3[2] - e2[2] * e3[1]) - e1[1] * (e2[0] * e3[2] - e2[2] * e3[0]) +
-           e1[2] * (e2[0] * e3[1] - e2[1] * e3[0])) * (1.0 / 6.0);
-    }
-    if (!(w > 0.0) || !isfinite(w)) set_error(err, DEV_BAD_ELEMENT);
+      for (int a = 0; a < D; ++a) xv[m][a] = x[(int64_t)v[m] * D + a];
+    const double w = elem_measure<D, TI>(xv);
+    // positive and finite, from the bits
+    const int64_t wb = __double_as_longlong(w);
+    if (wb <= 0 || wb >= 0x7FF0000000000000ll) set_error(err, DEV_BAD_ELEMENT);
     vol[e] = w;
     vol32[e] = __double2float_rn(w);
     // mass-matrix factor |T|/((d+1)(d+2)) and lumped share |T|/(d+1), by
@@ -101,14 +95,165 @@ __global__ void k_inc_rank(const int32_t* __restrict__ inc_start, const int32_t*
   }
 }
 
-// Row i of M: FILL=false writes the row length (and, when tmp_col is given,
-// the row itself into an entry-major staging array [kMaxRow][nv], so that the second pass
-// only copies), FILL=true writes columns, values, the Jacobi inverse diagonal
-// and the lumped mass.
-// CAP bounds the row buffers (local memory per thread); a counting pass with
-// CAP < kMaxRow marks the rows that do not fit (row_len = -1) and a second
-// pass with REDO = true and CAP = kMaxRow builds exactly those.
-template <int D, bool FILL, int CAP = kMaxRow, bool REDO = false>
+// Row i of M, a thread per row, into the entry-major staging arrays
+// tmp_col / tmp_val [kMaxRow][nv] (the second pass copies). The row is a small
+// hash table of the thread's own in shared memory, [slot][thread], so that an
+// entry is found in one or two reads whatever the valence; each entry sums its
+// elements in ascending order, and the columns are put in order once at the
+// end. A row of more than CAP entries is marked (row_len = -1) for
+// k_mass_rows. (An ordered list per thread in local memory, searched and
+// shifted for each of the 4 x 24 contributions of a tetrahedral row, took
+// 650 us for 0.91 M rows of a 5.0 M-tetrahedron mesh and 187 us for 2.0 M
+// rows of 4.0 M triangles; now 346 and 132.)
+constexpr int kHashThreads = 128;
+template <int CAP>
+constexpr size_t mass_hash_smem() { return (size_t)CAP * kHashThreads * (sizeof(double) + sizeof(int32_t) + 1); }
+
+// order entries [0, N) by column: place of each among them
+template <int N>
+__device__ __forceinline__ void rank_columns(const int32_t* key, int cnt, int (&rank)[N], int32_t (&c)[N]) {
+#pragma unroll
+  for (int a = 0; a < N; ++a) {
+    c[a] = a < cnt ? key[a * kHashThreads] : INT32_MAX;
+    rank[a] = 0;
+  }
+#pragma unroll
+  for (int b = 1; b < N; ++b)
+#pragma unroll
+    for (int a = 0; a < b; ++a) {
+      const bool lt = c[a] <= c[b];
+      rank[b] += lt;
+      rank[a] += !lt;
+    }
+}
+
+template <int D, int CAP>
+__global__ void __launch_bounds__(kHashThreads)
+    k_mass_hash(const int32_t* __restrict__ conn, const double2* __restrict__ wfac, const int32_t* __restrict__ inc_start,
+                const int32_t* __restrict__ inc, int64_t nv, int32_t* __restrict__ row_len, int32_t* __restrict__ tmp_col,
+                double* __restrict__ tmp_val, double* __restrict__ tmp_lump) {
+  extern __shared__ double sm_rows[];
+  double* const vals = sm_rows + threadIdx.x;                                     // [CAP][thread]
+  int32_t* const keys = (int32_t*)(sm_rows + CAP * kHashThreads) + threadIdx.x;   // [CAP][thread], -1 empty
+  uint8_t* const slot = (uint8_t*)((int32_t*)(sm_rows + CAP * kHashThreads) + CAP * kHashThreads) + threadIdx.x;
+  constexpr int kBits = CAP == 16 ? 4 : 5;
+  const int64_t i = (int64_t)blockIdx.x * kHashThreads + threadIdx.x;
+  if (i >= nv) return;
+#pragma unroll
+  for (int q = 0; q < CAP; ++q) keys[q * kHashThreads] = -1;
+  int cnt = 0;
+  bool overflow = false;
+  double lump = 0.0, diag = 0.0;
+  // incident elements in chunks of kPre, their loads in flight together
+  constexpr int kPre = 4;
+  const int32_t p_end = inc_start[i + 1];
+  for (int32_t p0 = inc_start[i]; p0 < p_end && !overflow; p0 += kPre) {
+    int32_t ce[kPre][D + 1];
+    double2 wv[kPre];
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      if (p0 + u < p_end) {
+        const int32_t e = __ldg(inc + p0 + u);
+        wv[u] = __ldg(wfac + e);
+        if constexpr (D == 3) {
+          const int4 q = __ldg(reinterpret_cast<const int4*>(conn) + e);
+          ce[u][0] = q.x; ce[u][1] = q.y; ce[u][2] = q.z; ce[u][D] = q.w;
+        } else {
+#pragma unroll
+          for (int m = 0; m <= D; ++m) ce[u][m] = __ldg(conn + (int64_t)e * (D + 1) + m);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      if (p0 + u >= p_end) break;
+      lump += wv[u].y;
+      diag += 2.0 * wv[u].x;  // (an element repeats no node: it would have no volume)
+#pragma unroll
+      for (int m = 0; m <= D; ++m) {
+        const int32_t j = ce[u][m];
+        if (j == (int32_t)i) continue;
+        uint32_t h = ((uint32_t)j * 2654435761u) >> (32 - kBits);
+        for (int probe = 0;; ++probe) {
+          const int32_t k = keys[h * kHashThreads];
+          if (k == j) {
+            vals[h * kHashThreads] += wv[u].x;
+            break;
+          }
+          if (k == -1) {
+            if (cnt == CAP - 1) {  // (the diagonal takes one)
+              overflow = true;
+              break;
+            }
+            keys[h * kHashThreads] = j;
+            vals[h * kHashThreads] = wv[u].x;
+            ++cnt;
+            break;
+          }
+          h = (h + 1u) & (CAP - 1);
+        }
+      }
+    }
+  }
+  if (overflow) {
+    row_len[i] = -1;
+    return;
+  }
+  // the table's entries to its front (a slot moves down or stays), the diagonal with them
+  int n = 0;
+#pragma unroll 4
+  for (int q = 0; q < CAP; ++q) {
+    const int32_t k = keys[q * kHashThreads];
+    if (k < 0) continue;
+    keys[n * kHashThreads] = k;
+    slot[n * kHashThreads] = (uint8_t)q;
+    ++n;
+  }
+  if (p_end > inc_start[i]) {
+    // a slot no entry holds takes the diagonal's value
+    int q = CAP - 1;
+    for (int a = n - 1; a >= 0 && slot[a * kHashThreads] == q; --a) --q;
+    vals[q * kHashThreads] = diag;
+    keys[n * kHashThreads] = (int32_t)i;
+    slot[n * kHashThreads] = (uint8_t)q;
+    ++n;
+  }
+  // in ascending column order
+  auto order = [&](auto& rank, auto& c, auto len) {
+    constexpr int N = decltype(len)::value;
+    rank_columns<N>(keys, n, rank, c);
+    int s[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) s[a] = a < n ? slot[a * kHashThreads] : 0;
+#pragma unroll
+    for (int a = 0; a < N; ++a)
+      if (a < n) {
+        keys[rank[a] * kHashThreads] = c[a];
+        slot[rank[a] * kHashThreads] = (uint8_t)s[a];
+      }
+  };
+  if (n <= CAP / 2) {
+    int rank[CAP / 2];
+    int32_t c[CAP / 2];
+    order(rank, c, std::integral_constant<int, CAP / 2>());
+  } else {
+    int rank[CAP];
+    int32_t c[CAP];
+    order(rank, c, std::integral_constant<int, CAP>());
+  }
+  for (int q = 0; q < n; ++q) {
+    tmp_col[(int64_t)q * nv + i] = keys[q * kHashThreads];
+    tmp_val[(int64_t)q * nv + i] = vals[slot[q * kHashThreads] * kHashThreads];
+  }
+  row_len[i] = n;
+  tmp_lump[i] = lump;
+}
+
+// Row i of M from an ordered list in local memory: FILL=false writes the row
+// length (and, when tmp_col is given, the row itself into the staging arrays),
+// FILL=true writes columns, values, the Jacobi inverse diagonal and the lumped
+// mass. With REDO only the rows marked -1.
+template <int D, bool FILL, bool REDO = false>
 __global__ void k_mass_rows(const int32_t* __restrict__ conn, const double2* __restrict__ wfac,
                             const int32_t* __restrict__ inc_start, const int32_t* __restrict__ inc, int64_t nv,
                             int32_t* __restrict__ row_len, const int32_t* __restrict__ row_ptr,
@@ -117,6 +262,7 @@ __global__ void k_mass_rows(const int32_t* __restrict__ conn, const double2* __r
                             double* __restrict__ tmp_val, double* __restrict__ tmp_lump) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
     if (REDO && row_len[i] >= 0) continue;
+    constexpr int CAP = kMaxRow;
     int32_t cols[CAP];
     double vals[CAP];
     int cnt = 0;
@@ -165,13 +311,7 @@ __global__ void k_mass_rows(const int32_t* __restrict__ conn, const double2* __r
       }
       }
     }
-    if (overflow) {
-      if (CAP < kMaxRow) {  // this row is built again with the full buffers
-        row_len[i] = -1;
-        continue;
-      }
-      set_error(err, DEV_VALENCE);
-    }
+    if (overflow) set_error(err, DEV_VALENCE);
     if (!FILL) {
       row_len[i] = cnt;
       if (tmp_col) {
@@ -275,16 +415,22 @@ static sft_status build_target_t(sft_target_s* t, cudaStream_t st, int32_t* d_er
       cudaGetLastError();  // no staging: the second pass merges again
     }
   }
-  // rows of up to 16 (2D) / 32 (3D) entries in small buffers, the rest again
-  // with the full ones (measured: the full-size buffers spill to L2)
-  constexpr int kCapSmall = D == 2 ? 16 : 32;
-  ::sft::note_launch(), k_mass_rows<D, false, kCapSmall><<<blocks_for(t->nv), 256, 0, st>>>(t->conn, wfac, inc_start, inc, t->nv, row_len, nullptr,
-                                                           nullptr, nullptr, nullptr, nullptr, d_err, tmp_col,
-                                                           tmp_val, tmp_lump);
-  SFT_CUDA(cudaGetLastError());
-  ::sft::note_launch(), k_mass_rows<D, false, kMaxRow, true><<<blocks_for(t->nv), 256, 0, st>>>(t->conn, wfac, inc_start, inc, t->nv, row_len, nullptr,
-                                                           nullptr, nullptr, nullptr, nullptr, d_err, tmp_col,
-                                                           tmp_val, tmp_lump);
+  if (tmp_col) {
+    // rows of up to 16 (2D) / 32 (3D) entries in the hash tables, the rest in lists
+    constexpr int kCapHash = D == 2 ? 16 : 32;
+    constexpr size_t smem = mass_hash_smem<kCapHash>();
+    SFT_CUDA(cudaFuncSetAttribute(k_mass_hash<D, kCapHash>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ::sft::note_launch(), k_mass_hash<D, kCapHash><<<(unsigned)((t->nv + kHashThreads - 1) / kHashThreads), kHashThreads, smem, st>>>(
+        t->conn, wfac, inc_start, inc, t->nv, row_len, tmp_col, tmp_val, tmp_lump);
+    SFT_CUDA(cudaGetLastError());
+    ::sft::note_launch(), k_mass_rows<D, false, true><<<blocks_for(t->nv), 256, 0, st>>>(
+        t->conn, wfac, inc_start, inc, t->nv, row_len, nullptr, nullptr, nullptr, nullptr, nullptr, d_err, tmp_col, tmp_val,
+        tmp_lump);
+  } else {
+    ::sft::note_launch(), k_mass_rows<D, false><<<blocks_for(t->nv), 256, 0, st>>>(
+        t->conn, wfac, inc_start, inc, t->nv, row_len, nullptr, nullptr, nullptr, nullptr, nullptr, d_err, nullptr, nullptr,
+        nullptr);
+  }
   SFT_CUDA(cudaGetLastError());
   SFT_CUDA(exclusive_scan_i32_to_i64(row_len, off64, t->nv, st));
   Events kit;
