@@ -5,7 +5,7 @@
 // error of a target field (Eq. relative_L2_error). It is the exact judge of
 // the Monte Carlo transfer at scale and the paper's comparison method.
 //
-// One thread per target triangle t, all arithmetic FP64:
+// All arithmetic FP64. Per target triangle t:
 //   1. locate t's centroid in the source (the location walk): the first
 //      source triangle s0 overlaps t with positive area;
 //   2. breadth-first over source face neighbours from s0: each visited source
@@ -15,21 +15,22 @@
 //      with positive area form a face-connected set (they tile the convex t),
 //      so the walk reaches all of them and touches only their face neighbours
 //      besides;
-//   3. b: three FP64 atomics per target triangle; L2: per-block partial sums.
+//   3. b: FP64 atomics per pair; L2: per-block partial sums.
 // The clipping runs in t's area coordinates A_m = 2 |t| lambda_m (cross
 // products with t's edges, exactly 0 at t's own vertices and on axis-parallel
 // edges) with the source field carried along as one more linear attribute of
 // each polygon vertex: whether a vertex is inside is the sign of a coordinate,
 // and both factors of every integrand are known at the polygon's vertices, so
 // int f g over a fan triangle is its area / 12 (sum f sum g + sum f g).
-// What bounds it: the FP64 pipe (one warp instruction per 16 cycles and SM;
-// 88 % busy), about 180 operations for an overlapping pair and 45 for a
-// neighbour that does not overlap, at 6 of 32 lanes (the lanes' walks and
-// polygons differ). Clipping in x, y with cross products at every stage and
-// the edge-midpoint rule through two barycentric maps per midpoint took about
-// 1,000 operations a pair: 1.0 M source, 0.5 M target triangles, load vector
-// 17.4 ms, L2 error 18.8 ms, now 5.6 and 5.7. Polygons and the first queue
-// entries are in shared memory (dynamic indices).
+// What bounds it: the FP64 pipe (one warp instruction per 16 cycles and SM).
+// A warp therefore keeps 32 targets' walks and fills its lanes with (target,
+// source triangle) pairs of any of them: the area coordinates of 32 queued
+// pairs at a time, then, 32 at a time again, the clipping of those that are
+// not outside an edge, with the at most two crossings of an edge line found
+// from the signs and computed together. The walks' bookkeeping stays with the
+// lane that owns the target. 1.0 M source, 0.5 M target triangles: load vector
+// 17.4 ms with clipping in x, y; 5.6 ms with a thread per target in area
+// coordinates (6 of 32 lanes active); now 2.1 (FP64 pipe 81 % busy). L2 error 18.8, 5.7, now 2.2.
 // Up to kMiQueue source triangles are visited per target triangle; beyond
 // that the kernel sets DEV_VALENCE and the call reports SFT_ERR_UNSUPPORTED.
 #include <algorithm>
@@ -41,7 +42,7 @@
 namespace sft {
 
 constexpr int kMiQueue = 256;
-constexpr int kMiThreads = 128;
+constexpr int kMiThreads = 64;
 
 struct P2 { double x, y; };
 
@@ -67,188 +68,322 @@ __device__ __forceinline__ PV lerp(const PV& a, const PV& b, double t) {
 }
 
 constexpr int kMiVerts = 6;      // vertices of a triangle clipped by three half-planes, at most
-constexpr int kMiQueueSm = 16;   // queue entries in shared memory
+constexpr int kMiQueueSm = 20;   // entries of a walk in shared memory, the rest in global
+constexpr int kMiBlocks = 5;     // per SM, by shared memory
+constexpr int kMiRefill = 8;     // idle lanes that make a warp take new targets
 
-template <bool L2>
-__global__ void __launch_bounds__(kMiThreads) k_mi_2d(
-    const double* __restrict__ sx, const int32_t* __restrict__ sconn, const int32_t* __restrict__ adj,
-    const double* __restrict__ svals, int snf, int field, const GridP<double>* __restrict__ gp,
-    const int32_t* __restrict__ cell_start, const int32_t* __restrict__ cell_items,
-    const int32_t* __restrict__ cell_first, const double* __restrict__ recs, const double* __restrict__ tx,
-    const int32_t* __restrict__ tconn, int64_t net, const double* __restrict__ u, double* __restrict__ b,
-    double* __restrict__ part, int32_t* err) {
-  __shared__ double spoly[2][kMiVerts][3][kMiThreads];
-  __shared__ int32_t squeue[kMiQueueSm][kMiThreads];
-  const int tid = threadIdx.x;
+// source triangle holding each target's centroid (it lies strictly inside t:
+// that triangle overlaps t with positive area)
+__global__ void k_mi_start(const GridP<double>* __restrict__ gp, const int32_t* __restrict__ cell_start,
+                           const int32_t* __restrict__ cell_items, const int32_t* __restrict__ cell_first,
+                           const double* __restrict__ recs, const int32_t* __restrict__ adj, const double* __restrict__ tx,
+                           const int32_t* __restrict__ tconn, int64_t net, int32_t* __restrict__ start, int32_t* err) {
   const GridP<double> g = *gp;
-  double e2 = 0.0, n2 = 0.0;
-  int32_t queue[kMiQueue - kMiQueueSm];
-  auto put = [&](int buf, int i, const PV& v) {
-    spoly[buf][i][0][tid] = v.a1;
-    spoly[buf][i][1][tid] = v.a2;
-    spoly[buf][i][2][tid] = v.f;
-  };
-  auto get = [&](int buf, int i) { return PV{spoly[buf][i][0][tid], spoly[buf][i][1][tid], spoly[buf][i][2][tid]}; };
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < net; t += (int64_t)gridDim.x * blockDim.x) {
     P2 tv[3];
-    int32_t tn[3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      tn[m] = __ldg(tconn + t * 3 + m);
-      tv[m] = P2{__ldg(tx + (int64_t)tn[m] * 2), __ldg(tx + (int64_t)tn[m] * 2 + 1)};
+      const double2 x = __ldg(reinterpret_cast<const double2*>(tx) + __ldg(tconn + t * 3 + m));
+      tv[m] = P2{x.x, x.y};
     }
-    // the centroid lies strictly inside t: the source triangle holding it
-    // overlaps t with positive area
     double c[2] = {__ddiv_rn(__dadd_rn(__dadd_rn(tv[0].x, tv[1].x), tv[2].x), 3.0),
                    __ddiv_rn(__dadd_rn(__dadd_rn(tv[0].y, tv[1].y), tv[2].y), 3.0)};
     double mu0[3];
     int status = 0;
     const int32_t s0 = locate_point<2, double>(g, cell_start, cell_items, cell_first, recs, adj, c, mu0, status);
-    if (s0 < 0) {
-      set_error(err, DEV_BAD_INDEX);
+    if (s0 < 0) set_error(err, DEV_BAD_INDEX);
+    start[t] = s0;
+  }
+}
+
+// what a warp keeps in shared memory
+struct alignas(16) MiWarp {
+  // targets: vertices 0..5, edges v0 -> v1, v1 -> v2, v2 -> v0 (A_2, A_0, A_1) 6..11,
+  // L2: 1 / (48 |t|) 12, u = u0 + A_1 g1 + A_2 g2 13..15; b: 1 / (12 |t|) 12, 1 / (96 |t|^2) 13
+  double tgt[16][32];
+  double poly[2 * kMiVerts - 1][3][32];  // clipped polygons: rows 0..5 and 6..10 in turn
+  double surv[12][64];             // pairs to clip: A_0, A_1, A_2, f at the source triangle's vertices
+  int32_t surv_s[64];
+  int32_t walk[kMiQueueSm][32];    // source triangles of the targets' walks, in the order found
+  int32_t len[32];                 // entries of the walk
+  int32_t node[3][32];             // the targets' nodes
+  int32_t inflight[32];            // pairs of the target in surv
+  int32_t pair_s[32];              // pairs of a batch, then the fans of the clipped ones
+  uint32_t hit;                    // pairs of the batch that overlap
+  uint8_t surv_t[64], pair_t[32];
+};
+
+template <bool L2>
+__global__ void __launch_bounds__(kMiThreads) k_mi_2d(
+    const double* __restrict__ sx, const int32_t* __restrict__ sconn, const int32_t* __restrict__ adj,
+    const double* __restrict__ svals, int snf, int field, const int32_t* __restrict__ start,
+    const double* __restrict__ tx, const int32_t* __restrict__ tconn, int64_t net, const double* __restrict__ u,
+    double* __restrict__ b, double* __restrict__ part, int32_t* __restrict__ far_walk, int32_t* err) {
+  __shared__ MiWarp smem[kMiThreads / 32];
+  constexpr uint32_t kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  MiWarp& w = smem[threadIdx.x >> 5];
+  // consecutive targets per warp
+  const int64_t nwarps = (int64_t)gridDim.x * (kMiThreads / 32), per = (net + nwarps - 1) / nwarps;
+  const int64_t wid = (int64_t)blockIdx.x * (kMiThreads / 32) + (threadIdx.x >> 5);
+  int64_t next = wid * per;
+  const int64_t end = next + per < net ? next + per : net;
+
+  double e2 = 0.0, n2 = 0.0;
+  int head = 0;                    // entries of the lane's walk that were taken
+  int qn = 0;                      // pairs in surv
+  int32_t* const far = far_walk + wid * (32 * (kMiQueue - kMiQueueSm));
+  w.inflight[lane] = 0;
+  w.len[lane] = 0;
+  __syncwarp();
+  auto entry = [&](int tl, int i) -> int32_t& {
+    return i < kMiQueueSm ? w.walk[i][tl] : far[(i - kMiQueueSm) * 32 + tl];
+  };
+
+  for (;;) {
+    // new targets for the lanes that are done with theirs
+    int pend = w.len[lane] - head;
+    const uint32_t idle = __ballot_sync(kAll, pend == 0 && w.inflight[lane] == 0);
+    int total = __reduce_add_sync(kAll, pend);
+    if (next < end && (__popc(idle) >= kMiRefill || total < 32)) {
+      const int64_t t = next + __popc(idle & ((1u << lane) - 1u));
+      if ((idle >> lane & 1u) && t < end) {
+        const int32_t s0 = __ldg(start + t);
+        int32_t tn[3];
+        P2 tv[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          tn[m] = __ldg(tconn + t * 3 + m);
+          w.node[m][lane] = tn[m];
+          const double2 x = __ldg(reinterpret_cast<const double2*>(tx) + tn[m]);
+          tv[m] = P2{x.x, x.y};
+        }
+        const double rD = 1.0 / cross3(tv[0], tv[1], tv[2]);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          w.tgt[2 * m][lane] = tv[m].x;
+          w.tgt[2 * m + 1][lane] = tv[m].y;
+          w.tgt[6 + 2 * m][lane] = tv[(m + 1) % 3].x - tv[m].x;
+          w.tgt[7 + 2 * m][lane] = tv[(m + 1) % 3].y - tv[m].y;
+        }
+        w.tgt[12][lane] = rD * (L2 ? 1.0 / 24.0 : 1.0 / 6.0);
+        if (!L2) {
+          w.tgt[13][lane] = rD * rD * (1.0 / 24.0);
+        } else {
+          const double u0 = __ldg(u + tn[0]);
+          w.tgt[13][lane] = u0;
+          w.tgt[14][lane] = (__ldg(u + tn[1]) - u0) * rD;
+          w.tgt[15][lane] = (__ldg(u + tn[2]) - u0) * rD;
+        }
+        w.walk[0][lane] = s0;
+        head = 0;
+        pend = s0 >= 0 ? 1 : 0;  // (a centroid outside is reported by k_mi_start)
+        w.len[lane] = pend;
+      }
+      next += __popc(idle);
+      total = __reduce_add_sync(kAll, pend);
+      if (total == 0 && qn == 0 && next < end) continue;
+    }
+    if (total == 0 && qn == 0) break;
+
+    if (qn < 32 && total > 0 && (total >= 32 || qn == 0)) {
+      // area coordinates of up to 32 queued pairs
+      int at = warp_inclusive_scan(pend, lane) - pend;
+      for (int left = pend; left > 0 && at < 32; --left) {
+        w.pair_s[at] = entry(lane, head++);
+        w.pair_t[at++] = (uint8_t)lane;
+      }
+      __syncwarp();
+      bool keep = false;
+      double a0[3], a1[3], a2[3], f[3];
+      int32_t s = 0;
+      int tl = 0;
+      if (lane < total) {
+        s = w.pair_s[lane];
+        tl = w.pair_t[lane];
+        double2 x[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          x[m] = __ldg(reinterpret_cast<const double2*>(sx) + __ldg(sconn + (int64_t)s * 3 + m));
+          f[m] = __ldg(svals + ((int64_t)s * snf + field) * 4 + m);
+        }
+        // separately rounded products: exactly 0 where x is an end of the edge
+        auto area = [&](int e, double dx, double dy) {
+          return __dsub_rn(__dmul_rn(w.tgt[6 + 2 * e][tl], dy), __dmul_rn(w.tgt[7 + 2 * e][tl], dx));
+        };
+        int in0 = 0, in1 = 0, in2 = 0;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          // v0 ends the edges of A_1 and A_2, v1 that of A_0
+          const double dx = __dsub_rn(x[m].x, w.tgt[0][tl]), dy = __dsub_rn(x[m].y, w.tgt[1][tl]);
+          a2[m] = area(0, dx, dy);
+          a0[m] = area(1, __dsub_rn(x[m].x, w.tgt[2][tl]), __dsub_rn(x[m].y, w.tgt[3][tl]));
+          a1[m] = area(2, dx, dy);
+          in0 |= not_neg(a0[m]);
+          in1 |= not_neg(a1[m]);
+          in2 |= not_neg(a2[m]);
+        }
+        keep = in0 && in1 && in2;  // else outside one edge: nothing left
+      }
+      const uint32_t kept = __ballot_sync(kAll, keep);
+      if (keep) {
+        const int q = qn + __popc(kept & ((1u << lane) - 1u));
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          w.surv[m][q] = a0[m];
+          w.surv[3 + m][q] = a1[m];
+          w.surv[6 + m][q] = a2[m];
+          w.surv[9 + m][q] = f[m];
+        }
+        w.surv_s[q] = s;
+        w.surv_t[q] = (uint8_t)tl;
+        atomicAdd(&w.inflight[tl], 1);
+      }
+      qn += __popc(kept);
+      __syncwarp();
       continue;
     }
-    const double D = cross3(tv[0], tv[1], tv[2]), rD = 1.0 / D;
-    // u = u0 + A_1 g1 + A_2 g2 on t
-    double u0 = 0.0, g1 = 0.0, g2 = 0.0;
-    if (L2) {
-      u0 = __ldg(u + tn[0]);
-      g1 = (__ldg(u + tn[1]) - u0) * rD;
-      g2 = (__ldg(u + tn[2]) - u0) * rD;
-    }
-    P2 te[3];  // edges v0 -> v1, v1 -> v2, v2 -> v0 (A_2, A_0, A_1)
+
+    // clip and integrate the last 32 pairs of surv
+    const int cnt = qn < 32 ? qn : 32;
+    qn -= cnt;
+    int tl = 0, k = 0, buf = 1;
+    int32_t s = 0;
+    if (lane < cnt) {
+      const int q = qn + lane;
+      tl = w.surv_t[q];
+      s = w.surv_s[q];
+      atomicSub(&w.inflight[tl], 1);
+      // axis 0 from surv, axes 1 and 2 from the polygon
+      k = 3;
 #pragma unroll
-    for (int m = 0; m < 3; ++m) te[m] = P2{tv[(m + 1) % 3].x - tv[m].x, tv[(m + 1) % 3].y - tv[m].y};
-    double q0 = 0.0, q1 = 0.0, q2 = 0.0;  // b: sums of (2 |piece| 2 |t|) f, f A_1, f A_2; L2: (f - u)^2, f^2
-    int n = 1, head = 0;
-    squeue[0][tid] = s0;
-    while (head < n) {
-      const int32_t s = head < kMiQueueSm ? squeue[head][tid] : queue[head - kMiQueueSm];
-      ++head;
-      PV pv[3];
-      double a0[3];
+      for (int ax = 0; ax < 3; ++ax) {
+        const int from = buf * kMiVerts, to = (buf ^ 1) * kMiVerts;
+        auto vert = [&](int i, int c) -> double {   // c: 0 A_1, 1 A_2, 2 f
+          return ax == 0 ? w.surv[3 + 3 * c + i][q] : w.poly[from + i][c][lane];
+        };
+        auto coord = [&](int i) -> double { return ax == 0 ? w.surv[i][q] : w.poly[from + i][ax - 1][lane]; };
+        uint32_t in = 0u;
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        const int32_t v = __ldg(sconn + (int64_t)s * 3 + m);
-        const double2 x = __ldg(reinterpret_cast<const double2*>(sx) + v);
-        pv[m].f = __ldg(svals + ((int64_t)s * snf + field) * 4 + m);
-        // separately rounded products: exactly 0 where x is an end of the edge
-        pv[m].a2 = __dsub_rn(__dmul_rn(te[0].x, __dsub_rn(x.y, tv[0].y)), __dmul_rn(te[0].y, __dsub_rn(x.x, tv[0].x)));
-        a0[m] = __dsub_rn(__dmul_rn(te[1].x, __dsub_rn(x.y, tv[1].y)), __dmul_rn(te[1].y, __dsub_rn(x.x, tv[1].x)));
-        pv[m].a1 = __dsub_rn(__dmul_rn(te[2].x, __dsub_rn(x.y, tv[2].y)), __dmul_rn(te[2].y, __dsub_rn(x.x, tv[2].x)));
-      }
-      const int in0 = (not_neg(a0[0]) ? 1 : 0) | (not_neg(a0[1]) ? 2 : 0) | (not_neg(a0[2]) ? 4 : 0);
-      const int in1 = (not_neg(pv[0].a1) ? 1 : 0) | (not_neg(pv[1].a1) ? 2 : 0) | (not_neg(pv[2].a1) ? 4 : 0);
-      const int in2 = (not_neg(pv[0].a2) ? 1 : 0) | (not_neg(pv[1].a2) ? 2 : 0) | (not_neg(pv[2].a2) ? 4 : 0);
-      if (in0 == 0 || in1 == 0 || in2 == 0) continue;  // outside one edge: nothing left
-      // clip by A_0 (from the registers), A_1, A_2
-      int k = 0, buf = 0;
+        for (int i = 0; i < 3 + ax; ++i)
+          if (i < k && not_neg(coord(i))) in |= 1u << i;
+        const uint32_t full = (1u << k) - 1u;
+        if (ax > 0 && in == full) continue;
+        // crossings of edge i -> i + 1; a vertex more than was there at most, by one run of
+        // signs (more runs than one, in a polygon thinner than the rounding: the rest is dropped)
+        const uint32_t x = (in ^ (in >> 1 | in << (k - 1))) & full;
+        const int kk = __popc(in) + __popc(x), most = k + 1;
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        constexpr int nx[3] = {1, 2, 0};
-        const bool ia = (in0 >> m) & 1, ib = (in0 >> nx[m]) & 1;
-        if (ia) put(0, k++, pv[m]);
-        if (ia != ib) put(0, k++, lerp(pv[m], pv[nx[m]], a0[m] / (a0[m] - a0[nx[m]])));
-      }
+        for (int i = 0; i < 3 + ax; ++i) {
+          if (!(in >> i & 1u)) continue;
+          const uint32_t below = (1u << i) - 1u;
+          const int o = __popc(in & below) + __popc(x & below);
+          if (o < most)
 #pragma unroll
-      for (int ax = 1; ax <= 2; ++ax) {
-        if ((ax == 1 ? in1 : in2) == 7) continue;  // every vertex of s inside: so is every point of s
-        int kk = 0;
-        const PV first = get(buf, 0);
-        PV cur = first;
-        for (int i = 0; i < k; ++i) {
-          const PV nxt = i + 1 < k ? get(buf, i + 1) : first;
-          const double ca = ax == 1 ? cur.a1 : cur.a2, cb = ax == 1 ? nxt.a1 : nxt.a2;
-          const bool ia = not_neg(ca), ib = not_neg(cb);
-          if (ia) put(buf ^ 1, kk++, cur);
-          if (ia != ib) {
-            PV x = lerp(cur, nxt, ca / (ca - cb));
-            if (ax == 1) x.a1 = 0.0;
-            else x.a2 = 0.0;
-            put(buf ^ 1, kk++, x);
-          }
-          cur = nxt;
+            for (int c = 0; c < 3; ++c) w.poly[to + o][c][lane] = vert(i, c);
         }
-        k = kk;
+        for (uint32_t rest = x; rest != 0u; rest &= rest - 1u) {
+          const int i = __ffs(rest) - 1, j = i + 1 < k ? i + 1 : 0;
+          const int o = __popc(in & ((2u << i) - 1u)) + __popc(x & ((1u << i) - 1u));
+          const double ca = coord(i), cb = coord(j), t = ca / (ca - cb);
+          PV v = lerp(PV{vert(i, 0), vert(i, 1), vert(i, 2)}, PV{vert(j, 0), vert(j, 1), vert(j, 2)}, t);
+          if (ax == 1) v.a1 = 0.0;
+          if (ax == 2) v.a2 = 0.0;
+          if (o < most) {
+            w.poly[to + o][0][lane] = v.a1;
+            w.poly[to + o][1][lane] = v.a2;
+            w.poly[to + o][2][lane] = v.f;
+          }
+        }
+        k = kk < most ? kk : most;
         buf ^= 1;
-        if (k == 0) break;
-      }
-      if (k < 3) continue;
-      bool overlap = false;
-      const PV o = get(buf, 0);
-      PV p = get(buf, 1);
-      // (f - u) at the vertices
-      double od = 0.0, pd = 0.0;
-      if (L2) {
-        od = o.f - fma(o.a2, g2, fma(o.a1, g1, u0));
-        pd = p.f - fma(p.a2, g2, fma(p.a1, g1, u0));
-      }
-      for (int i = 2; i < k; ++i) {  // fan from the first vertex
-        const PV q = get(buf, i);
-        double qd = 0.0;
-        if (L2) qd = q.f - fma(q.a2, g2, fma(q.a1, g1, u0));
-        const double cr = fma(p.a1 - o.a1, q.a2 - o.a2, -((p.a2 - o.a2) * (q.a1 - o.a1)));
-        if (positive(cr)) {
-          overlap = true;
-          const double sf = o.f + p.f + q.f;
-          if (L2) {
-            const double sd = od + pd + qd;
-            q0 = fma(cr, fma(sd, sd, fma(od, od, fma(pd, pd, qd * qd))), q0);
-            q1 = fma(cr, fma(sf, sf, fma(o.f, o.f, fma(p.f, p.f, q.f * q.f))), q1);
-          } else {
-            const double s1 = o.a1 + p.a1 + q.a1, s2 = o.a2 + p.a2 + q.a2;
-            q0 = fma(cr, sf, q0);
-            q1 = fma(cr, fma(s1, sf, fma(o.a1, o.f, fma(p.a1, p.f, q.a1 * q.f))), q1);
-            q2 = fma(cr, fma(s2, sf, fma(o.a2, o.f, fma(p.a2, p.f, q.a2 * q.f))), q2);
-          }
-        }
-        p = q;
-        pd = qd;
-      }
-      if (!overlap) continue;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        const int32_t nb = __ldg(adj + (int64_t)s * 3 + m);
-        if (nb < 0) continue;
-        bool seen = false;
-        for (int i = 0; i < n; ++i) seen = seen || (i < kMiQueueSm ? squeue[i][tid] : queue[i - kMiQueueSm]) == nb;
-        if (seen) continue;
-        if (n == kMiQueue) {
-          set_error(err, DEV_VALENCE);
-          head = n;  // stop this element; the call reports the overflow
-          break;
-        }
-        if (n < kMiQueueSm) squeue[n][tid] = nb;
-        else queue[n - kMiQueueSm] = nb;
-        ++n;
       }
     }
-    // a piece's area is cr / (2 D)
-    const double w12 = rD * (1.0 / 24.0);
-    if (L2) {
-      e2 = fma(q0, w12, e2);
-      n2 = fma(q1, w12, n2);
-    } else {
-      const double bf = q0 * (rD * (1.0 / 6.0)), b1 = q1 * (w12 * rD), b2 = q2 * (w12 * rD);
-      atomicAdd(b + tn[0], bf - b1 - b2);   // the three basis functions sum to 1
-      atomicAdd(b + tn[1], b1);
-      atomicAdd(b + tn[2], b2);
+    // the triangles of the fans from the first vertices, 32 at a time: polygon's lane, its rows, triangle
+    uint8_t* const fan = reinterpret_cast<uint8_t*>(w.pair_s);
+    const int nf = k > 2 ? k - 2 : 0;
+    const int incl = warp_inclusive_scan(nf, lane), nfan = __shfl_sync(kAll, incl, 31);
+    for (int i = 0; i < nf; ++i) fan[incl - nf + i] = (uint8_t)(lane | buf << 5 | i << 6);
+    if (lane == 0) w.hit = 0u;
+    __syncwarp();
+    for (int i = lane; i < nfan; i += 32) {
+      const int v = fan[i], pl = v & 31, row = (v >> 5 & 1) * kMiVerts, j = row + 1 + (v >> 6), ft = w.surv_t[qn + pl];
+      auto get = [&](int r) { return PV{w.poly[r][0][pl], w.poly[r][1][pl], w.poly[r][2][pl]}; };
+      const PV o = get(row), p = get(j), r = get(j + 1);
+      const double cr = fma(p.a1 - o.a1, r.a2 - o.a2, -((p.a2 - o.a2) * (r.a1 - o.a1)));
+      if (!positive(cr)) continue;
+      atomicOr(&w.hit, 1u << pl);
+      // the triangle's area is cr / (4 |t|)
+      const double sf = o.f + p.f + r.f, wt = cr * w.tgt[12][ft];
+      if (L2) {
+        const double u0 = w.tgt[13][ft], g1 = w.tgt[14][ft], g2 = w.tgt[15][ft];
+        // (f - u) at the vertices
+        const double od = o.f - fma(o.a2, g2, fma(o.a1, g1, u0)), pd = p.f - fma(p.a2, g2, fma(p.a1, g1, u0)),
+                     rd = r.f - fma(r.a2, g2, fma(r.a1, g1, u0)), sd = od + pd + rd;
+        e2 = fma(wt, fma(sd, sd, fma(od, od, fma(pd, pd, rd * rd))), e2);
+        n2 = fma(wt, fma(sf, sf, fma(o.f, o.f, fma(p.f, p.f, r.f * r.f))), n2);
+      } else {
+        const double s1 = o.a1 + p.a1 + r.a1, s2 = o.a2 + p.a2 + r.a2, w2 = cr * w.tgt[13][ft];
+        const double b1 = w2 * fma(s1, sf, fma(o.a1, o.f, fma(p.a1, p.f, r.a1 * r.f)));
+        const double b2 = w2 * fma(s2, sf, fma(o.a2, o.f, fma(p.a2, p.f, r.a2 * r.f)));
+        atomicAdd(b + w.node[0][ft], fma(wt, sf, -(b1 + b2)));   // the three basis functions sum to 1
+        atomicAdd(b + w.node[1][ft], b1);
+        atomicAdd(b + w.node[2][ft], b2);
+      }
+    }
+    __syncwarp();
+    const bool overlap = w.hit >> lane & 1u;
+    // face neighbours of an overlapping triangle that are new go to its target's walk
+    int32_t nb[3] = {-1, -1, -1};
+    if (overlap) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) nb[c] = __ldg(adj + (int64_t)s * 3 + c);
+    }
+    int known = 0;   // entries of the walk compared with
+    auto strike = [&] {
+      if (!overlap) return;
+      const int m = w.len[tl];
+      for (; known < m; ++known) {
+        const int32_t v = entry(tl, known);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          if (nb[c] == v) nb[c] = -1;
+      }
+    };
+    strike();
+    __syncwarp();  // (the fans were read)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      // of the pairs that bring the same one the first lane's does
+      const bool want = nb[c] >= 0;
+      const unsigned long long id = want ? (unsigned long long)tl << 32 | (uint32_t)nb[c] : ~0ull << 8 | (unsigned)lane;
+      const uint32_t same = __match_any_sync(kAll, id);
+      if (want && (same & ((1u << lane) - 1u)) == 0u) {
+        const int at = atomicAdd(&w.len[tl], 1);
+        if (at < kMiQueue) entry(tl, at) = nb[c];
+        else set_error(err, DEV_VALENCE);
+      }
+      __syncwarp();
+      // (beyond the limit the call fails and reports it: the walk ends there)
+      if (w.len[lane] > kMiQueue) w.len[lane] = kMiQueue;
+      __syncwarp();
+      if (c < 2) strike();
     }
   }
   if (L2) {
     __shared__ double sh[2][kMiThreads / 32];
     e2 = warp_sum<double>(e2);
     n2 = warp_sum<double>(n2);
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
       sh[0][threadIdx.x >> 5] = e2;
       sh[1][threadIdx.x >> 5] = n2;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
       double a = 0.0, c = 0.0;
-      for (int w = 0; w < kMiThreads / 32; ++w) {
-        a += sh[0][w];
-        c += sh[1][w];
+      for (int i = 0; i < kMiThreads / 32; ++i) {
+        a += sh[0][i];
+        c += sh[1][i];
       }
       part[blockIdx.x * 2] = a;
       part[blockIdx.x * 2 + 1] = c;
@@ -271,16 +406,24 @@ sft_status mesh_intersection_2d(sft_source_s* s, sft_target_s* t, int field, con
   int dev = 0, sms = 0;
   SFT_CUDA(cudaGetDevice(&dev));
   SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // warps with fewer targets where that fills the chip; a warp's last pairs leave lanes idle
   const int64_t want = (t->ne + kMiThreads - 1) / kMiThreads;
-  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 16));
+  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * kMiBlocks));
+  DevBuf<int32_t> start(st), far(st);
+  SFT_CUDA(start.alloc((size_t)t->ne));
+  SFT_CUDA(far.alloc((size_t)blocks * kMiThreads * (kMiQueue - kMiQueueSm)));
   DevBuf<double> part(st);
   SFT_CUDA(part.alloc((size_t)blocks * 2));
   if (!l2) SFT_CUDA(cudaMemsetAsync(b, 0, sizeof(double) * t->nv, st));
+  const double* const tx = (const double*)t->coordsP[SFT_PREC_FP64];
+  ::sft::note_launch(), k_mi_start<<<(unsigned)std::min<int64_t>((t->ne + 127) / 128, (int64_t)sms * 64), 128, 0, st>>>(
+      (const GridP<double>*)L.grid, L.cell_start, L.cell_items, L.cell_first, (const double*)L.recs, L.adj, tx, t->conn, t->ne,
+      start.p, d_err.p);
+  SFT_CUDA(cudaGetLastError());
   auto launch = [&](auto kern) {
-    ::sft::note_launch(), kern<<<blocks, kMiThreads, 0, st>>>(
-        (const double*)L.coordsP, s->conn, L.adj, (const double*)L.vals, s->nf, field, (const GridP<double>*)L.grid,
-        L.cell_start, L.cell_items, L.cell_first, (const double*)L.recs, (const double*)t->coordsP[SFT_PREC_FP64], t->conn,
-        t->ne, u, b, part.p, d_err.p);
+    ::sft::note_launch(), kern<<<blocks, kMiThreads, 0, st>>>((const double*)L.coordsP, s->conn, L.adj, (const double*)L.vals,
+                                                            s->nf, field, start.p, tx, t->conn, t->ne, u, b, part.p, far.p,
+                                                            d_err.p);
   };
   if (l2) launch(k_mi_2d<true>);
   else launch(k_mi_2d<false>);
