@@ -127,7 +127,7 @@ void sft_source_destroy(sft_source s) {
 void sft_target_destroy(sft_target t) {
   if (!t) return;
   cudaStream_t st = t->stream;
-  void* bufs[] = {t->coords, t->conn, t->coordsP[0], t->coordsP[1], t->vol, t->vol32, t->row_ptr, t->col, t->val, t->dinv, t->lumped, t->sc, t->val32s, t->jent, t->jval, t->mdiag, t->rinfo};
+  void* bufs[] = {t->coords, t->conn, t->coordsP[0], t->coordsP[1], t->vol, t->vol32, t->row_ptr, t->col, t->val, t->dinv, t->lumped, t->sc, t->jent, t->jval, t->mdiag, t->rinfo};
   for (void* p : bufs)
     if (p) cudaFreeAsync(p, st);
   delete t;

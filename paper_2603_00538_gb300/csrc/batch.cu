@@ -58,8 +58,14 @@ struct BSys {
   const int32_t* col;
   const double* val;
   const double* dinv;
-  const float* aval;  // FP32 values of S M S (mixed mode)
-  const double* sc;   // S = diag(M)^-1/2 (mixed mode)
+  // mixed mode: the off-diagonal entries of M and S M S as jagged diagonals of
+  // 32-row slices (see k_mixed), S = diag(M)^-1/2
+  const int2* jent;
+  const double* jval;
+  const double* mdiag;
+  const uint16_t* rinfo;
+  const double* sc;
+  int64_t roff;       // the request's first place in the FP32 work vectors ([row][field])
   const double* b;
   double* x;
   int64_t off;  // first global row
@@ -71,9 +77,7 @@ struct BSys {
 };
 
 // a block's share of the mixed-precision batched solve: matrix rows [i0, i1)
-// of one request with all its nf field systems s0 .. s0 + nf - 1 (the
-// fields of a matrix row are visited back to back, so the row's matrix
-// entries are read once from memory and again from cache for the others)
+// of one request with all its nf field systems s0 .. s0 + nf - 1
 struct BPiece {
   int32_t s0, nf;
   int64_t i0, i1;
@@ -540,38 +544,37 @@ __global__ void __launch_bounds__(kBatchThreads) k_batch_pcg(const BSys* __restr
 }
 
 
-// ---------------------------------------------------------------------------
 // Row phases of one piece of the batched mixed-precision solve. The piece's
-// field f is system P.s0 + f; the fields of one request share the matrix and
-// lie at stride S.n (S = the first field's system) in b, x and the work
-// vectors, so a row's matrix entries are loaded once for all fields. NFC
-// (1, 2, 4, 8) bounds the piece's field count; bit f of m marks the fields
-// that work in the phase. A thread sums its rows' dot-product terms per
-// field, and the warp adds them to its shared slots once per piece.
+// field f is system P.s0 + f. The FP64 vectors (b, x, t) hold the fields of a
+// request one after the other (stride S.n, S = the first field's system); the
+// FP32 work vectors interleave them, NFC (1, 2, 4, 8: the piece's fields
+// rounded up) values per row, so that a matrix entry's gather is one or two
+// vector loads for all fields. Bit f of m marks the fields that work in the
+// phase. A warp takes a slice of 32 rows (its jagged diagonals are coalesced
+// loads); at the ends of a piece the lanes whose rows belong to another block
+// only keep step.
 // ---------------------------------------------------------------------------
 template <int NFC>
-__device__ __forceinline__ void piece_flush(const double (&a)[NFC], const double (&c)[NFC], unsigned m,
-                                            double (*slot)[2], int j0) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void row_ld(const float* p, float (&v)[NFC]) {
+  if constexpr (NFC == 1) v[0] = *p;
+  else if constexpr (NFC == 2) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    v[0] = q.x; v[1] = q.y;
+  } else {
 #pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    if (!((m >> f) & 1u)) continue;
-    const double u = warp_sum<double>(a[f]), v = warp_sum<double>(c[f]);
-    if (lane == 0) {
-      slot[j0 + f][0] += u;
-      slot[j0 + f][1] += v;
+    for (int f = 0; f < NFC; f += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(p + f);
+      v[f] = q.x; v[f + 1] = q.y; v[f + 2] = q.z; v[f + 3] = q.w;
     }
   }
 }
-
 template <int NFC>
-__device__ __forceinline__ void piece_flush_f(const float (&a)[NFC], unsigned m, double (*slot)[2], int j0) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void row_st(float* p, const float (&v)[NFC]) {
+  if constexpr (NFC == 1) *p = v[0];
+  else if constexpr (NFC == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  else {
 #pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    if (!((m >> f) & 1u)) continue;
-    const float u = warp_sum<float>(a[f]);
-    if (lane == 0) slot[j0 + f][0] += (double)u;
+    for (int f = 0; f < NFC; f += 4) *reinterpret_cast<float4*>(p + f) = make_float4(v[f], v[f + 1], v[f + 2], v[f + 3]);
   }
 }
 
@@ -584,221 +587,157 @@ __device__ __forceinline__ void piece_R(const BPiece P, const BSys& S, unsigned 
   double a0[NFC], a1[NFC];
 #pragma unroll
   for (int f = 0; f < NFC; ++f) a0[f] = a1[f] = 0.0;
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
+  for (int64_t rb = (P.i0 & ~(int64_t)31) + warp * 32; rb < P.i1; rb += kBatchThreads) {
     double w[NFC];
 #pragma unroll
     for (int f = 0; f < NFC; ++f) w[f] = 0.0;
+    int64_t i = rb + lane;
+    bool mine = i >= P.i0 && i < P.i1;
     if (cyc > 0) {
-      const int32_t k0 = __ldg(S.rp + i), k1 = __ldg(S.rp + i + 1);
+      const int ri = S.rinfo[rb + lane], len = ri >> 5;
+      i = rb + (ri & 31);
+      mine = i >= P.i0 && i < P.i1;
+      const int maxlen = __shfl_sync(0xffffffffu, len, 0);
+      const int32_t base = __ldg(S.rp + rb);
+      const int2* e0 = S.jent + base + lane;
+      const double* m0 = S.jval + base + lane;
       // x of other blocks is visible to ordinary loads after the grid barrier
-      for (int32_t k = k0; k < k1; ++k) {
-        const double v = __ldg(S.val + k);
-        const int64_t c = __ldg(S.col + k);
+      if (mine) {
+        const double d = S.mdiag[i];
 #pragma unroll
         for (int f = 0; f < NFC; ++f)
-          if ((m >> f) & 1u) w[f] += v * S.x[f * n + c];
+          if ((m >> f) & 1u) w[f] = d * S.x[f * n + i];
+      }
+      constexpr int U = NFC <= 2 ? 4 : 2;
+      for (int q = 0; q < maxlen; q += U) {
+        int col[U];
+        double v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const bool has = len > q + u;
+          col[u] = -1;
+          v[u] = 0.0;
+          if (has && mine) {
+            col[u] = __ldg(&e0->x);
+            v[u] = __ldg(m0);
+          }
+          const int step = __popc(__ballot_sync(0xffffffffu, has));
+          e0 += step;
+          m0 += step;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (col[u] >= 0) {
+#pragma unroll
+            for (int f = 0; f < NFC; ++f)
+              if ((m >> f) & 1u) w[f] += v[u] * S.x[f * n + col[u]];
+          }
       }
     }
-    const double si = S.sc[i];
+    if (mine) {
+      const double si = S.sc[i];
 #pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t o = f * n + i;
-      if (cyc == 0) S.x[o] = 0.0;
-      const double ri = S.b[o] - w[f];
-      const double ti = si * ri;
-      t[S.off + o] = ti;
-      a0[f] += ri * ri;
-      a1[f] += ti * ti;
+      for (int f = 0; f < NFC; ++f) {
+        if (!((m >> f) & 1u)) continue;
+        const int64_t o = f * n + i;
+        if (cyc == 0) S.x[o] = 0.0;
+        const double ri = S.b[o] - w[f];
+        const double ti = si * ri;
+        t[S.off + o] = ti;
+        a0[f] += ri * ri;
+        a1[f] += ti * ti;
+      }
     }
   }
-  piece_flush<NFC>(a0, a1, m, slot, j0);
-}
-
-// I: c = t / ||t|| in FP32, y = p = q = 0; term c.c
-template <int NFC>
-__device__ __forceinline__ void piece_I(const BPiece P, const BSys& S, unsigned m, const double* t, float* r,
-                                        float* p, float* q, float* y, const double* isig, double (*slot)[2],
-                                        int j0) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = S.n;
-  float a[NFC];
-  double is[NFC];
 #pragma unroll
   for (int f = 0; f < NFC; ++f) {
-    a[f] = 0.f;
-    is[f] = (m >> f) & 1u ? isig[j0 + f] : 0.0;
-  }
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t gr = S.off + f * n + i;
-      const float ci = (float)(t[gr] * is[f]);
-      r[gr] = ci;
-      y[gr] = 0.f;
-      p[gr] = 0.f;
-      q[gr] = 0.f;
-      a[f] += ci * ci;
+    if (!((m >> f) & 1u)) continue;
+    const double u = warp_sum<double>(a0[f]), v = warp_sum<double>(a1[f]);
+    if (lane == 0) {
+      slot[j0 + f][0] += u;
+      slot[j0 + f][1] += v;
     }
   }
-  piece_flush_f<NFC>(a, m, slot, j0);
 }
 
-// A: w = A r, p = r + beta p, q = w + beta q (= A p); term p.q
+// x += ||t|| S y for the fields of m in row i
 template <int NFC>
-__device__ __forceinline__ void piece_A(const BPiece P, const BSys& S, unsigned m, float* r, float* p, float* q,
-                                        const float* beta, double (*slot)[2], int j0) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = S.n;
-  const float* rs = r + S.off;
-  float a[NFC], bt[NFC];
+__device__ __forceinline__ void row_U(const BSys& S, unsigned m, const double* sig, int j0, int64_t i, const float (&y)[NFC]) {
+  const double si = S.sc[i];
 #pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    a[f] = 0.f;
-    bt[f] = (m >> f) & 1u ? beta[j0 + f] : 0.f;
+  for (int f = 0; f < NFC; ++f)
+    if ((m >> f) & 1u) S.x[f * S.n + i] += (sig[j0 + f] * si) * f2d(y[f]);
+}
+
+// I: c = t / ||t|| in FP32, y_1 = c / theta (all of the solve for the fields of last)
+template <int NFC>
+__device__ __forceinline__ void piece_I(const BPiece P, const BSys& S, unsigned m, unsigned last, const double* t, float* c,
+                                        float* y, const double* isig, const double* sig, float ith, int j0) {
+  for (int64_t i = P.i0 + threadIdx.x; i < P.i1; i += kBatchThreads) {
+    float cv[NFC], yv[NFC];
+#pragma unroll
+    for (int f = 0; f < NFC; ++f) {
+      cv[f] = (m >> f) & 1u ? (float)(t[S.off + f * S.n + i] * isig[j0 + f]) : 0.f;
+      yv[f] = cv[f] * ith;
+    }
+    row_st<NFC>(c + S.roff + i * NFC, cv);
+    row_st<NFC>(y + S.roff + i * NFC, yv);
+    if (last) row_U<NFC>(S, last, sig, j0, i, yv);
   }
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
-    const int32_t k0 = __ldg(S.rp + i), k1 = __ldg(S.rp + i + 1);
+}
+
+// C: Chebyshev step, y_{k+1} = y_k + c1 (y_k - y_{k-1}) + c2 (c - A y_k) in the
+// place of y_{k-1} (0 for k = 1); for the fields of last straight into x
+template <int NFC>
+__device__ __forceinline__ void piece_C(const BPiece P, const BSys& S, unsigned m, unsigned last, const float* yk, float* yp,
+                                        const float* cvec, const double* sig, float c1, float c2, bool first, int j0) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  yk += S.roff;
+  yp += S.roff;
+  cvec += S.roff;
+  for (int64_t rb = (P.i0 & ~(int64_t)31) + warp * 32; rb < P.i1; rb += kBatchThreads) {
+    const int ri = S.rinfo[rb + lane], len = ri >> 5;
+    const int64_t i = rb + (ri & 31);
+    const bool mine = i >= P.i0 && i < P.i1;
+    const int maxlen = __shfl_sync(0xffffffffu, len, 0);
+    const int2* e0 = S.jent + __ldg(S.rp + rb) + lane;
     float w[NFC];
 #pragma unroll
     for (int f = 0; f < NFC; ++f) w[f] = 0.f;
-    // r was written by other blocks before the grid barrier (plain loads)
-    for (int32_t k = k0; k < k1; ++k) {
-      const float v = __ldg(S.aval + k);
-      const int64_t c = __ldg(S.col + k);
+    // y was written by other blocks before the grid barrier (plain loads)
+    constexpr int U = NFC <= 2 ? 8 : (NFC == 4 ? 4 : 2);
+    for (int q = 0; q < maxlen; q += U) {
+      int2 e[U];
 #pragma unroll
-      for (int f = 0; f < NFC; ++f)
-        if ((m >> f) & 1u) w[f] += v * rs[f * n + c];
+      for (int u = 0; u < U; ++u) {
+        const bool has = len > q + u;
+        e[u] = make_int2(-1, 0);
+        if (has && mine) e[u] = __ldg(e0);
+        e0 += __popc(__ballot_sync(0xffffffffu, has));
+      }
+      float g[U][NFC];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int f = 0; f < NFC; ++f) g[u][f] = 0.f;
+        if (e[u].x >= 0) row_ld<NFC>(yk + (int64_t)e[u].x * NFC, g[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int f = 0; f < NFC; ++f) w[f] = __fmaf_rn(__int_as_float(e[u].y), g[u][f], w[f]);
     }
+    if (!mine) continue;
+    float y1[NFC], y0[NFC], cv[NFC];
+    row_ld<NFC>(yk + i * NFC, y1);
+    row_ld<NFC>(cvec + i * NFC, cv);
 #pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t gr = S.off + f * n + i;
-      const float pn = r[gr] + bt[f] * p[gr];
-      const float qn = w[f] + bt[f] * q[gr];
-      p[gr] = pn;
-      q[gr] = qn;
-      a[f] += pn * qn;
-    }
-  }
-  piece_flush_f<NFC>(a, m, slot, j0);
-}
-
-// B: y += alpha p, r -= alpha q; term r.r
-template <int NFC>
-__device__ __forceinline__ void piece_B(const BPiece P, const BSys& S, unsigned m, float* r, const float* p,
-                                        const float* q, float* y, const float* alpha, double (*slot)[2], int j0) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = S.n;
-  float a[NFC], al[NFC];
+    for (int f = 0; f < NFC; ++f) y0[f] = 0.f;
+    if (!first) row_ld<NFC>(yp + i * NFC, y0);
 #pragma unroll
-  for (int f = 0; f < NFC; ++f) {
-    a[f] = 0.f;
-    al[f] = (m >> f) & 1u ? alpha[j0 + f] : 0.f;
-  }
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t gr = S.off + f * n + i;
-      y[gr] += al[f] * p[gr];
-      const float ri = r[gr] - al[f] * q[gr];
-      r[gr] = ri;
-      a[f] += ri * ri;
-    }
-  }
-  piece_flush_f<NFC>(a, m, slot, j0);
-}
-
-// Chebyshev I: c = t / ||t|| in FP32, r = c, y = 0, d = c / theta (in p)
-template <int NFC>
-__device__ __forceinline__ void piece_Ic(const BPiece P, const BSys& S, unsigned m, const double* t, float* r,
-                                         float* p, float* y, const double* isig, float ith, int j0) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = S.n;
-  double is[NFC];
-#pragma unroll
-  for (int f = 0; f < NFC; ++f) is[f] = (m >> f) & 1u ? isig[j0 + f] : 0.0;
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t gr = S.off + f * n + i;
-      const float ci = (float)(t[gr] * is[f]);
-      r[gr] = ci;
-      y[gr] = 0.f;
-      p[gr] = ci * ith;
-    }
-  }
-}
-
-// Chebyshev step: w = A d, y += d, r -= w, d' = c1 d + c2 r (d' in the
-// other buffer: the SpMV reads the d every block wrote in the step before)
-template <int NFC>
-__device__ __forceinline__ void piece_C(const BPiece P, const BSys& S, unsigned m, const float* dc, float* dn,
-                                        float* r, float* y, float c1, float c2, int j0) {
-  (void)j0;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = S.n;
-  const float* ds = dc + S.off;
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
-    const int32_t k0 = __ldg(S.rp + i), k1 = __ldg(S.rp + i + 1);
-    float w[NFC];
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) w[f] = 0.f;
-    // d was written by other blocks before the grid barrier (plain loads)
-    for (int32_t k = k0; k < k1; ++k) {
-      const float v = __ldg(S.aval + k);
-      const int64_t c = __ldg(S.col + k);
-#pragma unroll
-      for (int f = 0; f < NFC; ++f)
-        if ((m >> f) & 1u) w[f] += v * ds[f * n + c];
-    }
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t gr = S.off + f * n + i;
-      const float di = dc[gr];
-      y[gr] += di;
-      const float ri = r[gr] - w[f];
-      r[gr] = ri;
-      dn[gr] = c1 * di + c2 * ri;
-    }
-  }
-}
-
-// U: x += ||t|| S y
-template <int NFC>
-__device__ __forceinline__ void piece_U(const BPiece P, const BSys& S, unsigned m, const float* y,
-                                        const double* sig, int j0) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = S.n;
-  double sg[NFC];
-#pragma unroll
-  for (int f = 0; f < NFC; ++f) sg[f] = (m >> f) & 1u ? sig[j0 + f] : 0.0;
-  for (int64_t base = P.i0 + warp * 32; base < P.i1; base += kBatchThreads) {
-    const int64_t i = base + lane;
-    if (i >= P.i1) continue;
-    const double si = S.sc[i];
-#pragma unroll
-    for (int f = 0; f < NFC; ++f) {
-      if (!((m >> f) & 1u)) continue;
-      const int64_t o = f * n + i;
-      S.x[o] += (sg[f] * si) * (double)y[S.off + o];
-    }
+    for (int f = 0; f < NFC; ++f) y0[f] = y1[f] + (c1 * (y1[f] - y0[f]) + c2 * (cv[f] - (y1[f] + w[f])));
+    if (last != m) row_st<NFC>(yp + i * NFC, y0);
+    if (last) row_U<NFC>(S, last, sig, j0, i, y0);
   }
 }
 
@@ -809,53 +748,90 @@ __device__ __forceinline__ unsigned piece_mask(const BPiece& P, const int* flags
   return m;
 }
 
-// run phase PH on piece P (locals P, m, j0, sys) by its field class; with
-// MAXF = 4 a piece of more fields runs as two halves (field 4's system
-// starts the second), which bounds the registers the unrolled fields take
-#define SFT_PIECE_RUN(PH, MAXF, ...)                                             \
-  do {                                                                           \
-    if (P.nf <= 1) PH<1>(P, sys[P.s0], m, __VA_ARGS__, j0);                      \
-    else if (P.nf <= 2) PH<2>(P, sys[P.s0], m, __VA_ARGS__, j0);                 \
-    else if (P.nf <= 4) PH<4>(P, sys[P.s0], m, __VA_ARGS__, j0);                 \
-    else if ((MAXF) == 8) PH<8>(P, sys[P.s0], m, __VA_ARGS__, j0);               \
-    else {                                                                       \
-      const BPiece H{P.s0 + 4, P.nf - 4, P.i0, P.i1};                            \
-      if (m & 0xfu) PH<4>(P, sys[P.s0], m & 0xfu, __VA_ARGS__, j0);              \
-      if (m >> 4) PH<4>(H, sys[H.s0], m >> 4, __VA_ARGS__, j0 + 4);              \
-    }                                                                            \
+// run phase PH on piece P (locals P, m, j0, sys) by its field class
+#define SFT_PIECE_RUN(PH, ...)                                    \
+  do {                                                            \
+    if (P.nf <= 1) PH<1>(P, sys[P.s0], m, __VA_ARGS__, j0);       \
+    else if (P.nf <= 2) PH<2>(P, sys[P.s0], m, __VA_ARGS__, j0);  \
+    else if (P.nf <= 4) PH<4>(P, sys[P.s0], m, __VA_ARGS__, j0);  \
+    else PH<8>(P, sys[P.s0], m, __VA_ARGS__, j0);                 \
   } while (0)
-// field bound of the FP64 phase R and of the FP32 phases
-constexpr int kPieceFieldsR = 4, kPieceFields = 8;
+// the FP64 phase takes a piece of more than four fields as two halves (field
+// 4's system starts the second), which bounds its registers
+#define SFT_PIECE_RUN_R(...)                                              \
+  do {                                                                    \
+    if (P.nf <= 1) piece_R<1>(P, sys[P.s0], m, __VA_ARGS__, j0);          \
+    else if (P.nf <= 2) piece_R<2>(P, sys[P.s0], m, __VA_ARGS__, j0);     \
+    else if (P.nf <= 4) piece_R<4>(P, sys[P.s0], m, __VA_ARGS__, j0);     \
+    else {                                                                \
+      const BPiece H{P.s0 + 4, P.nf - 4, P.i0, P.i1};                     \
+      if (m & 0xfu) piece_R<4>(P, sys[P.s0], m & 0xfu, __VA_ARGS__, j0);  \
+      if (m >> 4) piece_R<4>(H, sys[H.s0], m >> 4, __VA_ARGS__, j0 + 4);  \
+    }                                                                     \
+  } while (0)
+
+// Grid barrier number `phase` (from 1) of the kernel: a counter that only
+// grows (a step waits for one message less than with a generation that the
+// last block publishes). The wait is limited; after the limit, or once the
+// error word is set, every block leaves.
+__device__ __forceinline__ bool batch_sync(BCgCtl* ctl, unsigned nb, unsigned& phase) {
+  __shared__ int ok;
+  ++phase;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = 1;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar.count) : "memory");
+    const uint32_t want = phase * nb;
+    const uint64_t t0 = globaltimer_ns();
+    for (;;) {
+      const int32_t e = *reinterpret_cast<volatile int32_t*>(&ctl->err);
+      uint32_t got;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&ctl->bar.count) : "memory");
+      if ((int32_t)(got - want) >= 0) break;
+      if (e != 0) { ok = 0; break; }
+      if (globaltimer_ns() - t0 > kDefaultWaitNs) {
+        set_error(&ctl->err, DEV_BARRIER_TIMEOUT);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
 
 // ---------------------------------------------------------------------------
 // Batched mixed-precision iterative refinement (the cg_mode MIXED solve of
-// every (request, field) system at once; see the single-system k_mixed_cg):
-// per refinement cycle an FP64 residual pass R, the FP32 right-hand side
-// pass I, the FP32 inner solve on S M S and the FP64 update U. The inner
-// solve is the Chebyshev iteration (one step phase per step; each system
-// takes the step count its spectrum interval fixes for its target), or CG
-// (phases A and B) when built with the CG alternative. All systems step
-// through the same phases; a system whose inner solve reached its target
-// (or that converged) skips the row work of the phase. Whether
-// any system still works is a flag summed over blocks, read after the next
-// grid barrier (three rotating flags: the one of decision d is cleared at
-// decision d + 2, when every block has read it).
+// every (request, field) system at once; the method is k_mixed's): per
+// refinement cycle an FP64 residual pass R, the FP32 right-hand side pass I
+// and the Chebyshev steps C on S M S in their three-term form, the last of
+// which adds to x. Every system takes the step count that its tolerance and
+// spectrum interval fix; a system that took its steps or that converged skips
+// the row work. The largest step count of a cycle (0: nothing left) goes
+// through a maximum over the blocks, read after the next grid barrier (three
+// rotating words: cycle c's is cleared in cycle c + 2, when every block has
+// read it).
+// What bounds it: a step's loads of A and y from L2 and L1 (37 MB of entries
+// for 4.6 M nonzeros) and the barrier's 2 us. With CSR rows by thread, fields
+// gathered one by one and separate update and vote passes 24 systems' worth of
+// requests (0.5 M rows, 1.9 M row fields) took 1,447 us, now 906.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_mixed(const BSys* __restrict__ sys,
                                                                const BPiece* __restrict__ pcs,
                                                                const int32_t* __restrict__ blk_pc,
                                                                const int32_t* __restrict__ blk_slo,
                                                                const int32_t* __restrict__ blk_shi, int maxs,
-                                                               double* t, float* r, float* p, float* q, float* y,
+                                                               double* t, float* ya, float* yb, float* cvec,
                                                                double* part, BSysOut* __restrict__ out, BCgCtl* ctl) {
   __shared__ double s_bn[kMaxLocalSys], s_prev[kMaxLocalSys], s_sig[kMaxLocalSys], s_isig[kMaxLocalSys],
       s_rel[kMaxLocalSys];
-  __shared__ float s_eta2[kMaxLocalSys], s_rr[kMaxLocalSys], s_alpha[kMaxLocalSys], s_beta[kMaxLocalSys];
-  __shared__ int s_live[kMaxLocalSys], s_act[kMaxLocalSys], s_conv[kMaxLocalSys], s_it[kMaxLocalSys];
-  __shared__ int s_ks[kMaxLocalSys];  // Chebyshev steps of the cycle
+  __shared__ int s_live[kMaxLocalSys], s_conv[kMaxLocalSys], s_it[kMaxLocalSys];
+  __shared__ int s_ks[kMaxLocalSys];  // Chebyshev steps of the cycle (0: none)
   __shared__ double s_w[kBatchWarps][kMaxLocalSys][2];
   __shared__ double s_g[kMaxLocalSys][2];
-  __shared__ int s_any;
+  __shared__ int s_kmax;
+  unsigned phase = 0;
   const unsigned nb = gridDim.x;
   const int b = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -864,7 +840,7 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_mixed(const BSys* __
   const int nloc = pc0 < pc1 ? shi - slo + 1 : 0;
   for (int j = threadIdx.x; j < nloc; j += blockDim.x) {
     s_live[j] = sys[slo + j].n > 0;
-    s_act[j] = 0;
+    s_ks[j] = 0;
     s_conv[j] = sys[slo + j].n == 0;
     s_it[j] = 0;
     s_rel[j] = 0.0;
@@ -902,19 +878,6 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_mixed(const BSys* __
     }
     __syncthreads();
   };
-  int dcount = 0;
-  // block's vote for decision dcount (s_any set by the per-system threads)
-  auto post = [&]() {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (b == 0) atomicExch(&ctl->flag[(dcount + 1) % 3], 0u);
-      if (s_any) atomicAdd(&ctl->flag[dcount % 3], 1u);
-    }
-    ++dcount;
-  };
-  auto voted = [&]() -> bool {
-    return *reinterpret_cast<volatile unsigned int*>(&ctl->flag[(dcount - 1) % 3]) != 0u;
-  };
   __syncthreads();
 
   for (int cyc = 0;; ++cyc) {
@@ -925,15 +888,16 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_mixed(const BSys* __
       const int j0 = P.s0 - slo;
       const unsigned m = piece_mask(P, s_live, j0);
       if (!m) continue;
-      SFT_PIECE_RUN(piece_R, kPieceFieldsR, cyc, t, s_w[warp]);
+      SFT_PIECE_RUN_R(cyc, t, s_w[warp]);
     }
     publish();
-    if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
+    if (!batch_sync(ctl, nb, phase)) return;
     gather_all();
-    if (threadIdx.x == 0) s_any = 0;
+    if (threadIdx.x == 0) s_kmax = 0;
     __syncthreads();
     if (threadIdx.x < nloc) {
       const int j = threadIdx.x;
+      s_ks[j] = 0;
       if (s_live[j]) {
         const BSys& S = sys[slo + j];
         const double rn = sqrt(s_g[j][0]), tn = sqrt(s_g[j][1]);
@@ -949,137 +913,54 @@ __global__ void __launch_bounds__(kBatchThreads, 4) k_batch_mixed(const BSys* __
           s_sig[j] = tn;
           s_isig[j] = 1.0 / tn;
           const double e = fmin(0.25, fmax(1e-5, 0.1 * S.tol * s_bn[j] / rn));
-          s_eta2[j] = (float)(e * e);
-          s_ks[j] = cheb_steps(e, cheb_coef(S.lmax).s1);
-          s_act[j] = 1;
-          atomicOr(&s_any, 1);
+          s_ks[j] = min(cheb_steps(e, cheb_coef(S.lmax).s1), S.max_iter - s_it[j]);
+          s_it[j] += s_ks[j];
+          atomicMax(&s_kmax, s_ks[j]);
         }
       }
     }
-    post();
-    if (kMixCheb) {
-      // I: r = c, y = 0, d = c / theta; the barrier makes d whole for the first step
-      for (int pc = pc0; pc < pc1; ++pc) {
-        const BPiece P = pcs[pc];
-        const int j0 = P.s0 - slo;
-        const unsigned m = piece_mask(P, s_act, j0);
-        if (!m) continue;
-        const float ith = 1.f / cheb_coef(sys[P.s0].lmax).theta;
-        SFT_PIECE_RUN(piece_Ic, kPieceFields, t, r, p, y, s_isig, ith);
-      }
-      if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
-      if (!voted()) break;  // no system left to refine
-      const ChebCoef c2d = cheb_coef(2.f), c3d = cheb_coef(2.5f);
-      float rho2 = 1.f / c2d.s1, rho3 = 1.f / c3d.s1;
-      for (int s = 0;; ++s) {
-        const float n2 = 1.f / (2.f * c2d.s1 - rho2), n3 = 1.f / (2.f * c3d.s1 - rho3);
-        const float a2 = n2 * rho2, b2 = n2 * (2.f / c2d.delta), a3 = n3 * rho3, b3 = n3 * (2.f / c3d.delta);
-        const float* dc = (s & 1) ? q : p;
-        float* dn = (s & 1) ? p : q;
-        for (int pc = pc0; pc < pc1; ++pc) {
-          const BPiece P = pcs[pc];
-          const int j0 = P.s0 - slo;
-          unsigned m = 0u;
-          for (int f = 0; f < P.nf; ++f) m |= s_act[j0 + f] && s < s_ks[j0 + f] ? 1u << f : 0u;
-          if (!m) continue;
-          const bool d3 = sys[P.s0].lmax > 2.25f;
-          SFT_PIECE_RUN(piece_C, kPieceFields, dc, dn, r, y, d3 ? a3 : a2, d3 ? b3 : b2);
-        }
-        rho2 = n2;
-        rho3 = n3;
-        if (threadIdx.x == 0) s_any = 0;
-        __syncthreads();
-        if (threadIdx.x < nloc) {
-          const int j = threadIdx.x;
-          if (s_act[j] && s < s_ks[j]) {
-            s_it[j] += 1;
-            if (s + 1 < s_ks[j] && s_it[j] < sys[slo + j].max_iter) atomicOr(&s_any, 1);
-            else s_act[j] = 0;
-          }
-        }
-        post();
-        if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
-        if (!voted()) break;  // every system took its steps
-      }
-    } else {
-    // I: c = t / ||t|| in FP32, y = p = q = 0; partial c.c
-    clear_slots();
     __syncthreads();
+    if (threadIdx.x == 0 && s_kmax > 0) atomicMax(&ctl->flag[cyc % 3], (unsigned)s_kmax);
     for (int pc = pc0; pc < pc1; ++pc) {
       const BPiece P = pcs[pc];
       const int j0 = P.s0 - slo;
-      const unsigned m = piece_mask(P, s_act, j0);
+      unsigned m = 0u, last = 0u;
+      for (int f = 0; f < P.nf; ++f) {
+        m |= s_ks[j0 + f] > 0 ? 1u << f : 0u;
+        last |= s_ks[j0 + f] == 1 ? 1u << f : 0u;
+      }
       if (!m) continue;
-      SFT_PIECE_RUN(piece_I, kPieceFields, t, r, p, q, y, s_isig, s_w[warp]);
+      const float ith = 1.f / cheb_coef(sys[P.s0].lmax).theta;
+      SFT_PIECE_RUN(piece_I, last, t, cvec, ya, s_isig, s_sig, ith);
     }
-    publish();
-    if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
-    if (!voted()) break;  // no system left to refine
-    gather_all();
-    if (threadIdx.x < nloc) {
-      const int j = threadIdx.x;
-      s_rr[j] = (float)s_g[j][0];
-      s_beta[j] = 0.f;
-    }
-    __syncthreads();
-
-    // FP32 CG on S M S y = c
-    for (int inner = 0;; ++inner) {
-      // A: w = A r, p = r + beta p, q = w + beta q; partial p.q
-      clear_slots();
+    if (!batch_sync(ctl, nb, phase)) return;
+    const int K = (int)*reinterpret_cast<volatile unsigned int*>(&ctl->flag[cyc % 3]);
+    if (b == 0 && threadIdx.x == 0) atomicExch(&ctl->flag[(cyc + 1) % 3], 0u);
+    if (K == 0) break;  // no system left to refine
+    const ChebCoef c2d = cheb_coef(2.f), c3d = cheb_coef(2.5f);
+    float rho2 = 1.f / c2d.s1, rho3 = 1.f / c3d.s1;
+    for (int k = 1; k < K; ++k) {   // y_{k+1} from y_k and y_{k-1}
+      const float n2 = 1.f / (2.f * c2d.s1 - rho2), n3 = 1.f / (2.f * c3d.s1 - rho3);
+      const float a2 = n2 * rho2, b2 = n2 * (2.f / c2d.delta), a3 = n3 * rho3, b3 = n3 * (2.f / c3d.delta);
+      const float* yk = (k & 1) ? ya : yb;
+      float* yp = (k & 1) ? yb : ya;
       for (int pc = pc0; pc < pc1; ++pc) {
         const BPiece P = pcs[pc];
         const int j0 = P.s0 - slo;
-        const unsigned m = piece_mask(P, s_act, j0);
-        if (!m) continue;
-        SFT_PIECE_RUN(piece_A, kPieceFields, r, p, q, s_beta, s_w[warp]);
-      }
-      publish();
-      if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
-      if (inner > 0 && !voted()) break;  // every inner solve reached its target
-      gather_all();
-      if (threadIdx.x < nloc) {
-        const int j = threadIdx.x;
-        s_alpha[j] = s_act[j] ? s_rr[j] / (float)s_g[j][0] : 0.f;
-      }
-      __syncthreads();
-      // B: y += alpha p, r -= alpha q; partial r.r
-      clear_slots();
-      for (int pc = pc0; pc < pc1; ++pc) {
-        const BPiece P = pcs[pc];
-        const int j0 = P.s0 - slo;
-        const unsigned m = piece_mask(P, s_act, j0);
-        if (!m) continue;
-        SFT_PIECE_RUN(piece_B, kPieceFields, r, p, q, y, s_alpha, s_w[warp]);
-      }
-      publish();
-      if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
-      gather_all();
-      if (threadIdx.x == 0) s_any = 0;
-      __syncthreads();
-      if (threadIdx.x < nloc) {
-        const int j = threadIdx.x;
-        if (s_act[j]) {
-          const float rn = (float)s_g[j][0];
-          s_it[j] += 1;
-          s_beta[j] = rn / s_rr[j];
-          s_rr[j] = rn;
-          if (rn <= s_eta2[j] || s_it[j] >= sys[slo + j].max_iter) s_act[j] = 0;
-          else atomicOr(&s_any, 1);
+        unsigned m = 0u, last = 0u;
+        for (int f = 0; f < P.nf; ++f) {
+          m |= s_ks[j0 + f] > k ? 1u << f : 0u;
+          last |= s_ks[j0 + f] == k + 1 ? 1u << f : 0u;
         }
+        if (!m) continue;
+        const bool d3 = sys[P.s0].lmax > 2.25f;
+        SFT_PIECE_RUN(piece_C, last, yk, yp, cvec, s_sig, d3 ? a3 : a2, d3 ? b3 : b2, k == 1);
       }
-      post();
+      rho2 = n2;
+      rho3 = n3;
+      if (!batch_sync(ctl, nb, phase)) return;
     }
-    }
-    // U: x += ||t|| S y for every system that refined in this cycle
-    for (int pc = pc0; pc < pc1; ++pc) {
-      const BPiece P = pcs[pc];
-      const int j0 = P.s0 - slo;
-      const unsigned m = piece_mask(P, s_live, j0);
-      if (!m) continue;
-      SFT_PIECE_RUN(piece_U, kPieceFields, y, s_sig);
-    }
-    if (!grid_sync(&ctl->bar, nb, &ctl->err)) return;
+    // (with one step x is whole after the pass I, whose barrier every block passed)
   }
   if (threadIdx.x < nloc) {
     const int j = threadIdx.x;
@@ -1252,13 +1133,11 @@ static sft_status enqueue_batch(sft_batch_s* B, cudaStream_t st) {
     cfg.numAttrs = 1;
     ::sft::note_launch();
     if (B->mixed) {
-      // FP32 work vectors packed into the FP64 ones: r | y in r, p | q in p; t in z
-      float* r32 = reinterpret_cast<float*>(B->r);
-      float* p32 = reinterpret_cast<float*>(B->p);
+      // t in z, the FP32 work vectors in the others
       SFT_CUDA(cudaLaunchKernelEx(&cfg, k_batch_mixed, (const BSys*)B->dsys, (const BPiece*)B->pcs,
                                   (const int32_t*)B->blk_pc, (const int32_t*)B->blk_slo, (const int32_t*)B->blk_shi,
-                                  B->maxs, B->z, r32, p32, p32 + B->ntot, r32 + B->ntot, B->part, B->sysout,
-                                  B->cgctl));
+                                  B->maxs, B->z, reinterpret_cast<float*>(B->r), reinterpret_cast<float*>(B->p),
+                                  reinterpret_cast<float*>(B->q), B->part, B->sysout, B->cgctl));
     } else {
       SFT_CUDA(cudaLaunchKernelEx(&cfg, k_batch_pcg, (const BSys*)B->dsys, B->nsys, B->ntot, B->rows_per_block,
                                   (const int32_t*)B->blk_slo, (const int32_t*)B->blk_shi, B->maxs, B->r, B->z, B->p,
@@ -1495,20 +1374,24 @@ static sft_status build_batch(sft_batch_s* B, const sft_options* opts, int autot
   // systems of the batched CG
   B->sys_first.resize(nreq + 1);
   for (int r = 0; r < nreq; ++r) B->mixed = B->mixed && opts[r].cg_mode == SFT_CG_MIXED;
-  int64_t off = 0;
+  int64_t off = 0, roff = 0;
   for (int r = 0; r < nreq; ++r) {
     B->sys_first[r] = (int)B->hsys.size();
     sft_target t = B->tgts[r];
     if (B->mixed)
-      if (sft_status e = scaled_matrix(t, st)) return e;
+      if (sft_status e = scaled_slices(t, st)) return e;
     for (int f = 0; f < B->hreq[r].nf; ++f) {
       BSys S;
       S.rp = t->row_ptr;
       S.col = t->col;
       S.val = t->val;
       S.dinv = t->dinv;
-      S.aval = t->val32s;
+      S.jent = t->jent;
+      S.jval = t->jval;
+      S.mdiag = t->mdiag;
+      S.rinfo = t->rinfo;
       S.sc = t->sc;
+      S.roff = roff;
       S.b = B->b + B->vec_off[r] + (int64_t)f * t->nv;
       S.x = B->u + B->vec_off[r] + (int64_t)f * t->nv;
       S.off = off;
@@ -1519,6 +1402,9 @@ static sft_status build_batch(sft_batch_s* B, const sft_options* opts, int autot
       off += t->nv;
       B->hsys.push_back(S);
     }
+    const int nf = B->hreq[r].nf;
+    const int64_t nfc = nf <= 2 ? nf : (nf <= 4 ? 4 : 8);
+    roff += (t->nv * nfc + 3) & ~(int64_t)3;   // rows start on whole vectors
   }
   B->sys_first[nreq] = (int)B->hsys.size();
   B->nsys = (int)B->hsys.size();
@@ -1631,10 +1517,11 @@ static sft_status build_batch(sft_batch_s* B, const sft_options* opts, int autot
   if (sft_status e = upload(&B->dsys, B->hsys, st)) return e;
   if (sft_status e = upload(&B->blk_slo, slo, st)) return e;
   if (sft_status e = upload(&B->blk_shi, shi, st)) return e;
-  SFT_CUDA(dalloc(&B->r, (size_t)B->ntot, st));
+  const size_t work = (size_t)std::max<int64_t>(B->ntot, B->mixed ? (roff + 1) / 2 : 0);
+  SFT_CUDA(dalloc(&B->r, work, st));
   SFT_CUDA(dalloc(&B->z, (size_t)B->ntot, st));
-  SFT_CUDA(dalloc(&B->p, (size_t)B->ntot, st));
-  SFT_CUDA(dalloc(&B->q, (size_t)B->ntot, st));
+  SFT_CUDA(dalloc(&B->p, work, st));
+  SFT_CUDA(dalloc(&B->q, work, st));
   SFT_CUDA(dalloc(&B->part, (size_t)B->nblocks * B->maxs * 2, st));
   SFT_CUDA(dalloc(&B->sysout, (size_t)std::max(1, B->nsys), st));
   SFT_CUDA(dalloc(&B->cgctl, 1, st));

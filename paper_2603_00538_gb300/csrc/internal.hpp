@@ -159,10 +159,9 @@ struct sft_target_s {
   double* val = nullptr;        // [nnz]
   double* dinv = nullptr;       // [nv]
   double* lumped = nullptr;     // [nv]
-  // symmetric Jacobi scaling for the mixed-precision solve (made on first use):
-  // sc = diag(M)^-1/2 and the FP32 values of sc_i M_ij sc_j
+  // symmetric Jacobi scaling for the mixed-precision solves (made on first use):
+  // sc = diag(M)^-1/2, entries of M and the FP32 values of sc_i M_ij sc_j
   double* sc = nullptr;         // [nv]
-  float* val32s = nullptr;      // [nnz] in CSR order (batched solve)
   int2* jent = nullptr;         // [nnz] off-diagonal entries as jagged diagonals (solve.cu): column, scaled value
   double* jval = nullptr;       // [nnz] the same entries of M
   double* mdiag = nullptr;      // [nv] diag(M)
@@ -222,12 +221,12 @@ struct SolveLate {
   bool pending = false;
 };
 sft_status finish_solve(const SolveLate& late, const CallStatus& host, SolveResult* res);
-// cg_mode: SFT_CG_MIXED (FP64 refinement around FP32 CG) or SFT_CG_FP64
+// cg_mode: SFT_CG_MIXED (FP64 refinement around an FP32 Chebyshev iteration) or SFT_CG_FP64
 sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, double tol, int max_iter,
                       cudaStream_t st, int32_t* d_err, SolveResult* res, int cg_mode = SFT_CG_MIXED,
                       SolveLate* late = nullptr, int warm = 0);
-// S = diag(M)^-1/2 and the FP32 values of S M S in CSR order on the target (made once, kept)
-sft_status scaled_matrix(sft_target_s* t, cudaStream_t st);
+// S = diag(M)^-1/2 and the jagged diagonals of M and S M S on the target (made once, kept)
+sft_status scaled_slices(sft_target_s* t, cudaStream_t st);
 constexpr unsigned kWsumBlocks = 304;
 sft_status weighted_sum_launch(const double* w, const double* u, int64_t n, double* part, cudaStream_t st);
 // conversions

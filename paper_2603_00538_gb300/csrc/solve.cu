@@ -848,16 +848,6 @@ __global__ void k_jacobi_sqrt(const double* __restrict__ dinv, int64_t n, double
     sc[i] = sqrt(dinv[i]);
 }
 
-// FP32 values of S M S in CSR order (the batched solve)
-__global__ void k_scaled_values(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                const double* __restrict__ val, const double* __restrict__ sc, int64_t n,
-                                float* __restrict__ out) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double si = sc[i];
-    for (int32_t k = rp[i]; k < rp[i + 1]; ++k) out[k] = (float)(val[k] * si * sc[col[k]]);
-  }
-}
-
 // the off-diagonal entries of S M S as jagged diagonals: one warp per slice
 __global__ void k_scaled_slices(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                                 const double* __restrict__ val, const double* __restrict__ sc, int64_t n,
@@ -928,18 +918,7 @@ static sft_status jacobi_scale(sft_target_s* t, cudaStream_t st) {
   return SFT_OK;
 }
 
-sft_status scaled_matrix(sft_target_s* t, cudaStream_t st) {
-  if (t->val32s) return SFT_OK;
-  const int64_t n = t->nv;
-  if (sft_status r = jacobi_scale(t, st)) return r;
-  SFT_CUDA(dalloc(&t->val32s, (size_t)std::max<int64_t>(t->nnz, 1), st));
-  const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
-  ::sft::note_launch(), k_scaled_values<<<nb, 256, 0, st>>>(t->row_ptr, t->col, t->val, t->sc, n, t->val32s);
-  SFT_CUDA(cudaGetLastError());
-  return SFT_OK;
-}
-
-static sft_status scaled_slices(sft_target_s* t, cudaStream_t st) {
+sft_status scaled_slices(sft_target_s* t, cudaStream_t st) {
   if (t->jent) return SFT_OK;
   const int64_t n = t->nv, ns = (n + kSlice - 1) / kSlice;
   if (sft_status r = jacobi_scale(t, st)) return r;

@@ -37,14 +37,6 @@ __device__ __forceinline__ T warp_inclusive_scan(T v, int lane) {
   return v;
 }
 
-// inner FP32 solver of the mixed-precision solves: 1 = Chebyshev iteration
-// on the proven spectrum bounds of A (one SpMV and one grid barrier per step,
-// no dot products), 0 = CG (two grid barriers and two reductions per step)
-#ifndef SFT_MIX_CHEBYSHEV
-#define SFT_MIX_CHEBYSHEV 1
-#endif
-constexpr bool kMixCheb = SFT_MIX_CHEBYSHEV != 0;
-
 // Chebyshev iteration on A y = c (A the Jacobi-scaled P1 mass matrix) with
 // the spectrum of A inside [a, b] (a = 1/2, b = 2 or 5/2, widened by 1e-3
 // relative for the FP32 rounding of A's entries): theta = (a + b) / 2,
