@@ -350,9 +350,11 @@ __device__ __forceinline__ int32_t cell_axis<float>(float x, float lo, float inv
 
 template <>
 __device__ __forceinline__ int32_t cell_axis<double>(double x, double lo, double inv, int32_t n) {
-  double s = __dmul_rn(__dsub_rn(x, lo), inv);
-  s = fmin(fmax(s, 0.0), 2251799813685248.0);
-  const double t = __dadd_rz(s, 4503599627370496.0);
+  // clamped by the bit pattern (FP64 minima and maxima use the FP64 pipe)
+  int64_t b = __double_as_longlong(__dmul_rn(__dsub_rn(x, lo), inv));
+  if (b < 0 || b > 0x7FF0000000000000ll) b = 0;                       // negative, NaN
+  if (b > 0x4320000000000000ll) b = 0x4320000000000000ll;             // 2^51
+  const double t = __dadd_rz(__longlong_as_double(b), 4503599627370496.0);
   const int64_t c = (int64_t)((uint64_t)__double_as_longlong(t) - 0x4330000000000000ull);
   return c < (int64_t)(n - 1) ? (int32_t)c : n - 1;
 }

@@ -155,11 +155,30 @@ __device__ __forceinline__ int64_t elem_cell_range(const GridP<P>& g, const P xv
   for (int a = 0; a < 3; ++a) { c0[a] = 0; c1[a] = 0; }
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    P lo = xv[0][a], hi = xv[0][a];
+    P lo, hi;
+    if constexpr (sizeof(P) == 8) {
+      // by the order of the bit patterns (FP64 comparisons use the FP64 pipe);
+      // -0 comes before +0, which is the same cell
+      auto key = [](double x) {
+        const int64_t b = __double_as_longlong(x);
+        return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
+      };
+      int64_t kl = key(xv[0][a]), kh = kl;
 #pragma unroll
-    for (int m = 1; m <= D; ++m) {
-      lo = xv[m][a] < lo ? xv[m][a] : lo;
-      hi = xv[m][a] > hi ? xv[m][a] : hi;
+      for (int m = 1; m <= D; ++m) {
+        const int64_t k = key(xv[m][a]);
+        kl = k < kl ? k : kl;
+        kh = k > kh ? k : kh;
+      }
+      lo = __longlong_as_double(kl ^ ((kl >> 63) & 0x7FFFFFFFFFFFFFFFll));
+      hi = __longlong_as_double(kh ^ ((kh >> 63) & 0x7FFFFFFFFFFFFFFFll));
+    } else {
+      lo = hi = xv[0][a];
+#pragma unroll
+      for (int m = 1; m <= D; ++m) {
+        lo = xv[m][a] < lo ? xv[m][a] : lo;
+        hi = xv[m][a] > hi ? xv[m][a] : hi;
+      }
     }
     c0[a] = cell_axis<P>(lo, g.lo[a], g.inv[a], g.n[a]);
     c1[a] = cell_axis<P>(hi, g.lo[a], g.inv[a], g.n[a]);
@@ -364,7 +383,8 @@ __device__ __forceinline__ bool cell_may_hold(const P* r, const P c[D], const P 
 // (8-byte (id, depth) entries filled one at a time with the full test again,
 // and read back for the start elements, took 1.60 ms for the 68 M
 // registrations of a 5.0 M-tetrahedron source, 0.43 ms for 4.0 M triangles;
-// now 1.07 ms and 0.36. Sorting a block's registrations by cell in shared
+// now 1.08 ms and 0.36; the count pass of 0.61 M FP64 triangles 242 us, now 87.
+// Sorting a block's registrations by cell in shared
 // memory, with one global atomic per block and cell, took 1.45 ms and 0.42:
 // the shared-memory atomics collide.)
 constexpr int kMaskCells = 64;
@@ -410,9 +430,9 @@ __device__ __forceinline__ P centre_depth(const P* r, const P (&cc)[D]) {
 
 // The coordinates of the box's cell centres as linear functions of the cell's
 // offset, in FP32, with a bound of their difference from the evaluation in P
-// by cell_may_hold and centre_depth. A cell is settled when it lies outside
-// the bound of the threshold and its centre is surely not in the element; the
-// others (one in ten) are decided in P. (In FP64 because its operations are
+// by cell_may_hold and centre_depth. What lies outside the bound is settled;
+// a cell at the threshold, and the depth of a centre that may be in the
+// element (one per element on average), are evaluated in P. (In FP64 because its operations are
 // 64 times as dear here, in FP32 because the full test takes four times the
 // instructions.)
 template <int D, typename P>
@@ -452,7 +472,8 @@ struct BoxFilter {
 #pragma unroll
     for (int a = 0; a < D; ++a) S += 0.5f * fabsf(col[a]);
   }
-  // cell at offset o[] of the box: 0 not held, 1 held and the centre outside, 2 undecided
+  // cell at offset o[] of the box: 0 not held, 1 held and the centre outside,
+  // 2 held and the centre perhaps inside, 3 undecided
   __device__ __forceinline__ int operator()(const float (&o)[3]) const {
     constexpr float eps = 0.0009765625f;
     float t[D], sum = 0.f;
@@ -471,7 +492,7 @@ struct BoxFilter {
     }
     lo += eps;
     if (lo < -band) return 0;
-    return lo > band && mn < -band ? 1 : 2;
+    return lo > band ? (mn < -band ? 1 : 2) : 3;
   }
 };
 
@@ -488,7 +509,7 @@ __global__ void __launch_bounds__(kRegThreads)
   constexpr int W = kRegThreads / 32;
   __shared__ unsigned long long smask[kRegThreads];         // cells settled in P
   __shared__ int32_t sbox[kRegThreads][4];                  // first box cell, nx | ny << 8
-  __shared__ uint16_t queue[W][64];                         // lane << 6 | k
+  __shared__ uint16_t queue[W][64];                         // undecided << 11 | lane << 6 | k
   __shared__ float gf[4];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const GridP<P> g = *gp;
@@ -546,27 +567,33 @@ __global__ void __launch_bounds__(kRegThreads)
   sbox[t][2] = c0[2];
   sbox[t][3] = nx | ny << 8;
   __syncwarp();
-  // the undecided cells of a warp are gathered and taken 32 at a time
+  // what a warp has to evaluate in P is gathered and taken 32 at a time
   auto settle = [&](int n) {
     __syncwarp();
     if (lane < n) {
-      const int q = queue[warp][lane], src = warp * 32 + (q >> 6), k = q & 63;
+      const int q = queue[warp][lane], src = warp * 32 + (q >> 6 & 31), k = q & 63;
       const int bx = sbox[src][3] & 255, by = sbox[src][3] >> 8;
       const int row = k / bx;
       const int32_t idx[3] = {sbox[src][0] + k - row * bx, sbox[src][1] + (D == 3 ? row % by : row),
                               sbox[src][2] + (D == 3 ? row / by : 0)};
       const int32_t e2 = (int32_t)(e0 + src);
-      P r2[RL], cc[D], w[D];
+      P r2[RL], cc[D];
       load_record<D, P>(recs, e2, r2);
 #pragma unroll
-      for (int a = 0; a < D; ++a) {
-        cc[a] = cell_centre<P>(g, a, idx[a]);
-        w[a] = Ar<P>::mul(g.h[a], P(0.5));
+      for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
+      const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
+      bool held = true;
+      if (q >> 11) {
+        P w[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) w[a] = Ar<P>::mul(g.h[a], P(0.5));
+        held = cell_may_hold<D, P>(r2, cc, w);
+        if (held) {
+          atomicOr(&smask[src], 1ull << k);
+          atomicAdd(cell_count + c, 1);
+        }
       }
-      if (cell_may_hold<D, P>(r2, cc, w)) {
-        const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
-        atomicOr(&smask[src], 1ull << k);
-        atomicAdd(cell_count + c, 1);
+      if (held) {
         const P depth = centre_depth<D, P>(r2, cc);
         if (depth >= P(0)) first_offer(first + c, depth, e2);
       }
@@ -581,15 +608,16 @@ __global__ void __launch_bounds__(kRegThreads)
   unsigned long long bits = 0ull;
   int qn = 0;
   for (int k = 0; k < kmax; ++k) {
-    int res = sane ? filter(o) : 2;
+    int res = sane ? filter(o) : 3;
     if (k >= nbox) res = 0;
-    if (res == 1) {
+    if (res == 1 || res == 2) {
       bits |= 1ull << k;
       atomicAdd(cell_count + c, 1);
     }
-    const uint32_t und = __ballot_sync(0xffffffffu, res == 2);
+    const uint32_t und = __ballot_sync(0xffffffffu, res >= 2);
     if (und != 0u) {
-      if (res == 2) queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)(lane << 6 | k);
+      if (res >= 2)
+        queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)((res == 3 ? 1 << 11 : 0) | lane << 6 | k);
       qn += __popc(und);
       if (qn >= 32) {
         settle(32);
