@@ -838,7 +838,7 @@ def run_surrogate(args):
             "exact_path": {"ms_per_step": float(np.mean(ex_ms)), "assembly_ms": ex["ms_assembly"],
                            "queries_per_s": (tgt.nelems * N + tgt.nnodes) / (float(np.mean(ex_ms)) / 1e3),
                            "surrogate_over_exact_time": ms_per_step / float(np.mean(ex_ms))},
-            "roofline": {"kernel": "sft::k_surrogate_net (with the decision and exact passes)", "bound": "tensor", "achieved": achieved,
+            "roofline": {"kernel": "sft::k_mlp_forward (with the sample, combine, decision and exact passes)", "bound": "tensor", "achieved": achieved,
                          "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                          "peak_source": which, "algorithmic_flops": flops, "network_queries": net_queries,
                          "flop_model": "0.395 MFLOP per network query: N per element that keeps the network "
