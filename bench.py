@@ -944,7 +944,7 @@ def mesh_intersection_leg(args, sc, sk, sv, tc, tk, u, N, tol):
     return {"E_L2": e / n, "load_vector_ms": float(np.median(ms)), "l2_error_ms": a.elapsed_time(z),
             "mc_assembly_ms": st["ms_assembly"],
             "b_mc_vs_exact_rel_l2": float(np.linalg.norm(bm - bx) / np.linalg.norm(bx)),
-            "method": "2D clipping of every overlapping (target, source) triangle pair, FP64, edge-midpoint rule"}
+            "method": "2D clipping of every overlapping (target, source) triangle pair, FP64, exact on every fan triangle"}
 
 
 def precision_comparison(args, sc, sk, sv, tc, tk, N, tol):
