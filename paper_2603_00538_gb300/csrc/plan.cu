@@ -113,7 +113,7 @@ sft_status sft_plan_create(sft_source s, sft_target t, const sft_options* o, sft
     if (e == cudaSuccess) e = cudaMemsetAsync(b.p, 0, sizeof(double) * nv * pl->nf, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(counters.p, 0, sizeof(int64_t) * 2, st);
     if (e != cudaSuccess) { r = cuda_fail(e, "plan scratch"); break; }
-    // step 1 recorded: node locations (and this round's control values)
+    // step 1 recorded: node locations (and this call's control values)
     if ((r = locate_points(s, prec, nv, t->coordsP[prec], prec == SFT_PREC_FP64, pl->node_elem, g.p,
                            prec == SFT_PREC_FP64, nv, counters.p, st, pl->nf, pl->node_mu)))
       break;
