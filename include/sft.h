@@ -97,7 +97,8 @@ typedef struct {
     const void* values;     /* source: [nfields][nnodes] of `dtype`; target: NULL */
     int32_t dtype;          /* sft_dtype of coords and values */
     int32_t device_ptrs;    /* 1: coords/conn/values are device pointers */
-    double grid_scale_L;    /* source: grid cells per axis = int(L * nelems^(1/dim)); <= 0 means 1 */
+    double grid_scale_L;    /* source: grid cells per axis = int(L * nelems^(1/dim)); <= 0 means 1;
+                               2^31 - 1 cells or more: SFT_ERR_UNSUPPORTED */
     void* cuda_stream;      /* cudaStream_t for the setup work */
 } sft_mesh_desc;
 

@@ -19,15 +19,17 @@
 
 namespace sft {
 
-// cells per axis: the largest n >= 1 with n^d <= L^d * ne
+// cells per axis: the largest n >= 1 with n^d <= L^d * ne; 0 when there would
+// be 2^31 - 1 cells or more (a cell's linear index is an int32 everywhere)
 static int32_t cells_per_axis(int dim, int64_t ne, double L) {
   const double target = (dim == 2 ? L * L : L * L * L) * (double)ne;
+  if (!(target < 1e12)) return 0;
   int64_t n = (int64_t)std::floor(dim == 2 ? std::sqrt(target) : std::cbrt(target));
   if (n < 1) n = 1;
   auto pw = [dim](double x) { return dim == 2 ? x * x : x * x * x; };
   while (pw((double)(n + 1)) <= target) ++n;
   while (n > 1 && pw((double)n) > target) --n;
-  return (int32_t)n;
+  return pw((double)n) < (double)INT32_MAX ? (int32_t)n : 0;
 }
 
 template <typename TI, typename TO>
@@ -841,14 +843,14 @@ template <int D, typename P>
 static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, int32_t* d_err) {
   Locator& L = s->loc[prec];
   constexpr int RL = RecLen<D>::value;
+  const int32_t n = cells_per_axis(D, s->ne, s->L);
+  if (n == 0) return fail(SFT_ERR_UNSUPPORTED, "grid too fine (2^31 - 1 cells or more)");
   // coordinates in P
   P* xP = nullptr;
   SFT_CUDA(dalloc(&xP, (size_t)s->nv * D, st));
   L.coordsP = xP;
   if (sft_status r = convert_coords(s->coords, s->dtype, xP, prec, s->nv * D, st)) return r;
   // grid box and parameters
-  const int32_t n = cells_per_axis(D, s->ne, s->L);
-  if (n >= (1 << 22)) return fail(SFT_ERR_UNSUPPORTED, "grid too fine (cells per axis >= 2^22)");
   L.n[0] = L.n[1] = L.n[2] = 1;
   L.ncells = 1;
   for (int a = 0; a < D; ++a) { L.n[a] = n; L.ncells *= n; }
