@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(192, 1) k_train_dw(const unsigned char* __rest
     for (int64_t c = 0; c < stages; ++c) {
       const int s = (int)(c % kDwStages);
       const uint32_t use = (uint32_t)(c / kDwStages);
-      if (use > 0 && !tc::mbar_wait(empty + s, (use - 1) & 1u, err)) break;
+      if (use > 0 && !warp_agrees(tc::mbar_wait(empty + s, (use - 1) & 1u, err))) break;
       if (leader) {
         const int64_t tile = blockIdx.x + (c / kPerTile) * gridDim.x;
         const unsigned char* src = img + tile * kTrainImages * (int64_t)kSmemA + (c % kPerTile) * (int64_t)kDwHalf;
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(192, 1) k_train_dw(const unsigned char* __rest
     const bool leader = tc::elect_one();
     for (int64_t c = 0; c < stages; ++c) {
       const int s = (int)(c % kDwStages);
-      if (!tc::mbar_wait(full + s, (uint32_t)(c / kDwStages) & 1u, err)) break;
+      if (!warp_agrees(tc::mbar_wait(full + s, (uint32_t)(c / kDwStages) & 1u, err))) break;
       tc::fence_after_sync();
       if (leader) {
         const uint32_t da = tc::smem_addr(sm + (size_t)s * 2 * kDwHalf);

@@ -185,7 +185,10 @@ __device__ __forceinline__ void group_sync(int grp) {
 // Bounded waits of the forward kernel. One that runs out sets *err and the
 // CTA's failed flag; from then on every wait returns at once and no copy or
 // MMA is issued, so the threads run through their loops, meet at the same
-// barriers, and leave together.
+// barriers, and leave together. The lanes of a warp each see for themselves
+// whether a wait ended or ran out and may differ at the limit, so a warp that
+// issues or copies goes by warp_agrees of their answers.
+__device__ __forceinline__ bool warp_agrees(bool ok) { return __all_sync(0xffffffffu, ok); }
 __device__ __forceinline__ bool turn_wait(const FwdSmem& S, volatile int* ctr, int v, int32_t* err) {
   if (*ctr == v) return true;
   const uint64_t t0 = globaltimer_ns();
@@ -318,14 +321,14 @@ __device__ __forceinline__ void layer_issue(const FwdSmem& S, int grp, uint32_t 
   const uint64_t b0 = tc::smem_desc(tc::smem_addr(S.B), 128u, (uint32_t)kKF * 16u);
   const int c0 = slot * kChunks;
   const bool leader = tc::elect_one();
-  if (!turn_wait(S, S.issued, slot, err)) return;
+  if (!warp_agrees(turn_wait(S, S.issued, slot, err))) return;
   __threadfence_block();
   tc::fence_after_sync();
 #pragma unroll 1
   for (int kc = 0; kc < kChunks; ++kc) {
     const int c = c0 + kc;
     const int b = c % kRing;
-    if (!fwd_wait(S, S.full + b, ((uint32_t)c / kRing) & 1u, err)) return;
+    if (!warp_agrees(fwd_wait(S, S.full + b, ((uint32_t)c / kRing) & 1u, err))) return;
     if (leader) {
 #pragma unroll
       for (int m = 0; m < kChunkK / kKF; ++m) {
@@ -354,7 +357,7 @@ __device__ __forceinline__ void layer_issue(const FwdSmem& S, int grp, uint32_t 
 template <int NL>
 __device__ __forceinline__ void refill_buffer(const FwdSmem& S, const LayerWeights<NL>& Wc, int slot, int b,
                                               int32_t* err) {
-  if (!turn_wait(S, S.copied + b, slot, err)) return;
+  if (!warp_agrees(turn_wait(S, S.copied + b, slot, err))) return;
   __threadfence_block();
   const bool leader = tc::elect_one();
   FwdStream& st = *S.st;
@@ -367,7 +370,7 @@ __device__ __forceinline__ void refill_buffer(const FwdSmem& S, const LayerWeigh
     const int u = c0 + kc;  // the chunk whose buffer the next one reuses
     const int c = u + kRing;
     if (c >= total) break;
-    if (!fwd_wait(S, S.mdone + b, ((uint32_t)u / kRing) & 1u, err)) return;
+    if (!warp_agrees(fwd_wait(S, S.mdone + b, ((uint32_t)u / kRing) & 1u, err))) return;
     if (leader) {
       copy_chunk(S, kc + kRing < kChunks ? w_this : w_next, c);
       st.next_copy[b] = c + kRing;
