@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libsft.
 #pragma once
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <cuda_runtime.h>
 #include "sft.h"
@@ -51,6 +52,26 @@ struct DevBuf {
   explicit DevBuf(cudaStream_t st) : s(st) {}
   cudaError_t alloc(size_t n) { return dalloc(&p, n, s); }
   ~DevBuf() { dfree(p, s); }
+};
+
+// Something to be done once on each device (kernel attributes belong to a
+// device): once(f) calls f unless it succeeded on the current device before.
+class PerDevice {
+  std::mutex mu_;
+  bool done_[64] = {};
+
+ public:
+  template <class F>
+  sft_status once(F&& f) {
+    int dev = 0;
+    SFT_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu_);
+    const bool listed = dev >= 0 && dev < 64;
+    if (listed && done_[dev]) return SFT_OK;
+    if (sft_status r = f()) return r;
+    if (listed) done_[dev] = true;
+    return SFT_OK;
+  }
 };
 
 // Byte offsets of several arrays in one allocation (each 256-byte aligned)

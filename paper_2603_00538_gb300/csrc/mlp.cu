@@ -523,12 +523,12 @@ struct TrainWs {
 };
 
 static sft_status train_attrs() {
-  static bool done = false;
-  if (done) return SFT_OK;
-  SFT_CUDA(cudaFuncSetAttribute(k_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTrain));
-  SFT_CUDA(cudaFuncSetAttribute(k_train_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDw));
-  done = true;
-  return SFT_OK;
+  static PerDevice attrs;
+  return attrs.once([]() -> sft_status {
+    SFT_CUDA(cudaFuncSetAttribute(k_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTrain));
+    SFT_CUDA(cudaFuncSetAttribute(k_train_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDw));
+    return SFT_OK;
+  });
 }
 
 // forward + backward of one batch of n rows, accumulating the gradient of
@@ -564,11 +564,12 @@ static sft_status batch_grad(sft_mlp_s* m, TrainWs& ws, const float* pts, const 
 
 sft_status mlp_forward_dev(sft_mlp_s* m, int64_t n, const float* pts, float* out, cudaStream_t st, int32_t* d_err) {
   if (n <= 0) return SFT_OK;
-  static bool attr_done = false;
-  if (!attr_done) {
-    SFT_CUDA(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFwd));
-    attr_done = true;
-  }
+  static PerDevice attrs;
+  if (sft_status r = attrs.once([]() -> sft_status {
+        SFT_CUDA(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFwd));
+        return SFT_OK;
+      }))
+    return r;
   int dev = 0, sms = 0;
   SFT_CUDA(cudaGetDevice(&dev));
   SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

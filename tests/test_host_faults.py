@@ -69,3 +69,23 @@ def test_the_largest_grids_are_still_built(fake, dim, L):
         sft.sft_source_create(m.coords, m.conn, m.values, grid_scale_L=L)
     assert e.value.status == sft.SFT_ERR_OOM
     assert fake.fake_live() == 0
+
+
+def test_network_calls_on_several_devices(fake):
+    """The kernels' shared-memory opt-in belongs to a device: first calls on each of three
+    (one beyond the table of devices), then again on the first."""
+    n = fake.sft_mlp_nparam()
+    params, pts = np.zeros(n, np.float32), np.zeros((300, 3), np.float32)
+    out, grad, loss = np.zeros(300, np.float32), np.zeros(n, np.float32), ctypes.c_double()
+    p = lambda a: ctypes.c_void_p(a.ctypes.data)
+    for dev in (0, 1, 70, 0):
+        fake.fake_device(dev)
+        h = ctypes.c_void_p()
+        assert fake.sft_mlp_create(p(params), 1, None, ctypes.byref(h)) == 0
+        ran = fake.fake_ran()
+        assert fake.sft_mlp_forward(h, 300, p(pts), p(out), 1, None) == 0, (dev, fake.sft_last_error())
+        assert fake.sft_mlp_loss_grad(h, 300, p(pts), p(out), p(grad), ctypes.byref(loss), 1, None) == 0, dev
+        assert fake.sft_mlp_train(h, 300, p(pts), p(out), 1, 128, 1e-3, 1e-4, None, 1, None) == 0, dev
+        assert fake.fake_ran() >= ran + 5
+        fake.sft_mlp_destroy(h)
+    assert fake.fake_live() == 0
