@@ -51,6 +51,11 @@ struct DevBuf {
   cudaStream_t s = nullptr;
   explicit DevBuf(cudaStream_t st) : s(st) {}
   cudaError_t alloc(size_t n) { return dalloc(&p, n, s); }
+  T* release() {
+    T* const q = p;
+    p = nullptr;
+    return q;
+  }
   ~DevBuf() { dfree(p, s); }
 };
 

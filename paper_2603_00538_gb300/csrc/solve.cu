@@ -908,28 +908,31 @@ __global__ void k_scaled_slices(const int32_t* __restrict__ rp, const int32_t* _
   }
 }
 
-static sft_status jacobi_scale(sft_target_s* t, cudaStream_t st) {
-  if (t->sc) return SFT_OK;
-  const int64_t n = t->nv;
-  SFT_CUDA(dalloc(&t->sc, (size_t)n, st));
-  const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
-  ::sft::note_launch(), k_jacobi_sqrt<<<nb, 256, 0, st>>>(t->dinv, n, t->sc);
-  SFT_CUDA(cudaGetLastError());
-  return SFT_OK;
-}
-
+// (the arrays become the target's together, once all are there and their
+// kernels are launched: a call that fails half-way leaves none behind)
 sft_status scaled_slices(sft_target_s* t, cudaStream_t st) {
   if (t->jent) return SFT_OK;
   const int64_t n = t->nv, ns = (n + kSlice - 1) / kSlice;
-  if (sft_status r = jacobi_scale(t, st)) return r;
-  SFT_CUDA(dalloc(&t->rinfo, (size_t)(ns * kSlice), st));
-  SFT_CUDA(dalloc(&t->jval, (size_t)std::max<int64_t>(t->nnz, 1), st));
-  SFT_CUDA(dalloc(&t->mdiag, (size_t)n, st));
-  SFT_CUDA(dalloc(&t->jent, (size_t)std::max<int64_t>(t->nnz, 1), st));
-  const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ns + 7) / 8, 152 * 16));
-  ::sft::note_launch(), k_scaled_slices<<<nb, 256, 0, st>>>(t->row_ptr, t->col, t->val, t->sc, n, ns, t->jent,
-                                                           t->jval, t->mdiag, t->rinfo);
+  DevBuf<double> sc(st), jval(st), mdiag(st);
+  DevBuf<uint16_t> rinfo(st);
+  DevBuf<int2> jent(st);
+  SFT_CUDA(sc.alloc((size_t)n));
+  SFT_CUDA(rinfo.alloc((size_t)(ns * kSlice)));
+  SFT_CUDA(jval.alloc((size_t)t->nnz));
+  SFT_CUDA(mdiag.alloc((size_t)n));
+  SFT_CUDA(jent.alloc((size_t)t->nnz));
+  const unsigned nbj = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
+  ::sft::note_launch(), k_jacobi_sqrt<<<nbj, 256, 0, st>>>(t->dinv, n, sc.p);
   SFT_CUDA(cudaGetLastError());
+  const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ns + 7) / 8, 152 * 16));
+  ::sft::note_launch(), k_scaled_slices<<<nb, 256, 0, st>>>(t->row_ptr, t->col, t->val, sc.p, n, ns, jent.p,
+                                                           jval.p, mdiag.p, rinfo.p);
+  SFT_CUDA(cudaGetLastError());
+  t->sc = sc.release();
+  t->rinfo = rinfo.release();
+  t->jval = jval.release();
+  t->mdiag = mdiag.release();
+  t->jent = jent.release();
   return SFT_OK;
 }
 

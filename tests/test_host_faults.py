@@ -89,3 +89,47 @@ def test_network_calls_on_several_devices(fake):
         assert fake.fake_ran() >= ran + 5
         fake.sft_mlp_destroy(h)
     assert fake.fake_live() == 0
+
+
+@pytest.mark.parametrize("what", ["alloc", "launch"])
+def test_a_solve_that_fails_half_way_can_be_repeated(fake, what):
+    """Each allocation and each launch of a target's first mixed solve fails once: nothing stays
+    behind, and the next solve launches the whole preparation."""
+    import paper_2603_00538_gb300 as sft
+
+    def solve(t):   # the fake's kernels do nothing, so a solve that ran reports no convergence
+        with pytest.raises(sft.SftError) as e:
+            sft.sft_mass_solve(t, np.ones((1, 9)), u_out=np.zeros((1, 9)))
+        return e.value.status
+
+    def first_solve():
+        m = _mesh(2)
+        return sft.sft_target_create(m.coords, m.conn)
+
+    t = first_solve()
+    live, ran = fake.fake_live(), fake.fake_ran()
+    assert solve(t) == sft.SFT_ERR_NOT_CONVERGED
+    kept, launches = fake.fake_live() - live, fake.fake_ran() - ran
+    assert launches == 3 and kept == 5
+    t.close()
+    for k in range(1, 20) if what == "alloc" else ("k_jacobi_sqrt", "k_scaled_slices", "k_mixed"):
+        t = first_solve()
+        live = fake.fake_live()
+        if what == "alloc":
+            fake.fake_fail_alloc(k)
+        else:
+            fake.fake_fail_launch(k.encode())
+        status = solve(t)
+        fake.fake_reset()
+        if status == sft.SFT_ERR_NOT_CONVERGED:   # the k-th allocation is beyond the call's last
+            assert what == "alloc" and k > kept
+            t.close()
+            break
+        assert status == (sft.SFT_ERR_OOM if what == "alloc" else sft.SFT_ERR_CUDA)
+        assert fake.fake_live() - live in (0, kept)
+        ran = fake.fake_ran()
+        prepared = fake.fake_live() - live == kept
+        assert solve(t) == sft.SFT_ERR_NOT_CONVERGED
+        assert fake.fake_ran() - ran == (1 if prepared else launches)
+        assert fake.fake_live() - live == kept
+        t.close()
