@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(kSolveThreads) k_pcg(const int32_t* __restrict
 // 0.71 / 0.68 ms on the 1.0 M-row 2D / 0.5 M-row 3D systems, 3e-6 and 1e-6
 // 0.74 / 0.71 ms: deeper FP32 solves cost more iterations than the extra
 // refinement cycle they save)
-constexpr float kEtaFloor = 1e-5f;
+constexpr double kEtaFloor = 1e-5f;
+constexpr int kMaxSteps = 16;  // steps of a cycle: at most 13 (tetrahedra)
 
 // Off-diagonal entries of A for the FP32 steps (A's diagonal is 1): rows in
 // slices of 32, each slice's rows sorted by length (longest first) over the
@@ -493,6 +494,11 @@ struct MixArgs {
   int warm;
   uint64_t wait_ns;
   float lmax;
+  // step counts of a cycle that asks for the reduction e = 0.1 tol ||b|| / ||r||
+  // (kEtaFloor to 1/4): the smallest K >= k_min with T_K(s1) >= 1 / e, which is
+  // reach[K] ||b||^2 >= ||r||^2 for K < k_max, with reach[K] = (0.1 tol T_K)^2
+  int k_min, k_max;
+  double reach[kMaxSteps];
   int spb;                // slices per block
   int cap;                // entries held in shared memory
   int c_smem;             // c held in shared memory
@@ -547,7 +553,6 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
   MixCtl* ctl = a.ctl;
   unsigned phase = 0;
   const ChebCoef ch = cheb_coef(a.lmax);
-  const float inv_acosh = 1.f / acoshf(ch.s1);
   YRef<TEAM, OWN> Y;
   Y.sm = ysm;
   Y.glob = a.ya;
@@ -717,31 +722,34 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
     put_partials(v, part);
     if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
     get_totals(part);
-    if (tid < nrhs) {
-      const int f = tid;
-      act[f] = 0;
-      ks[f] = 0;
-      if (live[f]) {
-        // tests on the squared norms (no square root or quotient on the way)
-        const double rn2 = shtot[2 * f], tn2 = shtot[2 * f + 1];
-        if (cyc == 0 && !a.warm) bn2[f] = rn2;
-        const double b2 = bn2[f], last2 = prev2[f];
-        prev2[f] = rn2;
-        itf[f] = it;
-        if (rn2 <= a.tol * a.tol * b2) {
-          live[f] = 0;
-          conv[f] = 1;
-        } else if ((cyc > 0 && rn2 > 0.25 * last2) || !(tn2 > 0.0)) {
-          // a cycle that did not halve the residual (FP64 rounding floor) or a
-          // residual on rows without diagonal ends the field unconverged
-          live[f] = 0;
-        } else {
-          const double is = rsqrt(tn2);
-          isig[f] = is;
-          sig[f] = tn2 * is;
-          const float e = fminf(0.25f, fmaxf(kEtaFloor, (float)(0.1 * a.tol) * sqrtf((float)(b2 / rn2))));
-          ks[f] = max(1, (int)ceilf(acoshf(1.f / e) * inv_acosh));
-          act[f] = 1;
+    if (warp < nrhs) {   // a warp per field; the lanes try the step counts
+      const int f = warp;
+      // tests on the squared norms (no square root or quotient on the way)
+      const double rn2 = shtot[2 * f], tn2 = shtot[2 * f + 1];
+      const double b2 = cyc == 0 && !a.warm ? rn2 : bn2[f], last2 = prev2[f];
+      const bool more = lane >= a.k_min && lane < a.k_max && a.reach[lane & (kMaxSteps - 1)] * b2 < rn2;
+      const int k = a.k_min + __popc(__ballot_sync(0xffffffffu, more));
+      if (lane == 0) {
+        act[f] = 0;
+        ks[f] = 0;
+        if (live[f]) {
+          bn2[f] = b2;
+          prev2[f] = rn2;
+          itf[f] = it;
+          if (rn2 <= a.tol * a.tol * b2) {
+            live[f] = 0;
+            conv[f] = 1;
+          } else if ((cyc > 0 && rn2 > 0.25 * last2) || !(tn2 > 0.0)) {
+            // a cycle that did not halve the residual (FP64 rounding floor) or a
+            // residual on rows without diagonal ends the field unconverged
+            live[f] = 0;
+          } else {
+            const double is = rsqrt(tn2);
+            isig[f] = is;
+            sig[f] = tn2 * is;
+            ks[f] = k;
+            act[f] = 1;
+          }
         }
       }
     }
@@ -1069,6 +1077,19 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
   a.warm = warm;
   a.wait_ns = t->wait_ns;
   a.lmax = t->dim == 2 ? 2.f : 2.5f;  // largest eigenvalue bound of S M S
+  {
+    const double s1 = cheb_coef(a.lmax).s1;
+    double t0 = 1.0, t1 = s1;   // T_{K-1}, T_K
+    a.k_min = a.k_max = 0;
+    for (int k = 1; k < kMaxSteps; ++k) {
+      a.reach[k] = (0.1 * tol * t1) * (0.1 * tol * t1);
+      if (!a.k_min && t1 >= 4.0) a.k_min = k;
+      if (!a.k_max && t1 * kEtaFloor >= 1.0) a.k_max = k;
+      const double t2 = 2.0 * s1 * t1 - t0;
+      t0 = t1;
+      t1 = t2;
+    }
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nblocks);
   cfg.blockDim = dim3(kMixThreads<NR>);

@@ -1,0 +1,52 @@
+"""Step counts of the mixed solve's first cycle at their edges. From u = 0 the
+cycle asks for e = 0.1 tol (clamped to 1e-5 .. 1/4), and takes the smallest K
+with T_K(s1) >= 1 / e (s1 of the spectrum interval, formed in FP32 as the
+kernel does). Tolerances 1e-9 to either side of 10 / T_K tell the counts of
+64-bit arithmetic from those of 32; an easy right-hand side (one smooth mode)
+converges within the cycle, so the reported iterations are the count. On a
+block, a cluster and the grid."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2603_00538_gb300 as sft  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+def _chebyshev(dim):
+    f = np.float32
+    a, b = f(0.5) * (f(1) - f(1e-3)), f(2.0 if dim == 2 else 2.5) * (f(1) + f(1e-3))
+    s1 = float((f(0.5) * (a + b)) / (f(0.5) * (b - a)))
+    t = [1.0, s1]
+    while len(t) < 16:
+        t.append(2 * s1 * t[-1] - t[-2])
+    return t
+
+
+def _steps(dim, tol):
+    t = _chebyshev(dim)
+    e = min(0.25, max(float(np.float32(1e-5)), 0.1 * tol))
+    return next(k for k in range(1, 16) if t[k] * e >= 1.0)
+
+
+@pytest.mark.parametrize("dim,n", [(2, 20), (2, 60), (2, 140), (3, 7), (3, 12), (3, 22)])
+def test_steps_of_the_first_cycle(orc, dim, n):
+    m = W.jittered_tri_mesh(n, 3) if dim == 2 else W.jittered_kuhn_mesh(n, 3)
+    t = sft.mesh_target(m, device=DEV)
+    rp, col, val = orc.mass_csr(m.coords, m.conn)
+    rows = np.repeat(np.arange(m.nnodes), np.diff(rp))
+    b = np.bincount(rows, weights=val, minlength=m.nnodes)[None]   # M 1
+    cheb = _chebyshev(dim)
+    tols = [10.0 / cheb[k] * (1 + s) for k in range(3, 13) for s in (1e-9, -1e-9)]
+    for tol in (x for x in tols if 1.001e-4 < x < 1.0):
+        _, it, rr = sft.sft_mass_solve(t, b, tol=tol, max_iter=100)
+        assert rr <= tol
+        assert it == _steps(dim, tol), tol
