@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
           bn2[f] = b2;
           prev2[f] = rn2;
           itf[f] = it;
-          if (rn2 <= a.tol * a.tol * b2) {
+          if (rn2 <= a.tol * (a.tol * b2)) {  // (in this order: b = 0 has converged for any tol)
             live[f] = 0;
             conv[f] = 1;
           } else if ((cyc > 0 && rn2 > 0.25 * last2) || !(tn2 > 0.0)) {

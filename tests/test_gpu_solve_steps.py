@@ -50,3 +50,11 @@ def test_steps_of_the_first_cycle(orc, dim, n):
         _, it, rr = sft.sft_mass_solve(t, b, tol=tol, max_iter=100)
         assert rr <= tol
         assert it == _steps(dim, tol), tol
+
+
+@pytest.mark.parametrize("tol", [0.0, 1e-12, 1e153, 1e160, 1e308])
+def test_zero_right_hand_side_converges_at_any_tolerance(tol):
+    """||r|| <= tol ||b|| holds with both zero, whatever tol (its square overflows above 1e154)."""
+    t = sft.mesh_target(W.jittered_tri_mesh(8, 3), device=DEV)
+    u, it, rr = sft.sft_mass_solve(t, np.zeros((2, 81)), tol=tol, max_iter=50)
+    assert it == 0 and rr == 0.0 and not u.any()
