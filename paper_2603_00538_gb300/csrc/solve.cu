@@ -977,6 +977,9 @@ constexpr int64_t kBlockWork = 10000;
 constexpr int64_t kClusterWork = 110000;
 constexpr int kClusterBlocks = 16;
 
+constexpr int64_t kThinShare = 8;      // share of A over what fits, from which little is held (launch_mixed)
+constexpr int kThinEntries = 12000;
+
 // Attributes of the solve kernels on the current device, set once per device;
 // false when a cluster of kClusterBlocks cannot be resident there.
 template <int NR>
@@ -1037,6 +1040,16 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
   // shared memory for the block's share of A (with room for uneven shares)
   const int64_t want = t->nnz * a.spb / std::max<int64_t>(ns, 1) * 5 / 4 + 1024;
   a.cap = (int)(std::min<int64_t>(want, ((int64_t)kMixSmemMax - fixed) / 8) & ~(int64_t)1);  // 16-byte multiple
+  // Where hardly any of the share fits and y is gathered from global memory,
+  // the gathers gain more from L1 than the held entries save: then only
+  // kThinEntries (96 KB) are held. Call times of k_mixed before it had the
+  // rule, with it, and of the kernel of four blocks per SM without shared
+  // memory that it replaced: 3.0 M rows 3D 3,066 / 2,825 / 3,165 us, 4.5 M
+  // 4,500 / 4,162 / 4,475, 8.0 M 7,790 / 7,180 / 7,700; 2 fields of 2.2 M
+  // 2,671 / 2,327 / 3,707. Below the line holding all that fits is better: 3.0 M
+  // rows 2D (a fifth held) 1,695 against 1,756, 4 fields of 1.4 M rows 3D 3,493
+  // against 3,532, of 0.64 M 1,226 against 1,466.
+  if (!own && want > kThinShare * (int64_t)a.cap) a.cap = std::min(a.cap, kThinEntries);
   const size_t smem = (size_t)a.cap * 8 + (size_t)fixed;
   const void* kern = team == kTeamBlock     ? (const void*)k_mixed<NR, kTeamBlock, true>
                      : team == kTeamCluster ? (const void*)k_mixed<NR, kTeamCluster, true>

@@ -58,3 +58,20 @@ def test_zero_right_hand_side_converges_at_any_tolerance(tol):
     t = sft.mesh_target(W.jittered_tri_mesh(8, 3), device=DEV)
     u, it, rr = sft.sft_mass_solve(t, np.zeros((2, 81)), tol=tol, max_iter=50)
     assert it == 0 and rr == 0.0 and not u.any()
+
+
+@pytest.mark.parametrize("n,nrhs", [(1960, 1), (1950, 2)])
+def test_systems_that_hold_little_of_their_matrix(n, nrhs):
+    """More than 26 M nonzeros: k_mixed keeps 12,000 entries of a block's 175,000. Against the FP64 CG
+    (each residual below tol ||b||, and cond(M) of this mesh's Jacobi-scaled matrix is at most 4;
+    the areas differ by less than a factor of 10, which bounds the unscaled one by 40)."""
+    t = sft.mesh_target(W.jittered_tri_mesh(n, 3), device=DEV)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(n)
+    b = torch.randn((nrhs, (n + 1) ** 2), dtype=torch.float64, device=DEV, generator=g)
+    u, v = torch.zeros_like(b), torch.zeros_like(b)
+    _, _, rr = sft.sft_mass_solve(t, b, tol=1e-11, u_out=u)
+    sft.sft_mass_solve(t, b, tol=1e-11, u_out=v, cg_mode=sft.SFT_CG_FP64)
+    assert rr <= 1e-11
+    for f in range(nrhs):
+        assert float((u[f] - v[f]).norm() / v[f].norm()) <= 2 * 40 * 1e-11
