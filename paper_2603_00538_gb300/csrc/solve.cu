@@ -505,6 +505,48 @@ struct MixArgs {
   int r_smem;             // rinfo held in shared memory
 };
 
+// a block's per-field state of the refinement cycles (shared memory)
+struct Cycle {
+  double tot[2 * kMaxFields];   // ||r||^2 and ||t||^2 by field
+  double bn2[kMaxFields], prev2[kMaxFields], sig[kMaxFields], isig[kMaxFields];
+  double reach[kMaxSteps];
+  int live[kMaxFields], act[kMaxFields], conv[kMaxFields], ks[kMaxFields], itf[kMaxFields];
+};
+
+// Field f after the residual of cycle cyc, by a warp: converged, given up, or
+// ||t||, 1 / ||t|| and the step count of its next inner solve (the lanes try
+// the counts). Out of line: inside k_mixed it changes the registers of the
+// steps (3.0 M rows 2D 1,660 us a call against 1,580, 4 fields of 636 k rows 3D
+// 1,160 against 1,110).
+__device__ __noinline__ void decide(Cycle& c, int f, int lane, int cyc, int warm, int it, double tol, int k_min, int k_max) {
+  // tests on the squared norms (no square root or quotient on the way)
+  const double rn2 = c.tot[2 * f], tn2 = c.tot[2 * f + 1];
+  const double b2 = cyc == 0 && !warm ? rn2 : c.bn2[f], last2 = c.prev2[f];
+  const bool more = lane >= k_min && lane < k_max && c.reach[lane & (kMaxSteps - 1)] * b2 < rn2;
+  const int k = k_min + __popc(__ballot_sync(0xffffffffu, more));
+  if (lane != 0) return;
+  c.act[f] = 0;
+  c.ks[f] = 0;
+  if (!c.live[f]) return;
+  c.bn2[f] = b2;
+  c.prev2[f] = rn2;
+  c.itf[f] = it;
+  if (rn2 <= tol * (tol * b2)) {  // (in this order: b = 0 has converged for any tol)
+    c.live[f] = 0;
+    c.conv[f] = 1;
+  } else if ((cyc > 0 && rn2 > 0.25 * last2) || !(tn2 > 0.0)) {
+    // a cycle that did not halve the residual (FP64 rounding floor) or a
+    // residual on rows without diagonal ends the field unconverged
+    c.live[f] = 0;
+  } else {
+    const double is = rsqrt(tn2);
+    c.isig[f] = is;
+    c.sig[f] = tn2 * is;
+    c.ks[f] = k;
+    c.act[f] = 1;
+  }
+}
+
 // blocks hold as much of their part of A as fits in shared memory for the
 // whole solve: bytes of it
 constexpr uint32_t kMixSmemMax = 212u * 1024u;
@@ -532,9 +574,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ int32_t s_off[kMaxStaged + 1];     // start of each held slice in ent
   __shared__ double shw[W][V];
-  __shared__ double shtot[V];
-  __shared__ double bn2[NR], prev2[NR], sig[NR], isig[NR];
-  __shared__ int live[NR], act[NR], conv[NR], ks[NR], itf[NR];
+  __shared__ Cycle C;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned nb = gridDim.x;
   const int64_t n = a.n;
@@ -569,11 +609,12 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
     if (lane == 0) s_off[sl + 1] = cnt;
   }
   if (tid == 0) s_off[0] = 0;
+  if (tid < kMaxSteps) C.reach[tid] = a.reach[tid];
   if (tid < NR) {
-    live[tid] = tid < nrhs;
-    act[tid] = 0;
-    conv[tid] = 0;
-    itf[tid] = 0;
+    C.live[tid] = tid < nrhs;
+    C.act[tid] = 0;
+    C.conv[tid] = 0;
+    C.itf[tid] = 0;
   }
   __syncthreads();
   if (warp == 0) {
@@ -605,7 +646,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
   __syncthreads();
 
   // per-block partial sums -> global; after the barrier every block adds all
-  // of them in the same order (totals in shtot)
+  // of them in the same order (totals in C.tot)
   auto put_partials = [&](double (&v)[V], double* part) {
     const double ws = warp_sums<V>(v, lane);
     if (lane % (32 / V) == 0) shw[warp][lane / (32 / V)] = ws;
@@ -620,7 +661,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
       double s = 0.0;
       for (int k = lane; k < (int)nb; k += 32) s += __ldcg(part + (int64_t)warp * nb + k);
       s = warp_sum<double>(s);
-      if (lane == 0) shtot[warp] = s;
+      if (lane == 0) C.tot[warp] = s;
     }
     __syncthreads();
   };
@@ -640,7 +681,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
     put_partials(v, a.partd);
     if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
     get_totals(a.partd);
-    if (tid < nrhs) bn2[tid] = shtot[2 * tid];
+    if (tid < nrhs) C.bn2[tid] = C.tot[2 * tid];
     __syncthreads();
   }
 
@@ -656,7 +697,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
 #pragma unroll
       for (int f = 0; f < NR; ++f) {
         if (f >= nrhs) break;
-        if (!live[f]) continue;
+        if (!C.live[f]) continue;
         const int64_t o = (int64_t)f * n + i;
         if (zero_x) a.x[o] = 0.0;
         const double ri = a.b[o] - s[f];
@@ -722,44 +763,14 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
     put_partials(v, part);
     if (!team_sync<TEAM>(ctl, nb, phase, a.wait_ns)) return;
     get_totals(part);
-    if (warp < nrhs) {   // a warp per field; the lanes try the step counts
-      const int f = warp;
-      // tests on the squared norms (no square root or quotient on the way)
-      const double rn2 = shtot[2 * f], tn2 = shtot[2 * f + 1];
-      const double b2 = cyc == 0 && !a.warm ? rn2 : bn2[f], last2 = prev2[f];
-      const bool more = lane >= a.k_min && lane < a.k_max && a.reach[lane & (kMaxSteps - 1)] * b2 < rn2;
-      const int k = a.k_min + __popc(__ballot_sync(0xffffffffu, more));
-      if (lane == 0) {
-        act[f] = 0;
-        ks[f] = 0;
-        if (live[f]) {
-          bn2[f] = b2;
-          prev2[f] = rn2;
-          itf[f] = it;
-          if (rn2 <= a.tol * (a.tol * b2)) {  // (in this order: b = 0 has converged for any tol)
-            live[f] = 0;
-            conv[f] = 1;
-          } else if ((cyc > 0 && rn2 > 0.25 * last2) || !(tn2 > 0.0)) {
-            // a cycle that did not halve the residual (FP64 rounding floor) or a
-            // residual on rows without diagonal ends the field unconverged
-            live[f] = 0;
-          } else {
-            const double is = rsqrt(tn2);
-            isig[f] = is;
-            sig[f] = tn2 * is;
-            ks[f] = k;
-            act[f] = 1;
-          }
-        }
-      }
-    }
+    if (warp < nrhs) decide(C, warp, lane, cyc, a.warm, it, a.tol, a.k_min, a.k_max);
     __syncthreads();
     // every active field takes the largest step count (more steps only
     // reduce its residual further)
     int K = 0;
 #pragma unroll
     for (int f = 0; f < NR; ++f)
-      if (f < nrhs && act[f] && ks[f] > K) K = ks[f];
+      if (f < nrhs && C.act[f] && C.ks[f] > K) K = C.ks[f];
     if (K == 0 || it >= a.max_iter) break;
     if (K > a.max_iter - it) K = a.max_iter - it;
 
@@ -769,7 +780,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
 #pragma unroll
       for (int f = 0; f < NR; ++f) {
         if (f >= nrhs) break;
-        if (act[f]) a.x[(int64_t)f * n + i] += (sig[f] * si) * f2d(y[f]);
+        if (C.act[f]) a.x[(int64_t)f * n + i] += (C.sig[f] * si) * f2d(y[f]);
       }
     };
     // I: c = t / ||t|| in FP32, y_1 = c / theta
@@ -779,7 +790,7 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
 #pragma unroll
       for (int f = 0; f < NR; ++f) {
         c[f] = 0.f;
-        if (f < nrhs && act[f]) c[f] = (float)(a.t[(int64_t)f * n + i] * isig[f]);
+        if (f < nrhs && C.act[f]) c[f] = (float)(a.t[(int64_t)f * n + i] * C.isig[f]);
         y[f] = c[f] * ith;
       }
       if (K == 1) {
@@ -844,9 +855,9 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
   }
   if (blockIdx.x == 0 && tid < nrhs) {
     if (tid == 0) ctl->cycles = cyc;
-    ctl->iters[tid] = itf[tid];
-    ctl->rel[tid] = bn2[tid] > 0.0 ? sqrt(prev2[tid] / bn2[tid]) : 0.0;
-    ctl->conv[tid] = conv[tid];
+    ctl->iters[tid] = C.itf[tid];
+    ctl->rel[tid] = C.bn2[tid] > 0.0 ? sqrt(C.prev2[tid] / C.bn2[tid]) : 0.0;
+    ctl->conv[tid] = C.conv[tid];
   }
 }
 
@@ -1044,9 +1055,9 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
   // the gathers gain more from L1 than the held entries save: then only
   // kThinEntries (96 KB) are held. Call times of k_mixed before it had the
   // rule, with it, and of the kernel of four blocks per SM without shared
-  // memory that it replaced: 3.0 M rows 3D 3,066 / 2,825 / 3,165 us, 4.5 M
-  // 4,500 / 4,162 / 4,475, 8.0 M 7,790 / 7,180 / 7,700; 2 fields of 2.2 M
-  // 2,671 / 2,327 / 3,707. Below the line holding all that fits is better: 3.0 M
+  // memory that it replaced: 3.0 M rows 3D 3,065 / 2,780 / 3,165 us, 4.5 M
+  // 4,415 / 4,035 / 4,475, 8.0 M 7,776 / 7,085 / 7,700; 2 fields of 2.2 M
+  // 2,667 / 2,266 / 3,707. Below the line holding all that fits is better: 3.0 M
   // rows 2D (a fifth held) 1,695 against 1,756, 4 fields of 1.4 M rows 3D 3,493
   // against 3,532, of 0.64 M 1,226 against 1,466.
   if (!own && want > kThinShare * (int64_t)a.cap) a.cap = std::min(a.cap, kThinEntries);
