@@ -58,6 +58,14 @@ __device__ __forceinline__ bool not_neg(double x) {
 }
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
 
+// x 2^k by the exponent (FP64 products use the FP64 pipe), |k| <= 1022
+__device__ __forceinline__ double scaled(double x, int k) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7FF;
+  if (e > 0 && (unsigned)(e + k - 1) < 2046u) return __longlong_as_double(b + ((long long)k << 52));
+  return b << 1 == 0 ? x : x * __longlong_as_double((long long)(1023 + k) << 52);
+}
+
 // a vertex of a clipped polygon: two area coordinates of the target triangle
 // and the source field
 struct PV { double a1, a2, f; };
@@ -98,8 +106,8 @@ __global__ void k_mi_start(const GridP<double>* __restrict__ gp, const int32_t* 
 
 // what a warp keeps in shared memory
 struct alignas(16) MiWarp {
-  // targets: vertices 0..5, edges v0 -> v1, v1 -> v2, v2 -> v0 (A_2, A_0, A_1) 6..11,
-  // L2: 1 / (48 |t|) 12, u = u0 + A_1 g1 + A_2 g2 13..15; b: 1 / (12 |t|) 12, 1 / (96 |t|^2) 13
+  // targets: vertices 0..5, c (edges v0 -> v1, v1 -> v2, v2 -> v0) (A_2, A_0, A_1) 6..11; of the scaled
+  // coordinates L2: 1 / (48 |t|) 12, u = u0 + A_1 g1 + A_2 g2 13..15; b: 1 / (12 |t|) 12, 1 / (96 |t|^2) 13
   double tgt[16][32];
   double poly[2 * kMiVerts - 1][3][32];  // clipped polygons: rows 0..5 and 6..10 in turn
   double surv[12][64];             // pairs to clip: A_0, A_1, A_2, f at the source triangle's vertices
@@ -158,22 +166,27 @@ __global__ void __launch_bounds__(kMiThreads) k_mi_2d(
           const double2 x = __ldg(reinterpret_cast<const double2*>(tx) + tn[m]);
           tv[m] = P2{x.x, x.y};
         }
-        const double rD = 1.0 / cross3(tv[0], tv[1], tv[2]);
+        // the coordinates are kept as c A_m with c the power of two that brings
+        // 2 |t| to d in [1, 2): their products (fourth powers of lengths) then
+        // keep clear of FP64's range at any scale of the mesh, with the same bits
+        const double D = cross3(tv[0], tv[1], tv[2]);
+        const int k = 1023 - min(max((int)(__double_as_longlong(D) >> 52), 1), 2045);   // c = 2^k
+        const double rd = 1.0 / scaled(D, k);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
           w.tgt[2 * m][lane] = tv[m].x;
           w.tgt[2 * m + 1][lane] = tv[m].y;
-          w.tgt[6 + 2 * m][lane] = tv[(m + 1) % 3].x - tv[m].x;
-          w.tgt[7 + 2 * m][lane] = tv[(m + 1) % 3].y - tv[m].y;
+          w.tgt[6 + 2 * m][lane] = scaled(tv[(m + 1) % 3].x - tv[m].x, k);
+          w.tgt[7 + 2 * m][lane] = scaled(tv[(m + 1) % 3].y - tv[m].y, k);
         }
-        w.tgt[12][lane] = rD * (L2 ? 1.0 / 24.0 : 1.0 / 6.0);
+        w.tgt[12][lane] = scaled(rd * (L2 ? 1.0 / 24.0 : 1.0 / 6.0), -k);
         if (!L2) {
-          w.tgt[13][lane] = rD * rD * (1.0 / 24.0);
+          w.tgt[13][lane] = scaled(rd * rd * (1.0 / 24.0), -k);
         } else {
           const double u0 = __ldg(u + tn[0]);
           w.tgt[13][lane] = u0;
-          w.tgt[14][lane] = (__ldg(u + tn[1]) - u0) * rD;
-          w.tgt[15][lane] = (__ldg(u + tn[2]) - u0) * rD;
+          w.tgt[14][lane] = (__ldg(u + tn[1]) - u0) * rd;
+          w.tgt[15][lane] = (__ldg(u + tn[2]) - u0) * rd;
         }
         w.walk[0][lane] = s0;
         head = 0;
