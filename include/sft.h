@@ -244,12 +244,19 @@ sft_status sft_mass_solve(sft_target tgt, int32_t nrhs, const double* b, double*
                           int32_t device_ptrs, double tol, int32_t max_iter, int32_t cg_mode,
                           void* cuda_stream, int32_t* iters_out, double* rel_resid_out);
 
-/* Limit of every device wait in the solves on this target (the grid barriers
- * of the cooperative CG kernels of step 7, Eq. cv_galerkin_system, reached
+/* Limit of every device wait in the solves on this target (the barriers
+ * between the blocks of the kernels of step 7, Eq. cv_galerkin_system, reached
  * through sft_transfer, sft_plan_transfer and sft_mass_solve): a wait that
  * runs past it sets the kernel's error word, every block of the launch
  * returns, and the call reports SFT_ERR_DEVICE_STATUS; the stream and the
- * context stay usable. Default 2 s; `seconds` in (0, 3600], else SFT_ERR_ARG.
+ * context stay usable. How a wait ends depends on the size of the system:
+ * - blocks over the whole GPU wait on a counter and leave at the limit;
+ * - MIXED solves of up to 110,000 nonzeros x fields (fields rounded up to 1, 2,
+ *   4, 8) run on one cluster of blocks, whose hardware barrier cannot be left
+ *   early: its blocks are resident together and none waits for anything else,
+ *   and a barrier that took longer than the limit ends the launch at the next;
+ * - up to 10,000 they run on one block, which waits for no other: no limit.
+ * Default 2 s; `seconds` in (0, 3600], else SFT_ERR_ARG.
  * The paper has no counterpart (failure detection of the device path). */
 sft_status sft_target_set_wait_limit(sft_target tgt, double seconds);
 
