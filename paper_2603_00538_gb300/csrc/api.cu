@@ -305,7 +305,7 @@ sft_status sft_transfer(sft_source s, sft_target t, const sft_options* o, double
   }
   SolveResult sr;
   SolveLate late(status->solve);  // the solve's status is read with the final readback below
-  if (sft_status r = mass_solve(t, nf, b, u_dev, o->cg_tol, o->cg_max_iter, st, &status->err, &sr, o->cg_mode, &late,
+  if (sft_status r = mass_solve(t, nf, b, u_dev, o->cg_tol, o->cg_max_iter, st, &sr, o->cg_mode, &late,
                                 o->cg_warm_start))
     return r;
   ev.record(4, st);
@@ -438,7 +438,7 @@ sft_status sft_mass_solve(sft_target t, int32_t nrhs, const double* b, double* u
     ud = ut.p;
   }
   SolveResult sr;
-  if (sft_status r = mass_solve(t, nrhs, bd, ud, tol, max_iter, st, nullptr, &sr, cg_mode)) return r;
+  if (sft_status r = mass_solve(t, nrhs, bd, ud, tol, max_iter, st, &sr, cg_mode)) return r;
   if (!device_ptrs) SFT_CUDA(cudaMemcpyAsync(u, ud, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
   SFT_CUDA(cudaStreamSynchronize(st));
   if (iters_out) *iters_out = sr.iters;

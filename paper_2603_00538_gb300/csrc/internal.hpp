@@ -249,7 +249,7 @@ struct SolveLate {
 sft_status finish_solve(const SolveLate& late, const CallStatus& host, SolveResult* res);
 // cg_mode: SFT_CG_MIXED (FP64 refinement around an FP32 Chebyshev iteration) or SFT_CG_FP64
 sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, double tol, int max_iter,
-                      cudaStream_t st, int32_t* d_err, SolveResult* res, int cg_mode = SFT_CG_MIXED,
+                      cudaStream_t st, SolveResult* res, int cg_mode = SFT_CG_MIXED,
                       SolveLate* late = nullptr, int warm = 0);
 // S = diag(M)^-1/2 and the jagged diagonals of M and S M S on the target (made once, kept)
 sft_status scaled_slices(sft_target_s* t, cudaStream_t st);

@@ -53,24 +53,11 @@ constexpr float kNegLog2e = -1.4426950408889634f;
 // u + u tanh(u), u = z/2, loses accuracy to cancellation for z << 0: its
 // absolute error |u| 2^-11 exceeds the BF16 rounding of the activation.)
 __device__ __forceinline__ float sigmoid_f(float z) { return rcp_sfu(1.0f + ex2_sfu(kNegLog2e * z)); }
-// SiLU z sigma(z): two special-function operations per activation
-__device__ __forceinline__ float silu_f(float z) { return z * sigmoid_f(z); }
-
-// (packed FP32 pair helpers f2_*: common.cuh)
-// silu_f of both lanes of z2 (the same operations in the same order)
-__device__ __forceinline__ void silu_pair(uint64_t z2, float& h0, float& h1) {
-  float t0, t1;
-  f2_unpack(f2_mul(z2, f2_pack(kNegLog2e, kNegLog2e)), t0, t1);
-  float d0, d1;
-  f2_unpack(f2_add(f2_pack(1.0f, 1.0f), f2_pack(ex2_sfu(t0), ex2_sfu(t1))), d0, d1);
-  f2_unpack(f2_mul(z2, f2_pack(rcp_sfu(d0), rcp_sfu(d1))), h0, h1);
-}
 // d silu / dz = sigma(z) (1 + z (1 - sigma(z)))
 __device__ __forceinline__ float silu_grad(float z) {
   const float sg = sigmoid_f(z);
   return sg * __fmaf_rn(z, 1.0f - sg, 1.0f);
 }
-__device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 // The first layer in shared memory, pair-interleaved for the packed FMAs:
 // outputs 2m and 2m + 1 take entries 2m = {W1[2m][0], W1[2m+1][0], W1[2m][1],
@@ -384,8 +371,9 @@ __device__ __forceinline__ void refill_buffer(const FwdSmem& S, const LayerWeigh
   __syncwarp();
 }
 
-// SiLU of N pairs, rounded to BF16 pairs: each operation over all pairs
-// before the next, so the special-function latencies overlap
+// SiLU z sigma(z) of N pairs, rounded to BF16 pairs: each operation over all
+// pairs (f2_*: common.cuh) before the next, so the special-function latencies
+// overlap
 template <int N>
 __device__ __forceinline__ void silu_pairs(const uint64_t (&z)[N], uint32_t (&h)[N]) {
   float t[2 * N];

@@ -225,7 +225,7 @@ sft_status sft_plan_transfer(sft_plan pl, double* u_out, double* b_out, double* 
   }
   SolveResult sr;
   SolveLate late(status->solve);  // the solve's status is read with the final readback
-  if (sft_status r = mass_solve(t, nf, b, u_dev, o.cg_tol, o.cg_max_iter, st, &status->err, &sr, o.cg_mode, &late,
+  if (sft_status r = mass_solve(t, nf, b, u_dev, o.cg_tol, o.cg_max_iter, st, &sr, o.cg_mode, &late,
                                 o.cg_warm_start))
     return r;
   ev.record(4, st);

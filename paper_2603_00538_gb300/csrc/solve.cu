@@ -267,7 +267,6 @@ struct MixCtl {
   uint32_t arrived;      // grid barrier: arrivals so far (never reset)
   int32_t err;
   int32_t late[2];       // cluster barriers that overran the wait limit, by parity
-  int32_t cycles;
   int32_t iters[kMaxFields];
   int32_t conv[kMaxFields];
   double rel[kMaxFields];
@@ -854,7 +853,6 @@ __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
     it += K;
   }
   if (blockIdx.x == 0 && tid < nrhs) {
-    if (tid == 0) ctl->cycles = cyc;
     ctl->iters[tid] = C.itf[tid];
     ctl->rel[tid] = C.bn2[tid] > 0.0 ? sqrt(C.prev2[tid] / C.bn2[tid]) : 0.0;
     ctl->conv[tid] = C.conv[tid];
@@ -1148,8 +1146,7 @@ static sft_status launch_mixed(sft_target_s* t, int nrhs, const double* b, doubl
 }
 
 sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, double tol, int max_iter,
-                      cudaStream_t st, int32_t* d_err, SolveResult* res, int cg_mode, SolveLate* late, int warm) {
-  (void)d_err;
+                      cudaStream_t st, SolveResult* res, int cg_mode, SolveLate* late, int warm) {
   res->iters = 0;
   res->rel_resid = 0.0;
   res->converged = 1;

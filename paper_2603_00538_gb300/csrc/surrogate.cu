@@ -46,7 +46,7 @@ struct SurParams {
   int has_exact;
   PhiloxKey key;
   uint32_t stream_id;
-  float alpha, tau, cdet, cmc;
+  float alpha, cdet, cmc;
   Strat st;              // sampling scheme
 };
 
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
     const int32_t* __restrict__ cell_start, const int32_t* __restrict__ cell_items,
     const int32_t* __restrict__ cell_first, const float* __restrict__ recs,
     const int32_t* __restrict__ adj, const float* __restrict__ vals, SurParams p, double* __restrict__ b, int32_t* __restrict__ fb_out,
-    float* __restrict__ sample_f, int64_t* __restrict__ counters, int32_t* err) {
+    float* __restrict__ sample_f, int64_t* __restrict__ counters) {
   constexpr int K = DT + 1;
   extern __shared__ __align__(1024) unsigned char sm[];
   float(*piece)[8] = reinterpret_cast<float(*)[8]>(sm);  // [row][s_i, e_i]
@@ -99,8 +99,7 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
   int64_t n_exact = 0;
   int n_empty = 0;
   Acc<float> acc_long;  // N > 128: thread i < K carries node i's sum over the element's tiles
-  const int row = threadIdx.x & (kTileM - 1);
-  const bool lead = threadIdx.x < kTileM;
+  const int row = threadIdx.x;
 
   for (int64_t unit = blockIdx.x; unit < p.nunits; unit += gridDim.x) {
     acc_long = Acc<float>();
@@ -142,8 +141,7 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
       // exact queries (the fallback pass takes the subsample's values from
       // the decision pass)
       float fe = 0.f;
-      const bool sub = lead && p.has_exact && valid;
-      if (sub) {
+      if (p.has_exact && valid) {
         if (p.sub_f && j < p.s) {
           fe = __ldg(p.sub_f + t * p.s + j);
         } else {
@@ -154,12 +152,11 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
       }
       const float f = fe;
       if (valid && c == 0 && j == 0 && fb_out) fb_out[t] = 1;
-      if (lead && valid && sample_f) sample_f[t * p.N + j] = f;
+      if (valid && sample_f) sample_f[t * p.N + j] = f;
 
       // residual against the P1 control and its basis-weighted partials
       Acc<float> a[K];
-      const bool mine = lead && valid;
-      if (mine) {
+      if (valid) {
         float gX = __fmul_rn(__ldg(g + v[0]), lam[0]);
 #pragma unroll
         for (int m = 1; m < K; ++m) gX = __fmaf_rn(__ldg(g + v[m]), lam[m], gX);
@@ -168,7 +165,7 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
         for (int i = 0; i < K; ++i) a[i].add(__fmul_rn(r, lam[i]));
       }
       // warp-segmented suffix combine over rows of the same element
-      const int seg = mine ? el : -1;
+      const int seg = valid ? el : -1;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int seg2 = __shfl_down_sync(0xffffffffu, seg, o);
@@ -181,7 +178,7 @@ __global__ void __launch_bounds__(kTileM, 8) k_surrogate_exact(
         }
       }
       const int seg_prev = __shfl_up_sync(0xffffffffu, seg, 1);
-      const bool head = mine && (lane == 0 || seg_prev != seg);
+      const bool head = valid && (lane == 0 || seg_prev != seg);
       if (head) {
 #pragma unroll
         for (int i = 0; i < K; ++i) {
@@ -582,7 +579,7 @@ static sft_status net_pass(sft_mlp_s* m, sft_target_s* t, const SurParams& p, co
 
 template <int DT, int DS>
 static sft_status launch_exact(sft_source_s* s, sft_target_s* t, const SurParams& p, const float* g, double* b,
-                               int32_t* fb, float* sf, int64_t* counters, int32_t* err, cudaStream_t st) {
+                               int32_t* fb, float* sf, int64_t* counters, cudaStream_t st) {
   int dev = 0, sms = 0;
   SFT_CUDA(cudaGetDevice(&dev));
   SFT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -593,7 +590,7 @@ static sft_status launch_exact(sft_source_s* s, sft_target_s* t, const SurParams
       (const float*)t->coordsP[SFT_PREC_FP32], t->conn, t->vol32, g,
       L ? (const GridP<float>*)L->grid : nullptr, L ? L->cell_start : nullptr, L ? L->cell_items : nullptr,
       L ? L->cell_first : nullptr, L ? (const float*)L->recs : nullptr, L ? L->adj : nullptr,
-      L ? (const float*)L->vals : nullptr, p, b, fb, sf, counters, err);
+      L ? (const float*)L->vals : nullptr, p, b, fb, sf, counters);
   SFT_CUDA(cudaGetLastError());
   return SFT_OK;
 }
@@ -742,7 +739,6 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   p.key.k1 = (uint32_t)(o->seed >> 32);
   p.stream_id = o->stream_id;
   p.alpha = (float)o->alpha;
-  p.tau = so->tau;
   p.cdet = (float)(o->alpha / (double)((t->dim + 1) * (t->dim + 2)));
   p.cmc = (float)(1.0 / (double)N);
   p.st = strat_for(t->dim, N, o->sampling);
@@ -763,9 +759,9 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
     if (with_net)
       return t->dim == 2 ? net_pass<2>(net, t, q, g.p, b.p, fbp, sf, d_err, st)
                          : net_pass<3>(net, t, q, g.p, b.p, fbp, sf, d_err, st);
-    if (t->dim == 2) return launch_exact<2, 2>(exact, t, q, g.p, b.p, fbp, sf, counters, d_err, st);
-    if (ds == 2) return launch_exact<3, 2>(exact, t, q, g.p, b.p, fbp, sf, counters, d_err, st);
-    return launch_exact<3, 3>(exact, t, q, g.p, b.p, fbp, sf, counters, d_err, st);
+    if (t->dim == 2) return launch_exact<2, 2>(exact, t, q, g.p, b.p, fbp, sf, counters, st);
+    if (ds == 2) return launch_exact<3, 2>(exact, t, q, g.p, b.p, fbp, sf, counters, st);
+    return launch_exact<3, 3>(exact, t, q, g.p, b.p, fbp, sf, counters, st);
   };
   sft_status lr = SFT_OK;
   int64_t n_fallback = net ? 0 : ne;
@@ -838,7 +834,7 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   }
   SolveResult sr;
   SolveLate late(status.p->solve);  // the solve's status is read with the final readback
-  if (sft_status r = mass_solve(t, 1, b.p, u_dev, o->cg_tol, o->cg_max_iter, st, d_err, &sr, o->cg_mode, &late,
+  if (sft_status r = mass_solve(t, 1, b.p, u_dev, o->cg_tol, o->cg_max_iter, st, &sr, o->cg_mode, &late,
                                 o->cg_warm_start))
     return r;
   ev.record(4, st);
