@@ -196,8 +196,9 @@ sft_status sft_transfer(sft_source src, sft_target tgt, const sft_options* opt,
  * Sec. 3, Intersection-Based Galerkin Projection: every target triangle is
  * partitioned by the source triangles it overlaps (Eq. partition_ts); each
  * piece is clipped (Sutherland-Hodgman), split into a fan from its first
- * vertex and integrated with the edge-midpoint rule, exact for the products
- * of two functions linear on the piece; all arithmetic FP64. A target
+ * vertex and integrated from the values at the fan triangles' vertices, exact
+ * for the products of two functions linear on the piece; all arithmetic FP64
+ * (lengths from about 1e-150 to 1e150). A target
  * triangle's pieces are found by a walk over source face neighbours from
  * the source triangle holding its centroid (at most 256 source triangles
  * visited per target triangle, else SFT_ERR_UNSUPPORTED).
@@ -209,7 +210,8 @@ sft_status sft_transfer(sft_source src, sft_target tgt, const sft_options* opt,
  * out2[0] = ||f^s - f^t||_L2, out2[1] = ||f^s||_L2 (host array of 2).
  * Both need 2D meshes (SFT_ERR_UNSUPPORTED otherwise), return
  * SFT_ERR_OUTSIDE if a target centroid lies in no source triangle, and
- * synchronise `cuda_stream`. */
+ * synchronise `cuda_stream`. Work space of a call: 4 bytes per target triangle
+ * and up to 46 MB. */
 sft_status sft_mi_load_vector(sft_source src, sft_target tgt, int32_t field, double* b_out,
                               int32_t out_device, void* cuda_stream);
 sft_status sft_mi_l2_error(sft_source src, sft_target tgt, int32_t field, const double* u,
@@ -239,7 +241,9 @@ sft_status sft_locate(sft_source src, int32_t precision, int64_t n, const double
  * `cg_mode`. max_iter bounds the iterations (FP32 inner Chebyshev steps
  * summed over the refinement cycles in MIXED mode). iters_out / rel_resid_out (host,
  * may be NULL) get the worst field; rel_resid is the true FP64 residual of the
- * returned u in MIXED mode, the recurrence residual in FP64 mode. */
+ * returned u in MIXED mode, the recurrence residual in FP64 mode. The first
+ * MIXED solve on a target makes its scaled matrix, which the target keeps:
+ * 16 bytes per nonzero and 18 per node (130 MB at 1.0 M nodes in 2D). */
 sft_status sft_mass_solve(sft_target tgt, int32_t nrhs, const double* b, double* u,
                           int32_t device_ptrs, double tol, int32_t max_iter, int32_t cg_mode,
                           void* cuda_stream, int32_t* iters_out, double* rel_resid_out);
@@ -310,7 +314,7 @@ sft_status sft_batch_result(sft_batch b, int32_t req, double* u_out, double* b_o
 sft_status sft_batch_groups(sft_batch plan, int32_t* out);
 void sft_batch_destroy(sft_batch b);
 
-/* ---- learned surrogate source (spec item 4; no counterpart in the
+/* ---- learned surrogate source (no counterpart in the
  * paper beyond its motivation: black-box sources "such as machine-learned
  * surrogates") ----
  * Network x in R^3 -> 256 -> 256 -> 256 -> 256 -> 1, SiLU after each hidden
@@ -330,7 +334,8 @@ sft_status sft_mlp_forward(sft_mlp m, int64_t n, const float* pts, float* out, i
  * respect to every parameter (grad_out [nparam] FP32) and the loss value
  * (host double); all arrays device memory. Hand-written BF16 forward and
  * backward on the tensor cores (activations and activation gradients in
- * BF16, FP32 accumulation, FP32 gradient). */
+ * BF16, FP32 accumulation, FP32 gradient). Work space of a call: 393 kB per 128
+ * points, at most 280 MB. */
 sft_status sft_mlp_loss_grad(sft_mlp m, int64_t n, const float* pts, const float* targets, float* grad_out,
                              double* loss_out, int32_t device_ptrs, void* cuda_stream);
 /* Adam training (beta 0.9 / 0.999, eps 1e-8) on device data: `epochs` passes
@@ -401,7 +406,7 @@ typedef struct {
     int64_t fallback_elems;  /* elements that used exact queries */
     int64_t empty_queries;   /* exact queries that landed in an empty grid cell (value 0) */
     float ms_control;        /* step 1: control values at the target nodes */
-    float ms_assembly;       /* steps 2-6: fused sample / network / fallback / scatter kernel */
+    float ms_assembly;       /* steps 2-6: samples, network, fallback and scatter */
     float ms_solve;          /* step 7 */
     float ms_total;
 } sft_surrogate_stats;
@@ -415,7 +420,9 @@ typedef struct {
  * sft_transfer: u_out, b_out, g_out [nnodes] FP64, fallback_out and
  * sample_f_out host or device per opt->out_device. Samples are those of
  * sft_transfer with the same seed / stream_id / N (Philox counters of the
- * target dimension), so both paths see identical points. */
+ * target dimension), so both paths see identical points. The network pass
+ * works through chunks of at most 4 Mi samples (one element where N is more),
+ * with 16 bytes of work space per sample of a chunk. */
 sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target tgt, const sft_options* opt,
                                   const sft_surrogate_opts* sopt, double* u_out, double* b_out, double* g_out,
                                   sft_surrogate_stats* stats);

@@ -1,5 +1,5 @@
 /*
- * Oracle: the surrogate source network (spec item 4 reshaping the black
+ * Oracle: the surrogate source network (reshaping the black
  * box of Sec. 4 step 4 into a learned field) in plain FP64.
  * TEST INFRASTRUCTURE ONLY (see oracle.h).
  *

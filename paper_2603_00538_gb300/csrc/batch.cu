@@ -1424,12 +1424,14 @@ static sft_status build_batch(sft_batch_s* B, const sft_options* opts, int autot
   if (B->mixed) {
     // pieces: whole matrix rows of one request with all its fields, in
     // request order (so a request's systems are owned by consecutive
-    // blocks), an equal share of the estimated row cost per block. A row of
-    // a request with z matrix entries per row and nf fields costs about
-    // 8 z (its FP32 entries and columns, loaded once for all fields) +
-    // nf (44 + 4 z) (per field the CG vectors of the two FP32 phases and
-    // the z gathered entries of r): 3D rows (z ~ 15) cost about twice 2D
-    // rows (z ~ 7), and a field of an 8-field row 0.6 of a lone field.
+    // blocks), an equal share of the estimated row cost per block: 8 z +
+    // nf (44 + 4 z) for a row of z matrix entries and nf fields. The 8 z are
+    // its FP32 entries and columns, read once for all fields; the rest was
+    // fitted to a solve that kept four FP32 vectors and gathered every
+    // field's entries one by one. The steps now keep three and gather a
+    // row's fields together, so a field of a wide row costs less than this
+    // says and its blocks finish earlier; 3D rows (z ~ 15) remain about twice
+    // 2D rows (z ~ 7).
     std::vector<BPiece> hp;
     std::vector<int32_t> hbpc(B->nblocks + 1);
     std::vector<double> rcost(nreq, 0.0);

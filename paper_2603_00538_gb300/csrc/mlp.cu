@@ -1,4 +1,4 @@
-// The surrogate source network (spec item 4): a learned black-box
+// The surrogate source network: a learned black-box
 // field x in R^3 -> 256 -> 256 -> 256 -> 256 -> 1 with SiLU, BF16 weights of
 // the three 256x256 layers and BF16 hidden activations, FP32 accumulation.
 // The 256x256 layers run on the 5th-generation tensor cores (tcgen05.mma,
@@ -79,8 +79,9 @@ __global__ void __launch_bounds__(2 * kGroupThreads, 1) k_mlp_forward(const floa
 // ---------------------------------------------------------------------------
 constexpr int kTrainLayers = 6;
 constexpr int kTrainImages = 6;                 // h1, h2, h3, dz4, dz3, dz2
-constexpr int64_t kTrainTiles = 4 * 152;         // tiles per pass over the two kernels (240 MB of images; half as
-                                                // many: 313 us against 274 at 70,001 points)
+// tiles per pass over the two kernels: four a SM, 240 MB of images (half as many: 313 us against 274 at
+// 70,001 points). 77,824 points are one pass: 309 us a call, 78,000 two: 415, 100,000 426, 400,000 (six) 1,331
+constexpr int64_t kTrainTiles = 4 * 152;
 constexpr int kTrainSums = 8;                   // column sums: c1..c4, w5, W1 by input
 constexpr uint32_t kSmemTrain = kSmemFwd + kTrainSums * kH * 4 + 2 * kTileM * 4;
 static_assert(kSmemTrain <= 227u * 1024u, "training tile exceeds the shared memory of one CTA");

@@ -1,7 +1,8 @@
 // The surrogate source network: x in R^3 -> 256 -> 256 -> 256 -> 256 -> 1
 // with SiLU, BF16 weights of the three 256x256 layers and BF16 hidden
 // activations, FP32 accumulation in tensor memory. Device pieces shared by
-// the forward kernel, the training kernels and the fused surrogate assembly.
+// the forward kernel and the training kernels (the network pass of a surrogate
+// transfer runs the forward).
 //
 // Parameter vector (FP32, kNParam): W1 [256][3], c1 [256], W2 [256][256],
 // c2, W3, c3, W4, c4, w5 [256], c5 [1]; weights row-major [out][in].
@@ -110,7 +111,7 @@ constexpr int kChunkK = 64;                     // K of a ring chunk
 constexpr uint32_t kChunkBytes = kH * kChunkK * 2;
 constexpr int kChunks = kH / kChunkK;           // chunks per layer
 constexpr int kRing = 2;                        // chunk buffers
-constexpr int kGroupThreads = kTPR * kTileM;    // 512
+constexpr int kGroupThreads = kTPR * kTileM;    // 256
 constexpr uint32_t kSmemBars = 256;             // mbarriers, TMEM slot, failed flag, turn counters, stream state
 constexpr uint32_t kSmemYH = 2 * kTileM * 4;    // partial outputs of the column halves
 constexpr uint32_t kSmemFwd = 2 * kSmemA + kRing * kChunkBytes + kSmemW1 + kSmemBias + 2 * kSmemYH + kSmemBars;

@@ -563,9 +563,9 @@ constexpr int kMixThreads = NR <= 2 ? 1024 : 512;
 // grid), large ones the shared-memory loads and issue of the steps (12 us a
 // step at 1.0 M rows) and the FP64 pipe of the residual (38 us a cycle there
 // against 25 of pure FP64 work). Kernel time, before (grid of 4 blocks per SM
-// over CSR rows, all vectors in L2) and now: 1.0 M rows 2D 648 -> 431 us,
-// 0.51 M 3D 574 -> 429, 0.37 M 2D 350 -> 177, 10 k 2D 179 -> 62, 784 2D
-// 140 -> 46, 227 k 3D with 8 fields 1,739 -> 618.
+// over CSR rows, all vectors in L2) and now: 1.0 M rows 2D 648 -> 421 us,
+// 0.51 M 3D 574 -> 422, 0.37 M 2D 350 -> 176, 10 k 2D 179 -> 62, 784 2D
+// 140 -> 46, 227 k 3D with 8 fields 1,739 -> 615.
 template <int NR, int TEAM, bool OWN>
 __global__ void __launch_bounds__(kMixThreads<NR>, 1) k_mixed(const MixArgs a) {
   constexpr int T = kMixThreads<NR>, W = T / 32, V = 2 * NR;

@@ -375,7 +375,7 @@ __global__ void k_dataset(int64_t n, PhiloxKey key, uint32_t stream_id, float3 l
 }
 
 // The network pass (the elements that keep the network; no exact queries), in
-// chunks of at most kNetChunk samples: k_net_points forms the sample points
+// chunks of at most kNetChunk samples (one element where N is more): k_net_points forms the sample points
 // of the chunk's elements (Philox, map; the FP32 points of the assembly),
 // the standalone forward evaluates them, k_net_combine turns the values into
 // residuals and adds them into b. The points and values of a chunk (16 bytes a
@@ -719,7 +719,7 @@ sft_status sft_transfer_surrogate(sft_mlp net, sft_source exact, sft_target t, c
   }
   ev.record(2, st);
 
-  // steps 2-6: fused sample / network / fallback / scatter
+  // steps 2-6: sample / network / fallback / scatter
   SurParams p{};
   p.nv = nv;
   p.ne = ne;

@@ -3,10 +3,11 @@
 // quadrature gives the closed form |T| (1 + delta_ij) / ((d+1)(d+2)).
 //
 // CSR build without a global sort: node -> element incidence lists by a
-// counting sort (atomics + per-node insertion sort, ascending element id);
-// then one thread per row merges the vertices of its incident elements into a
-// sorted, de-duplicated column list, summing contributions in ascending
-// element order (deterministic values).
+// counting sort, each list put in ascending element order by ranks; then one
+// thread per row sums its incident elements in that order (deterministic
+// values) into a hash table in shared memory, whose columns are ordered once
+// at the end (k_mass_hash); rows too long for it, and all rows where the
+// staging arrays cannot be had, into an ordered list (k_mass_rows).
 #include <type_traits>
 #include <vector>
 #include "internal.hpp"

@@ -43,11 +43,12 @@ __device__ __forceinline__ T warp_inclusive_scan(T v, int lane) {
 // delta = (b - a) / 2, s1 = theta / delta.
 // From y0 = 0, r0 = c, d0 = c / theta, rho0 = 1 / s1, each step takes
 //   y += d, r -= A d, rho' = 1 / (2 s1 - rho), d' = rho' rho d + (2 rho' / delta) r
-// and leaves r_k = P_k(A) c with max |P_k| on [a, b] = 1 / T_k(s1) (the
+// (the solves run it on y alone, y_{k+1} from y_k and y_{k-1}) and leaves
+// r_k = P_k(A) c with max |P_k| on [a, b] = 1 / T_k(s1) (the
 // scaled Chebyshev polynomial of degree k; Saad, Iterative Methods for Sparse
 // Linear Systems, Sec. 12.3). So ||r_k|| <= eta ||c|| after
 // k = ceil(acosh(1 / eta) / acosh(s1)) steps: 12 for eta = 1e-5 on
-// triangles, 13 on tetrahedra.
+// triangles, 13 on tetrahedra (the single solve finds k from the T_k: solve.cu).
 struct ChebCoef {
   float theta, delta, s1;
 };
