@@ -331,6 +331,10 @@ __global__ void __launch_bounds__(2 * kGroupThreads, 1) k_train_tile(const Train
   }
 }
 
+// whether a bounded wait ended for all lanes of the warp (at the limit they may
+// differ: the warp leaves its loop as a whole or not at all)
+__device__ __forceinline__ bool warp_agrees(bool ok) { return __all_sync(0xffffffffu, ok); }
+
 // dW of square layer blockIdx.y (W2, W3, W4) over tiles blockIdx.x, + gridDim.x, ...
 constexpr int kDwRows = 32;                               // batch rows a stage
 constexpr uint32_t kDwHalf = kDwRows * kH * 2;            // 16 KiB: one operand's rows
