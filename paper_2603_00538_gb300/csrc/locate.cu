@@ -380,8 +380,9 @@ __device__ __forceinline__ bool cell_may_hold(const P* r, const P c[D], const P 
 //          with an atomic maximum of (depth, id);
 //   fill   from the masks alone, four registrations of an element in flight:
 //          the atomic on the cell's cursor returns the place.
-// Elements with more than kMaskCells box cells go to a list that a warp per
-// element takes after the others.
+// Elements with more box cells than their mask has bits go to a list that
+// k_register_big takes after the others. A mask is one word (MW = 1), or on fine
+// grids, where the boxes of ordinary elements are larger, up to kMaskWords.
 // (8-byte (id, depth) entries filled one at a time with the full test again,
 // and read back for the start elements, took 1.60 ms for the 68 M
 // registrations of a 5.0 M-tetrahedron source, 0.43 ms for 4.0 M triangles;
@@ -389,7 +390,8 @@ __device__ __forceinline__ bool cell_may_hold(const P* r, const P c[D], const P 
 // Sorting a block's registrations by cell in shared
 // memory, with one global atomic per block and cell, took 1.45 ms and 0.42:
 // the shared-memory atomics collide.)
-constexpr int kMaskCells = 64;
+constexpr int kMaskCells = 64;   // bits of a mask word
+constexpr int kMaskWords = 16;   // of an element at most
 constexpr int kRegThreads = 128;
 
 // best (depth, id) at a cell's centre so far: largest depth, lowest id
@@ -474,6 +476,29 @@ struct BoxFilter {
 #pragma unroll
     for (int a = 0; a < D; ++a) S += 0.5f * fabsf(col[a]);
   }
+  // coordinates beyond FP32's range for this leave all cells undecided
+  __device__ __forceinline__ bool sane(const float* gf, float mag) const {
+    bool ok = band < 1e30f && mag < 1e15f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) ok = ok && gf[a] > 1e-30f;
+#pragma unroll
+    for (int m = 0; m < D; ++m) ok = ok && fabsf(t0[m]) < 1e30f && sp[m] < 1e30f;
+    return ok;
+  }
+  // the filter that lane j of the warp holds
+  __device__ __forceinline__ BoxFilter from_lane(int j) const {
+    BoxFilter f;
+#pragma unroll
+    for (int m = 0; m < D; ++m) {
+      f.t0[m] = __shfl_sync(0xffffffffu, t0[m], j);
+      f.sp[m] = __shfl_sync(0xffffffffu, sp[m], j);
+#pragma unroll
+      for (int a = 0; a < D; ++a) f.st[m][a] = __shfl_sync(0xffffffffu, st[m][a], j);
+    }
+    f.S = __shfl_sync(0xffffffffu, S, j);
+    f.band = __shfl_sync(0xffffffffu, band, j);
+    return f;
+  }
   // cell at offset o[] of the box: 0 not held, 1 held and the centre outside,
   // 2 held and the centre perhaps inside, 3 undecided
   __device__ __forceinline__ int operator()(const float (&o)[3]) const {
@@ -498,20 +523,21 @@ struct BoxFilter {
   }
 };
 
-// an element's bounding-box cells: linear index of the first, nx | ny << 8
+// an element's bounding-box cells: linear index of the first, nx - 1 | ny - 1 << 10 |
+// words of its mask << 20
 struct ElemBox { int32_t lin0, dims; };
 
-template <int D, typename P>
+template <int D, typename P, int MW>
 __global__ void __launch_bounds__(kRegThreads)
     k_register_count(const P* __restrict__ x, const int32_t* __restrict__ conn, const P* __restrict__ recs, int64_t nv,
                      int64_t ne, const GridP<P>* __restrict__ gp, int32_t* __restrict__ cell_count,
                      FirstKey<P>* __restrict__ first, unsigned long long* __restrict__ mask, ElemBox* __restrict__ box,
-                     int32_t* __restrict__ big, int32_t* __restrict__ nbig) {
+                     int32_t* __restrict__ big, int32_t* __restrict__ nbig, int words) {
   constexpr int RL = RecLen<D>::value;
   constexpr int W = kRegThreads / 32;
-  __shared__ unsigned long long smask[kRegThreads];         // cells settled in P
-  __shared__ int32_t sbox[kRegThreads][4];                  // first box cell, nx | ny << 8
-  __shared__ uint16_t queue[W][64];                         // undecided << 11 | lane << 6 | k
+  __shared__ unsigned long long smask[MW][kRegThreads];     // cells settled in P
+  __shared__ int32_t sbox[kRegThreads][4];                  // first box cell, nx - 1 | ny - 1 << 10
+  __shared__ uint16_t queue[W][64];                         // undecided << 15 | lane << 10 | k
   __shared__ float gf[4];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const GridP<P> g = *gp;
@@ -541,7 +567,7 @@ __global__ void __launch_bounds__(kRegThreads)
     elem_vertices<D, P>(x, conn, e, xv);
     const int64_t nb = elem_cell_range<D, P>(g, xv, c0, c1);
     ok = c1[0] >= c0[0] && c1[1] >= c0[1] && c1[2] >= c0[2];  // (non-finite coordinates)
-    if (ok && nb > kMaskCells) {
+    if (ok && nb > (MW == 1 ? 1 : words) * kMaskCells) {
       big[atomicAdd(nbig, 1)] = (int32_t)e;
       ok = false;
     }
@@ -557,24 +583,20 @@ __global__ void __launch_bounds__(kRegThreads)
     const int nc[3] = {nx, ny, c1[2] - c0[2] + 1};
     filter.init(g, r, c0, gf, gf[3], nc);
   }
-  // coordinates beyond FP32's range for this leave all cells undecided
-  bool sane = ok && filter.band < 1e30f && gf[3] < 1e15f;
+  const bool sane = ok && filter.sane(gf, gf[3]);
 #pragma unroll
-  for (int a = 0; a < D; ++a) sane = sane && gf[a] > 1e-30f;
-#pragma unroll
-  for (int m = 0; m < D; ++m) sane = sane && fabsf(filter.t0[m]) < 1e30f && filter.sp[m] < 1e30f;
-  smask[t] = 0ull;
+  for (int w = 0; w < MW; ++w) smask[w][t] = 0ull;
   sbox[t][0] = c0[0];
   sbox[t][1] = c0[1];
   sbox[t][2] = c0[2];
-  sbox[t][3] = nx | ny << 8;
+  sbox[t][3] = (nx - 1) | (ny - 1) << 10;
   __syncwarp();
   // what a warp has to evaluate in P is gathered and taken 32 at a time
   auto settle = [&](int n) {
     __syncwarp();
     if (lane < n) {
-      const int q = queue[warp][lane], src = warp * 32 + (q >> 6 & 31), k = q & 63;
-      const int bx = sbox[src][3] & 255, by = sbox[src][3] >> 8;
+      const int q = queue[warp][lane], src = warp * 32 + (q >> 10 & 31), k = q & 1023;
+      const int bx = (sbox[src][3] & 1023) + 1, by = (sbox[src][3] >> 10) + 1;
       const int row = k / bx;
       const int32_t idx[3] = {sbox[src][0] + k - row * bx, sbox[src][1] + (D == 3 ? row % by : row),
                               sbox[src][2] + (D == 3 ? row / by : 0)};
@@ -585,13 +607,13 @@ __global__ void __launch_bounds__(kRegThreads)
       for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
       const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
       bool held = true;
-      if (q >> 11) {
+      if (q >> 15) {
         P w[D];
 #pragma unroll
         for (int a = 0; a < D; ++a) w[a] = Ar<P>::mul(g.h[a], P(0.5));
         held = cell_may_hold<D, P>(r2, cc, w);
         if (held) {
-          atomicOr(&smask[src], 1ull << k);
+          atomicOr(&smask[MW == 1 ? 0 : k >> 6][src], 1ull << (k & 63));
           atomicAdd(cell_count + c, 1);
         }
       }
@@ -613,13 +635,13 @@ __global__ void __launch_bounds__(kRegThreads)
     int res = sane ? filter(o) : 3;
     if (k >= nbox) res = 0;
     if (res == 1 || res == 2) {
-      bits |= 1ull << k;
+      bits |= 1ull << (MW == 1 ? k : k & 63);
       atomicAdd(cell_count + c, 1);
     }
     const uint32_t und = __ballot_sync(0xffffffffu, res >= 2);
     if (und != 0u) {
       if (res >= 2)
-        queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)((res == 3 ? 1 << 11 : 0) | lane << 6 | k);
+        queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)((res == 3 ? 1 << 15 : 0) | lane << 10 | k);
       qn += __popc(und);
       if (qn >= 32) {
         settle(32);
@@ -627,6 +649,11 @@ __global__ void __launch_bounds__(kRegThreads)
         if (lane < qn) queue[warp][lane] = queue[warp][32 + lane];
         __syncwarp();
       }
+    }
+    if (MW > 1 && (k & 63) == 63) {   // (the word is the warp's own: its lanes meet in settle)
+      smask[k >> 6][t] |= bits;
+      bits = 0ull;
+      __syncwarp();
     }
     o[0] += 1.f;
     ++c;
@@ -643,83 +670,238 @@ __global__ void __launch_bounds__(kRegThreads)
   }
   settle(qn);
   if (e >= ne) return;
-  mask[e] = bits | smask[t];
+  const int mine = (nbox + kMaskCells - 1) / kMaskCells;
+  if constexpr (MW == 1) {
+    mask[e] = bits | smask[0][t];
+  } else {
+    for (int w = 0; w < mine; ++w) mask[(int64_t)w * ne + e] = smask[w][t] | (w == kmax >> 6 ? bits : 0ull);
+  }
   box[e].lin0 = lin0;
-  box[e].dims = nx | ny << 8;
+  box[e].dims = (nx - 1) | (ny - 1) << 10 | mine << 20;
 }
 
-// the elements with large boxes: FILL = false counts them, true fills them
-// (cell_count then holds the cells' cursors)
+// The elements beyond their masks: FILL = false counts them, true fills them
+// (cell_count then holds the cells' cursors). A warp takes up to 32 of them:
+// each lane prepares the box of one (in FP64 also the filter), then the warp
+// goes through the boxes one after the other, 32 cells at a time. FP64 settles
+// by the filter in both passes what it can, and evaluates the rest in P 32 at a
+// time; FP32 evaluates every cell (its test costs less than the filter and what
+// follows from it: 162 k tetrahedra at L = 6, source build 3.26 ms, with the
+// filter 4.82). One element at a time with every cell in P and 64-bit indices
+// took 3.80 ms there in FP32 and 44.0 in FP64 (now 6.3), a thread per element
+// 5.20 and 85.8.
+constexpr int kBigThreads = 256;
+
+// Words of the masks at grid scale L: an element of a structured mesh takes about
+// (1.4 L + 1)^2 cells of a 2D grid, (1.8 L + 1)^3 of a 3D one. One word up to 60
+// cells of that (elements a little larger than most are then few), else twice the
+// cells, so that few elements are left for k_register_big. Source builds with one
+// word and the list / with the words / with 8-byte entries filled one at a time,
+// in ms: 2.06 M tetrahedra at L = 2 4.65 / 2.52 / 3.33, at L = 3 9.11 / 5.95 /
+// 7.86, in FP64 at L = 2 68.4 / 3.8 / 55.9; 2.0 M triangles at L = 6 4.79 / 3.52 /
+// 3.92, in FP64 43.2 / 5.54 / 25.8. Up to the line (L = 1.5 in 3D, 3 in 2D) most
+// elements need one word, and the two-word mask gains nothing.
+static int mask_words(int dim, double L) {
+  const double c = (dim == 2 ? 1.4 : 1.8) * L + 1.0, cells = dim == 2 ? c * c : c * c * c;
+  return cells <= 60.0 ? 1 : (int)std::fmin(kMaskWords, std::ceil(2.0 * cells / kMaskCells));
+}
+
 template <int D, typename P, bool FILL>
-__global__ void k_register_big(const P* __restrict__ x, const int32_t* __restrict__ conn, const P* __restrict__ recs,
-                               const GridP<P>* __restrict__ gp, const int32_t* __restrict__ big,
-                               const int32_t* __restrict__ nbig, int32_t* __restrict__ cell_count,
-                               FirstKey<P>* __restrict__ first, int32_t* __restrict__ items) {
+__global__ void __launch_bounds__(kBigThreads, D == 2 || sizeof(P) == 4 ? 3 : 2)
+    k_register_big(const P* __restrict__ x, const int32_t* __restrict__ conn, const P* __restrict__ recs,
+                   const GridP<P>* __restrict__ gp, const int32_t* __restrict__ big, const int32_t* __restrict__ nbig,
+                   int32_t* __restrict__ cell_count, FirstKey<P>* __restrict__ first, int32_t* __restrict__ items) {
   constexpr int RL = RecLen<D>::value;
+  constexpr uint32_t kAll = 0xffffffffu;
+  constexpr bool kFilter = sizeof(P) == 8;
+  __shared__ uint32_t queue[kFilter ? kBigThreads / 32 : 1][64];   // undecided << 31 | cell of the box
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nb = *nbig;
-  // a warp per element, its box cells over the lanes
-  const int lane = threadIdx.x & 31;
-  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb;
-       b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int32_t e = big[b];
-    const GridP<P> g = *gp;
-    P xv[D + 1][D];
-    elem_vertices<D, P>(x, conn, e, xv);
-    int32_t c0[3], c1[3];
-    const int64_t nbox = elem_cell_range<D, P>(g, xv, c0, c1);
-    P r[RL], w[D];
-    load_record<D, P>(recs, e, r);
+  const int nwarps = (int)gridDim.x * (kBigThreads / 32), wid = (int)blockIdx.x * (kBigThreads / 32) + warp;
+  const int per = min(32, (nb + nwarps - 1) / nwarps);   // elements a warp prepares together
+  if (nb == 0) return;
+  const GridP<P> g = *gp;
+  float gf[D], mag = 0.f;
 #pragma unroll
-    for (int a = 0; a < D; ++a) w[a] = Ar<P>::mul(g.h[a], P(0.5));
-    const int64_t nx = c1[0] - c0[0] + 1, ny = c1[1] - c0[1] + 1;
-    for (int64_t k = lane; k < nbox; k += 32) {
-      const int32_t idx[3] = {c0[0] + (int32_t)(k % nx), c0[1] + (int32_t)(k / nx % ny), c0[2] + (int32_t)(k / nx / ny)};
-      P cc[D];
+  for (int a = 0; a < D; ++a) {
+    gf[a] = (float)g.h[a];
+    mag = fmaxf(mag, fabsf((float)g.lo[a]) + fabsf((float)g.h[a]) * (float)g.n[a]);
+  }
+  for (int64_t b0 = (int64_t)wid * per; b0 < nb; b0 += (int64_t)nwarps * per) {
+    int32_t my_e = 0, my_c0[3] = {0, 0, 0}, my_nx = 1, my_ny = 1;
+    int64_t my_box = 0;
+    bool my_sane = false;
+    BoxFilter<D, P> mine;
+    if (lane < per && b0 + lane < nb) {
+      my_e = big[b0 + lane];
+      P xv[D + 1][D];
+      elem_vertices<D, P>(x, conn, my_e, xv);
+      int32_t c1[3];
+      my_box = elem_cell_range<D, P>(g, xv, my_c0, c1);
+      my_nx = c1[0] - my_c0[0] + 1;
+      my_ny = c1[1] - my_c0[1] + 1;
+      if constexpr (kFilter) {
+        P r[RL];
+        load_record<D, P>(recs, my_e, r);
+        const int nc[3] = {my_nx, my_ny, c1[2] - my_c0[2] + 1};
+        mine.init(g, r, my_c0, gf, mag, nc);
+        my_sane = mine.sane(gf, mag);
+      }
+    }
+    const int m = min((int64_t)per, nb - b0);
+    for (int j = 0; j < m; ++j) {
+      const int32_t e = __shfl_sync(kAll, my_e, j);
+      const int nx = __shfl_sync(kAll, my_nx, j), ny = __shfl_sync(kAll, my_ny, j);
+      const int64_t nbox = __shfl_sync(kAll, my_box, j);
+      int32_t c0[3];
 #pragma unroll
-      for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
-      if (!cell_may_hold<D, P>(r, cc, w)) continue;
-      const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
-      if (FILL) {
-        items[atomicAdd(cell_count + c, 1)] = e;
+      for (int a = 0; a < 3; ++a) c0[a] = __shfl_sync(kAll, my_c0[a], j);
+      bool sane = false;
+      BoxFilter<D, P> filter;
+      P r[RL];
+      if constexpr (kFilter) {
+        sane = __shfl_sync(kAll, (int)my_sane, j) != 0;
+        filter = mine.from_lane(j);
       } else {
-        atomicAdd(cell_count + c, 1);
-        const P depth = centre_depth<D, P>(r, cc);
-        if (depth >= P(0)) first_offer(first + c, depth, e);
+        load_record<D, P>(recs, e, r);
+      }
+      // a cell of the box in P: held? and its centre's depth
+      auto place = [&](int ox, int oy, int oz) { return ((c0[2] + oz) * g.n[1] + c0[1] + oy) * g.n[0] + c0[0] + ox; };
+      auto in_p = [&](int ox, int oy, int oz, bool test, P& depth) {
+        const int32_t idx[3] = {c0[0] + ox, c0[1] + oy, c0[2] + oz};
+        P cc[D], w[D];
+        if constexpr (kFilter) load_record<D, P>(recs, e, r);
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          cc[a] = cell_centre<P>(g, a, idx[a]);
+          w[a] = Ar<P>::mul(g.h[a], P(0.5));
+        }
+        if (test && !cell_may_hold<D, P>(r, cc, w)) return false;
+        if (!FILL) depth = centre_depth<D, P>(r, cc);
+        return true;
+      };
+      auto settle = [&](int n) {
+        __syncwarp();
+        if (lane < n) {
+          const uint32_t q = queue[warp][lane], k = q & 0x7fffffffu, row = k / (uint32_t)nx;
+          const int ox = (int)(k - row * (uint32_t)nx), oz = (int)(row / (uint32_t)ny), oy = (int)row - oz * ny;
+          P depth;
+          if (in_p(ox, oy, oz, q >> 31, depth)) {
+            const int32_t c = place(ox, oy, oz);
+            if (q >> 31) atomicAdd(cell_count + c, 1);
+            if (depth >= P(0)) first_offer(first + c, depth, e);
+          }
+        }
+        __syncwarp();
+      };
+      // the lane's first cell, and 32 cells on, by axis
+      int ox = lane % nx, oy = lane / nx % ny, oz = lane / nx / ny;
+      const int dx = 32 % nx, dy = 32 / nx % ny, dz = 32 / nx / ny;
+      auto decide = [&](int64_t k) {
+        const float o[3] = {(float)ox, (float)oy, (float)oz};
+        return k >= nbox ? 0 : kFilter && sane ? filter(o) : 3;
+      };
+      auto step = [&] {
+        ox += dx;
+        oy += dy;
+        oz += dz;
+        if (ox >= nx) {
+          ox -= nx;
+          ++oy;
+        }
+        if (oy >= ny) {
+          oy -= ny;
+          ++oz;
+        }
+      };
+      if constexpr (FILL) {
+        constexpr int U = 4;   // cells of a lane in flight
+        for (int64_t k0 = lane; k0 - lane < nbox; k0 += 32 * U) {
+          int32_t* at[U];
+          int32_t pos[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int res = decide(k0 + 32 * u);
+            P none;
+            at[u] = res == 1 || res == 2 || (res == 3 && in_p(ox, oy, oz, true, none)) ? cell_count + place(ox, oy, oz)
+                                                                                       : nullptr;
+            step();
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (at[u]) pos[u] = atomicAdd(at[u], 1);
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (at[u]) items[pos[u]] = e;
+        }
+      } else if constexpr (!kFilter) {
+        for (int64_t k = lane; k < nbox; k += 32) {
+          P depth;
+          if (in_p(ox, oy, oz, true, depth)) {
+            const int32_t c = place(ox, oy, oz);
+            atomicAdd(cell_count + c, 1);
+            if (depth >= P(0)) first_offer(first + c, depth, e);
+          }
+          step();
+        }
+      } else {
+        int qn = 0;
+        for (int64_t k0 = 0; k0 < nbox; k0 += 32) {
+          const int res = decide(k0 + lane);
+          if (res == 1 || res == 2) atomicAdd(cell_count + place(ox, oy, oz), 1);
+          const uint32_t und = __ballot_sync(kAll, res >= 2);
+          if (und != 0u) {
+            if (res >= 2)
+              queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (res == 3 ? 0x80000000u : 0u) | (uint32_t)(k0 + lane);
+            qn += __popc(und);
+            if (qn >= 32) {
+              settle(32);
+              qn -= 32;
+              if (lane < qn) queue[warp][lane] = queue[warp][32 + lane];
+              __syncwarp();
+            }
+          }
+          step();
+        }
+        settle(qn);
       }
     }
   }
 }
 
 // cursor: place of each cell's next registration (its start before the first)
-template <int D>
+template <int D, int MW>
 __global__ void k_register_fill(int64_t ne, int32_t gnx, int32_t gny, const unsigned long long* __restrict__ mask,
                                 const ElemBox* __restrict__ box, int32_t* __restrict__ cursor, int32_t* __restrict__ items) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
-    unsigned long long rest = __ldg(mask + e);
     const int2 bx = __ldg(reinterpret_cast<const int2*>(box) + e);
-    const uint32_t nx = bx.y & 255, ny = bx.y >> 8;
-    // division of k < 64 by n <= 64 as (k * ceil(2^16 / n)) >> 16: exact
-    const uint32_t inx = (65535u + nx) / nx, iny = D == 3 ? (65535u + ny) / ny : 0u;
-    while (rest != 0ull) {
-      constexpr int U = 4;
-      int32_t* at[U];
-      int32_t pos[U];
+    const uint32_t nx = (bx.y & 1023) + 1, ny = (bx.y >> 10 & 1023) + 1;
+    const int words = bx.y >> 20;
+    // division of k < 1024 by n <= 1024 as (k * ceil(2^20 / n)) >> 20: exact
+    const uint32_t inx = (1048575u + nx) / nx, iny = D == 3 ? (1048575u + ny) / ny : 0u;
+    for (int w = 0; w < (MW == 1 ? 1 : words); ++w) {
+      unsigned long long rest = MW == 1 || words > w ? __ldg(mask + (int64_t)w * ne + e) : 0ull;
+      while (rest != 0ull) {
+        constexpr int U = 4;
+        int32_t* at[U];
+        int32_t pos[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        at[u] = nullptr;
-        if (rest != 0ull) {
-          const uint32_t k = (uint32_t)__ffsll((long long)rest) - 1u;
-          rest &= rest - 1ull;
-          const uint32_t row = (k * inx) >> 16, lay = D == 3 ? (row * iny) >> 16 : 0u;
-          at[u] = cursor + (bx.x + (int32_t)(k - row * nx) + gnx * (int32_t)(row - lay * ny + gny * lay));
+        for (int u = 0; u < U; ++u) {
+          at[u] = nullptr;
+          if (rest != 0ull) {
+            const uint32_t k = (uint32_t)(w * kMaskCells) + (uint32_t)__ffsll((long long)rest) - 1u;
+            rest &= rest - 1ull;
+            const uint32_t row = (k * inx) >> 20, lay = D == 3 ? (row * iny) >> 20 : 0u;
+            at[u] = cursor + (bx.x + (int32_t)(k - row * nx) + gnx * (int32_t)(row - lay * ny + gny * lay));
+          }
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (at[u]) pos[u] = atomicAdd(at[u], 1);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (at[u]) items[pos[u]] = (int32_t)e;
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (at[u]) pos[u] = atomicAdd(at[u], 1);
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (at[u]) items[pos[u]] = (int32_t)e;
     }
   }
 }
@@ -893,7 +1075,8 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
   const size_t o_count = lay.add(sizeof(int32_t) * (size_t)L.ncells);
   const size_t o_key = lay.add(sizeof(FirstKey<P>) * (size_t)L.ncells);
   const size_t o_nbig = lay.add(sizeof(int32_t)), zeroed = lay.total;
-  const size_t o_mask = lay.add(sizeof(unsigned long long) * (size_t)s->ne);
+  const int mw = mask_words(D, s->L);
+  const size_t o_mask = lay.add(sizeof(unsigned long long) * (size_t)s->ne * mw);
   const size_t o_box = lay.add(sizeof(ElemBox) * (size_t)s->ne);
   const size_t o_big = lay.add(sizeof(int32_t) * (size_t)s->ne);
   SFT_CUDA(ws.alloc(lay.total));
@@ -906,10 +1089,10 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
   const unsigned reg_blocks = (unsigned)((s->ne + kRegThreads - 1) / kRegThreads);
   constexpr unsigned kBigBlocks = 152 * 4;
   SFT_CUDA(cudaMemsetAsync(ws.p, 0, zeroed, st));
-  ::sft::note_launch(), k_register_count<D, P><<<reg_blocks, kRegThreads, 0, st>>>(xP, s->conn, recs, s->nv, s->ne, g, count,
-                                                                                  key, mask, box, big, nbig);
+  ::sft::note_launch(), (mw == 1 ? k_register_count<D, P, 1> : k_register_count<D, P, kMaskWords>)<<<reg_blocks, kRegThreads, 0, st>>>(
+      xP, s->conn, recs, s->nv, s->ne, g, count, key, mask, box, big, nbig, mw);
   SFT_CUDA(cudaGetLastError());
-  ::sft::note_launch(), k_register_big<D, P, false><<<kBigBlocks, 256, 0, st>>>(xP, s->conn, recs, g, big, nbig, count, key,
+  ::sft::note_launch(), k_register_big<D, P, false><<<kBigBlocks, kBigThreads, 0, st>>>(xP, s->conn, recs, g, big, nbig, count, key,
                                                                               nullptr);
   SFT_CUDA(cudaGetLastError());
   SFT_CUDA(exclusive_scan_i32_to_i64(count, start64.p, L.ncells, st));
@@ -930,10 +1113,10 @@ static sft_status build_locator_t(sft_source_s* s, int prec, cudaStream_t st, in
   // fill (arbitrary order within a cell), then each cell's start element
   SFT_CUDA(dalloc(&L.cell_items, (size_t)total, st));
   SFT_CUDA(cudaMemcpyAsync(count, L.cell_start, sizeof(int32_t) * (size_t)L.ncells, cudaMemcpyDeviceToDevice, st));
-  ::sft::note_launch(), k_register_fill<D><<<grid_for(s->ne), 256, 0, st>>>(s->ne, L.n[0], L.n[1], mask, box, count,
-                                                                          L.cell_items);
+  ::sft::note_launch(), (mw == 1 ? k_register_fill<D, 1> : k_register_fill<D, kMaskWords>)<<<grid_for(s->ne), 256, 0, st>>>(
+      s->ne, L.n[0], L.n[1], mask, box, count, L.cell_items);
   SFT_CUDA(cudaGetLastError());
-  ::sft::note_launch(), k_register_big<D, P, true><<<kBigBlocks, 256, 0, st>>>(xP, s->conn, recs, g, big, nbig, count, key,
+  ::sft::note_launch(), k_register_big<D, P, true><<<kBigBlocks, kBigThreads, 0, st>>>(xP, s->conn, recs, g, big, nbig, count, key,
                                                                              L.cell_items);
   SFT_CUDA(cudaGetLastError());
   SFT_CUDA(dalloc(&L.cell_first, (size_t)L.ncells, st));
