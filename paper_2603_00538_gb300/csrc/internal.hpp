@@ -98,16 +98,24 @@ struct CallStatus {
   alignas(16) unsigned char solve[256];  // the solve's control block (solve.cu)
 };
 
-// Host resources of one call: timing events and a page-locked copy of the
-// status words (a copy to pageable memory costs the call some 10 us more).
+// What a call reads back: its status words, or sums of fields and the partial
+// sums of a weighted sum
+constexpr unsigned kWsumBlocks = 304;
+struct CallHost {
+  CallStatus status;
+  double sums[kMaxFields + kWsumBlocks];
+};
+
+// Host resources of one call: timing events and page-locked memory for what it
+// reads back (a copy to pageable memory costs the call some 10 us more).
 // Kits are lent out for the length of a call, one caller at a time, and at
 // most kMaxKits idle ones per process are kept (util.cu); sft_trim_memory
 // frees those.
 struct CallKit {
   int dev = 0;
   cudaEvent_t e[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  CallStatus* host = nullptr;  // page-locked, or &own
-  CallStatus own;
+  CallHost* host = nullptr;  // page-locked, or &own
+  CallHost own;
   bool timing = false;
 };
 CallKit* kit_acquire();
@@ -120,7 +128,8 @@ struct Events {
   ~Events() { kit_release(kit); }
   Events(const Events&) = delete;
   Events& operator=(const Events&) = delete;
-  CallStatus& host() { return *kit->host; }
+  CallStatus& host() { return kit->host->status; }
+  double* sums() { return kit->host->sums; }
   void record(int i, cudaStream_t st) {
     if (ok) cudaEventRecord(kit->e[i], st);
   }
@@ -202,12 +211,11 @@ sft_status build_locator(sft_source_s* s, int prec, cudaStream_t st, int32_t* d_
 sft_status locate_points(sft_source_s* s, int prec, int64_t n, const void* pts, int pts_are_double,
                          int32_t* elem_out, void* val_out, int val_is_double, int64_t val_stride,
                          int64_t* d_counters, cudaStream_t st, int nf_out = -1, void* mu_out = nullptr);
-// integrals of every source field and a weighted sum: per-block partials
-// ([kIntegralBlocks][kMaxFields], [kWsumBlocks]) and their final sums in a
-// fixed order (out[0 .. kMaxFields - 1] the fields, out[kMaxFields] the sum)
+// integrals of every source field: per-block partials
+// [kIntegralBlocks][kMaxFields] and their sums by field in a fixed order
 constexpr unsigned kIntegralBlocks = 152 * 8;
 sft_status source_integrals_launch(sft_source_s* s, double* part, cudaStream_t st);
-sft_status final_sums_launch(const double* part, int nf, const double* wpart, int n_w, double* out, cudaStream_t st);
+sft_status final_sums_launch(const double* part, int nf, double* out, cudaStream_t st);
 sft_status refresh_value_copies(sft_source_s* s, cudaStream_t st);
 // target.cu
 sft_status build_target(sft_target_s* t, cudaStream_t st, int32_t* d_err);
@@ -253,7 +261,7 @@ sft_status mass_solve(sft_target_s* t, int nrhs, const double* b, double* x, dou
                       SolveLate* late = nullptr, int warm = 0);
 // S = diag(M)^-1/2 and the jagged diagonals of M and S M S on the target (made once, kept)
 sft_status scaled_slices(sft_target_s* t, cudaStream_t st);
-constexpr unsigned kWsumBlocks = 304;
+// kWsumBlocks partial sums of w u, added by the caller in their order
 sft_status weighted_sum_launch(const double* w, const double* u, int64_t n, double* part, cudaStream_t st);
 // conversions
 sft_status convert_coords(const void* in, int in_dtype, void* out, int out_prec, int64_t n, cudaStream_t st);

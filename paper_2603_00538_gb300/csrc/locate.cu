@@ -1364,23 +1364,19 @@ sft_status source_integrals_launch(sft_source_s* s, double* part, cudaStream_t s
   return SFT_OK;
 }
 
-// Final sums in a fixed order: warp f < nf adds field f's partials, warp
-// kMaxFields the n_w partials of a weighted sum, into out[0 .. kMaxFields]
-__global__ void __launch_bounds__(32 * (kMaxFields + 1)) k_final_sums(const double* __restrict__ part, int nf,
-                                                                     const double* __restrict__ wpart, int n_w,
-                                                                     double* __restrict__ out) {
+// Sums of the partials in a fixed order: warp f < nf adds field f's into out[f]
+__global__ void __launch_bounds__(32 * kMaxFields) k_final_sums(const double* __restrict__ part, int nf,
+                                                               double* __restrict__ out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp >= nf) return;
   double s = 0.0;
-  if (warp < nf)
-    for (unsigned k = lane; k < kIntegralBlocks; k += 32) s += part[(int64_t)k * kMaxFields + warp];
-  if (warp == kMaxFields)
-    for (int k = lane; k < n_w; k += 32) s += wpart[k];
+  for (unsigned k = lane; k < kIntegralBlocks; k += 32) s += part[(int64_t)k * kMaxFields + warp];
   s = warp_sum<double>(s);
   if (lane == 0) out[warp] = s;
 }
 
-sft_status final_sums_launch(const double* part, int nf, const double* wpart, int n_w, double* out, cudaStream_t st) {
-  ::sft::note_launch(), k_final_sums<<<1, 32 * (kMaxFields + 1), 0, st>>>(part, nf, wpart, n_w, out);
+sft_status final_sums_launch(const double* part, int nf, double* out, cudaStream_t st) {
+  ::sft::note_launch(), k_final_sums<<<1, 32 * kMaxFields, 0, st>>>(part, nf, out);
   SFT_CUDA(cudaGetLastError());
   return SFT_OK;
 }

@@ -73,7 +73,7 @@ CallKit* kit_acquire() {
   k->timing = true;
   for (auto& x : k->e) k->timing = k->timing && cudaEventCreate(&x) == cudaSuccess;
   void* p = nullptr;
-  k->host = cudaMallocHost(&p, sizeof(CallStatus)) == cudaSuccess ? (CallStatus*)p : &k->own;
+  k->host = cudaMallocHost(&p, sizeof(CallHost)) == cudaSuccess ? (CallHost*)p : &k->own;
   cudaGetLastError();
   return k;
 }
