@@ -537,7 +537,8 @@ __global__ void __launch_bounds__(kRegThreads)
   constexpr int W = kRegThreads / 32;
   __shared__ unsigned long long smask[MW][kRegThreads];     // cells settled in P
   __shared__ int32_t sbox[kRegThreads][4];                  // first box cell, nx - 1 | ny - 1 << 10
-  __shared__ uint16_t queue[W][64];                         // undecided << 15 | lane << 10 | k
+  constexpr int kB = MW == 1 ? 6 : 10;                      // bits of k
+  __shared__ uint16_t queue[W][64];                         // undecided << (kB + 5) | lane << kB | k
   __shared__ float gf[4];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const GridP<P> g = *gp;
@@ -595,7 +596,7 @@ __global__ void __launch_bounds__(kRegThreads)
   auto settle = [&](int n) {
     __syncwarp();
     if (lane < n) {
-      const int q = queue[warp][lane], src = warp * 32 + (q >> 10 & 31), k = q & 1023;
+      const int q = queue[warp][lane], src = warp * 32 + (q >> kB & 31), k = q & ((1 << kB) - 1);
       const int bx = (sbox[src][3] & 1023) + 1, by = (sbox[src][3] >> 10) + 1;
       const int row = k / bx;
       const int32_t idx[3] = {sbox[src][0] + k - row * bx, sbox[src][1] + (D == 3 ? row % by : row),
@@ -607,7 +608,7 @@ __global__ void __launch_bounds__(kRegThreads)
       for (int a = 0; a < D; ++a) cc[a] = cell_centre<P>(g, a, idx[a]);
       const int64_t c = ((int64_t)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
       bool held = true;
-      if (q >> 15) {
+      if (q >> (kB + 5)) {
         P w[D];
 #pragma unroll
         for (int a = 0; a < D; ++a) w[a] = Ar<P>::mul(g.h[a], P(0.5));
@@ -641,7 +642,7 @@ __global__ void __launch_bounds__(kRegThreads)
     const uint32_t und = __ballot_sync(0xffffffffu, res >= 2);
     if (und != 0u) {
       if (res >= 2)
-        queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)((res == 3 ? 1 << 15 : 0) | lane << 10 | k);
+        queue[warp][qn + __popc(und & ((1u << lane) - 1u))] = (uint16_t)((res == 3 ? 1 << (kB + 5) : 0) | lane << kB | k);
       qn += __popc(und);
       if (qn >= 32) {
         settle(32);
